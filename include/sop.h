@@ -180,9 +180,9 @@ int sop_channel_norms_static(const float* X_dev, long long T, long long K, long 
  *   candidate in neither mask is absent: every table entry that involves it is marked undefined and
  *   its shift is reported as 0.  The masks must be disjoint and not both empty.  At most 8 distinct
  *   tables may be evaluated per call (an atom and its negation share one).  The lookup tables of the
- *   evaluated candidates live in shared memory; when a fine-grained alphabet would not fit beside the
- *   staging tile, the lookup grid is coarsened and the tables that then share a cell between thresholds are
- *   searched exactly instead (slower, same results): no alphabet within the limits above is refused for size.
+ *   evaluated candidates live in shared memory; when a large alphabet would not fit, the lookup grid is coarsened,
+ *   and candidates with more than three decision points in one cell are searched exactly instead (slower, same
+ *   results): no alphabet within the limits above is refused for size.
  * flags: SOP_SEARCH_SINGLES_ONLY fills only the diagonal (and best_single): enough to choose the
  *   primary codebook FMTa before the Lloyd refinement.  SOP_SEARCH_SELECT_MSE (paragraph "Pair-search
  *   design axes", axis ii): in every two-way and signed entry the block goes to the candidate with the

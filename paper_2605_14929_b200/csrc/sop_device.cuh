@@ -3,6 +3,7 @@
 // is one IEEE-754 operation rounded to nearest even and reproducible bit for bit.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -163,6 +164,24 @@ __device__ __forceinline__ float fp_quantize(float u) {
   const float magic = __uint_as_float(max(__float_as_uint(au) & 0x7F800000u, (uint32_t)min_eb << 23) + (20u << 23));
   const float q = __fsub_rn(__fadd_rn(au, magic), magic);
   return __uint_as_float(__float_as_uint(q) | (__float_as_uint(u) & 0x80000000u));
+}
+
+// The same for two values at once through the conversion instructions of the two formats (round to nearest even, saturating,
+// sign of zero kept; every E2M3 and E4M3 value is an fp16 number): fp_quantize<KIND> and fp_code<KIND> of x and y, compared for
+// every finite fp32 pattern.  The codes come back as bytes, x in the lower one.
+template <int KIND>
+__device__ __forceinline__ float2 fp_quantize2(float x, float y, uint32_t& codes) {
+  unsigned short c;
+  uint32_t h;
+  if (KIND == SOP_KIND_FP_E2M3) {
+    asm("cvt.rn.satfinite.e2m3x2.f32 %0, %1, %2;" : "=h"(c) : "f"(y), "f"(x));
+    asm("cvt.rn.f16x2.e2m3x2 %0, %1;" : "=r"(h) : "h"(c));
+  } else {
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(c) : "f"(y), "f"(x));
+    asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h) : "h"(c));
+  }
+  codes = c;
+  return __half22float2(*reinterpret_cast<const __half2*>(&h));
 }
 
 // Element grid given by parameters (SOP_KIND_FP_GRID): min_eb = biased fp32 exponent of the smallest normal

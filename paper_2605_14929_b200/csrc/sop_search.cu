@@ -6,10 +6,12 @@
 //                    histogram and the layer power-of-two scale for "^0" candidates.
 //   kselect_kernel   that last step alone: the shifts of another scale format from the histogram a prepass of the
 //                    same layer left in the workspace (SOP_SEARCH_REUSE_PREPASS).
-//   sweep_kernel     persistent, one thread per 16-element block: evaluates every candidate of the call
-//                    in registers (cell-table lookup of the reconstruction value, packed f32x2
-//                    fused multiply-adds for the block metric, fixed quad-tree order) and writes
-//                    the per-block cosine and squared error of each as one column.          (ALU-bound)
+//   sweep_kernel     persistent, one thread per 16-element block: evaluates every candidate of the call.  Table candidates of
+//                    one class are evaluated together (up to eight: a "group"): their decision points are merged, an element
+//                    looks up the interval it lies in once and reads all eight reconstruction values as one row of shared
+//                    memory; packed f32x2 multiply-adds form the block metric in the fixed quad-tree order.  Element formats
+//                    go through the conversion instructions.  Writes the per-block cosine and squared error of each candidate
+//                    as one column.                                          (bound by register operands and issue)
 //   reduce_kernel    reads the columns of every candidate present in the call (those just written
 //                    and those an earlier call wrote) tile by tile into shared memory and forms
 //                    the table entries: a warp owns a few "tasks" (one anchor column against up to
@@ -26,17 +28,15 @@
 
 namespace sop {
 
-constexpr int TB = 512;             // threads per CTA of the sweep kernel
+constexpr int TB = 512;             // threads per CTA of the sweep kernel (one CTA per SM; two where it has no table candidates)
 constexpr int MAX_SLOTS = 192;      // pair slots per call: 16 singles + 120 pairs + 36 signed < 192
 constexpr int MAX_GRID = 1024;
 constexpr float MAGIC = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
 
-struct CandDev { unsigned char cls, kind, neg, table; };
+struct CandDev { unsigned char cls, kind, neg, pad; };
 struct ClassDev {
   float tmax;
-  float invh;        // cells per unit of u (a power of two)
   int scope, kind;   // kind of the quantiser: LUT, E2M3, E4M3
-  int c_half;        // table rows = 2 * c_half + 1
   int auto_k;        // 1: k* from the histogram
   int n_cand;                            // candidates evaluated in this call
   unsigned char cand[SOP_MAX_ATOMS];
@@ -44,6 +44,16 @@ struct ClassDev {
   unsigned char mem[SOP_MAX_ATOMS];
   int k_src;                             // candidate whose shift an earlier result holds (k from result), or -1
   GridDev grid;                          // kind SOP_KIND_FP_GRID: the grid's parameters
+};
+// Up to eight table candidates of one class that the sweep evaluates together (see build_group): their joint rows and the
+// cell grid that finds the row of a scaled value.
+constexpr int GROUP_CAND = 8;
+struct GroupDev {
+  unsigned char cls, n, np, pad;             // n candidates in np pairs (an odd one is paired with itself)
+  unsigned char cand[GROUP_CAND];
+  unsigned row_off, cell_off, plane_bytes;   // shared-memory offsets; bytes of the rows of two pairs of candidates
+  int n_cells;                               // cells 0 .. n_cells
+  float inv_range;                           // cell = rint(n_cells * saturate(u * inv_range + 1/2))
 };
 struct SlotDev { unsigned char type, i0, i1, pad; };  // type 0: pair (i0, i1) (i0 == i1: single); 1: signed (i0, i0+1, i1, i1+1)
 
@@ -70,19 +80,15 @@ struct SeatsDev {
 };
 
 struct Plan {
-  int n_atoms, n_classes, n_tables, n_slots, n_pair_slots;
-  int k_mode, rows, a_pad;
+  int n_atoms, n_classes, n_groups, n_slots, n_pair_slots;
+  int k_mode;
   unsigned eval_mask, load_mask;   // candidates evaluated here / read from the per-block arrays of an earlier call
   int k_from_result;               // 1: shifts and max|W| come from the result block of an earlier call, no prepass
   int n_bases;                               // base atoms (each followed by its negation) of the signed table
   unsigned char base_atom[SOP_MAX_ATOMS];    // signed-best column n_atoms + b holds the better of base_atom[b] and its negation
   CandDev cand[SOP_MAX_ATOMS];
   ClassDev cls[SOP_MAX_CLASSES];
-  unsigned char table_atom[SOP_MAX_TABLES];   // atom whose lut fills the table
-  unsigned char table_cls[SOP_MAX_TABLES];
-  unsigned char table_pos[SOP_MAX_TABLES];    // candidate that uses the table as it is (255: none)
-  unsigned char table_neg[SOP_MAX_TABLES];    // candidate that uses the negated table (255: none)
-  unsigned char cls_tables[SOP_MAX_CLASSES];  // bit t: table t belongs to the class
+  GroupDev groups[SOP_MAX_CLASSES];
   SlotDev slots[MAX_SLOTS];
   int keep_loaded;                            // entries among loaded candidates stay as the tables hold them
   int n_tasks;
@@ -120,6 +126,8 @@ __device__ __forceinline__ void load_block_bits(const uint16_t* p, uint32_t (&v)
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
   v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
+
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ float absmax_bits(const uint32_t (&v)[8]) {
   // bf16 magnitudes order like their bit patterns: the maximum of the sixteen 15-bit patterns, two per word at a time
@@ -242,191 +250,543 @@ __device__ void kselect_body(const Plan& P, const FmtDev& F, const unsigned* his
 }
 
 // ---------------------------------------------------------------------------------------------
-// Phase-1 evaluators.  Element layout inside a thread: index idx = 2 * i + p holds, as a float2,
-// element i of quads 2p (x) and 2p + 1 (y): the two lanes of a packed f32x2 operation are two
-// independent sequential chains, which is exactly the quad-tree summation order.
+// Evaluators of the sweep.
+//
+// Table candidates.  The candidates of one class see the same scaled value u of an element, so the decision points of up to
+// eight of them (a "group") are merged into one ascending list: between two neighbouring points every candidate's nearest
+// entry is fixed, and the eight values of that interval form one row.  Finding the row (a cell of a uniform grid on u, then
+// at most three comparisons) and loading it is then paid once per element instead of once per element and candidate, and no
+// candidate needs a comparison, a selection or an unpacking of its own: what remains per candidate are the five products and
+// sums of its metric, as packed f32x2 operations whose two lanes are two candidates.
+// What bounds it: the packed operations read six registers each, and the register file, not the FMA units, limits them (3.2
+// cycles each where the units would take 2); the metric of eight candidates alone takes 900 of the 1640 cycles that a warp
+// spends on 32 blocks.  More resident warps do not help (256, 384 and 512 threads per SM take the same time).  8192 x 8192 at
+// E5M6, eight candidates: 188 us (310 us with a lookup, a comparison and a selection per element and candidate); two
+// candidates: 85 us (127 us).
 // ---------------------------------------------------------------------------------------------
-struct BlockRegs {
-  float2 w[8], c[8], u[8];
-  unsigned off[16]; // byte offset of the element's cell row: row * (n_tables * 128) + (lane & 15) * 8; table t adds t * 128
+constexpr int SLOW_STEPS = 8;                        // a binary search over at most 255 decision points
+
+// Shared-memory scratch: while the tables are built, the candidates' values and decision points; for the sweep the merged
+// decision points (for a group that is searched).
+struct __align__(16) ColumnPtr { char *cos, *sse; };      // a candidate's columns
+struct GroupScratch {
+  ColumnPtr col[SOP_MAX_CLASSES][GROUP_CAND];
+  float vals[GROUP_CAND][32];          // the values of a candidate, in ascending order of u
+  float breaks[GROUP_CAND][32];        // the value index of u is the number of these below u (+inf padded)
+  float u[SOP_MAX_CLASSES][256];       // merged decision points per group, without repeats (+inf padded)
+  unsigned short cell[256];            // their cells
+  float sorted[256];                   // the points before repeats are dropped, and which of them is the first of its value
+  unsigned char first[256];
+  unsigned warp_count[8];
+  int n_breaks[SOP_MAX_CLASSES];       // distinct merged decision points
+  int per_cell[SOP_MAX_CLASSES];       // the most of them that a cell holds (4: more than three)
 };
 
+__device__ __forceinline__ unsigned group_cell(float u, float inv_range, float n_cells) {
+  return __float_as_uint(__fmaf_rn(__saturatef(__fmaf_rn(u, inv_range, 0.5f)), n_cells, MAGIC));     // cell number + bits of MAGIC
+}
+
+__device__ __forceinline__ int count_not_above(const float* breaks, float u) {      // entries <= u of 31 sorted ones
+  int pos = 0;
+#pragma unroll
+  for (int step = 16; step >= 1; step >>= 1)
+    if (breaks[pos + step - 1] <= u) pos += step;
+  return pos;
+}
+
+// Builds the rows and cells of one group (the whole CTA; at least 256 threads).
+//   A candidate is brought into ascending order of u: value index = number of its points below u.  For a negated candidate
+//   (the table run on -u) the values are -lut in reverse; its points are the thresholds' negatives, where a tie goes to the
+//   upper value (the lower table index), so each moves down by one fp32 step.
+//   Row r holds the candidates' values for u in (point r - 1, point r], those of every two pairs in a plane of their own; it is
+//   stored in 8 copies of 16 bytes (16 of 8 bytes for a single pair) so that the lanes that load together never meet in a bank.
+//   A cell entry is {up to three points of the cell, byte offset of this copy of the row below the first of them}, in as many copies.
+__device__ void build_group(const Plan& P, const AtomsDev& A, int g, unsigned char* smem, GroupScratch& S) {
+  const GroupDev& G = P.groups[g];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+  for (int i = tid; i < GROUP_CAND * 32; i += nt) {
+    const int q = i >> 5, j = i & 31, a = G.cand[q], ne = A.atoms[a].n_entries;
+    const bool neg = A.atoms[a].negated != 0;
+    const float* lut = ((A.dd_mask >> a) & 1u) ? A.dd_lut : A.atoms[a].lut;
+    const int jj = min(j, ne - 1);
+    const float v = lut[neg ? ne - 1 - jj : jj];
+    S.vals[q][j] = neg ? -v : v;
+    // threshold of the table below entry t (the rule of build_thresholds: the largest fp32 <= the midpoint, a repeated
+    // entry takes the threshold above it, +inf from the last entry on)
+    float x = __int_as_float(0x7F800000);
+    if (j < ne - 1) {
+      int t = neg ? ne - 2 - j : j;
+      while (t < ne - 1 && lut[t] == lut[t + 1]) ++t;
+      if (t < ne - 1) x = __double2float_rd(0.5 * ((double)lut[t] + (double)lut[t + 1]));
+      if (neg) {
+        const float y = -x;
+        const unsigned b = __float_as_uint(y);
+        x = (b << 1) == 0u ? __uint_as_float(0x80000001u)                      // below zero: the smallest negative number
+            : b == 0xFF800000u ? y                                              // -inf: below every u
+            : __uint_as_float((b >> 31) ? b + 1u : b - 1u);
+      }
+    }
+    S.breaks[q][j] = x;
+  }
+  if (tid < 256) S.u[g][tid] = __int_as_float(0x7F800000);
+  if (tid == 0) S.per_cell[g] = 0;
+  __syncthreads();
+  // merge: thread (q, j) finds the place of its point among all, equal points in the order of (q, j); repeats are dropped
+  float mine = __int_as_float(0x7F800000);
+  int place = 0;
+  bool first = false;
+  if (tid < GROUP_CAND * 32 && (tid >> 5) < G.n) {
+    const int q = tid >> 5, j = tid & 31;
+    mine = S.breaks[q][j];
+    if (mine < __int_as_float(0x7F800000)) {
+      first = j == 0 || S.breaks[q][j - 1] != mine;
+#pragma unroll
+      for (int b = 0; b < GROUP_CAND; ++b) {
+        if (b >= G.n) break;
+        const int lt = count_below<5>(S.breaks[b], mine), le = count_not_above(S.breaks[b], mine);
+        place += b < q ? le : lt;
+        if (b < q && le != lt) first = false;
+      }
+      place += j - count_below<5>(S.breaks[q], mine);
+    }
+  }
+  if (tid < 256) S.first[tid] = 0;
+  __syncthreads();
+  if (mine < __int_as_float(0x7F800000)) { S.sorted[place] = mine; S.first[place] = first ? 1 : 0; }
+  __syncthreads();
+  if (tid < 256) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, S.first[tid] != 0);
+    if (lane == 0) S.warp_count[warp] = (unsigned)__popc(m);
+  }
+  __syncthreads();
+  if (tid < 256) {
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, S.first[tid] != 0);
+    unsigned at = (unsigned)__popc(m & ((1u << lane) - 1u)), total = 0;
+    for (int w = 0; w < 8; ++w) { if (w < warp) at += S.warp_count[w]; total += S.warp_count[w]; }
+    if (S.first[tid]) {
+      S.u[g][at] = S.sorted[tid];
+      S.cell[at] = (unsigned short)(group_cell(S.sorted[tid], G.inv_range, (float)G.n_cells) - __float_as_uint(MAGIC));
+    }
+    if (tid == 0) S.n_breaks[g] = (int)total;
+  }
+  __syncthreads();
+  const int R = S.n_breaks[g];
+  for (int i = tid; i < (R + 1) * GROUP_CAND; i += nt) {
+    const int r = i >> 3, q = i & 7;
+    if (q >= 2 * G.np) continue;
+    const float v = S.vals[q][count_below<5>(S.breaks[q], r < R ? S.u[g][r] : __int_as_float(0x7F800000))];
+    unsigned char* row = smem + G.row_off + (q >> 2) * G.plane_bytes + r * 128;
+    if (G.np == 1) {
+      for (int c = 0; c < 16; ++c) *reinterpret_cast<float*>(row + 8 * ((c + r) & 15) + 4 * q) = v;      // (neighbouring threads in different banks)
+    } else {
+      for (int c = 0; c < 8; ++c) *reinterpret_cast<float*>(row + 16 * ((c + (i >> 2)) & 7) + 4 * (q & 3)) = v;
+    }
+  }
+  for (int k = tid; k <= G.n_cells; k += nt) {
+    int lo = 0;                                    // points in lower cells
+#pragma unroll
+    for (int step = 128; step >= 1; step >>= 1)
+      if (lo + step <= R && (int)S.cell[lo + step - 1] < k) lo += step;
+    float t[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) t[x] = lo + x < R && (int)S.cell[lo + x] == k ? S.u[g][lo + x] : __int_as_float(0x7F800000);
+    int most = 0;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) most += lo + x < R && (int)S.cell[lo + x] == k ? 1 : 0;
+    if (most > 1) atomicMax(&S.per_cell[g], most);
+    const int copies = G.np == 1 ? 16 : 8;
+    float4* dst = reinterpret_cast<float4*>(smem + G.cell_off) + (size_t)k * copies;
+    for (int x = 0; x < copies; ++x) {
+      const int c = (x + k) & (copies - 1);
+      dst[c] = make_float4(t[0], t[1], t[2], __uint_as_float((unsigned)lo * 128u + (unsigned)c * (128u / copies)));
+    }
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ float4 lds_f4(unsigned addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Cosines of two candidates at once: RN(dot / RN(sqrt(RN(nw nq)))), the value of block_cosine.  Square root and quotient by
+// Newton steps with exact fused residuals and a final correction (P. Markstein, "Computation of elementary functions on the
+// IBM RISC System/6000 processor", 1990): from the reciprocal root y the pair g ~ sqrt(x), h ~ 1 / (2 sqrt(x)) is refined once
+// and g corrected by its residual x - g^2; 2 h, refined once against the rounded root, is its rounded reciprocal, with which the
+// quotient is corrected by its residual.  The signs are chosen so that no operand needs a negation: G = -g, S = -sqrt(x).
+// Valid for x in [2^-80, 2^80] and |dot| >= 2^-60 (no intermediate result leaves the normal range); the caller checks.
+constexpr float COS_LO = 8.271806125530277e-25f, COS_HI = 1.2089258196146292e24f, COS_DOT = 8.673617379884035e-19f;
+__device__ __forceinline__ float2 cosine_pair(const float2 nx, const float2 dot) {       // nx = -(nw nq)
+  const float2 y = make_float2(rsqrt_approx(-nx.x), rsqrt_approx(-nx.y));
+  const float2 half = make_float2(0.5f, 0.5f), one = make_float2(1.0f, 1.0f);
+  float2 G = __fmul2_rn(nx, y), h = __fmul2_rn(y, half);
+  const float2 r = __ffma2_rn(G, h, half);
+  G = __ffma2_rn(G, r, G);
+  h = __ffma2_rn(h, r, h);
+  const float2 D = __ffma2_rn(G, G, nx);
+  const float2 S = __ffma2_rn(D, h, G);
+  float2 z = __fadd2_rn(h, h);
+  const float2 e = __ffma2_rn(S, z, one);
+  z = __ffma2_rn(z, e, z);
+  const float2 q = __fmul2_rn(dot, z);
+  const float2 m = __ffma2_rn(S, q, dot);
+  return __ffma2_rn(m, z, q);
+}
+
+__device__ __forceinline__ float cosine_one(float nx, float dot) {      // the same steps for one candidate
+  const float y = rsqrt_approx(-nx);
+  float G = __fmul_rn(nx, y), h = __fmul_rn(y, 0.5f);
+  const float r = __fmaf_rn(G, h, 0.5f);
+  G = __fmaf_rn(G, r, G);
+  h = __fmaf_rn(h, r, h);
+  const float S = __fmaf_rn(__fmaf_rn(G, G, nx), h, G);
+  float z = __fadd_rn(h, h);
+  z = __fmaf_rn(z, __fmaf_rn(S, z, 1.0f), z);
+  const float q = __fmul_rn(dot, z);
+  return __fmaf_rn(__fmaf_rn(S, q, dot), z, q);
+}
+
+__device__ __noinline__ float block_cosine_any(float nw, float nq, float dot) { return block_cosine(nw, nq, dot); }
+
+// Rounding of a scale in its usual range, with what does not change from block to block worked out beforehand: the pattern of
+// sigma, rounded to nearest even on y mantissa bits by one integer addition (see scale_quantize).
+struct ScaleFast {
+  unsigned lo, span;          // patterns lo .. lo + span - 1 take the fast path
+  unsigned half, mask;        // half a step less one, the bits that are dropped
+  int sh;
+  __device__ __forceinline__ void init(const FmtDev& F, int k) {
+    const int e0 = max(F.emin + 127 - k, 4), e1 = min(F.emax + 127 - k, 250);      // normal, below the top binade, reciprocal normal
+    const bool ok = F.y >= 1 && e1 > e0;
+    lo = ok ? (unsigned)e0 << 23 : 0u;
+    span = ok ? (unsigned)(e1 - e0) << 23 : 0u;
+    sh = 23 - F.y;
+    half = (1u << (sh - 1)) - 1u;
+    mask = (1u << sh) - 1u;
+  }
+};
+
+// 1 / s rounded to nearest for a normal s whose reciprocal is normal: a Newton step with a fused residual (Markstein 1990, as
+// above; compared with the correctly rounded reciprocal for every significand).
+__device__ __forceinline__ float reciprocal_scale(float s) {
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(s));
+  return __fmaf_rn(y, __fmaf_rn(-s, y, 1.0f), y);
+}
+
+// What the block loops of one class share: the class's scale rule and the thread's walk over the rows of its column block.
+struct SweepCtx {
+  const unsigned char* smem;
+  unsigned c_addr;                 // shared-memory address of the thread's channel norms: four, then TB * 16 bytes on the next four
+  // scale
+  float tmax, pot;
+  bool block_scope;
+  int k;
+  ScaleFast fast;
+  // blocks
+  const uint16_t* w0;
+  long long w_step;
+  unsigned n_rows, off0, off_step; // this thread's blocks, the byte offset of the first in a column, the step
+  unsigned n_iter;                 // blocks of the thread that has the most
+
+  __device__ __forceinline__ void scale(float amax, const FmtDev& F, float& s_hat, float& rcp) const {
+    const float sigma = tmax == 1.0f ? amax : __fdiv_rn(amax, tmax);
+    const unsigned b = __float_as_uint(sigma);
+    if (block_scope && b - fast.lo < fast.span) {
+      s_hat = __uint_as_float((b + fast.half + ((b >> fast.sh) & 1u)) & ~fast.mask);
+      rcp = reciprocal_scale(s_hat);
+    } else {
+      s_hat = !block_scope ? (amax > 0.0f ? pot : 0.0f) : scale_quantize(sigma, k, F).s_hat;
+      rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
+    }
+  }
+};
+
+constexpr unsigned C_STEP = TB * 16u;
+
+// The metrics of NP pairs of candidates on one block: row offsets of its elements in `off` (elements 8 p + i and 8 p + 4 + i
+// in the halves of word 4 p + i), their rows at `plane`.  The sums run in the order of the quad tree: four quads of consecutive
+// elements, sequential inside a quad, (Q0 + Q1) + (Q2 + Q3).
+template <int NP>
+__device__ __forceinline__ void sweep_pass(const unsigned char* __restrict__ plane, const uint32_t (&wb)[8], const uint32_t (&off)[8],
+                                           unsigned c_addr, float s_hat, float2 (&nq)[NP], float2 (&dot)[NP], float2 (&sse)[NP]) {
+  const float2 ns = make_float2(-s_hat, -s_hat);
+  float2 n2[NP], d2[NP], s2[NP];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    float2 n[NP], d[NP], s[NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) n[p] = d[p] = s[p] = make_float2(0.0f, 0.0f);
+    const float4 cc = lds_f4(c_addr + (unsigned)h * C_STEP);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = 4 * h + r;
+      const float c = r == 0 ? cc.x : r == 1 ? cc.y : r == 2 ? cc.z : cc.w;
+      const float w = (i & 1) ? bf16hi(wb[i >> 1]) : bf16lo(wb[i >> 1]);
+      const uint32_t o = off[4 * (h >> 1) + r];
+      const unsigned char* row = plane + ((h & 1) ? o >> 16 : o & 0xFFFFu);
+      float2 q[NP];
+      if (NP == 1) {
+        q[0] = *reinterpret_cast<const float2*>(row);
+      } else {
+        const float4 a = *reinterpret_cast<const float4*>(row);
+        q[0] = make_float2(a.x, a.y);
+        q[NP - 1] = make_float2(a.z, a.w);
+      }
+      const float2 w2 = make_float2(w, w), c2 = make_float2(c, c);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const float2 cq = __fmul2_rn(c2, q[p]);
+        n[p] = __ffma2_rn(cq, q[p], n[p]);
+        d[p] = __ffma2_rn(cq, w2, d[p]);
+        const float2 e = __ffma2_rn(ns, q[p], w2);
+        s[p] = __ffma2_rn(e, e, s[p]);
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      if (h == 0) { nq[p] = n[p]; dot[p] = d[p]; sse[p] = s[p]; }
+      if (h == 1) { nq[p] = __fadd2_rn(nq[p], n[p]); dot[p] = __fadd2_rn(dot[p], d[p]); sse[p] = __fadd2_rn(sse[p], s[p]); }
+      if (h == 2) { n2[p] = n[p]; d2[p] = d[p]; s2[p] = s[p]; }
+      if (h == 3) {
+        nq[p] = __fadd2_rn(nq[p], __fadd2_rn(n2[p], n[p]));
+        dot[p] = __fadd2_rn(dot[p], __fadd2_rn(d2[p], d[p]));
+        sse[p] = __fadd2_rn(sse[p], __fadd2_rn(s2[p], s[p]));
+      }
+    }
+  }
+}
+
+// The cosines of NP pairs from their sums, then both per-block values into the columns.
+template <int NP>
+__device__ __forceinline__ void sweep_emit(float nw, float2 (&nq)[NP], float2 (&dot)[NP], float2 (&sse)[NP], const ColumnPtr* cols,
+                                           unsigned at, bool on) {
+  float2 nx[NP];
+  float lo = 3.0e38f, hi = 0.0f, dl = 3.0e38f;
+  const float2 nnw = make_float2(-nw, -nw);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    nx[p] = __fmul2_rn(nnw, nq[p]);
+    lo = fminf(lo, fminf(-nx[p].x, -nx[p].y));
+    hi = fmaxf(hi, fmaxf(-nx[p].x, -nx[p].y));
+    dl = fminf(dl, fminf(fabsf(dot[p].x), fabsf(dot[p].y)));
+  }
+  if (lo >= COS_LO && hi <= COS_HI && dl >= COS_DOT) {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) dot[p] = cosine_pair(nx[p], dot[p]);
+  } else {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) dot[p] = make_float2(block_cosine_any(nw, nq[p].x, dot[p].x), block_cosine_any(nw, nq[p].y, dot[p].y));
+  }
+  if (on) {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const ColumnPtr a = cols[2 * p], b = cols[2 * p + 1];          // (the last candidate again where their number is odd)
+      *reinterpret_cast<float*>(a.cos + at) = dot[p].x;
+      *reinterpret_cast<float*>(a.sse + at) = sse[p].x;
+      *reinterpret_cast<float*>(b.cos + at) = dot[p].y;
+      *reinterpret_cast<float*>(b.sse + at) = sse[p].y;
+    }
+  }
+}
+
+// The candidates of one group on every block of the thread: first the rows of its sixteen elements (kept as 16-bit offsets),
+// then the metrics of two pairs of candidates at a time -- the sums of all eight at once would take more registers than leave
+// enough warps resident.
+//   KT: decision points per cell that are compared (0: the group is searched).
+template <int NP, int KT>
+__device__ __forceinline__ void sweep_group(const SweepCtx& X, const FmtDev& F, const GroupDev& G, const float* merged, const ColumnPtr* cols) {
+  const int lane = threadIdx.x & 31;
+  const unsigned copy = NP == 1 ? (unsigned)(lane & 15) * 8u : (unsigned)(lane & 7) * 16u;
+  constexpr unsigned CELL = NP == 1 ? 256u : 128u;
+  const unsigned cells = G.cell_off + (NP == 1 ? 2u : 1u) * copy - __float_as_uint(MAGIC) * CELL;      // modulo 2^32
+  const unsigned char* plane = X.smem + G.row_off;
+  const unsigned plane_bytes = G.plane_bytes;
+  const float inv_range = G.inv_range, n_cells = (float)G.n_cells;
+  const uint16_t* wp = X.w0;
+  unsigned at = X.off0;
+  uint32_t wn[8];
+  load_block_bits(wp, wn);
+#pragma unroll 1
+  for (unsigned it = 0; it < X.n_iter; ++it) {
+    uint32_t wb[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) wb[q] = wn[q];
+    // the next row's block, one iteration ahead; a thread past its last row keeps the block and stores nothing more
+    if (it + 1 < X.n_rows) wp += X.w_step;
+    load_block_bits(wp, wn);
+    float s_hat, rcp;
+    X.scale(absmax_bits(wb), F, s_hat, rcp);
+    uint32_t off[8];
+    float nw4[4];
+    const float2 r2 = make_float2(rcp, rcp);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const float4 ca = lds_f4(X.c_addr + (unsigned)(2 * p) * C_STEP), cb = lds_f4(X.c_addr + (unsigned)(2 * p + 1) * C_STEP);
+      const float a4[4] = {ca.x, ca.y, ca.z, ca.w}, b4[4] = {cb.x, cb.y, cb.z, cb.w};
+      nw4[2 * p] = nw4[2 * p + 1] = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int ix = 8 * p + i, iy = ix + 4;
+        const float2 w = make_float2((ix & 1) ? bf16hi(wb[ix >> 1]) : bf16lo(wb[ix >> 1]), (iy & 1) ? bf16hi(wb[iy >> 1]) : bf16lo(wb[iy >> 1]));
+        const float2 u2 = __fmul2_rn(w, r2);
+        nw4[2 * p] = __fmaf_rn(__fmul_rn(a4[i], w.x), w.x, nw4[2 * p]);
+        nw4[2 * p + 1] = __fmaf_rn(__fmul_rn(b4[i], w.y), w.y, nw4[2 * p + 1]);
+        unsigned o[2];
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+          const float u = y ? u2.y : u2.x;
+          if (KT == 0) {
+            unsigned pos = 0;
+#pragma unroll
+            for (int step = 1 << (SLOW_STEPS - 1); step >= 1; step >>= 1)
+              if (merged[pos + step - 1] < u) pos += step;
+            o[y] = pos * 128u + copy;
+          } else {
+            const float4 e = *reinterpret_cast<const float4*>(X.smem + (cells + group_cell(u, inv_range, n_cells) * CELL));
+            o[y] = __float_as_uint(e.w);
+            if (u > e.x) o[y] += 128u;
+            if (u > e.y) o[y] += 128u;
+            if (KT > 2 && u > e.z) o[y] += 128u;
+          }
+        }
+        off[4 * p + i] = o[0] + (o[1] << 16);
+      }
+    }
+    const float nw = quad_tree(nw4);
+#pragma unroll
+    for (int b = 0; b < NP; b += 2) {
+      constexpr int LAST = NP % 2 ? 1 : 2;
+      if (b + 2 <= NP) {
+        float2 nq[2], dot[2], sse[2];
+        sweep_pass<2>(plane + (b / 2) * plane_bytes, wb, off, X.c_addr, s_hat, nq, dot, sse);
+        sweep_emit<2>(nw, nq, dot, sse, cols + 2 * b, at, it < X.n_rows);
+      } else {
+        float2 nq[LAST], dot[LAST], sse[LAST];
+        sweep_pass<LAST>(plane + (b / 2) * plane_bytes, wb, off, X.c_addr, s_hat, nq, dot, sse);
+        sweep_emit<LAST>(nw, nq, dot, sse, cols + 2 * b, at, it < X.n_rows);
+      }
+    }
+    at += X.off_step;
+  }
+}
+
+// Element-format candidates (no table): element layout as float2 over elements i of quads 2p (x) and 2p + 1 (y), so that the
+// two lanes of a packed operation are two independent sequential chains.
+//   MODE: E2M3, E4M3 or a grid given by parameters.  PAIRED: the channel norms lie in shared memory in that layout too.
 __device__ __forceinline__ float fold(const float2 a, const float2 b) {
   return __fadd_rn(__fadd_rn(a.x, a.y), __fadd_rn(b.x, b.y));
 }
 
-struct Metric { float nq, dot, sse; };
-
-// One cell entry is {threshold, hi bf16 : lo bf16}: the reconstruction value is hi when u lies
-// strictly above the threshold, else lo.  A negated candidate runs the base table on -u (mirrored
-// row) and flips the sign of the dot product and of the scale in the error term.
-template <bool NEG>
-__device__ __forceinline__ Metric eval_lut_cells(const unsigned char* __restrict__ tp, unsigned moff, const BlockRegs& B, float s_hat) {
-  float2 nq[2], dot[2], sse[2];
-  nq[0] = nq[1] = dot[0] = dot[1] = sse[0] = sse[1] = make_float2(0.0f, 0.0f);
-  const float sg = NEG ? s_hat : -s_hat;
-  const float2 ns = make_float2(sg, sg);
+template <int MODE, bool PAIRED>
+__device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F, const ClassDev& K, size_t NB, float* __restrict__ block_cos,
+                                             float* __restrict__ block_sse) {
+  const uint16_t* wp = X.w0;
+  unsigned at = X.off0;
+  const int n_cand = K.n_cand;
+  uint32_t wn[8];
+  load_block_bits(wp, wn);
+#pragma unroll 1
+  for (unsigned it = 0; it < X.n_iter; ++it) {
+    uint32_t wb[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+    for (int q = 0; q < 8; ++q) wb[q] = wn[q];
+    if (it + 1 < X.n_rows) wp += X.w_step;
+    load_block_bits(wp, wn);
+    float s_hat, rcp;
+    X.scale(absmax_bits(wb), F, s_hat, rcp);
+    float cc[16];
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const int idx = 2 * i + p;
-      const uint2 ea = *reinterpret_cast<const uint2*>(tp + (NEG ? moff - B.off[2 * idx] : B.off[2 * idx]));
-      const uint2 eb = *reinterpret_cast<const uint2*>(tp + (NEG ? moff - B.off[2 * idx + 1] : B.off[2 * idx + 1]));
-      const bool pa = NEG ? (-B.u[idx].x > __uint_as_float(ea.x)) : (B.u[idx].x > __uint_as_float(ea.x));
-      const bool pb = NEG ? (-B.u[idx].y > __uint_as_float(eb.x)) : (B.u[idx].y > __uint_as_float(eb.x));
-      float2 q;
-      q.x = __uint_as_float(__byte_perm(ea.y, 0u, pa ? 0x3244u : 0x1044u));
-      q.y = __uint_as_float(__byte_perm(eb.y, 0u, pb ? 0x3244u : 0x1044u));
-      const float2 cq = __fmul2_rn(B.c[idx], q);
-      nq[p] = __ffma2_rn(cq, q, nq[p]);
-      dot[p] = __ffma2_rn(cq, B.w[idx], dot[p]);
-      const float2 e = __ffma2_rn(ns, q, B.w[idx]);
-      sse[p] = __ffma2_rn(e, e, sse[p]);
+    for (int h = 0; h < 4; ++h) {
+      const float4 v = lds_f4(X.c_addr + (unsigned)h * C_STEP);
+      if (PAIRED) { const int i = 8 * (h >> 1) + 2 * (h & 1); cc[i] = v.x; cc[i + 4] = v.y; cc[i + 1] = v.z; cc[i + 5] = v.w; }
+      else { cc[4 * h] = v.x; cc[4 * h + 1] = v.y; cc[4 * h + 2] = v.z; cc[4 * h + 3] = v.w; }
     }
-  }
-  Metric m;
-  m.nq = fold(nq[0], nq[1]);
-  const float d = fold(dot[0], dot[1]);
-  m.dot = NEG ? -d : d;
-  m.sse = fold(sse[0], sse[1]);
-  return m;
-}
-
-// mode 0: table through binary search over the thresholds (any table); mode 1 / 2: E2M3 / E4M3 grid;
-// mode 3: grid given by parameters
-template <int MODE, bool NEG>
-__device__ __forceinline__ Metric eval_generic(const float* __restrict__ tau, const float* __restrict__ lutv, const BlockRegs& B, float s_hat,
-                                               const GridDev grid = GridDev()) {
-  float2 nq[2], dot[2], sse[2];
-  nq[0] = nq[1] = dot[0] = dot[1] = sse[0] = sse[1] = make_float2(0.0f, 0.0f);
-  const float sg = NEG ? s_hat : -s_hat;
-  const float2 ns = make_float2(sg, sg);
+    float2 nw2[2], nq[2], dot[2], sse[2];
+    nw2[0] = nw2[1] = nq[0] = nq[1] = dot[0] = dot[1] = sse[0] = sse[1] = make_float2(0.0f, 0.0f);
+    const float2 ns = make_float2(-s_hat, -s_hat), r2 = make_float2(rcp, rcp);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 4; ++i) {
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const int idx = 2 * i + p;
-      const float ux = B.u[idx].x, uy = B.u[idx].y;
-      float2 q;
-      if constexpr (MODE == 0) {
-        q.x = lutv[count_below(tau, NEG ? -ux : ux)];
-        q.y = lutv[count_below(tau, NEG ? -uy : uy)];
-      } else if constexpr (MODE == SOP_KIND_FP_GRID) {
-        q.x = grid_quantize(ux, grid);
-        q.y = grid_quantize(uy, grid);
-      } else {
-        q.x = fp_quantize<MODE>(ux);
-        q.y = fp_quantize<MODE>(uy);
+      for (int p = 0; p < 2; ++p) {
+        const int ix = 8 * p + i, iy = ix + 4;
+        const float2 w = make_float2((ix & 1) ? bf16hi(wb[ix >> 1]) : bf16lo(wb[ix >> 1]), (iy & 1) ? bf16hi(wb[iy >> 1]) : bf16lo(wb[iy >> 1]));
+        const float2 c = make_float2(cc[ix], cc[iy]);
+        const float2 u = __fmul2_rn(w, r2);
+        float2 q;
+        if constexpr (MODE == SOP_KIND_FP_GRID) { q.x = grid_quantize(u.x, K.grid); q.y = grid_quantize(u.y, K.grid); }
+        else { uint32_t codes; q = fp_quantize2<MODE>(u.x, u.y, codes); }
+        nw2[p] = __ffma2_rn(__fmul2_rn(c, w), w, nw2[p]);
+        const float2 cq = __fmul2_rn(c, q);
+        nq[p] = __ffma2_rn(cq, q, nq[p]);
+        dot[p] = __ffma2_rn(cq, w, dot[p]);
+        const float2 e = __ffma2_rn(ns, q, w);
+        sse[p] = __ffma2_rn(e, e, sse[p]);
       }
-      const float2 cq = __fmul2_rn(B.c[idx], q);
-      nq[p] = __ffma2_rn(cq, q, nq[p]);
-      dot[p] = __ffma2_rn(cq, B.w[idx], dot[p]);
-      const float2 e = __ffma2_rn(ns, q, B.w[idx]);
-      sse[p] = __ffma2_rn(e, e, sse[p]);
     }
-  }
-  Metric m;
-  m.nq = fold(nq[0], nq[1]);
-  const float d = fold(dot[0], dot[1]);
-  m.dot = NEG ? -d : d;
-  m.sse = fold(sse[0], sse[1]);
-  return m;
-}
-
-// Build the shared-memory tables of one CTA: table values and thresholds, then the cell tables.
-// A cell row r (k = r - c_half) covers the u values that round to k: u * invh in [k - 1/2, k + 1/2];
-// row 0 and the last row extend to -inf / +inf.  A row is usable when at most one distinct threshold
-// falls inside its closed interval and both neighbouring table values are bf16 numbers (they are
-// stored as one 32-bit pair); otherwise the whole table is marked slow and its candidates take the
-// binary-search path.  Every row is stored 16 times (128 bytes): lanes l and l + 16 read copy l & 15,
-// so a 64-bit load of any 32 rows by a warp is free of bank conflicts.  The tables are interleaved
-// row by row ([row][table][copy]): a thread keeps one offset per element and the table is an
-// immediate displacement of the load.
-__device__ void build_tables(const Plan& P, const AtomsDev& A, uint2* cell, float* tau, float* lutv, int* fast) {
-  const int tid = threadIdx.x;
-  for (int i = tid; i < P.n_tables * 32; i += blockDim.x) {
-    const int t = i >> 5, j = i & 31;
-    const int a = P.table_atom[t];
-    const int ne = A.atoms[a].n_entries;
-    const int jj = min(j, ne - 1);
-    lutv[i] = ((A.dd_mask >> a) & 1u) ? A.dd_lut[jj] : A.atoms[a].lut[jj];
-  }
-  if (tid < SOP_MAX_TABLES) fast[tid] = 1;
-  __syncthreads();
-  // decision thresholds, one thread per entry (the rule of build_thresholds: the largest fp32 <= the midpoint,
-  // a repeated entry takes the threshold above it, +inf from the last entry on)
-  for (int i = tid; i < P.n_tables * 32; i += blockDim.x) {
-    const int t = i >> 5, j = i & 31;
-    const int ne = A.atoms[P.table_atom[t]].n_entries;
-    const float* lv = lutv + t * 32;
-    int jj = j;
-    while (jj < ne - 1 && lv[jj] == lv[jj + 1]) ++jj;
-    tau[i] = jj < ne - 1 ? __double2float_rd(0.5 * ((double)lv[jj] + (double)lv[jj + 1])) : __int_as_float(0x7F800000);
-  }
-  __syncthreads();
-  const int rows = P.rows;
-  for (int i = tid; i < P.n_tables * rows; i += blockDim.x) {
-    const int t = i / rows, r = i - t * rows;
-    const ClassDev& C = P.cls[P.table_cls[t]];
-    const int ne = A.atoms[P.table_atom[t]].n_entries;
-    const int nrow = 2 * C.c_half + 1;
-    uint2 entry = make_uint2(0x7F800000u, 0u);
-    if (r < nrow) {
-      const float hh = __fdiv_rn(1.0f, C.invh);                     // cell width in u (a power of two)
-      const float kf = (float)(r - C.c_half);
-      const float lo_edge = r == 0 ? -INFINITY : __fmul_rn(kf - 0.5f, hh);
-      const float hi_edge = r == nrow - 1 ? INFINITY : __fmul_rn(kf + 0.5f, hh);
-      const float* tt = tau + t * 32;
-      const float* lv = lutv + t * 32;
-      int nbelow = 0, ninside = 0, ndistinct = 0;
-      float prev = 0.0f;
-      for (int j = 0; j < ne - 1; ++j) {
-        const float x = tt[j];
-        if (x < lo_edge) ++nbelow;
-        else if (x <= hi_edge) {
-          if (ninside == 0 || x != prev) ++ndistinct;
-          prev = x;
-          ++ninside;
-        }
+    const float nw = fold(nw2[0], nw2[1]), nqs = fold(nq[0], nq[1]), dots = fold(dot[0], dot[1]), err = fold(sse[0], sse[1]);
+    const float x = __fmul_rn(nw, nqs);
+    const float cosv = x >= COS_LO && x <= COS_HI && fabsf(dots) >= COS_DOT ? cosine_one(-x, dots) : block_cosine_any(nw, nqs, dots);
+    if (it < X.n_rows)
+      for (int ci = 0; ci < n_cand; ++ci) {      // (candidates of one format and scale have the same values)
+        const size_t col = (size_t)K.cand[ci] * NB + (at >> 2);
+        block_cos[col] = cosv;
+        block_sse[col] = err;
       }
-      const float lo = lv[nbelow], hi = lv[min(nbelow + ninside, ne - 1)];
-      const uint32_t lb = __float_as_uint(lo), hb = __float_as_uint(hi);
-      const bool ok = ndistinct <= 1 && (lb & 0xFFFFu) == 0 && (hb & 0xFFFFu) == 0;
-      if (!ok) atomicAnd(&fast[t], 0);
-      entry.x = ninside ? __float_as_uint(prev) : 0x7F800000u;
-      entry.y = (hb & 0xFFFF0000u) | (lb >> 16);
-    }
-    uint2* dst = cell + ((size_t)r * P.n_tables + t) * 16;
-    for (int l = 0; l < 16; ++l) dst[l] = entry;
-  }
-  __syncthreads();
-}
-
-// One evaluated candidate of one block: the cosine, then both per-block values into their columns.
-__device__ __forceinline__ void emit(float* __restrict__ block_cos, float* __restrict__ block_sse, size_t col_off, bool on, float nw,
-                                     const Metric& mt) {
-  const float cosv = block_cosine(nw, mt.nq, mt.dot);
-  if (on) {
-    block_cos[col_off] = cosv;
-    block_sse[col_off] = mt.sse;
+    at += X.off_step;
   }
 }
 
-// Evaluates the candidates of eval_mask on every block and writes their columns of block_cos / block_sse.
-__global__ void __launch_bounds__(TB, 1) sweep_kernel(LayerArgs L, Plan P, AtomsDev A, FmtDev F, const WsHeader* __restrict__ hdr,
+// Evaluates the candidates of eval_mask on every block and writes their columns of block_cos / block_sse: group by group, then
+// format by format (W is read again for each: it is a tenth of the time of one).
+template <int MAX_NP>
+__global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArgs L, Plan P, AtomsDev A, FmtDev F, const WsHeader* __restrict__ hdr,
                                                       float* __restrict__ block_cos, float* __restrict__ block_sse,
-                                                      const sop_search_result* __restrict__ prev) {
+                                                      const sop_search_result* __restrict__ prev, unsigned c_off, unsigned tba) {
   extern __shared__ __align__(128) unsigned char smem[];
-  uint2* cell = reinterpret_cast<uint2*>(smem);
-  float* tau = reinterpret_cast<float*>(cell + (size_t)P.n_tables * P.rows * 16);
-  float* lutv = tau + SOP_MAX_TABLES * 32;
-  int* fast = reinterpret_cast<int*>(lutv + SOP_MAX_TABLES * 32);
-  int* cls_k = fast + SOP_MAX_TABLES;
-  float* cls_pot = reinterpret_cast<float*>(cls_k + SOP_MAX_CLASSES);
+  GroupScratch& S = *reinterpret_cast<GroupScratch*>(smem);
+  __shared__ int cls_k[SOP_MAX_CLASSES];
+  __shared__ float cls_pot[SOP_MAX_CLASSES];
 
-  const int tid = threadIdx.x, lane = tid & 31;
-  build_tables(P, A, cell, tau, lutv, fast);
+  const int tid = threadIdx.x;
+  // thread -> fixed column block j, rows m = r0, r0 + R, ...; its sixteen channel norms stay in shared memory.  Control flow is
+  // uniform: a thread with fewer rows evaluates its last block once more and stores nothing.
+  const unsigned nbk = (unsigned)L.nbk, M = (unsigned)L.M;       // the block count fits 31 bits
+  const unsigned R = gridDim.x * tba / nbk;                      // rows in flight (host guarantees R >= 1)
+  const unsigned gt = blockIdx.x * tba + min((unsigned)tid, tba - 1u);
+  const unsigned r0 = gt / nbk, j = gt - r0 * nbk;
+  SweepCtx X;
+  X.smem = smem;
+  X.c_addr = smem_u32(smem) + c_off + (unsigned)tid * 16u;
+  X.n_iter = (M + R - 1) / R;
+  X.n_rows = r0 < R && r0 < M ? (M - r0 + R - 1) / R : 0u;
+  X.w0 = L.W + (size_t)j * SOP_G + (long long)min(r0, M - 1) * L.ldw;
+  X.w_step = (long long)R * L.ldw;
+  X.off0 = (r0 * nbk + j) * 4u;                                  // at most 2^27 blocks
+  X.off_step = R * nbk * 4u;
+  for (int i = tid; i < P.n_groups * GROUP_CAND; i += TB) {
+    const size_t at = (size_t)P.groups[i / GROUP_CAND].cand[i % GROUP_CAND] * (size_t)L.NB;
+    S.col[i / GROUP_CAND][i % GROUP_CAND] = {reinterpret_cast<char*>(block_cos + at), reinterpret_cast<char*>(block_sse + at)};
+  }
+  {
+    const float4* cp = reinterpret_cast<const float4*>(L.c + (size_t)j * SOP_G);
+    float4* dst = reinterpret_cast<float4*>(smem + c_off);
+    const float4 v0 = __ldg(cp), v1 = __ldg(cp + 1), v2 = __ldg(cp + 2), v3 = __ldg(cp + 3);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(X.w0));          // the first block arrives while the tables are built
+    if (MAX_NP == 0) {
+      dst[tid] = make_float4(v0.x, v1.x, v0.y, v1.y);
+      dst[TB + tid] = make_float4(v0.z, v1.z, v0.w, v1.w);
+      dst[2 * TB + tid] = make_float4(v2.x, v3.x, v2.y, v3.y);
+      dst[3 * TB + tid] = make_float4(v2.z, v3.z, v2.w, v3.w);
+    } else {
+      dst[tid] = v0; dst[TB + tid] = v1; dst[2 * TB + tid] = v2; dst[3 * TB + tid] = v3;
+    }
+  }
   if (tid < SOP_MAX_CLASSES) {
     if (P.k_from_result) {
       const bool live = tid < P.n_classes;
@@ -437,129 +797,35 @@ __global__ void __launch_bounds__(TB, 1) sweep_kernel(LayerArgs L, Plan P, Atoms
       cls_pot[tid] = hdr->cls_pot[tid];
     }
   }
+
+  for (int g = 0; g < P.n_groups; ++g) build_group(P, A, g, smem, S);
   __syncthreads();
+  if ((unsigned)tid >= tba) return;                              // (whole warps: they only helped with the tables)
 
-  // thread -> fixed column block j, rows m = r0, r0 + R, ...
-  const long long GT = (long long)gridDim.x * TB;
-  const long long R = GT / L.nbk;                 // rows in flight (host guarantees R >= 1)
-  const long long gt = (long long)blockIdx.x * TB + tid;
-  const bool lane_on = gt < R * L.nbk;
-  const long long j = lane_on ? gt % L.nbk : 0;
-  const long long r0 = gt / L.nbk;
-  const long long n_iter = (L.M + R - 1) / R;
-
-  BlockRegs B;
-  {
-    const float4* cp = reinterpret_cast<const float4*>(L.c + j * SOP_G);
-    float cc[16];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 v = __ldg(cp + q);
-      cc[4 * q] = v.x; cc[4 * q + 1] = v.y; cc[4 * q + 2] = v.z; cc[4 * q + 3] = v.w;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) B.c[2 * i + p] = make_float2(cc[8 * p + i], cc[8 * p + 4 + i]);
+#pragma unroll 1
+  for (int x = 0; x < P.n_groups + P.n_classes; ++x) {
+    const int cl = x < P.n_groups ? P.groups[x].cls : x - P.n_groups;
+    const ClassDev& K = P.cls[cl];
+    if (x >= P.n_groups && (K.kind == SOP_KIND_LUT || K.n_cand == 0)) continue;
+    X.tmax = K.tmax; X.pot = cls_pot[cl]; X.block_scope = K.scope != 0; X.k = cls_k[cl];
+    X.fast.init(F, X.k);
+    if (x < P.n_groups) {
+      const GroupDev& G = P.groups[x];
+      const float* merged = S.u[x];
+      const int per_cell = S.per_cell[x];
+#define SOP_RUN_GROUP(NP)                                                    \
+  if constexpr (NP <= MAX_NP) {                                              \
+    if (G.np == NP) {                                                        \
+      if (per_cell <= 2) sweep_group<NP, 2>(X, F, G, merged, S.col[x]);            \
+      else if (per_cell == 3) sweep_group<NP, 3>(X, F, G, merged, S.col[x]);       \
+      else sweep_group<NP, 0>(X, F, G, merged, S.col[x]);                          \
+    }                                                                        \
   }
-  const int copy_off = (lane & 15) * 8;
-  const unsigned char* cell_bytes = reinterpret_cast<const unsigned char*>(cell);
-
-  // Warp-uniform control flow: every thread evaluates a block in every iteration (a thread without
-  // work re-evaluates a valid block and stores nothing), so the class / candidate loops below are
-  // uniform branches.
-  const unsigned fast_mask = __ballot_sync(0xFFFFFFFFu, fast[lane & (SOP_MAX_TABLES - 1)] != 0);
-  const uint16_t* wcol = L.W + j * SOP_G;
-  uint32_t wb[8];
-  load_block_bits(wcol + min(r0, L.M - 1) * L.ldw, wb);
-  const size_t NBs = (size_t)L.NB;
-
-  for (long long it = 0; it < n_iter; ++it) {
-    const long long m = r0 + it * R;
-    const bool on = lane_on && m < L.M;
-    // ---- unpack, block statistics ----
-    float wf[16];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) { wf[2 * q] = bf16lo(wb[q]); wf[2 * q + 1] = bf16hi(wb[q]); }
-    const float amax = absmax_bits(wb);
-    load_block_bits(wcol + min(m + R, L.M - 1) * L.ldw, wb);   // prefetch the next row's block
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) B.w[2 * i + p] = make_float2(wf[8 * p + i], wf[8 * p + 4 + i]);
-    float2 nw2[2];
-    nw2[0] = nw2[1] = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        const float2 cw = __fmul2_rn(B.c[2 * i + p], B.w[2 * i + p]);
-        nw2[p] = __ffma2_rn(cw, B.w[2 * i + p], nw2[p]);
-      }
-    const float nw = fold(nw2[0], nw2[1]);
-    const size_t blk = (size_t)(m * L.nbk + j);
-
-    for (int cl = 0; cl < P.n_classes; ++cl) {
-      const ClassDev& C = P.cls[cl];
-      if (C.n_cand == 0) continue;
-      float s_hat;
-      if (C.scope == 0) {
-        s_hat = amax > 0.0f ? cls_pot[cl] : 0.0f;
-      } else {
-        const float sigma = C.tmax == 1.0f ? amax : __fdiv_rn(amax, C.tmax);
-        s_hat = scale_quantize(sigma, cls_k[cl], F).s_hat;
-      }
-      const float rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
-      const float2 r2 = make_float2(rcp, rcp);
-#pragma unroll
-      for (int idx = 0; idx < 8; ++idx) B.u[idx] = __fmul2_rn(B.w[idx], r2);
-      if (C.kind == SOP_KIND_LUT) {
-        const float tlo = MAGIC, thi = MAGIC + (float)(2 * C.c_half), toff = MAGIC + (float)C.c_half;
-        const float invh = C.invh;
-        const unsigned pitch = (unsigned)P.n_tables * 128u;
-        const unsigned cbias = (unsigned)copy_off - __float_as_uint(MAGIC) * pitch;   // modulo 2^32
-#pragma unroll
-        for (int idx = 0; idx < 8; ++idx) {
-          const float tx = fminf(fmaxf(__fmaf_rn(B.u[idx].x, invh, toff), tlo), thi);
-          const float ty = fminf(fmaxf(__fmaf_rn(B.u[idx].y, invh, toff), tlo), thi);
-          B.off[2 * idx] = __float_as_uint(tx) * pitch + cbias;
-          B.off[2 * idx + 1] = __float_as_uint(ty) * pitch + cbias;
-        }
-        const unsigned moff = 2u * (unsigned)C.c_half * pitch + 2u * (unsigned)copy_off;
-        // tables of this class with a usable cell grid: the table slot is a compile-time displacement
-        const unsigned cls_fast = P.cls_tables[cl] & fast_mask;
-#pragma unroll
-        for (int T = 0; T < SOP_MAX_TABLES; ++T) {
-          if ((cls_fast >> T) & 1u) {
-            const unsigned char* tp = cell_bytes + T * 128;
-            const int ap = P.table_pos[T], an = P.table_neg[T];
-            if (ap != 255) emit(block_cos, block_sse, (size_t)ap * NBs + blk, on, nw, eval_lut_cells<false>(tp, moff, B, s_hat));
-            if (an != 255) emit(block_cos, block_sse, (size_t)an * NBs + blk, on, nw, eval_lut_cells<true>(tp, moff, B, s_hat));
-          }
-        }
-        // tables without a usable cell grid: binary search over the thresholds
-        if (P.cls_tables[cl] & ~fast_mask) {
-          for (int ci = 0; ci < C.n_cand; ++ci) {
-            const int a = C.cand[ci];
-            const int t = P.cand[a].table;
-            if ((fast_mask >> t) & 1u) continue;
-            const Metric mt = P.cand[a].neg ? eval_generic<0, true>(tau + t * 32, lutv + t * 32, B, s_hat)
-                                            : eval_generic<0, false>(tau + t * 32, lutv + t * 32, B, s_hat);
-            emit(block_cos, block_sse, (size_t)a * NBs + blk, on, nw, mt);
-          }
-        }
-      } else if (C.kind == SOP_KIND_FP_E2M3) {
-        for (int ci = 0; ci < C.n_cand; ++ci)
-          emit(block_cos, block_sse, (size_t)C.cand[ci] * NBs + blk, on, nw, eval_generic<SOP_KIND_FP_E2M3, false>(nullptr, nullptr, B, s_hat));
-      } else if (C.kind == SOP_KIND_FP_GRID) {
-        for (int ci = 0; ci < C.n_cand; ++ci)
-          emit(block_cos, block_sse, (size_t)C.cand[ci] * NBs + blk, on, nw,
-               eval_generic<SOP_KIND_FP_GRID, false>(nullptr, nullptr, B, s_hat, C.grid));
-      } else {
-        for (int ci = 0; ci < C.n_cand; ++ci)
-          emit(block_cos, block_sse, (size_t)C.cand[ci] * NBs + blk, on, nw, eval_generic<SOP_KIND_FP_E4M3, false>(nullptr, nullptr, B, s_hat));
-      }
-    }
+      SOP_RUN_GROUP(1) SOP_RUN_GROUP(2) SOP_RUN_GROUP(3) SOP_RUN_GROUP(4)
+#undef SOP_RUN_GROUP
+    } else if (K.kind == SOP_KIND_FP_E2M3) sweep_format<SOP_KIND_FP_E2M3, MAX_NP == 0>(X, F, K, (size_t)L.NB, block_cos, block_sse);
+    else if (K.kind == SOP_KIND_FP_GRID) sweep_format<SOP_KIND_FP_GRID, MAX_NP == 0>(X, F, K, (size_t)L.NB, block_cos, block_sse);
+    else sweep_format<SOP_KIND_FP_E4M3, MAX_NP == 0>(X, F, K, (size_t)L.NB, block_cos, block_sse);
   }
 }
 
@@ -585,8 +851,6 @@ constexpr int RTB = 256;              // threads per CTA of the reduction: eight
 constexpr int RTILE = 256;            // blocks per tile: eight per lane
 constexpr int ENT = TASK_PART + 1;    // entries of a task: the anchor alone, then its partners
 constexpr int MAX_STAGE = 4;           // tile buffers of the ring
-
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
 __device__ void finalize_body(const LayerArgs& L, const Plan& P, int grid, const Partial* partials, sop_pair_stat* s_pair, sop_pair_stat* s_sig,
                               Partial* s_red, sop_pair_stat* pair_table, sop_pair_stat* signed_table, sop_search_result* res,
@@ -1029,20 +1293,6 @@ static bool same_table(const sop_atom& a, const sop_atom& b) {
   return a.n_entries == b.n_entries && memcmp(a.lut, b.lut, sizeof(float) * a.n_entries) == 0;
 }
 
-// smallest gap between distinct decision thresholds of a host-known table (in u)
-static double min_threshold_gap(const sop_atom& a) {
-  double prev = 0, best = 1e30;
-  bool have = false;
-  for (int j = 0; j + 1 < a.n_entries; ++j) {
-    if (a.lut[j] == a.lut[j + 1]) continue;
-    const double t = 0.5 * ((double)a.lut[j] + (double)a.lut[j + 1]);
-    if (have && t > prev) best = fmin(best, t - prev);
-    prev = t;
-    have = true;
-  }
-  return best;
-}
-
 int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mask, unsigned load_mask, int singles_only, int keep_loaded, Plan* P) {
   memset(P, 0, sizeof(*P));
   const int n = A.n_atoms;
@@ -1051,6 +1301,7 @@ int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mas
   P->eval_mask = eval_mask;
   P->load_mask = load_mask;
   const unsigned present = eval_mask | load_mask;
+  int n_tables = 0, table_atom[SOP_MAX_TABLES], table_signs[SOP_MAX_TABLES];
   // classes
   for (int i = 0; i < n; ++i) {
     const sop_atom& a = A.atoms[i];
@@ -1067,62 +1318,45 @@ int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mas
       cl = P->n_classes++;
       P->cls[cl].scope = a.scope; P->cls[cl].tmax = a.tmax; P->cls[cl].kind = a.kind;
       P->cls[cl].auto_k = (k_mode == SOP_K_AUTO && a.scope != 0) ? 1 : 0;
-      P->cls[cl].invh = 1.0f; P->cls[cl].c_half = 0;
       P->cls[cl].grid.min_eb = 128 - a.grid_bias; P->cls[cl].grid.sh = 23 - a.grid_man_bits;
       P->cls[cl].grid.vpos = a.tmax; P->cls[cl].grid.vneg = a.grid_neg_max;
     }
     ClassDev& C = P->cls[cl];
     C.mem[C.n_mem++] = (unsigned char)i;
     P->cand[i].cls = (unsigned char)cl;
-    P->cand[i].table = 0;
     if (!((eval_mask >> i) & 1u)) continue;
     C.cand[C.n_cand++] = (unsigned char)i;
     if (a.kind != SOP_KIND_LUT) continue;
+    // distinct tables of the call (an atom and its negation share one)
     const bool dd = (A.dd_mask >> i) & 1u;
     int t = -1;
-    for (int q = 0; q < P->n_tables; ++q) {
-      const int o = P->table_atom[q];
-      const bool odd = (A.dd_mask >> o) & 1u;
-      if (P->table_cls[q] != cl || odd != dd) continue;
-      if ((a.negated ? P->table_neg[q] : P->table_pos[q]) != 255) continue;   // one candidate per table and sign
+    for (int q = 0; q < n_tables; ++q) {
+      const int o = table_atom[q];
+      if (P->cand[o].cls != cl || (((A.dd_mask >> o) & 1u) != 0) != dd || ((table_signs[q] >> a.negated) & 1)) continue;
       if (dd ? (A.atoms[o].n_entries == a.n_entries) : same_table(A.atoms[o], a)) t = q;
     }
     if (t < 0) {
-      if (P->n_tables == SOP_MAX_TABLES) return SOP_ERR_ALPHABET;
-      t = P->n_tables++;
-      P->table_atom[t] = (unsigned char)i;
-      P->table_cls[t] = (unsigned char)cl;
-      P->table_pos[t] = P->table_neg[t] = 255;
+      if (n_tables == SOP_MAX_TABLES) return SOP_ERR_ALPHABET;
+      t = n_tables++;
+      table_atom[t] = i;
+      table_signs[t] = 0;
     }
-    (a.negated ? P->table_neg[t] : P->table_pos[t]) = (unsigned char)i;
-    P->cls_tables[cl] |= (unsigned char)(1u << t);
-    P->cand[i].table = (unsigned char)t;
+    table_signs[t] |= 1 << a.negated;
   }
-  // cell geometry per LUT class: cell width (in u) below the smallest threshold gap, a power of two
-  int rows = 1;
+  // groups of up to eight table candidates of one class (never more groups than distinct tables: eight candidates that differ
+  // have at least four)
   for (int c = 0; c < P->n_classes; ++c) {
-    ClassDev& C = P->cls[c];
-    if (C.kind != SOP_KIND_LUT) continue;
-    double gap = 1e30;
-    bool any_dd = false;
-    for (int q = 0; q < P->n_tables; ++q) {
-      if (P->table_cls[q] != c) continue;
-      const int o = P->table_atom[q];
-      if ((A.dd_mask >> o) & 1u) { any_dd = true; continue; }
-      gap = fmin(gap, min_threshold_gap(A.atoms[o]));
+    if (P->cls[c].kind != SOP_KIND_LUT) continue;
+    for (int i = 0; i < P->cls[c].n_cand; i += GROUP_CAND) {
+      if (P->n_groups == SOP_MAX_CLASSES) return SOP_ERR_ALPHABET;
+      GroupDev& G = P->groups[P->n_groups++];
+      G.cls = (unsigned char)c;
+      G.n = (unsigned char)(P->cls[c].n_cand - i < GROUP_CAND ? P->cls[c].n_cand - i : GROUP_CAND);
+      G.np = (unsigned char)((G.n + 1) / 2);
+      for (int q = 0; q < GROUP_CAND; ++q) G.cand[q] = P->cls[c].cand[i + (q < G.n ? q : G.n - 1)];
+      G.inv_range = (float)(1.0 / (2.5 * (double)P->cls[c].tmax));       // the cells cover |u| <= 1.25 tmax, the end cells everything beyond
     }
-    if (gap > C.tmax) gap = C.tmax / 8.0;
-    if (any_dd) gap = fmin(gap, C.tmax / 48.0);           // a data-derived table: assume a finer grid
-    int e = (int)floor(log2(gap * 0.999));
-    double h = ldexp(1.0, e);
-    const double reach = 1.25 * C.tmax;                    // scale rounding can push |u| a little above tmax
-    while (2 * (int)ceil(reach / h) + 1 > 257) h *= 2.0;   // bound the table size
-    C.c_half = (int)ceil(reach / h);
-    C.invh = (float)(1.0 / h);
-    rows = rows > 2 * C.c_half + 1 ? rows : 2 * C.c_half + 1;
   }
-  P->rows = rows;
-  P->a_pad = n | 1;
   // slots: pair-type first (singles as (a, a)), then signed.  With keep_loaded an entry whose candidates were all
   // evaluated by an earlier call is not formed again: the tables hold it.
   P->keep_loaded = keep_loaded;
@@ -1260,10 +1494,27 @@ static int deal_tasks(const Plan& P, int task0, int n, SeatsDev* seats) {
   return tpw > 0 ? tpw : 1;
 }
 
-size_t sweep_smem_bytes(const Plan& P) {
-  size_t b = (size_t)P.n_tables * P.rows * 16 * 8;
-  b += SOP_MAX_TABLES * 32 * 4 * 2 + SOP_MAX_TABLES * 4 + SOP_MAX_CLASSES * 8;
-  return (b + 15) & ~(size_t)15;
+// Shared memory of the sweep: per group its rows (one more than its decision points) and its cells, 128 bytes per cell and
+// 128 or 256 per row with the copies; every group gets the same number of cells, the largest of 1280, 640, 320, ... that fits
+// `limit` bytes in all (a cell then rarely holds more than three decision points; a group where one does is searched instead).
+constexpr size_t SWEEP_C_BYTES = (size_t)TB * SOP_G * sizeof(float);
+static size_t sweep_layout(const AtomsDev& A, Plan* P, size_t limit) {
+  for (int cells = 640;; cells /= 2) {
+    size_t b = (sizeof(GroupScratch) + 127) & ~(size_t)127;
+    for (int g = 0; g < P->n_groups; ++g) {
+      GroupDev& G = P->groups[g];
+      int breaks = 0;
+      for (int q = 0; q < G.n; ++q) breaks += A.atoms[G.cand[q]].n_entries - 1;
+      G.row_off = (unsigned)b;
+      G.plane_bytes = (unsigned)(breaks + 1) * 128u;
+      b += (size_t)G.plane_bytes * (size_t)((G.np + 1) / 2);
+      G.cell_off = (unsigned)b;
+      G.n_cells = cells;
+      b += (size_t)(cells + 1) * (G.np == 1 ? 256 : 128);
+    }
+    b += SWEEP_C_BYTES;                           // the threads' channel norms
+    if (b <= limit || cells <= 20) return b;
+  }
 }
 
 // the ring of tile buffers, the signed-best columns, the lanes' accumulators; at least the room the closing
@@ -1276,27 +1527,9 @@ static size_t reduce_smem_bytes(const SeatsDev& S, int n_stage, bool pair = fals
   return ((b > fin ? b : fin) + 127) & ~(size_t)127;
 }
 
-// Doubles the cell width of the LUT class with the most rows (its tables then hold several thresholds per cell
-// where they are dense, and such tables take the exact binary search).  False when no class can shrink further.
 // Two tiles per step in the reduction (see reduce_kernel) wherever the shared memory allows; sop_pair_search_tuning
 // turns it off (tests compare both paths: the results are the same bit for bit).
 static bool g_reduce_pairs = true;
-
-static bool coarsen_cells(Plan* P) {
-  int pick = -1;
-  for (int c = 0; c < P->n_classes; ++c)
-    if (P->cls[c].kind == SOP_KIND_LUT && P->cls[c].c_half > 1 && (pick < 0 || P->cls[c].c_half > P->cls[pick].c_half)) pick = c;
-  if (pick < 0) return false;
-  ClassDev& C = P->cls[pick];
-  C.invh *= 0.5f;
-  C.c_half = (int)ceil(1.25 * (double)C.tmax * (double)C.invh);
-  if (C.c_half < 1) C.c_half = 1;
-  int rows = 1;
-  for (int c = 0; c < P->n_classes; ++c)
-    if (P->cls[c].kind == SOP_KIND_LUT) rows = rows > 2 * P->cls[c].c_half + 1 ? rows : 2 * P->cls[c].c_half + 1;
-  P->rows = rows;
-  return true;
-}
 
 }  // namespace sop
 
@@ -1370,14 +1603,19 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
 
   // everything that can refuse the call is decided before the first enqueue
   constexpr size_t SMEM_MAX = 226 * 1024;   // 227 KB per CTA minus the kernels' few static bytes
-  size_t smem = sweep_smem_bytes(P);
-  while (smem > SMEM_MAX && coarsen_cells(&P)) smem = sweep_smem_bytes(P);   // cell tables too large: coarser cells, exact search where needed
+  int max_np = 0;
+  for (int g = 0; g < P.n_groups; ++g) max_np = P.groups[g].np > max_np ? P.groups[g].np : max_np;
+  const size_t smem = sweep_layout(A, &P, SMEM_MAX);
   if (smem > SMEM_MAX) return SOP_ERR_ALPHABET;
   const int sms = num_sms();
   // persistent grid: one CTA per SM, fewer when the layer is small; at least enough threads for one row
-  long long grid = (L.NB + TB - 1) / TB;
-  if (grid > sms) grid = sms;
-  const long long min_grid = (L.nbk + TB - 1) / TB;
+  // (a small layer is spread over all of them: its CTAs build the tables with all their threads and evaluate with tba)
+  long long tba = ((L.NB + sms - 1) / sms + 31) / 32 * 32;
+  if (tba > TB) tba = TB;
+  long long grid = (L.NB + tba - 1) / tba;
+  const long long resident = (long long)sms * (max_np == 0 ? 2 : 1);
+  if (grid > resident) grid = resident;
+  const long long min_grid = (L.nbk + tba - 1) / tba;
   if (grid < min_grid) grid = min_grid;
   if (grid > MAX_GRID) return SOP_ERR_SHAPE;
   // the reduction: up to MAX_TPW tasks per warp and launch, more launches for more tasks; persistent grid over tiles.
@@ -1408,7 +1646,11 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   if ((rc = profile_mark(SOP_PROFILE_PREPASS, 1, st))) return rc;
   DeviceFacts* facts = device_facts();
   if (!facts->search_attr_set) {
-    SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
 #define SOP_REDUCE_ATTR(SE, T, BK, PR) \
   SOP_CUDA_TRY(cudaFuncSetAttribute(reduce_kernel<SE, T, BK, PR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX))
     SOP_REDUCE_ATTR(false, 1, false, false); SOP_REDUCE_ATTR(false, 2, false, false); SOP_REDUCE_ATTR(false, 3, false, false);
@@ -1422,7 +1664,14 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   }
   if ((rc = profile_mark(SOP_PROFILE_SWEEP, 0, st))) return rc;
   if (eval_mask) {
-    sweep_kernel<<<(int)grid, TB, smem, st>>>(L, P, A, F, hdr, cos_cols, sse_cols, prev_result_dev);
+    const unsigned c_off = (unsigned)(smem - SWEEP_C_BYTES);
+#define SOP_LAUNCH_SWEEP(NP) sweep_kernel<NP><<<(int)grid, TB, smem, st>>>(L, P, A, F, hdr, cos_cols, sse_cols, prev_result_dev, c_off, (unsigned)tba)
+    if (max_np == 0) SOP_LAUNCH_SWEEP(0);
+    else if (max_np == 1) SOP_LAUNCH_SWEEP(1);
+    else if (max_np == 2) SOP_LAUNCH_SWEEP(2);
+    else if (max_np == 3) SOP_LAUNCH_SWEEP(3);
+    else SOP_LAUNCH_SWEEP(4);
+#undef SOP_LAUNCH_SWEEP
     SOP_CUDA_TRY(cudaGetLastError());
   }
   if ((rc = profile_mark(SOP_PROFILE_SWEEP, 1, st))) return rc;

@@ -1,0 +1,52 @@
+"""GPU parity of the sweep's joint evaluation of table candidates where it can go wrong: more candidates of a class than one
+group holds, an odd number of them, table values that are no bf16 numbers, lookup cells with three and with more decision
+points, and block sums outside the range of the fast cosine.  Per-block values bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_14929_b200 import inputs as I
+
+from .test_gpu_parity import B, check_search  # noqa: F401  (B is a fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def _table(name, lut, n_bits=4):
+    return I.Atom(name, n_bits, I.KIND_LUT, 0, 16, float(np.abs(lut).max()), np.sort(np.asarray(lut, dtype=np.float32)))
+
+
+def _dense(step, n):
+    """16 entries, n + 1 of them `step` apart around 0.3 (n decision points `step` apart), the rest spread out."""
+    return np.concatenate([np.linspace(-1.0, 0.1, 15 - n), 0.3 + step * np.arange(n + 1)[:n], [1.0]])
+
+
+def _alphabet(kind):
+    rng = np.random.default_rng(11)
+    if kind == "twelve":          # one class, twelve candidates: a group of eight and one of four
+        extra = [_table(f"r{i}", np.concatenate([[-1.0, 1.0], I.snap_bf16(rng.uniform(-0.95, 0.95, 14))])) for i in range(2)]
+        return I.alphabet(["NF4", "SH4", "BOF4", "Split87"]) + [x for a in extra for x in (a, a.negation())]
+    if kind == "odd":             # five candidates without negations, values with full fp32 significands
+        return [_table(f"f{i}", np.concatenate([[-1.0, 1.0], rng.uniform(-0.99, 0.99, 14)])) for i in range(5)]
+    if kind == "cell3":           # a cell with three decision points (cells are 2.5 / 640 wide)
+        return [_table("c3", _dense(5e-4, 4))] + I.alphabet(["NF4"])
+    if kind == "cell6":           # more than three: the group is searched
+        a = _table("c6", _dense(2e-4, 7))
+        return [a, a.negation()] + I.alphabet(["NF4", "SH4"])
+    return I.alphabet(["NF5", "SH5", "BOF5", "E2M2"])      # two classes: six candidates and two
+
+
+@pytest.mark.parametrize("kind,fmt_name", [("twelve", "E5M6"), ("odd", "UE4M4"), ("cell3", "E4M5"), ("cell6", "UE4M6"), ("classes", "E4M3")])
+def test_groups_of_candidates_match_oracle(B, kind, fmt_name):
+    check_search(B, I.tiny_layer(21, 37, 272), fmt_name, _alphabet(kind))
+
+
+@pytest.mark.parametrize("fmt_name", ["E8M7", "UE4M4", "UE8M0"])
+def test_block_sums_of_any_magnitude(B, fmt_name):
+    # rows from 2^-64 to 2^60: norms and dot products from below 2^-80 to above 2^80 take the general cosine, the others the
+    # fast one; a zero row, a row with one non-zero weight per block
+    L = I.tiny_layer(22, 24, 256)
+    W = L.W.float() * (2.0 ** torch.linspace(-64, 60, 24).round())[:, None]
+    W[5] = 0
+    W[6] = torch.where(torch.arange(256) % 16 == 3, W[6], torch.zeros(256))
+    check_search(B, I.Layer(W.to(torch.bfloat16), L.X), fmt_name, I.alphabet(["NF4", "SH4"], fp=["E2M3", "E4M3"]))
