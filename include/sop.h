@@ -199,8 +199,10 @@ int sop_channel_norms_static(const float* X_dev, long long T, long long K, long 
  *   candidate of load_mask (SOP_ERR_RANGE otherwise). */
 int sop_pair_search_workspace(long long M, long long K, int n_atoms, size_t* bytes);
 /* Launch shape of the reduction of the table entries (no counterpart in the paper): reduce_tile_pairs = 1 (the
- * default) lets a CTA work on two tiles of 256 blocks at a time where its shared memory allows, 0 keeps it to one.
- * The additions and their order are the same: results do not depend on it.  SOP_ERR_RANGE for other values. */
+ * default) lets a CTA fill as many tile buffers ahead of its arithmetic as its shared memory holds (up to four), 0 keeps
+ * it to two.  The additions and their order are the same: results do not depend on it.  SOP_ERR_RANGE for other values.
+ * Inside the reduction the warps of a CTA wait for copies into those buffers; every wait is bounded.  Should one give
+ * up, every entry that the call forms is left undefined (n_sel1 = -1). */
 int sop_pair_search_tuning(int reduce_tile_pairs);
 int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, const float* c_dev, int g,
                     const sop_scale_fmt* fmt, int k_mode, const sop_atom* atoms, int n_atoms,

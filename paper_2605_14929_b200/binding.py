@@ -311,7 +311,7 @@ def sop_wr_extract(W: torch.Tensor, c: torch.Tensor, fmt, atoms: Sequence, codes
 
 
 def pair_search_tuning(reduce_tile_pairs: bool = True) -> None:
-    """Launch shape of the reduction kernel (results do not depend on it)."""
+    """Tile buffers of the reduction kernel: as many as fit, or two (results do not depend on it)."""
     _check(lib().sop_pair_search_tuning(1 if reduce_tile_pairs else 0), "sop_pair_search_tuning")
 
 

@@ -13,16 +13,15 @@
 //                    go through the conversion instructions.  Writes the per-block cosine and squared error of each candidate
 //                    as one column.                                          (bound by register operands and issue)
 //   reduce_kernel    reads the columns of every candidate present in the call (those just written
-//                    and those an earlier call wrote) tile by tile into shared memory and forms
-//                    the table entries: a warp owns a few "tasks" (one anchor column against up to
-//                    four partner columns, so five columns are fetched for up to five entries), a
-//                    lane owns eight blocks of every tile, the sums of those eight are fp32 and go
-//                    to FP64 accumulators after every tile (two tiles per step where the shared
-//                    memory allows: the accumulators are then touched once per sixteen blocks).
+//                    and those an earlier call wrote) tile by tile into shared memory by bulk copies and forms
+//                    the table entries: a warp owns a bundle of entries among up to six columns and keeps their
+//                    sums in registers (fp32 over eight blocks, then FP64).
 //                    The CTA that finishes last adds the per-CTA partials in a fixed order
 //                    (deterministic), writes the tables and picks the best pair / best single.
 #include <math.h>
 #include <string.h>
+
+#include <vector>
 
 #include "sop_device.cuh"
 
@@ -30,7 +29,7 @@ namespace sop {
 
 constexpr int TB = 512;             // threads per CTA of the sweep kernel (one CTA per SM; two where it has no table candidates)
 constexpr int MAX_SLOTS = 192;      // pair slots per call: 16 singles + 120 pairs + 36 signed < 192
-constexpr int MAX_GRID = 1024;
+constexpr int MAX_GRID = 1056;
 constexpr float MAGIC = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
 
 struct CandDev { unsigned char cls, kind, neg, pad; };
@@ -57,42 +56,40 @@ struct GroupDev {
 };
 struct SlotDev { unsigned char type, i0, i1, pad; };  // type 0: pair (i0, i1) (i0 == i1: single); 1: signed (i0, i0+1, i1, i1+1)
 
-// One unit of work of the reduction: an anchor candidate against up to four partners.  Entry q is the table slot
-// slot[q] of the pair {anchor, part[q]}; rev = 0: the anchor is the first candidate of all its entries (it keeps a
-// tie), rev = 1: it is the second one.  self_slot is the slot of the anchor alone (255: none).  sgn = 1: anchor and
-// partners are base atoms and stand for the better of the atom and its negation (a signed four-way entry).
-constexpr int TASK_PART = 4;
-constexpr int MAX_TASKS = 96;
-constexpr int MAX_TPW = 3;             // tasks per warp and launch
-struct TaskDev {
-  unsigned char anchor, n_part, self_slot, sgn, rev, pad[3];
-  unsigned char part[TASK_PART], slot[TASK_PART];
+// One unit of work of the reduction (see reduce_run): up to six columns and the entries among them that a warp forms.
+// shape 0: a[0..3], their singles and pairs (0,1) (0,2) (0,3) (1,2) (1,3) (2,3); 1: the same of a[0..1]; 2: entry 4 j + i pairs
+// a[i] (first candidate) with b[j]; 3: the same with b[0] alone; 4: as 2 with a[i] as the second candidate.  slot: the table slot
+// of every entry (255: none).  sgn = 1: the columns stand for base atoms (neg: the column of the negation).
+constexpr int RTB = 512;                           // threads per CTA of the reduction (one CTA per SM): fifteen warps form
+constexpr int RED_WARPS = 15;                      // entries, one issues the copies
+constexpr int BUNDLE_ENT = 10, MAX_BUNDLES = RED_WARPS;
+struct BundleDev {
+  unsigned char shape, sgn, first_warp, n_warps;
+  unsigned char a[4], b[2], neg[6];
+  unsigned char slot[BUNDLE_ENT];
 };
-// One launch of the reduction: per warp its tasks (255: empty seat) and the first accumulator seat of each; the
-// candidates whose columns the launch fetches (col_slot: candidate -> column of the tile buffers, 255: not fetched)
-// and the base atoms whose signed-best column it forms (sb_slot likewise).
-struct SeatsDev {
-  unsigned char task[8][MAX_TPW];
-  unsigned short acc0[8][MAX_TPW];
-  unsigned char col_slot[SOP_MAX_ATOMS], sb_slot[SOP_MAX_ATOMS];
-  unsigned char cols[SOP_MAX_ATOMS], bases[SOP_MAX_ATOMS];      // the inverse lists
-  int n_cols, n_bases, n_seats;
+// One launch of the reduction: its bundles, the bundle of every warp, the candidates whose columns it fetches.
+struct BundlesDev {
+  int n_bundles, n_cols, n_warps;
+  unsigned char warp_bundle[RED_WARPS], cols[SOP_MAX_ATOMS];
+  BundleDev bundle[MAX_BUNDLES];
+};
+struct RedPlan {                            // what the reduction knows of the call
+  int n_atoms, n_classes, n_slots, k_from_result, keep_loaded;
+  unsigned eval_mask, load_mask, lut_mask;
+  unsigned char cls_of[SOP_MAX_ATOMS];
+  signed char k_src[SOP_MAX_CLASSES];
+  SlotDev slots[MAX_SLOTS];
 };
 
 struct Plan {
-  int n_atoms, n_classes, n_groups, n_slots, n_pair_slots;
+  int n_atoms, n_classes, n_groups;
   int k_mode;
   unsigned eval_mask, load_mask;   // candidates evaluated here / read from the per-block arrays of an earlier call
   int k_from_result;               // 1: shifts and max|W| come from the result block of an earlier call, no prepass
-  int n_bases;                               // base atoms (each followed by its negation) of the signed table
-  unsigned char base_atom[SOP_MAX_ATOMS];    // signed-best column n_atoms + b holds the better of base_atom[b] and its negation
   CandDev cand[SOP_MAX_ATOMS];
   ClassDev cls[SOP_MAX_CLASSES];
   GroupDev groups[SOP_MAX_CLASSES];
-  SlotDev slots[MAX_SLOTS];
-  int keep_loaded;                            // entries among loaded candidates stay as the tables hold them
-  int n_tasks;
-  TaskDev tasks[MAX_TASKS];
 };
 
 struct WsHeader {
@@ -100,16 +97,19 @@ struct WsHeader {
   int cls_k[SOP_MAX_CLASSES];
   float cls_pot[SOP_MAX_CLASSES];
   unsigned done_prepass, done_reduce;  // CTAs that have finished (the last one does the serial tail)
-  int pad[5];
+  unsigned reduce_error;               // a wait of the reduction gave up
+  int pad[4];
 };
-struct Partial { double gap, sse; long long n1, nneg; };
+// Sums of one entry over a CTA's blocks: gap and error, blocks of the second candidate and of a negated winner (31 bits each).
+// Kept as two arrays [CTA][slot] so that the reads of the closing reduction are contiguous.
+struct PartialSums { double2* sums; uint2* counts; };
 
 static size_t ws_hist_off() { return 256; }
 // after the histograms: max|W| as the prepass found it (the header is cleared by every call, the histograms and this
 // word stay until the next prepass)
 static size_t ws_wmax_off() { return 256 + sizeof(unsigned) * SOP_MAX_CLASSES * SOP_HIST_BINS; }
 static size_t ws_part_off() { return ws_wmax_off() + 256; }
-static size_t ws_total() { return ((ws_part_off() + sizeof(Partial) * (size_t)MAX_GRID * MAX_SLOTS) + 255) & ~(size_t)255; }
+static size_t ws_total() { return ((ws_part_off() + (sizeof(double2) + sizeof(uint2)) * (size_t)MAX_GRID * MAX_SLOTS) + 255) & ~(size_t)255; }
 
 struct LayerArgs {
   const uint16_t* W;
@@ -831,365 +831,349 @@ __global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArg
 
 // ---------------------------------------------------------------------------------------------
 // The reduction of the per-block columns into table entries.
-//   A CTA takes tiles of RTILE blocks.  The columns (cosines and errors of every candidate that a task of the
-//   launch touches) of a tile are brought into a ring of shared-memory buffers by 16-byte asynchronous copies
-//   (cp.async, every thread a few), up to three tiles ahead of the arithmetic; a thread waits for its own copy
-//   groups and the one barrier per tile makes everybody's visible.  (One-dimensional bulk copies with an
-//   mbarrier, one kilobyte per column, were measured first: the per-request cost of twenty small requests per
-//   tile bound the kernel.)  16-byte copies need aligned addresses, which holds when the number of blocks is a
-//   multiple of four and the arrays are 16-byte aligned; otherwise (odd small layers) the tile is fetched with
-//   plain loads.  Nothing in this kernel spins on a flag.
-//   A warp owns up to three tasks.  A lane owns eight blocks of the tile (two runs of four): per
-//   entry it sums eight gaps 1 - cos (exact in fp32 for cos in [0.5, 1]) and eight errors in fp32, then adds
-//   both to the lane's FP64 accumulators of that entry, which live in shared memory.  At the end the 32 lanes'
-//   accumulators of an entry are added in lane order: the result depends on the grid size only.
-//   A signed four-way entry {i, -i, j, -j} is the two-way entry of "the better of i and -i" and "the better of
-//   j and -j" (ties to the atom; the sign of the error marks a negated winner), formed on the fly from the two
-//   columns of each base atom.  A block beyond the end of the layer reads as (cos 1, error 0): it adds nothing.
+//   A CTA takes tiles of 768 blocks (256 in a small layer).  The columns (cosines and errors of every candidate that the launch
+//   needs) of a tile are brought into a ring of up to four shared-memory buffers by bulk copies, one per row, that one thread
+//   issues; per buffer an mbarrier says that it has landed and another that its readers are done.
+//   The entries are grouped into "bundles": a few columns and the entries among them that a warp forms with everything in
+//   registers -- four columns with their singles and six pairs, or four first candidates against two second ones.  A bundle
+//   belongs to one or more warps (dealt by its cost), which take every n-th run of 128 blocks, four blocks per lane.
+//   An entry costs one comparison and five predicated additions per block (no selections: both outcomes are additions under
+//   opposite predicates, so that only the comparison runs on the ALU); its gap 1 - cos and error are summed in fp32 over eight
+//   blocks (gaps exactly, for cosines in [0.5, 1]) and then go to FP64 registers of the lane.
+//   At the end the lanes' sums are added by a fixed shuffle tree, a bundle's warps in order: the result depends on the launch
+//   shape only.
+//   A signed four-way entry {i, -i, j, -j} is the two-way entry of "the better of i and -i" and "the better of j and -j"
+//   (ties to the atom), formed on the fly from the two columns of each base atom.
+//   A block beyond the end of the layer reads as (cos 1, error 0): it adds nothing.
+// What bounds it: at an unsigned format the copies (28672 x 8192, both calls of a pass: 2.1 GB of columns in 407 us, 325 us at the
+// measured copy rate; 523 us with tasks whose sums lived in shared memory), at a signed format issue (8192 x 8192: 92 + 80 us, 148 +
+// 125 us before).  A lane of the copying warp per row matters: one thread issuing twenty copies a tile took 30 % longer; so does the
+// tail of the last CTA (see finalize_body): 256 x 1024 takes 11 us, 16 us with the serial tail.
 // ---------------------------------------------------------------------------------------------
-constexpr int RTB = 256;              // threads per CTA of the reduction: eight warps
-constexpr int RTILE = 256;            // blocks per tile: eight per lane
-constexpr int ENT = TASK_PART + 1;    // entries of a task: the anchor alone, then its partners
-constexpr int MAX_STAGE = 4;           // tile buffers of the ring
+constexpr int RUNIT = 128;            // blocks of a run: four per lane
+constexpr int MAX_STAGE = 4;          // tile buffers of the ring
 
-__device__ void finalize_body(const LayerArgs& L, const Plan& P, int grid, const Partial* partials, sop_pair_stat* s_pair, sop_pair_stat* s_sig,
-                              Partial* s_red, sop_pair_stat* pair_table, sop_pair_stat* signed_table, sop_search_result* res,
-                              const int* cls_k, float wmax);
+__device__ void finalize_body(const LayerArgs& L, const RedPlan& P, int grid, PartialSums partials, unsigned char* smem, sop_pair_stat* pair_table,
+                              sop_pair_stat* signed_table, sop_search_result* res, const sop_search_result* prev, WsHeader* hdr);
 
-constexpr int ACC_BYTES = 32 * 20;     // accumulators of one entry: 32 lanes x (two FP64 sums, two 16-bit counts)
-
-__device__ __forceinline__ void lds128(unsigned addr, float (&v)[4]) {
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(addr));
+// Sums over the 32 lanes of N values each: in every step a lane hands half of its values to its partner and adds the partner's share
+// of the other half, so that N values take about N + 5 exchanges.  Afterwards the lane whose return value is q >= 0 holds the sum of
+// value q in v[0] (lanes in pairs hold the same one); -1: the lane holds none.
+template <int N, int O>
+__device__ __forceinline__ void lane_sums_step(double* v, int lane, int& idx, int& cnt) {
+  if constexpr (O > 0) {
+    constexpr int H = (N + 1) / 2;
+    const bool up = (lane & O) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const double hi = i + H < N ? v[i + H] : 0.0;
+      const double got = __shfl_xor_sync(0xFFFFFFFFu, N > 1 ? (up ? v[i] : hi) : v[i], O);
+      v[i] = (N > 1 && up ? hi : v[i]) + got;
+    }
+    if (N > 1) { idx += up ? H : 0; cnt = up ? cnt - H : min(cnt, H); }
+    lane_sums_step<H, O / 2>(v, lane, idx, cnt);
+  }
+}
+template <int N>
+__device__ __forceinline__ int lane_sums(double (&v)[N], int lane) {
+  int idx = 0, cnt = N;
+  lane_sums_step<N, 16>(v, lane, idx, cnt);
+  return cnt > 0 ? idx : -1;
 }
 
-// The accumulators of one entry and lane, in shared memory: FP64 sums (gap, error) at sums + seat * 512 + lane * 16 and
-// counts (second candidate chosen, negated winner; 16 bits each: a lane sees at most 8 blocks per tile and a CTA a few
-// thousand tiles) at counts + seat * 128 + lane * 4.
-// NT = 1: the sums of one tile; NT = 2: of two tiles, added one after the other (the same additions in the same order
-// as two calls, with one load and one store of the accumulators).
-template <int NT>
-__device__ __forceinline__ void acc_add(unsigned sums, unsigned counts, const float (&cg)[NT], const float (&ce)[NT], const int (&n1)[NT],
-                                        const int (&nn)[NT]) {
-  double g, e;
-  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(g), "=d"(e) : "r"(sums));
-#pragma unroll
-  for (int t = 0; t < NT; ++t) { g += (double)cg[t]; e += (double)ce[t]; }
-  asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(sums), "d"(g), "d"(e) : "memory");
-  unsigned c;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(c) : "r"(counts));
-#pragma unroll
-  for (int t = 0; t < NT; ++t) c += (unsigned)n1[t] + ((unsigned)nn[t] << 16);       // neither half can carry: both stay below 2^16
-  asm volatile("st.shared.u32 [%0], %1;" ::"r"(counts), "r"(c) : "memory");
+// One entry on one block: the second candidate takes the block when it is strictly better.  v1 / v0: what the count gains
+// when the second / first candidate wins (unsigned entries: 1 and nothing).
+template <bool SEL_ERR, bool SGN>
+__device__ __forceinline__ void entry_add(float& g, float& e, float& n, float c0, float c1, float g0, float g1, float e0, float e1, float v0, float v1) {
+  const float x = SEL_ERR ? e0 : c1, y = SEL_ERR ? e1 : c0;            // strictly better: x > y
+  if (SGN)
+    asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %3, %4;\n\t@p add.rn.f32 %0, %0, %6;\n\t@!p add.rn.f32 %0, %0, %5;\n\t@p add.rn.f32 %1, %1, %8;\n\t"
+        "@!p add.rn.f32 %1, %1, %7;\n\t@p add.rn.f32 %2, %2, %10;\n\t@!p add.rn.f32 %2, %2, %9;\n\t}"
+        : "+f"(g), "+f"(e), "+f"(n) : "f"(x), "f"(y), "f"(g0), "f"(g1), "f"(e0), "f"(e1), "f"(v0), "f"(v1));
+  else
+    asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %3, %4;\n\t@p add.rn.f32 %0, %0, %6;\n\t@!p add.rn.f32 %0, %0, %5;\n\t@p add.rn.f32 %1, %1, %8;\n\t"
+        "@!p add.rn.f32 %1, %1, %7;\n\t@p add.rn.f32 %2, %2, 0f3F800000;\n\t}"
+        : "+f"(g), "+f"(e), "+f"(n) : "f"(x), "f"(y), "f"(g0), "f"(g1), "f"(e0), "f"(e1));
 }
 
-// One task on the lane's eight blocks of one tile (blocks 4 lane .. 4 lane + 3 and the same 128 further on: two 128-bit
-// loads per column and array).  The code is the same for every warp and task -- tasks differ in data only -- and small:
-// a loop over the task's partners whose body handles the eight blocks.  Per entry the eight gaps and errors are summed
-// in fp32 and added to the lane's FP64 accumulators.
-//   cos_base / sse_base: shared-memory addresses of the tile's columns (for a signed task the signed-best columns);
-//   tk: the task (in shared memory); sums / counts: shared-memory addresses of this lane's accumulators of the task's
-//   first seat: the anchor alone if the task has that entry, then the partners.
-//   NT = 2: the same task on two tiles at once -- the tile in work and the one `pair_off` bytes further on in shared
-//   memory -- so that the accumulators are loaded and stored once for both.
-template <bool SEL_ERR, bool SGN, bool REV, int NT>
-__device__ __forceinline__ void run_task(const TaskDev* __restrict__ tk, unsigned cos_base, unsigned sse_base, unsigned pair_off, int lane,
-                                         unsigned sums, unsigned counts) {
-  constexpr unsigned COL = RTILE * 4u;          // bytes of one column
-  const unsigned lane_off = (unsigned)lane * 16u;
-  float ac0[NT][4], ac1[NT][4], ae0[NT][4], ae1[NT][4], ga0[NT][4], ga1[NT][4];
-#pragma unroll
-  for (int t = 0; t < NT; ++t) {
-    const unsigned a = (unsigned)tk->anchor * COL + lane_off + (unsigned)t * pair_off;
-    lds128(cos_base + a, ac0[t]); lds128(cos_base + a + 512u, ac1[t]);
-    lds128(sse_base + a, ae0[t]); lds128(sse_base + a + 512u, ae1[t]);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) { ga0[t][r] = __fsub_rn(1.0f, ac0[t][r]); ga1[t][r] = __fsub_rn(1.0f, ac1[t][r]); }
-  }
-  if (tk->self_slot != 255) {
-    float cg[NT], ce[NT];
-    int n1[NT], nn[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      cg[t] = 0.0f; ce[t] = 0.0f; n1[t] = 0; nn[t] = 0;
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        cg[t] = __fadd_rn(cg[t], ga0[t][r]); ce[t] = __fadd_rn(ce[t], fabsf(ae0[t][r]));
-        cg[t] = __fadd_rn(cg[t], ga1[t][r]); ce[t] = __fadd_rn(ce[t], fabsf(ae1[t][r]));
-        if (SGN) nn[t] += (int)(__float_as_uint(ae0[t][r]) >> 31) + (int)(__float_as_uint(ae1[t][r]) >> 31);
-      }
+struct ReduceCtx {
+  long long NB;
+  unsigned n_tiles;                    // tiles of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...
+  int n_cols, units, n_stage;
+  int row_len;                         // floats from one row of a tile buffer to the next
+  const float* ring;                   // [stage][column][cosines, errors][row_len]
+  unsigned full, empty;                // shared-memory addresses of the stages' barriers (8 bytes each)
+  const int* row_off;                  // first float of every row in a tile buffer
+  WsHeader* hdr;
+};
+
+// Waits for the phase of an mbarrier that completes with the given parity.  Bounded: a warp that gives up raises the error flag and
+// goes on without waiting; the tables of the call are then marked undefined.
+__device__ __forceinline__ void mbar_wait(unsigned bar, unsigned parity, WsHeader* hdr) {
+  for (unsigned tries = 0;; ++tries) {
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return;
+    if (tries > (1u << 20) || ((tries & 1023u) == 1023u && *(volatile unsigned*)&hdr->reduce_error)) {
+      atomicExch(&hdr->reduce_error, 1u);
+      return;
     }
-    acc_add<NT>(sums, counts, cg, ce, n1, nn);
-    sums += 512u; counts += 128u;            // the partners' seats follow
-  }
-  const int np = tk->n_part;
-#pragma unroll 1
-  for (int q = 0; q < np; ++q) {
-    float cg[NT], ce[NT];
-    int n1[NT], nn[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const unsigned b = (unsigned)tk->part[q] * COL + lane_off + (unsigned)t * pair_off;
-      float bc0[4], bc1[4], be0[4], be1[4];
-      lds128(cos_base + b, bc0); lds128(cos_base + b + 512u, bc1);
-      lds128(sse_base + b, be0); lds128(sse_base + b + 512u, be1);
-      cg[t] = 0.0f; ce[t] = 0.0f; n1[t] = 0; nn[t] = 0;
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        // mu: the entry's second candidate is strictly better and takes the block.  REV = false: the anchor is the
-        // first candidate and the partner the second; REV = true: the other way round.
-        bool mu0, mu1;
-        float g0, g1, e0, e1;
-        if (!REV) {
-          mu0 = SEL_ERR ? fabsf(be0[r]) < fabsf(ae0[t][r]) : bc0[r] > ac0[t][r];
-          mu1 = SEL_ERR ? fabsf(be1[r]) < fabsf(ae1[t][r]) : bc1[r] > ac1[t][r];
-          g0 = mu0 ? __fsub_rn(1.0f, bc0[r]) : ga0[t][r]; e0 = mu0 ? be0[r] : ae0[t][r];
-          g1 = mu1 ? __fsub_rn(1.0f, bc1[r]) : ga1[t][r]; e1 = mu1 ? be1[r] : ae1[t][r];
-        } else {
-          mu0 = SEL_ERR ? fabsf(ae0[t][r]) < fabsf(be0[r]) : ac0[t][r] > bc0[r];
-          mu1 = SEL_ERR ? fabsf(ae1[t][r]) < fabsf(be1[r]) : ac1[t][r] > bc1[r];
-          g0 = mu0 ? ga0[t][r] : __fsub_rn(1.0f, bc0[r]); e0 = mu0 ? ae0[t][r] : be0[r];
-          g1 = mu1 ? ga1[t][r] : __fsub_rn(1.0f, bc1[r]); e1 = mu1 ? ae1[t][r] : be1[r];
-        }
-        cg[t] = __fadd_rn(cg[t], g0); ce[t] = __fadd_rn(ce[t], fabsf(e0));
-        cg[t] = __fadd_rn(cg[t], g1); ce[t] = __fadd_rn(ce[t], fabsf(e1));
-        n1[t] += (mu0 ? 1 : 0) + (mu1 ? 1 : 0);
-        if (SGN) nn[t] += (int)(__float_as_uint(e0) >> 31) + (int)(__float_as_uint(e1) >> 31);
-      }
-    }
-    acc_add<NT>(sums + (unsigned)q * 512u, counts + (unsigned)q * 128u, cg, ce, n1, nn);
   }
 }
 
-// PAIR (with VEC and a ring of four buffers): the CTA works on two tiles at a time -- buffers (0, 1), then (2, 3) while
-// (0, 1) are refilled -- so that a lane owns sixteen blocks per step and touches its accumulators half as often.  The
-// additions and their order are those of the one-tile path: the results are the same bit for bit.
-template <bool SEL_ERR, int TPW, bool VEC, bool PAIR>
-__global__ void __launch_bounds__(RTB, 2) reduce_kernel(LayerArgs L, Plan P, SeatsDev seats, int n_stage, int do_final, WsHeader* __restrict__ hdr,
-                                                     Partial* __restrict__ partials, const float* __restrict__ block_cos,
-                                                     const float* __restrict__ block_sse, sop_pair_stat* pair_table,
-                                                     sop_pair_stat* signed_table, sop_search_result* __restrict__ res,
-                                                     const sop_search_result* __restrict__ prev) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  const int A = seats.n_cols;                                            // columns of a tile buffer
-  const int NBUF = VEC ? n_stage : 1;                                    // tile buffers: a ring, filled n_stage - 1 tiles ahead
-  float* cos0 = reinterpret_cast<float*>(smem);                          // [NBUF][A][RTILE]
-  float* sse0 = cos0 + (size_t)NBUF * A * RTILE;                         // [NBUF][A][RTILE]
-  // signed-best columns of the tile in work
-  constexpr int NSB = PAIR ? 2 : 1;                                      // tiles in work at a time
-  float* scos = sse0 + (size_t)NBUF * A * RTILE;                         // [NSB][n_bases][RTILE]
-  float* ssse = scos + (size_t)NSB * seats.n_bases * RTILE;              // [NSB][n_bases][RTILE]
-  double2* acc_sums = reinterpret_cast<double2*>(ssse + (size_t)NSB * seats.n_bases * RTILE);   // [n_seats][32]: seat-major, then lane
-  unsigned* acc_counts = reinterpret_cast<unsigned*>(acc_sums + (size_t)seats.n_seats * 32);   // [n_seats][32]: two 16-bit counts
-  __shared__ unsigned long long s_coloff[SOP_MAX_ATOMS];   // first element of every fetched column in the arrays
-  __shared__ TaskDev s_task[RTB / 32][TPW];        // anchors and partners translated to columns of the buffers
-  __shared__ int s_acc0[RTB / 32][TPW];
-
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (lane < TPW) {
-    const int ti = seats.task[warp][lane];
-    TaskDev t;
-    if (ti != 255) {
-      t = P.tasks[ti];
-      const unsigned char* map = t.sgn ? seats.sb_slot : seats.col_slot;
-      t.anchor = map[t.anchor];
-      for (int q = 0; q < t.n_part; ++q) t.part[q] = map[t.part[q]];
-    } else { t.anchor = 0; t.n_part = 0; t.self_slot = 255; t.sgn = 2; }   // sgn 2: an empty seat
-    s_task[warp][lane] = t;
-    s_acc0[warp][lane] = seats.acc0[warp][lane];
+// The copies of this CTA's tiles by one warp, a lane per row (column, array; at most 32): one bulk copy per row and tile, started at
+// the 16-byte boundary at or below its first float and rounded up to whole 16 bytes (the neighbouring floats belong to the same
+// 16-byte granule of the array's allocation; what lies beyond the layer is masked by its readers).
+__device__ __forceinline__ void reduce_produce(const ReduceCtx& X, unsigned long long row_src) {
+  const int tile_len = X.units * RUNIT, rows = 2 * X.n_cols, lane = threadIdx.x & 31;
+  const unsigned row_bytes = 4u * (unsigned)X.row_len, dst0 = smem_u32(X.ring) + (unsigned)lane * row_bytes;
+  const unsigned skew = (unsigned)(row_src & 15u);       // (tiles are multiples of four blocks)
+  int stage = 0;
+  unsigned parity = 1;                                   // a fresh barrier passes a wait for the phase before its first
+  for (unsigned t = 0; t < X.n_tiles; ++t) {
+    const long long blk0 = ((long long)blockIdx.x + (long long)t * gridDim.x) * tile_len;
+    const unsigned len = 4u * (unsigned)min((long long)tile_len, X.NB - blk0);
+    const unsigned bytes = lane < rows ? (skew + len + 15u) & ~15u : 0u;
+    const unsigned total = __reduce_add_sync(0xFFFFFFFFu, bytes);
+    const unsigned bar = X.full + 8u * stage;
+    mbar_wait(X.empty + 8u * stage, parity, X.hdr);
+    if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(total) : "memory");
+    __syncwarp();
+    if (lane < rows)
+      asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   ::"r"(dst0 + (unsigned)(stage * rows) * row_bytes), "l"(row_src - skew + 4ull * (unsigned long long)blk0), "r"(bytes), "r"(bar) : "memory");
+    if (++stage == X.n_stage) { stage = 0; parity ^= 1u; }
   }
-  for (int i = tid; i < seats.n_seats * 32; i += RTB) { acc_sums[i] = make_double2(0.0, 0.0); acc_counts[i] = 0u; }
-  if (tid < seats.n_cols) s_coloff[tid] = (unsigned long long)seats.cols[tid] * (unsigned long long)L.NB;
-  __syncthreads();
-  const int ncols = seats.n_cols, nbases = seats.n_bases;
-  const long long n_tiles = (L.NB + RTILE - 1) / RTILE;
+}
 
-  // Every thread's share of the 16-byte copies of one tile into buffer b.  Chunk c = (column, array, run of four blocks);
-  // thread t takes the chunks t, t + 256, ...: always the same array and run, every second column.  Runs beyond the
-  // end of the layer are filled with (cos 1, error 0) instead.  One commit group per tile.
-  const int f_arr = (tid >> 6) & 1, f_ch = tid & 63;
-  const float* f_src = (f_arr ? block_sse : block_cos) + 4 * f_ch;
-  const unsigned f_dst = smem_u32(f_arr ? sse0 : cos0) + (unsigned)(((tid >> 7) * RTILE + 4 * f_ch) * 4);
-  auto fetch = [&](long long tile, int b) {
-    if (tile < n_tiles) {
-      const long long blk0 = tile * RTILE;
-      const bool live = blk0 + 4 * f_ch < L.NB;
-      unsigned dst = f_dst + (unsigned)(b * A * RTILE * 4);
-      for (int i = tid >> 7; i < ncols; i += 2, dst += 2u * RTILE * 4u) {
-        if (live) {
-          const float* src = f_src + s_coloff[i] + blk0;
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-        } else {
-          const float v = f_arr ? 0.0f : 1.0f;
-          asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "f"(v) : "memory");
-        }
-      }
-    } else if (PAIR) {
-      // the second tile of the last pair does not exist: it reads as (cos 1, error 0) and adds nothing
-      unsigned dst = f_dst + (unsigned)(b * A * RTILE * 4);
-      const float v = f_arr ? 0.0f : 1.0f;
-      for (int i = tid >> 7; i < ncols; i += 2, dst += 2u * RTILE * 4u)
-        asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "f"(v) : "memory");
+struct BundleSums {              // what a warp hands to the CTA: the sums of its bundle's entries
+  double2 sums[BUNDLE_ENT];
+  uint2 counts[BUNDLE_ENT];
+  int n_warps;                   // of the bundle, this one the first (the only one with slots)
+  unsigned char slot[BUNDLE_ENT + 2];
+};
+
+// The loop of one warp (k-th of nk of its bundle) over its runs, SHAPE 0: four columns, their singles and pairs; 1: the same of
+// two; 2: four first candidates against two second ones; 3: against one; 4: four second candidates against two first ones.
+// The runs of all tiles are dealt in one sequence (run k, k + nk, ...): a warp that has little of one tile has more of the next,
+// and the ring lets the warps drift apart by its length.
+//   VEC: rows start at 16-byte boundaries, a lane owns four consecutive blocks of a run; else every 32nd.
+template <int SHAPE, bool SGN, bool SEL_ERR, bool VEC>
+__device__ __forceinline__ void reduce_run(const ReduceCtx& X, const BundleDev& B, int k, int nk, BundleSums* part) {
+  constexpr int NA = SHAPE == 1 ? 2 : 4, NBC = SHAPE == 2 || SHAPE == 4 ? 2 : SHAPE == 3 ? 1 : 0, NC = NA + NBC;
+  constexpr int NE = SHAPE == 0 ? 10 : SHAPE == 1 ? 3 : SHAPE == 3 ? 4 : 8;
+  constexpr int BL = SGN ? 2 : 4;                   // blocks per lane and step: the registers of a signed bundle hold two
+  constexpr float NEG = 4096.0f;                    // a count gains 1 for the second candidate, 4096 for a negated winner
+  const int lane = threadIdx.x & 31, row_len = X.row_len, lane0 = VEC ? BL * lane : lane;
+  int col[SGN ? 2 * NC : NC];                       // VEC: first float of the columns in a tile buffer; else their first row
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    const int c = 2 * (i < NA ? B.a[i] : B.b[i - NA]);
+    col[SGN ? 2 * i : i] = VEC ? c * row_len + lane0 : c;
+    if (SGN) col[2 * i + 1] = VEC ? 2 * B.neg[i] * row_len + lane0 : 2 * B.neg[i];
+  }
+  double dg[NE], de[NE];
+  float g[NE], e[NE], n[NE];
+#pragma unroll
+  for (int q = 0; q < NE; ++q) { dg[q] = de[q] = 0.0; g[q] = e[q] = n[q] = 0.0f; }
+  auto load = [&](const float* bu, int cc, int arr, float (&v)[BL]) {
+    if constexpr (VEC) {
+      const float* p = bu + cc + arr * row_len;
+      if constexpr (BL == 4) { const float4 t = *reinterpret_cast<const float4*>(p); v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; }
+      else { const float2 t = *reinterpret_cast<const float2*>(p); v[0] = t.x; v[1] = t.y; }
+    } else {
+      const float* p = bu + X.row_off[cc + arr] + lane0;
+#pragma unroll
+      for (int r = 0; r < BL; ++r) v[r] = p[32 * r];
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-
-  if constexpr (PAIR) {
-    const long long step = gridDim.x;
-    long long tile = blockIdx.x;
-    fetch(tile, 0);
-    fetch(tile + step, 1);
-    int ps = 0;                  // the pair of buffers in work: (0, 1) or (2, 3)
-    for (; tile < n_tiles; tile += 2 * step) {
-      float* cosb = cos0 + (size_t)(2 * ps) * A * RTILE;
-      float* sseb = sse0 + (size_t)(2 * ps) * A * RTILE;
-      asm volatile("cp.async.wait_group 0;" ::: "memory");       // this thread's copies of both tiles have landed
-      if (nbases) {
-        __syncthreads();                                          // ... and everybody's; the previous pair's readers are done
-        for (int t = 0; t < 2; ++t)
-          for (int i = 0; i < nbases; ++i) {
-            const int a = seats.bases[i], cp = seats.col_slot[a], cn = seats.col_slot[a + 1];
-            const float* cb = cosb + (size_t)t * A * RTILE;
-            const float* sb = sseb + (size_t)t * A * RTILE;
-            const float pc = cb[cp * RTILE + tid], pe = sb[cp * RTILE + tid];
-            const float nc = cb[cn * RTILE + tid], ne = sb[cn * RTILE + tid];
-            const bool neg = SEL_ERR ? ne < pe : nc > pc;
-            scos[((size_t)t * nbases + i) * RTILE + tid] = neg ? nc : pc;
-            ssse[((size_t)t * nbases + i) * RTILE + tid] = neg ? -ne : pe;
-          }
-      }
-      __syncthreads();
-      // the other pair of buffers is free (everybody has passed the barrier, so nobody reads the previous pair any more)
-      fetch(tile + 2 * step, 2 * (ps ^ 1));
-      fetch(tile + 3 * step, 2 * (ps ^ 1) + 1);
+  auto fold_sums = [&]() {
+#pragma unroll
+    for (int q = 0; q < NE; ++q) { dg[q] += (double)g[q]; de[q] += (double)e[q]; g[q] = e[q] = 0.0f; }
+  };
+  int stage = 0, run = k, half = 0;                 // run: of this tile, counted from its first
+  unsigned parity = 0;
+  const unsigned last_full = (unsigned)(X.NB / (X.units * RUNIT));      // tiles below this one are whole
+  for (unsigned t = 0; t < X.n_tiles; ++t) {
+    mbar_wait(X.full + 8u * stage, parity, X.hdr);
+    const float* buf = X.ring + (size_t)stage * (2 * X.n_cols) * row_len;
+    const long long tile = (long long)blockIdx.x + (long long)t * gridDim.x;
+    const int live = tile < last_full ? 1 << 30 : (int)(X.NB - tile * (X.units * RUNIT));       // blocks of this tile
 #pragma unroll 1
-      for (int k = 0; k < TPW; ++k) {
-        const TaskDev* tk = &s_task[warp][k];
-        const unsigned sums = smem_u32(acc_sums) + (unsigned)(s_acc0[warp][k] * 32 + lane) * 16u;
-        const unsigned counts = smem_u32(acc_counts) + (unsigned)(s_acc0[warp][k] * 32 + lane) * 4u;
-        const int sgn = tk->sgn;
-        const int rev = tk->rev;
-        const unsigned poff = (unsigned)(A * RTILE * 4), soff = (unsigned)(nbases * RTILE * 4);
-        if (sgn == 0) {
-          if (rev) run_task<SEL_ERR, false, true, 2>(tk, smem_u32(cosb), smem_u32(sseb), poff, lane, sums, counts);
-          else run_task<SEL_ERR, false, false, 2>(tk, smem_u32(cosb), smem_u32(sseb), poff, lane, sums, counts);
-        } else if (sgn == 1) {
-          if (rev) run_task<SEL_ERR, true, true, 2>(tk, smem_u32(scos), smem_u32(ssse), soff, lane, sums, counts);
-          else run_task<SEL_ERR, true, false, 2>(tk, smem_u32(scos), smem_u32(ssse), soff, lane, sums, counts);
+    for (; run < X.units; run += nk) {
+#pragma unroll 1
+      for (int h = 0; h < 4 / BL; ++h) {
+        const int at = run * RUNIT + h * (32 * BL);
+        const float* bu = buf + at;
+        float c[NC][BL], er[NC][BL], va[NC][BL];
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          load(bu, col[SGN ? 2 * i : i], 0, c[i]);
+          load(bu, col[SGN ? 2 * i : i], 1, er[i]);
+          if constexpr (SGN) {
+            float mc[BL], me[BL];
+            load(bu, col[2 * i + 1], 0, mc);
+            load(bu, col[2 * i + 1], 1, me);
+#pragma unroll
+            for (int r = 0; r < BL; ++r) {
+              const bool neg = SEL_ERR ? me[r] < er[i][r] : mc[r] > c[i][r];                    // ties to the atom
+              c[i][r] = neg ? mc[r] : c[i][r]; er[i][r] = neg ? me[r] : er[i][r]; va[i][r] = neg ? NEG : 0.0f;
+            }
+          } else {
+#pragma unroll
+            for (int r = 0; r < BL; ++r) va[i][r] = 0.0f;
+          }
+        }
+        if (at + 32 * BL > live) {                   // blocks beyond the layer: cosine 1, error 0
+#pragma unroll
+          for (int i = 0; i < NC; ++i)
+#pragma unroll
+            for (int r = 0; r < BL; ++r)
+              if (at + lane0 + (VEC ? r : 32 * r) >= live) { c[i][r] = 1.0f; er[i][r] = va[i][r] = 0.0f; }
+        }
+#pragma unroll
+        for (int r = 0; r < BL; ++r) {
+          float gp[NC];
+#pragma unroll
+          for (int i = 0; i < NC; ++i) gp[i] = __fsub_rn(1.0f, c[i][r]);
+          int q = 0;
+          if (SHAPE < 2) {
+#pragma unroll
+            for (int i = 0; i < NA; ++i, ++q) {
+              g[q] = __fadd_rn(g[q], gp[i]); e[q] = __fadd_rn(e[q], er[i][r]);
+              if (SGN) n[q] = __fadd_rn(n[q], va[i][r]);
+            }
+#pragma unroll
+            for (int i = 0; i < NA; ++i)
+#pragma unroll
+              for (int j = i + 1; j < NA; ++j, ++q)
+                entry_add<SEL_ERR, SGN>(g[q], e[q], n[q], c[i][r], c[j][r], gp[i], gp[j], er[i][r], er[j][r], va[i][r], SGN ? __fadd_rn(va[j][r], 1.0f) : 1.0f);
+          } else {
+#pragma unroll
+            for (int j = NA; j < NC; ++j)
+#pragma unroll
+              for (int i = 0; i < NA; ++i, ++q) {
+                const int x = SHAPE == 4 ? j : i, y = SHAPE == 4 ? i : j;        // first and second candidate
+                entry_add<SEL_ERR, SGN>(g[q], e[q], n[q], c[x][r], c[y][r], gp[x], gp[y], er[x][r], er[y][r], va[x][r], SGN ? __fadd_rn(va[y][r], 1.0f) : 1.0f);
+              }
+          }
         }
       }
-      ps ^= 1;
+      half ^= 1;
+      if (!half) fold_sums();                        // eight blocks per lane
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");         // nothing of this CTA's is in flight when it leaves
-  } else {
-    long long tile = blockIdx.x;
-    if (VEC)
-      for (int b = 0; b < n_stage - 1; ++b) fetch(tile + (long long)b * gridDim.x, b);
-    int cur = 0;                 // buffer of the tile in work
-    for (; tile < n_tiles; tile += gridDim.x) {
-      float* cosb = cos0 + (size_t)cur * A * RTILE;
-      float* sseb = sse0 + (size_t)cur * A * RTILE;
-      if (VEC) {
-        // this thread's copies of the tile in work are complete when at most n_stage - 2 newer groups are still pending
-        if (n_stage == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
-        else if (n_stage == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
-        else asm volatile("cp.async.wait_group 0;" ::: "memory");
-      } else {
-        const long long blk0 = tile * RTILE;
-        const int nv = (int)min((long long)RTILE, L.NB - blk0);
-        __syncthreads();                                      // everybody has finished the previous tile
-        for (int i = 0; i < ncols; ++i) {
-          const size_t a = seats.cols[i];
-          cosb[i * RTILE + tid] = tid < nv ? __ldg(block_cos + a * L.NB + blk0 + tid) : 1.0f;
-          sseb[i * RTILE + tid] = tid < nv ? __ldg(block_sse + a * L.NB + blk0 + tid) : 0.0f;
-        }
-      }
-      if (nbases) {
-        // Signed-best columns: this thread's block.  The values come from other threads' copies, and the previous tile's
-        // readers of these columns must be done first: hence the barrier.
-        __syncthreads();
-        for (int i = 0; i < nbases; ++i) {
-          const int a = seats.bases[i], cp = seats.col_slot[a], cn = seats.col_slot[a + 1];     // the atom and its negation
-          const float pc = cosb[cp * RTILE + tid], pe = sseb[cp * RTILE + tid];
-          const float nc = cosb[cn * RTILE + tid], ne = sseb[cn * RTILE + tid];
-          const bool neg = SEL_ERR ? ne < pe : nc > pc;           // ties to the atom; a negative error marks a negated winner
-          scos[i * RTILE + tid] = neg ? nc : pc;
-          ssse[i * RTILE + tid] = neg ? -ne : pe;
-        }
-      }
-      // One barrier per tile: the tile is complete for everybody, and everybody has finished the previous tile, whose
-      // buffer (the one before this in the ring) the next copies refill.
-      __syncthreads();
-      if (VEC) fetch(tile + (long long)(n_stage - 1) * gridDim.x, cur == 0 ? n_stage - 1 : cur - 1);
-  #pragma unroll 1
-      for (int k = 0; k < TPW; ++k) {
-        const TaskDev* tk = &s_task[warp][k];
-        const unsigned sums = smem_u32(acc_sums) + (unsigned)(s_acc0[warp][k] * 32 + lane) * 16u;
-        const unsigned counts = smem_u32(acc_counts) + (unsigned)(s_acc0[warp][k] * 32 + lane) * 4u;
-        const int sgn = tk->sgn;
-        const int rev = tk->rev;
-        if (sgn == 0) {
-          if (rev) run_task<SEL_ERR, false, true, 1>(tk, smem_u32(cosb), smem_u32(sseb), 0u, lane, sums, counts);
-          else run_task<SEL_ERR, false, false, 1>(tk, smem_u32(cosb), smem_u32(sseb), 0u, lane, sums, counts);
-        } else if (sgn == 1) {
-          if (rev) run_task<SEL_ERR, true, true, 1>(tk, smem_u32(scos), smem_u32(ssse), 0u, lane, sums, counts);
-          else run_task<SEL_ERR, true, false, 1>(tk, smem_u32(scos), smem_u32(ssse), 0u, lane, sums, counts);
-        }
-      }
-      if (VEC && ++cur == n_stage) cur = 0;
+    run -= X.units;
+    __syncwarp();
+    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(X.empty + 8u * stage) : "memory");
+    if (++stage == X.n_stage) { stage = 0; parity ^= 1u; }
+  }
+  fold_sums();
+  unsigned n1 = 0, nn = 0, slot = 255;
+#pragma unroll
+  for (int q = 0; q < NE; ++q) {
+    const unsigned c = __float2uint_rn(n[q]);                  // exact: below 2^24
+    const unsigned a = __reduce_add_sync(0xFFFFFFFFu, SGN ? c & 4095u : c), b = SGN ? __reduce_add_sync(0xFFFFFFFFu, c >> 12) : 0u;
+    if (lane == q) { n1 = a; nn = b; slot = k == 0 ? B.slot[q] : 255u; }
+  }
+  if (lane < BUNDLE_ENT) { part->counts[lane] = make_uint2(n1, nn); part->slot[lane] = (unsigned char)slot; }
+  if (lane == 0) part->n_warps = nk;
+  const int q = lane_sums<NE>(dg, lane);
+  lane_sums<NE>(de, lane);
+  if (q >= 0) part->sums[q] = make_double2(dg[0], de[0]);
+}
+
+template <bool SEL_ERR, bool VEC>
+__global__ void __launch_bounds__(RTB, 1) reduce_kernel(LayerArgs L, RedPlan P, BundlesDev Q, int units, int n_stage, int do_final,
+                                                        WsHeader* __restrict__ hdr, PartialSums partials, const float* __restrict__ block_cos,
+                                                        const float* __restrict__ block_sse, sop_pair_stat* pair_table, sop_pair_stat* signed_table,
+                                                        sop_search_result* __restrict__ res, const sop_search_result* __restrict__ prev) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ BundleSums s_part[RED_WARPS];
+  __shared__ unsigned long long s_row[2 * SOP_MAX_ATOMS];      // address of every fetched row: a column's cosines, its errors
+  __shared__ int s_off[2 * SOP_MAX_ATOMS];
+  __shared__ __align__(8) unsigned long long s_bar[2 * MAX_STAGE];
+  __shared__ int s_last;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  ReduceCtx X;
+  X.NB = L.NB; X.n_cols = Q.n_cols; X.units = units; X.n_stage = n_stage;
+  X.row_len = units * RUNIT + (VEC ? 0 : 4);
+  const unsigned tiles = (unsigned)((L.NB + units * RUNIT - 1) / (units * RUNIT));
+  X.n_tiles = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
+  X.ring = reinterpret_cast<const float*>(smem);
+  X.full = smem_u32(s_bar); X.empty = X.full + 8u * MAX_STAGE;
+  X.row_off = s_off; X.hdr = hdr;
+  if (tid < 2 * Q.n_cols) {
+    const unsigned long long a = reinterpret_cast<unsigned long long>(((tid & 1) ? block_sse : block_cos) + (size_t)Q.cols[tid >> 1] * (size_t)L.NB);
+    s_row[tid] = a;
+    s_off[tid] = tid * X.row_len + (int)((a & 15u) >> 2);      // (tiles are multiples of four blocks)
+  }
+  if (tid == 0) {
+    for (int i = 0; i < n_stage; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(X.full + 8u * i) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(X.empty + 8u * i), "r"(Q.n_warps) : "memory");
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  __syncthreads();
+  BundleSums* mine = s_part + (warp < RED_WARPS ? warp : 0);
+  if (warp == RED_WARPS) {
+    reduce_produce(X, s_row[tid & 31]);
+  } else if (warp < Q.n_warps) {
+    const BundleDev& B = Q.bundle[Q.warp_bundle[warp]];
+    const int k = warp - B.first_warp, nk = B.n_warps;
+    switch (2 * B.shape + B.sgn) {
+      case 0: reduce_run<0, false, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 1: reduce_run<0, true, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 2: reduce_run<1, false, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 3: reduce_run<1, true, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 4: reduce_run<2, false, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 5: reduce_run<2, true, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 6: reduce_run<3, false, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 7: reduce_run<3, true, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      case 8: reduce_run<4, false, SEL_ERR, VEC>(X, B, k, nk, mine); break;
+      default: reduce_run<4, true, SEL_ERR, VEC>(X, B, k, nk, mine); break;
     }
   }
-
-  // ---- per-CTA partials: lane (k, q) of a warp adds the 32 lanes' sums of entry q of the warp's task k, in lane order ----
-  __syncwarp();
-  if (lane < TPW * ENT) {
-    const int k = lane / ENT, q = lane - k * ENT;
-    const TaskDev t = s_task[warp][k];
-    const int slot = t.sgn == 2 ? 255 : (q == 0 ? t.self_slot : (q - 1 < t.n_part ? t.slot[q - 1] : 255));
-    if (slot != 255) {
-      Partial p; p.gap = 0.0; p.sse = 0.0; p.n1 = 0; p.nneg = 0;
-      const int seat = s_acc0[warp][k] + (q == 0 ? 0 : q - 1 + (t.self_slot != 255 ? 1 : 0));
-      for (int l = 0; l < 32; ++l) {
-        const double2 a = acc_sums[(size_t)seat * 32 + l];
-        const unsigned c = acc_counts[(size_t)seat * 32 + l];
-        p.gap += a.x; p.sse += a.y; p.n1 += (long long)(c & 0xFFFFu); p.nneg += (long long)(c >> 16);
-      }
-      partials[(size_t)blockIdx.x * MAX_SLOTS + slot] = p;
+  __syncthreads();                      // every copy has landed: the warps have waited for each
+  // ---- per-CTA partials: a bundle's warps in order ----
+  if (tid < Q.n_warps * BUNDLE_ENT) {
+    const BundleSums* p = s_part + tid / BUNDLE_ENT;
+    const int q = tid % BUNDLE_ENT;
+    const unsigned slot = p->slot[q];
+    if (slot != 255u) {
+      double2 v = p->sums[q];
+      uint2 c = p->counts[q];
+      const int n = p->n_warps;
+#pragma unroll 1
+      for (int w = 1; w < n; ++w) { const double2 o = p[w].sums[q]; const uint2 oc = p[w].counts[q]; v.x += o.x; v.y += o.y; c.x += oc.x; c.y += oc.y; }
+      partials.sums[(size_t)blockIdx.x * MAX_SLOTS + slot] = v;
+      partials.counts[(size_t)blockIdx.x * MAX_SLOTS + slot] = c;
     }
   }
   if (!do_final) return;
   // the CTA that arrives last adds everybody's partials and writes the tables; nobody waits for anybody
-  __shared__ int s_last;
   __threadfence();
   __syncthreads();
   if (tid == 0) s_last = atomicAdd(&hdr->done_reduce, 1u) == gridDim.x - 1 ? 1 : 0;
   __syncthreads();
-  if (s_last) {
-    __threadfence();
-    __shared__ int cls_k[SOP_MAX_CLASSES];
-    if (tid < SOP_MAX_CLASSES) {
-      const bool live = tid < P.n_classes;
-      cls_k[tid] = P.k_from_result ? (live && P.cls[tid].k_src >= 0 ? prev->k[P.cls[tid].k_src] : 0) : __ldcg(&hdr->cls_k[tid]);
-    }
-    const float wmax = P.k_from_result ? prev->layer_absmax : __uint_as_float(__ldcg(&hdr->wmax_bits));
-    __syncthreads();
-    sop_pair_stat* s_pair = reinterpret_cast<sop_pair_stat*>(smem);
-    sop_pair_stat* s_sig = s_pair + SOP_MAX_ATOMS * SOP_MAX_ATOMS;
-    finalize_body(L, P, (int)gridDim.x, partials, s_pair, s_sig, reinterpret_cast<Partial*>(s_sig + SOP_MAX_ATOMS * SOP_MAX_ATOMS), pair_table,
-                  signed_table, res, cls_k, wmax);
-  }
+  if (s_last) finalize_body(L, P, (int)gridDim.x, partials, smem, pair_table, signed_table, res, prev, hdr);
 }
 
-// One warp.  The defined entry of `tab` ([A x A]) with the largest acos, ties to the smallest index: among the
-// entries above the diagonal (diag = 0) or among the diagonal entries of the candidates in lut_mask (diag = 1).  -1: none.
+// One warp.  The defined entry of `tab` ([A x A]) with the largest acos, ties to the smallest index: among the entries above the
+// diagonal (diag = 0) or among the diagonal entries of the candidates in lut_mask (diag = 1).  -1: none.
 __device__ __noinline__ int warp_best(const sop_pair_stat* tab, int A, int diag, unsigned lut_mask) {
   const int lane = threadIdx.x & 31;
+  const unsigned per = 65536u / (unsigned)A + 1u;             // i / A = i per >> 16 for i < 256
   int best = -1;
   double bv = 0.0;
 #pragma unroll 1
-  for (int i = lane; i < A * A; i += 32) {
-    const int a = i / A, b = i - a * A;
-    const bool in = diag ? (b == a && ((lut_mask >> a) & 1u)) : b > a;
-    if (in && tab[i].n_sel1 >= 0 && (best < 0 || tab[i].acos > bv)) { best = i; bv = tab[i].acos; }
+  for (int i = lane; i < (diag ? A : A * A); i += 32) {
+    const int a = diag ? i : (int)((unsigned)i * per >> 16), b = diag ? i : i - a * A;
+    const bool in = diag ? ((lut_mask >> a) & 1u) != 0u : b > a;
+    const int at = a * A + b;
+    if (in && tab[at].n_sel1 >= 0 && (best < 0 || tab[at].acos > bv)) { best = at; bv = tab[at].acos; }
   }
 #pragma unroll 1
   for (int o = 16; o; o >>= 1) {
@@ -1200,88 +1184,102 @@ __device__ __noinline__ int warp_best(const sop_pair_stat* tab, int A, int diag,
   return best;
 }
 
-// Run by one whole CTA of TB threads.  Thread (slot, chunk) adds the partials of CTAs chunk, chunk + C,
-// ... in that order (C = min(TB / n_slots, ceil(grid / 4)) chunks, loads coalesced over the slots and issued four at a
-// time), the chunks are then added in chunk order: the result depends only on the grid size, not on
-// scheduling.  s_pair / s_sig (n_atoms^2 entries each) and s_red (TB entries) are shared-memory staging.
-__device__ void finalize_body(const LayerArgs& L, const Plan& P, int grid, const Partial* partials, sop_pair_stat* s_pair, sop_pair_stat* s_sig,
-                              Partial* s_red, sop_pair_stat* pair_table, sop_pair_stat* signed_table, sop_search_result* res,
-                              const int* cls_k, float wmax) {
+// Run by one whole CTA of RTB threads, the last one to arrive: its time is added to every search, so what does not depend on one
+// another is loaded together and the three selections run in warps of their own (the serial form took 12 to 20 us of a launch).
+// Thread (slot, chunk) adds the partials of CTAs chunk, chunk + C, ... in that order (C = min(RTB / n_slots, ceil(grid / 4)) chunks,
+// loads coalesced over the slots and issued eight at a time), the chunks are then added in chunk order: the result depends only on
+// the grid size, not on scheduling.
+struct FinalSmem {
+  sop_pair_stat pair[SOP_MAX_ATOMS * SOP_MAX_ATOMS], sig[SOP_MAX_ATOMS * SOP_MAX_ATOMS];
+  double2 sums[RTB];
+  uint2 counts[RTB];
+};
+__device__ void finalize_body(const LayerArgs& L, const RedPlan& P, int grid, PartialSums partials, unsigned char* smem, sop_pair_stat* pair_table,
+                              sop_pair_stat* signed_table, sop_search_result* res, const sop_search_result* prev, WsHeader* hdr) {
+  __threadfence();
+  FinalSmem& S = *reinterpret_cast<FinalSmem*>(smem);
   const int A = P.n_atoms, tid = threadIdx.x, n_slots = P.n_slots;
-  for (int i = tid; i < A * A; i += blockDim.x) {
-    sop_pair_stat u; u.acos = 0.0; u.mse = 0.0; u.n_sel1 = -1; u.n_neg = -1;
-    // entries among candidates that an earlier call evaluated stay as that call left them in the tables
-    const int a = i / A, b = i - a * A;
-    const bool keep = P.keep_loaded && ((P.load_mask >> a) & 1u) && ((P.load_mask >> b) & 1u);
-    s_pair[i] = keep ? pair_table[i] : u;
-    s_sig[i] = keep && signed_table ? signed_table[i] : u;
-  }
-  __syncthreads();
-  const int n_chunks = max(1, min((int)blockDim.x / max(n_slots, 1), (grid + 3) / 4));   // at best one round of four loads per thread
-  const int slot = tid % max(n_slots, 1), chunk = tid / max(n_slots, 1);
+  const bool failed = *(volatile unsigned*)&hdr->reduce_error != 0u;
+  const int n_chunks = max(1, min(RTB / max(n_slots, 1), (grid + 3) / 4));
+  const int chunk = tid / max(n_slots, 1), slot = tid - chunk * n_slots;
   if (chunk < n_chunks && n_slots > 0) {
-    Partial t; t.gap = 0.0; t.sse = 0.0; t.n1 = 0; t.nneg = 0;
+    double2 t = make_double2(0.0, 0.0);
+    uint2 c = make_uint2(0u, 0u);
 #pragma unroll 1
-    for (int g0 = chunk; g0 < grid; g0 += 4 * n_chunks) {
-      double2 a[4];
-      longlong2 b[4];
+    for (int g0 = chunk; g0 < grid; g0 += 8 * n_chunks) {
+      double2 a[8];
+      uint2 b[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int g = g0 + u * n_chunks;
-        a[u] = make_double2(0.0, 0.0);
-        b[u] = make_longlong2(0, 0);
-        if (g < grid) {
-          const double2* q = reinterpret_cast<const double2*>(partials + (size_t)g * MAX_SLOTS + slot);
-          a[u] = __ldcg(q);
-          b[u] = __ldcg(reinterpret_cast<const longlong2*>(q + 1));
-        }
+      for (int u = 0; u < 8; ++u) {
+        const size_t at = (size_t)(g0 + u * n_chunks) * MAX_SLOTS + slot;
+        const bool in = g0 + u * n_chunks < grid;
+        a[u] = in ? __ldcg(partials.sums + at) : make_double2(0.0, 0.0);
+        b[u] = in ? __ldcg(partials.counts + at) : make_uint2(0u, 0u);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (g0 + u * n_chunks < grid) { t.gap += a[u].x; t.sse += a[u].y; t.n1 += b[u].x; t.nneg += b[u].y; }
+      for (int u = 0; u < 8; ++u) { t.x += a[u].x; t.y += a[u].y; c.x += b[u].x; c.y += b[u].y; }
     }
-    s_red[tid] = t;
+    S.sums[tid] = t;
+    S.counts[tid] = c;
   }
+  for (int i = tid; i < 2 * SOP_MAX_ATOMS * SOP_MAX_ATOMS; i += RTB) {
+    // entries among candidates that an earlier call evaluated stay as that call left them in the tables
+    const int w = i / (SOP_MAX_ATOMS * SOP_MAX_ATOMS), e = i - w * (SOP_MAX_ATOMS * SOP_MAX_ATOMS);
+    if (e >= A * A) continue;
+    const int a = e / A, b = e - a * A;
+    const sop_pair_stat* tab = w ? signed_table : pair_table;
+    sop_pair_stat u; u.acos = 0.0; u.mse = 0.0; u.n_sel1 = -1; u.n_neg = -1;
+    if (P.keep_loaded && tab && ((P.load_mask >> a) & 1u) && ((P.load_mask >> b) & 1u)) u = tab[e];
+    (w ? S.sig : S.pair)[e] = u;
+  }
+  int k = 0;
+  float wmax = 0.0f;
+  if (tid >= RTB - 32) {
+    const int i = tid - (RTB - 32);
+    if (i < A && (((P.eval_mask | P.load_mask) >> i) & 1u)) {
+      const int cl = P.cls_of[i];
+      k = P.k_from_result ? (P.k_src[cl] >= 0 ? prev->k[P.k_src[cl]] : 0) : __ldcg(&hdr->cls_k[cl]);
+    }
+    wmax = P.k_from_result ? prev->layer_absmax : __uint_as_float(__ldcg(&hdr->wmax_bits));
+  }
+  SlotDev sd = {0, 0, 0, 0};
+  if (tid < n_slots) sd = P.slots[tid];
   __syncthreads();
-  if (tid < n_slots) {
-    Partial t = s_red[tid];
-#pragma unroll 1
-    for (int c = 1; c < n_chunks; ++c) {
-      const Partial q = s_red[c * n_slots + tid];
-      t.gap += q.gap; t.sse += q.sse; t.n1 += q.n1; t.nneg += q.nneg;
+  if (tid < n_slots && !failed) {      // (a wait that gave up: every entry formed here stays undefined)
+    double2 t = S.sums[tid];
+    uint2 c = S.counts[tid];
+#pragma unroll 4
+    for (int q = 1; q < n_chunks; ++q) {
+      const double2 o = S.sums[q * n_slots + tid];
+      const uint2 oc = S.counts[q * n_slots + tid];
+      t.x += o.x; t.y += o.y; c.x += oc.x; c.y += oc.y;
     }
     sop_pair_stat st;
-    st.acos = ((double)L.NB - t.gap) / (double)L.NB;
-    st.mse = t.sse / ((double)L.M * (double)L.K);
-    st.n_sel1 = t.n1;
-    const SlotDev sd = P.slots[tid];
-    if (sd.type == 0) { st.n_neg = 0; s_pair[sd.i0 * A + sd.i1] = st; }
-    else { st.n_neg = t.nneg; s_sig[sd.i0 * A + sd.i1] = st; }
+    st.acos = ((double)L.NB - t.x) / (double)L.NB;
+    st.mse = t.y / ((double)L.M * (double)L.K);
+    st.n_sel1 = (long long)c.x;
+    st.n_neg = sd.type ? (long long)c.y : 0;
+    (sd.type ? S.sig : S.pair)[sd.i0 * A + sd.i1] = st;
   }
   __syncthreads();
-  for (int i = tid; i < A * A; i += blockDim.x) {
-    pair_table[i] = s_pair[i];
-    if (signed_table) signed_table[i] = s_sig[i];
-  }
-  if (tid < SOP_MAX_ATOMS) {
-    const bool present = tid < A && (((P.eval_mask | P.load_mask) >> tid) & 1u);
-    res->k[tid] = present ? cls_k[P.cand[tid].cls] : 0;
-  }
-  // best two-codebook pair, best single LUT candidate, best signed pair: largest ACos, ties to the smallest
-  // (a, b).  One warp, one small routine called three times: this code runs once per launch, so its size
-  // (instruction fetches that miss) costs more than its arithmetic.
-  if (tid < 32) {
-    unsigned lut_mask = 0;
-    for (int a = 0; a < A; ++a) lut_mask |= P.cand[a].kind == SOP_KIND_LUT ? 1u << a : 0u;
-    const int ip = warp_best(s_pair, A, 0, lut_mask);
-    const int is = warp_best(s_pair, A, 1, lut_mask);
-    const int isg = signed_table ? warp_best(s_sig, A, 0, lut_mask) : -1;
-    if (tid == 0) {
-      res->layer_absmax = wmax;
-      res->reserved[0] = res->reserved[1] = 0;
-      res->best_a = ip >= 0 ? ip / A : -1; res->best_b = ip >= 0 ? ip % A : -1;
-      res->best_single = is >= 0 ? is / A : -1;
-      res->best_sa = isg >= 0 ? isg / A : -1; res->best_sb = isg >= 0 ? isg % A : -1;
+  // best two-codebook pair, best single LUT candidate, best signed pair: largest ACos, ties to the smallest (a, b)
+  if (tid < 96) {
+    const int w = tid >> 5;
+    const int best = w == 2 && !signed_table ? -1 : warp_best(w == 2 ? S.sig : S.pair, A, w == 1, P.lut_mask);
+    if ((tid & 31) == 0) {
+      const int a = best >= 0 ? best / A : -1, b = best >= 0 ? best - a * A : -1;
+      if (w == 0) { res->best_a = a; res->best_b = b; }
+      else if (w == 1) res->best_single = a;
+      else { res->best_sa = a; res->best_sb = b; }
+    }
+  } else if (tid >= RTB - 32) {
+    const int i = tid - (RTB - 32);
+    if (i < SOP_MAX_ATOMS) res->k[i] = k;
+    if (i == 0) { res->layer_absmax = wmax; res->reserved[0] = res->reserved[1] = 0; }
+  } else {
+    for (int i = tid - 96; i < A * A; i += RTB - 128) {
+      pair_table[i] = S.pair[i];
+      if (signed_table) signed_table[i] = S.sig[i];
     }
   }
 }
@@ -1293,8 +1291,9 @@ static bool same_table(const sop_atom& a, const sop_atom& b) {
   return a.n_entries == b.n_entries && memcmp(a.lut, b.lut, sizeof(float) * a.n_entries) == 0;
 }
 
-int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mask, unsigned load_mask, int singles_only, int keep_loaded, Plan* P) {
+int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mask, unsigned load_mask, int singles_only, int keep_loaded, Plan* P, RedPlan* Rp) {
   memset(P, 0, sizeof(*P));
+  memset(Rp, 0, sizeof(*Rp));
   const int n = A.n_atoms;
   P->n_atoms = n;
   P->k_mode = k_mode;
@@ -1359,21 +1358,20 @@ int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mas
   }
   // slots: pair-type first (singles as (a, a)), then signed.  With keep_loaded an entry whose candidates were all
   // evaluated by an earlier call is not formed again: the tables hold it.
-  P->keep_loaded = keep_loaded;
+  Rp->keep_loaded = keep_loaded;
   int ns = 0;
   auto has = [present](int i) { return ((present >> i) & 1u) != 0; };
   auto old = [keep_loaded, load_mask](int i) { return keep_loaded && ((load_mask >> i) & 1u) != 0; };
   for (int a = 0; a < n; ++a) {
     if (!has(a) || old(a)) continue;
-    P->slots[ns].type = 0; P->slots[ns].i0 = P->slots[ns].i1 = (unsigned char)a; ++ns;
+    Rp->slots[ns].type = 0; Rp->slots[ns].i0 = Rp->slots[ns].i1 = (unsigned char)a; ++ns;
   }
   for (int a = 0; a < n && !singles_only; ++a)
     for (int b = a + 1; b < n; ++b) {
       if (!has(a) || !has(b) || (old(a) && old(b))) continue;
       if (A.atoms[a].kind != SOP_KIND_LUT || A.atoms[b].kind != SOP_KIND_LUT || A.atoms[a].n_bits != A.atoms[b].n_bits) continue;
-      P->slots[ns].type = 0; P->slots[ns].i0 = (unsigned char)a; P->slots[ns].i1 = (unsigned char)b; ++ns;
+      Rp->slots[ns].type = 0; Rp->slots[ns].i0 = (unsigned char)a; Rp->slots[ns].i1 = (unsigned char)b; ++ns;
     }
-  P->n_pair_slots = ns;
   if (F.sign_bits && !singles_only) {
     bool base[SOP_MAX_ATOMS];
     for (int i = 0; i < n; ++i) {
@@ -1385,113 +1383,142 @@ int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mas
       base[i] = (da && db && a.n_entries == b.n_entries) || (!da && !db && same_table(a, b));
     }
     for (int i = 0; i < n; ++i)
-      if (base[i]) P->base_atom[P->n_bases++] = (unsigned char)i;
-    for (int i = 0; i < n; ++i)
       for (int j = i; j < n; ++j) {
         if (!base[i] || !base[j] || A.atoms[i].n_bits != A.atoms[j].n_bits) continue;
         if (old(i) && old(i + 1) && old(j) && old(j + 1)) continue;
-        P->slots[ns].type = 1; P->slots[ns].i0 = (unsigned char)i; P->slots[ns].i1 = (unsigned char)j; ++ns;   // base atoms
+        Rp->slots[ns].type = 1; Rp->slots[ns].i0 = (unsigned char)i; Rp->slots[ns].i1 = (unsigned char)j; ++ns;   // base atoms
       }
   }
   if (ns > MAX_SLOTS) return SOP_ERR_ALPHABET;
-  P->n_slots = ns;
-  // tasks of the reduction: repeatedly the candidate with the most entries still to form on one side of it (as their
-  // first candidate, the one that keeps a tie, or as their second) becomes an anchor and takes up to four of them as
-  // partners; its own (single) entry rides with its first task.  Signed entries (type 1) make tasks of their own.
-  {
-    bool done[MAX_SLOTS];
-    int self_of[2][SOP_MAX_ATOMS];
-    bool self_used[2][SOP_MAX_ATOMS];
-    for (int ty = 0; ty < 2; ++ty)
-      for (int c = 0; c < SOP_MAX_ATOMS; ++c) { self_of[ty][c] = -1; self_used[ty][c] = false; }
-    for (int i = 0; i < ns; ++i) {
-      done[i] = P->slots[i].i0 == P->slots[i].i1;
-      if (done[i]) self_of[P->slots[i].type][P->slots[i].i0] = i;
-    }
-    int nt = 0;
-    for (;;) {
-      int cnt[2][2][SOP_MAX_ATOMS] = {};          // [type][side][candidate]; side 0: the candidate is the entry's first
-      for (int i = 0; i < ns; ++i)
-        if (!done[i]) { ++cnt[P->slots[i].type][0][P->slots[i].i0]; ++cnt[P->slots[i].type][1][P->slots[i].i1]; }
-      int pt = -1, pside = 0, pc = 0;
-      for (int ty = 0; ty < 2; ++ty)
-        for (int side = 0; side < 2; ++side)
-          for (int c = 0; c < SOP_MAX_ATOMS; ++c) {
-            // at most four partners ride with one anchor, so more than four entries count like four
-            const int v = cnt[ty][side][c] < TASK_PART ? cnt[ty][side][c] : TASK_PART;
-            const int best = pt < 0 ? 0 : (cnt[pt][pside][pc] < TASK_PART ? cnt[pt][pside][pc] : TASK_PART);
-            if (v > best) { pt = ty; pside = side; pc = c; }
-          }
-      if (pt < 0) break;
-      if (nt == MAX_TASKS) return SOP_ERR_ALPHABET;
-      TaskDev& t = P->tasks[nt++];
-      memset(&t, 0, sizeof(t));
-      t.anchor = (unsigned char)pc;
-      t.sgn = (unsigned char)pt;
-      t.rev = (unsigned char)pside;
-      t.self_slot = 255;
-      if (self_of[pt][pc] >= 0 && !self_used[pt][pc]) { t.self_slot = (unsigned char)self_of[pt][pc]; self_used[pt][pc] = true; }
-      for (int i = 0; i < ns && t.n_part < TASK_PART; ++i) {
-        if (done[i] || P->slots[i].type != pt || (pside ? P->slots[i].i1 : P->slots[i].i0) != pc) continue;
-        const int q = t.n_part++;
-        t.part[q] = pside ? P->slots[i].i0 : P->slots[i].i1;
-        t.slot[q] = (unsigned char)i;
-        done[i] = true;
-      }
-    }
-    for (int ty = 0; ty < 2; ++ty)
-      for (int c = 0; c < SOP_MAX_ATOMS; ++c) {
-        if (self_of[ty][c] < 0 || self_used[ty][c]) continue;
-        if (nt == MAX_TASKS) return SOP_ERR_ALPHABET;
-        TaskDev& t = P->tasks[nt++];
-        memset(&t, 0, sizeof(t));
-        t.anchor = (unsigned char)c; t.sgn = (unsigned char)ty; t.self_slot = (unsigned char)self_of[ty][c];
-      }
-    // heaviest first (a signed task costs about twice as much per entry: two columns per candidate)
-    auto weight = [](const TaskDev& t) { return (2 + 3 * (int)t.n_part) * (t.sgn ? 2 : 1); };
-    for (int i = 1; i < nt; ++i)
-      for (int j = i; j > 0 && weight(P->tasks[j]) > weight(P->tasks[j - 1]); --j) { const TaskDev x = P->tasks[j]; P->tasks[j] = P->tasks[j - 1]; P->tasks[j - 1] = x; }
-    P->n_tasks = nt;
+  Rp->n_slots = ns;
+  Rp->n_atoms = n; Rp->n_classes = P->n_classes; Rp->eval_mask = eval_mask; Rp->load_mask = load_mask;
+  for (int i = 0; i < n; ++i) {
+    Rp->cls_of[i] = P->cand[i].cls;
+    if (A.atoms[i].kind == SOP_KIND_LUT) Rp->lut_mask |= 1u << i;
   }
   return SOP_OK;
 }
 
-// Seats of one launch of the reduction: tasks [task0, task0 + n) dealt to the eight warps, always to the warp with the
-// least work so far that still has a free seat; the columns to fetch and their places in the tile buffers; one
-// accumulator seat per entry.  Returns the largest number of tasks on one warp.
-static int deal_tasks(const Plan& P, int task0, int n, SeatsDev* seats) {
-  int load[8] = {0}, used[8] = {0};
-  memset(seats, 0, sizeof(*seats));
-  memset(seats->task, 255, sizeof(seats->task));
-  memset(seats->col_slot, 255, sizeof(seats->col_slot));
-  memset(seats->sb_slot, 255, sizeof(seats->sb_slot));
-  int tpw = 0;
-  unsigned cand = 0, bases = 0;
-  for (int i = 0; i < n; ++i) {
-    const TaskDev& t = P.tasks[task0 + i];
-    int w = -1;
-    for (int x = 0; x < 8; ++x)
-      if (used[x] < MAX_TPW && (w < 0 || load[x] < load[w])) w = x;
-    seats->task[w][used[w]++] = (unsigned char)(task0 + i);
-    load[w] += 2 + 3 * (int)t.n_part;
-    tpw = tpw > used[w] ? tpw : used[w];
-    unsigned m = 1u << t.anchor;
-    for (int q = 0; q < t.n_part; ++q) m |= 1u << t.part[q];
-    if (t.sgn) { bases |= m; cand |= m | (m << 1); }     // a base atom stands for itself and its negation
-    else cand |= m;
-  }
-  for (int a = 0; a < P.n_atoms; ++a) {
-    if ((cand >> a) & 1u) { seats->col_slot[a] = (unsigned char)seats->n_cols; seats->cols[seats->n_cols++] = (unsigned char)a; }
-    if ((bases >> a) & 1u) { seats->sb_slot[a] = (unsigned char)seats->n_bases; seats->bases[seats->n_bases++] = (unsigned char)a; }
-  }
-  for (int w = 0; w < 8; ++w)
-    for (int k = 0; k < MAX_TPW; ++k) {
-      if (seats->task[w][k] == 255) continue;
-      seats->acc0[w][k] = (unsigned short)seats->n_seats;
-      const TaskDev& t = P.tasks[seats->task[w][k]];
-      seats->n_seats += (t.self_slot != 255 ? 1 : 0) + t.n_part;
+// The bundles that form the slots of a plan.  Per kind of entry (two-way, signed): first the candidates with a single entry in
+// fours (twos for a rest of two) with the pairs among them, then the remaining pairs as rectangles -- the second candidate with
+// the most pairs left and the one that shares the most first candidates with it, against up to four of those; where one first
+// candidate meets many second ones the rectangle is taken the other way round.
+static void build_bundles(const RedPlan& P, std::vector<BundleDev>* out) {
+  for (int ty = 0; ty < 2; ++ty) {
+    int slot_of[SOP_MAX_ATOMS][SOP_MAX_ATOMS];
+    for (int i = 0; i < SOP_MAX_ATOMS; ++i)
+      for (int j = 0; j < SOP_MAX_ATOMS; ++j) slot_of[i][j] = 255;
+    int single[SOP_MAX_ATOMS], n_single = 0;
+    for (int s = 0; s < P.n_slots; ++s)
+      if (P.slots[s].type == ty) slot_of[P.slots[s].i0][P.slots[s].i1] = s;
+    for (int i = 0; i < SOP_MAX_ATOMS; ++i)
+      if (slot_of[i][i] != 255) single[n_single++] = i;
+    auto make = [&](int shape) {
+      BundleDev B;
+      memset(&B, 0, sizeof(B));
+      memset(B.slot, 255, sizeof(B.slot));
+      B.shape = (unsigned char)shape; B.sgn = (unsigned char)ty;
+      return B;
+    };
+    for (int at = 0; at < n_single;) {
+      const int take = n_single - at < 4 ? n_single - at : 4;
+      const int na = take <= 2 ? 2 : 4;
+      BundleDev B = make(take <= 2 ? 1 : 0);
+      for (int i = 0; i < na; ++i) B.a[i] = (unsigned char)single[at + (i < take ? i : take - 1)];
+      int q = 0;
+      for (int i = 0; i < na; ++i, ++q)
+        if (i < take) { B.slot[q] = (unsigned char)slot_of[B.a[i]][B.a[i]]; slot_of[B.a[i]][B.a[i]] = 255; }
+      for (int i = 0; i < na; ++i)
+        for (int j = i + 1; j < na; ++j, ++q)
+          if (j < take) { B.slot[q] = (unsigned char)slot_of[B.a[i]][B.a[j]]; slot_of[B.a[i]][B.a[j]] = 255; }
+      out->push_back(B);
+      at += take;
     }
-  return tpw > 0 ? tpw : 1;
+    for (;;) {
+      // rev = 0: x is the second candidate of its pairs (column of the matrix), rev = 1: the first (row)
+      auto left = [&](int rev, int x, int y) { return (rev ? slot_of[x][y] : slot_of[y][x]) != 255; };
+      int best = 0, brev = 0, bx = 0;
+      for (int rev = 0; rev < 2; ++rev)
+        for (int x = 0; x < SOP_MAX_ATOMS; ++x) {
+          int c = 0;
+          for (int y = 0; y < SOP_MAX_ATOMS; ++y) c += left(rev, x, y) ? 1 : 0;
+          if ((c < 4 ? c : 4) > best) { best = c < 4 ? c : 4; brev = rev; bx = x; }
+        }
+      if (!best) break;
+      int b2 = -1, shared = 0;
+      for (int x = 0; x < SOP_MAX_ATOMS; ++x) {
+        if (x == bx) continue;
+        int c = 0;
+        for (int y = 0; y < SOP_MAX_ATOMS; ++y) c += left(brev, bx, y) && left(brev, x, y) ? 1 : 0;
+        if ((c < 4 ? c : 4) > shared) { shared = c < 4 ? c : 4; b2 = x; }
+      }
+      if (2 * shared < best) b2 = -1;                 // hardly anything in common: one at a time
+      BundleDev B = make(brev ? 4 : b2 < 0 ? 3 : 2);
+      B.b[0] = (unsigned char)bx; B.b[1] = (unsigned char)(b2 < 0 ? bx : b2);
+      int n = 0;
+      for (int pass = 0; pass < 2 && n < 4; ++pass)    // what both share first
+        for (int y = 0; y < SOP_MAX_ATOMS && n < 4; ++y) {
+          const bool both = b2 >= 0 && left(brev, bx, y) && left(brev, b2, y);
+          if (left(brev, bx, y) && (pass == 0 ? both || b2 < 0 : !both && b2 >= 0)) B.a[n++] = (unsigned char)y;
+        }
+      for (int i = n; i < 4; ++i) B.a[i] = B.a[n - 1];
+      for (int j = 0; j < (b2 < 0 ? 1 : 2); ++j)
+        for (int i = 0; i < n; ++i) {
+          int& s = brev ? slot_of[B.b[j]][B.a[i]] : slot_of[B.a[i]][B.b[j]];
+          B.slot[4 * j + i] = (unsigned char)s;
+          s = 255;
+        }
+      out->push_back(B);
+    }
+  }
+}
+
+// One launch of up to fifteen bundles: the columns it fetches, the columns' places in the bundles, and the warps dealt to them,
+// always to the bundle whose warps have the most to do (instructions per run).
+static void deal_bundles(const BundleDev* b, int n, BundlesDev* Q) {
+  memset(Q, 0, sizeof(*Q));
+  Q->n_bundles = n;
+  unsigned cand = 0;
+  auto cols_of = [](const BundleDev& B) { return B.shape == 0 ? 4 : B.shape == 1 ? 2 : B.shape == 3 ? 5 : 6; };
+  auto col = [](const BundleDev& B, int i) { const int na = B.shape == 1 ? 2 : 4; return i < na ? (int)B.a[i] : (int)B.b[i - na]; };
+  for (int i = 0; i < n; ++i)
+    for (int c = 0; c < cols_of(b[i]); ++c) cand |= (b[i].sgn ? 3u : 1u) << col(b[i], c);
+  int place[SOP_MAX_ATOMS + 1] = {0};
+  for (int a = 0; a < SOP_MAX_ATOMS; ++a)
+    if ((cand >> a) & 1u) { place[a] = Q->n_cols; Q->cols[Q->n_cols++] = (unsigned char)a; }
+  int cost[MAX_BUNDLES], nw[MAX_BUNDLES];
+  for (int i = 0; i < n; ++i) {
+    BundleDev B = b[i];
+    const int nc = cols_of(B), ne = B.shape == 0 ? 10 : B.shape == 1 ? 3 : B.shape == 3 ? 4 : 8;
+    cost[i] = B.sgn ? 15 * ne + 24 * nc : 13 * ne + 6 * nc;
+    nw[i] = 1;
+    const int na = B.shape == 1 ? 2 : 4;
+    for (int c = 0; c < nc; ++c) {
+      const int a = col(b[i], c);
+      (c < na ? B.a[c] : B.b[c - na]) = (unsigned char)place[a];
+      if (B.sgn) B.neg[c] = (unsigned char)place[a + 1];
+    }
+    Q->bundle[i] = B;
+  }
+  for (int w = n; w < RED_WARPS && n; ++w) {
+    int pick = 0;
+    for (int i = 1; i < n; ++i)
+      if (cost[i] * nw[pick] > cost[pick] * nw[i]) pick = i;
+    ++nw[pick];
+  }
+  int at = 0;
+  for (int i = 0; i < n; ++i) {
+    Q->bundle[i].first_warp = (unsigned char)at; Q->bundle[i].n_warps = (unsigned char)nw[i];
+    for (int w = 0; w < nw[i]; ++w) Q->warp_bundle[at++] = (unsigned char)i;
+  }
+  Q->n_warps = at;
+}
+
+// the ring of tile buffers; at least the room the closing reduction of the last CTA needs
+static size_t reduce_smem_bytes(int n_cols, int units, int n_stage) {
+  const size_t ring = (size_t)n_stage * n_cols * 2 * (units * RUNIT + 4) * sizeof(float);
+  const size_t fin = sizeof(FinalSmem);
+  return ((ring > fin ? ring : fin) + 127) & ~(size_t)127;
 }
 
 // Shared memory of the sweep: per group its rows (one more than its decision points) and its cells, 128 bytes per cell and
@@ -1517,19 +1544,9 @@ static size_t sweep_layout(const AtomsDev& A, Plan* P, size_t limit) {
   }
 }
 
-// the ring of tile buffers, the signed-best columns, the lanes' accumulators; at least the room the closing
-// reduction of the last CTA needs
-static size_t reduce_smem_bytes(const SeatsDev& S, int n_stage, bool pair = false) {
-  const size_t tiles = ((size_t)n_stage * S.n_cols + (pair ? 2 : 1) * (size_t)S.n_bases) * 2 * RTILE * sizeof(float);
-  const size_t acc = (size_t)S.n_seats * ACC_BYTES;
-  const size_t fin = sizeof(Partial) * (size_t)RTB + 2 * sizeof(sop_pair_stat) * SOP_MAX_ATOMS * SOP_MAX_ATOMS;
-  const size_t b = tiles + acc;
-  return ((b > fin ? b : fin) + 127) & ~(size_t)127;
-}
-
-// Two tiles per step in the reduction (see reduce_kernel) wherever the shared memory allows; sop_pair_search_tuning
-// turns it off (tests compare both paths: the results are the same bit for bit).
-static bool g_reduce_pairs = true;
+// sop_pair_search_tuning(0): a ring of two tile buffers instead of as many as fit, up to four (tests compare both: the results
+// are the same bit for bit).
+static bool g_reduce_ring = true;
 
 }  // namespace sop
 
@@ -1537,7 +1554,7 @@ extern "C" {
 
 int sop_pair_search_tuning(int reduce_tile_pairs) {
   if (reduce_tile_pairs != 0 && reduce_tile_pairs != 1) return SOP_ERR_RANGE;
-  sop::g_reduce_pairs = reduce_tile_pairs != 0;
+  sop::g_reduce_ring = reduce_tile_pairs != 0;
   return SOP_OK;
 }
 
@@ -1581,13 +1598,15 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   const bool reuse_prepass = (flags & SOP_SEARCH_REUSE_PREPASS) && !k_from_result;
   const int keep_loaded = (flags & SOP_SEARCH_KEEP_LOADED_ENTRIES) && load_mask ? 1 : 0;
   Plan P;
-  if ((rc = build_plan(A, F, k_from_result ? 0 : k_mode, eval_mask, load_mask, flags & SOP_SEARCH_SINGLES_ONLY, keep_loaded, &P))) return rc;
-  P.k_from_result = k_from_result ? 1 : 0;
+  RedPlan Rp;
+  if ((rc = build_plan(A, F, k_from_result ? 0 : k_mode, eval_mask, load_mask, flags & SOP_SEARCH_SINGLES_ONLY, keep_loaded, &P, &Rp))) return rc;
+  P.k_from_result = Rp.k_from_result = k_from_result ? 1 : 0;
   for (int c = 0; c < P.n_classes; ++c) {
     // the shift of a class is read from a candidate of that class that the earlier call had
     P.cls[c].k_src = -1;
     for (int i = 0; i < P.cls[c].n_mem; ++i)
       if ((load_mask >> P.cls[c].mem[i]) & 1u) { P.cls[c].k_src = P.cls[c].mem[i]; break; }
+    Rp.k_src[c] = (signed char)P.cls[c].k_src;
     if (k_from_result && P.cls[c].scope != 0 && P.cls[c].k_src < 0) return SOP_ERR_RANGE;
   }
 
@@ -1597,7 +1616,9 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   unsigned char* ws = (unsigned char*)workspace_dev;
   WsHeader* hdr = (WsHeader*)ws;
   unsigned* hist = (unsigned*)(ws + ws_hist_off());
-  Partial* partials = (Partial*)(ws + ws_part_off());
+  PartialSums partials;
+  partials.sums = (double2*)(ws + ws_part_off());
+  partials.counts = (uint2*)(partials.sums + (size_t)MAX_GRID * MAX_SLOTS);
   float* cos_cols = own_columns ? (float*)(ws + ws_total()) : block_cos_dev;
   float* sse_cols = own_columns ? (float*)(ws + ws_total() + col_bytes) : block_sse_dev;
 
@@ -1605,6 +1626,7 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   constexpr size_t SMEM_MAX = 226 * 1024;   // 227 KB per CTA minus the kernels' few static bytes
   int max_np = 0;
   for (int g = 0; g < P.n_groups; ++g) max_np = P.groups[g].np > max_np ? P.groups[g].np : max_np;
+  constexpr size_t RED_SMEM_MAX = 220 * 1024;
   const size_t smem = sweep_layout(A, &P, SMEM_MAX);
   if (smem > SMEM_MAX) return SOP_ERR_ALPHABET;
   const int sms = num_sms();
@@ -1618,17 +1640,17 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   const long long min_grid = (L.nbk + tba - 1) / tba;
   if (grid < min_grid) grid = min_grid;
   if (grid > MAX_GRID) return SOP_ERR_SHAPE;
-  // the reduction: up to MAX_TPW tasks per warp and launch, more launches for more tasks; persistent grid over tiles.
-  // 16-byte copies need 16-byte aligned column starts and runs: a block count that is a multiple of four.
-  constexpr int PER_LAUNCH = (RTB / 32) * MAX_TPW;
-  const int n_launch = P.n_tasks ? (P.n_tasks + PER_LAUNCH - 1) / PER_LAUNCH : 1;
+  // the reduction: up to fifteen bundles per launch; persistent grid over tiles of 768 blocks, 256 where those would leave SMs
+  // without one.  16-byte copies need 16-byte aligned column starts and runs: a block count that is a multiple of four.
+  std::vector<BundleDev> bundles;
+  build_bundles(Rp, &bundles);
+  const int n_launch = bundles.empty() ? 1 : (int)((bundles.size() + MAX_BUNDLES - 1) / MAX_BUNDLES);
   const bool vec = (L.NB % 4) == 0 && (((uintptr_t)cos_cols | (uintptr_t)sse_cols) & 15u) == 0;
-  const long long n_tiles = (L.NB + RTILE - 1) / RTILE;
-  long long rgrid = n_tiles < (long long)sms * 2 ? n_tiles : (long long)sms * 2;
-  if (rgrid < 1) rgrid = 1;
-  // a lane counts at most 8 blocks per tile in 16 bits: a CTA takes fewer than 8000 tiles (never near it on a GPU with
-  // a hundred SMs: 2^19 tiles at most)
-  if (n_tiles / rgrid >= 8000) rgrid = (n_tiles + 7999) / 8000;
+  const int units = L.NB >= (long long)sms * 6 * RUNIT ? 6 : 2;
+  const long long n_tiles = (L.NB + units * RUNIT - 1) / (units * RUNIT);
+  long long rgrid = n_tiles < (long long)sms ? n_tiles : (long long)sms;
+  // a lane counts its blocks in 12 bits: at most 4095 of them even where a bundle has one warp only
+  while (((n_tiles + rgrid - 1) / rgrid) * units * (RUNIT / 32) > 4095) ++rgrid;
 
   // the header always starts from zero; the histograms (and max|W| behind them) only when this call fills them
   SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, (k_from_result || reuse_prepass) ? ws_hist_off() : ws_part_off(), st));
@@ -1651,15 +1673,10 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
     SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
     SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
     SOP_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
-#define SOP_REDUCE_ATTR(SE, T, BK, PR) \
-  SOP_CUDA_TRY(cudaFuncSetAttribute(reduce_kernel<SE, T, BK, PR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX))
-    SOP_REDUCE_ATTR(false, 1, false, false); SOP_REDUCE_ATTR(false, 2, false, false); SOP_REDUCE_ATTR(false, 3, false, false);
-    SOP_REDUCE_ATTR(false, 1, true, false); SOP_REDUCE_ATTR(false, 2, true, false); SOP_REDUCE_ATTR(false, 3, true, false);
-    SOP_REDUCE_ATTR(true, 1, false, false); SOP_REDUCE_ATTR(true, 2, false, false); SOP_REDUCE_ATTR(true, 3, false, false);
-    SOP_REDUCE_ATTR(true, 1, true, false); SOP_REDUCE_ATTR(true, 2, true, false); SOP_REDUCE_ATTR(true, 3, true, false);
-    SOP_REDUCE_ATTR(false, 1, true, true); SOP_REDUCE_ATTR(false, 2, true, true); SOP_REDUCE_ATTR(false, 3, true, true);
-    SOP_REDUCE_ATTR(true, 1, true, true); SOP_REDUCE_ATTR(true, 2, true, true); SOP_REDUCE_ATTR(true, 3, true, true);
-#undef SOP_REDUCE_ATTR
+    SOP_CUDA_TRY(cudaFuncSetAttribute(reduce_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RED_SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(reduce_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RED_SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(reduce_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RED_SMEM_MAX));
+    SOP_CUDA_TRY(cudaFuncSetAttribute(reduce_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RED_SMEM_MAX));
     facts->search_attr_set = true;
   }
   if ((rc = profile_mark(SOP_PROFILE_SWEEP, 0, st))) return rc;
@@ -1678,26 +1695,18 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   if ((rc = profile_mark(SOP_PROFILE_REDUCE, 0, st))) return rc;
   const bool sel_err = (flags & SOP_SEARCH_SELECT_MSE) != 0;
   for (int l = 0; l < n_launch; ++l) {
-    const int task0 = l * PER_LAUNCH;
-    const int nt = P.n_tasks - task0 < PER_LAUNCH ? P.n_tasks - task0 : PER_LAUNCH;
-    SeatsDev seats;
-    const int tpw = deal_tasks(P, task0, nt, &seats);
-    // as many tile buffers as still let two CTAs share an SM (at most 16 columns, 8 signed-best ones and 120 seats: two
-    // buffers always fit one CTA)
-    int n_stage = vec ? MAX_STAGE : 1;
-    while (n_stage > 2 && reduce_smem_bytes(seats, n_stage) > SMEM_MAX / 2) --n_stage;
-    // two tiles at a time when the ring has its four buffers and the second set of signed-best columns still fits
-    const bool pair = vec && n_stage == MAX_STAGE && reduce_smem_bytes(seats, n_stage, true) <= SMEM_MAX / 2 && g_reduce_pairs;
-    const size_t rs = reduce_smem_bytes(seats, n_stage, pair);
+    const int b0 = l * MAX_BUNDLES, nb = (int)bundles.size() - b0 < MAX_BUNDLES ? (int)bundles.size() - b0 : MAX_BUNDLES;
+    BundlesDev Q;
+    deal_bundles(bundles.data() + b0, nb, &Q);
+    int n_stage = g_reduce_ring ? MAX_STAGE : 2;             // (sixteen columns: two buffers of 98 KB)
+    while (n_stage > 2 && reduce_smem_bytes(Q.n_cols, units, n_stage) > RED_SMEM_MAX) --n_stage;
+    const size_t rs = reduce_smem_bytes(Q.n_cols, units, n_stage);
     const int fin = l == n_launch - 1 ? 1 : 0;
-#define SOP_LAUNCH_REDUCE(SE, T, BK, PR)                                                                                      \
-  reduce_kernel<SE, T, BK, PR><<<(int)rgrid, RTB, rs, st>>>(L, P, seats, n_stage, fin, hdr, partials, cos_cols, sse_cols, pair_table_dev, \
-                                                            signed_table_dev, result_dev, prev_result_dev)
-#define SOP_LAUNCH_REDUCE_T(SE, BK, PR) \
-  do { if (tpw == 1) SOP_LAUNCH_REDUCE(SE, 1, BK, PR); else if (tpw == 2) SOP_LAUNCH_REDUCE(SE, 2, BK, PR); else SOP_LAUNCH_REDUCE(SE, 3, BK, PR); } while (0)
-    if (sel_err) { if (pair) SOP_LAUNCH_REDUCE_T(true, true, true); else if (vec) SOP_LAUNCH_REDUCE_T(true, true, false); else SOP_LAUNCH_REDUCE_T(true, false, false); }
-    else { if (pair) SOP_LAUNCH_REDUCE_T(false, true, true); else if (vec) SOP_LAUNCH_REDUCE_T(false, true, false); else SOP_LAUNCH_REDUCE_T(false, false, false); }
-#undef SOP_LAUNCH_REDUCE_T
+#define SOP_LAUNCH_REDUCE(SE, VC)                                                                                                   \
+  reduce_kernel<SE, VC><<<(int)rgrid, RTB, rs, st>>>(L, Rp, Q, units, n_stage, fin, hdr, partials, cos_cols, sse_cols, pair_table_dev, \
+                                                     signed_table_dev, result_dev, prev_result_dev)
+    if (sel_err) { if (vec) SOP_LAUNCH_REDUCE(true, true); else SOP_LAUNCH_REDUCE(true, false); }
+    else { if (vec) SOP_LAUNCH_REDUCE(false, true); else SOP_LAUNCH_REDUCE(false, false); }
 #undef SOP_LAUNCH_REDUCE
     SOP_CUDA_TRY(cudaGetLastError());
   }

@@ -1,0 +1,69 @@
+"""The reduction of the per-block values into table entries, recomputed in FP64 from the per-block arrays of the same call: block
+counts around a tile of 256 or 768 blocks and around one tile per SM, rows of the columns that start off a 16-byte boundary, and
+alphabets whose entries make every kind of bundle (a rest of one, two or three candidates, one second candidate, many)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_14929_b200 import inputs as I
+
+from .test_gpu_parity import B, dev  # noqa: F401  (B is a fixture)
+
+pytestmark = pytest.mark.gpu
+
+# fp32 sums of eight gaps or errors (relative 8 * 2^-24 of non-negative terms), everything after them in FP64
+TOL = 8 * 2.0 ** -24
+
+
+def _expect(cos, sse, atoms, signed, by_error):
+    def pick(second, first):
+        return sse[second] < sse[first] if by_error else cos[second] > cos[first]
+    A, pair, four = len(atoms), {}, {}
+    lut = [a.kind == I.KIND_LUT for a in atoms]
+    for a in range(A):
+        for b in range(a, A):
+            if a != b and not (lut[a] and lut[b] and atoms[a].n_bits == atoms[b].n_bits):
+                continue
+            mu = pick(b, a)
+            pair[a, b] = (np.where(mu, cos[b], cos[a]), np.where(mu, sse[b], sse[a]), int(mu.sum()), 0)
+    base = [i for i in range(A - 1) if lut[i] and not atoms[i].negated and atoms[i + 1].negated] if signed else []
+    best = {}
+    for i in base:
+        neg = pick(i + 1, i)
+        best[i] = (np.where(neg, cos[i + 1], cos[i]), np.where(neg, sse[i + 1], sse[i]), neg)
+    for x, i in enumerate(base):
+        for j in base[x:]:
+            (ci, ei, ni), (cj, ej, nj) = best[i], best[j]
+            mu = (ej < ei if by_error else cj > ci) if i != j else np.zeros(len(ci), bool)
+            four[i, j] = (np.where(mu, cj, ci), np.where(mu, ej, ei), int(mu.sum()), int(np.where(mu, nj, ni).sum()))
+    return pair, four
+
+
+@pytest.mark.parametrize("M,K", [(1, 16), (3, 64), (17, 240), (48, 256), (61, 1040), (1776, 1024), (1777, 1040)])
+@pytest.mark.parametrize("rom,fp,by_error", [(["NF4"], [], False), (["NF4", "SH4", "BOF4", "Split87"], ["E2M3", "E4M3"], False),
+                                             (["NF4", "SH4", "BOF4"], ["E2M3"], True)])
+def test_table_entries_match_the_per_block_values(B, M, K, rom, fp, by_error):
+    L = I.student_layer(5, 0, M, K, 4, 4.0, device="cuda")
+    atoms = I.alphabet(rom, fp=fp)
+    A, NB = len(atoms), M * K // 16
+    c = torch.rand(K, device=dev()) + 0.1
+    for fmt_name in ("E5M6", "UE4M4"):
+        fmt = I.scale_format(fmt_name)
+        pt, st, res = B.new_pair_table(A, dev()), B.new_pair_table(A, dev()), B.new_result(dev())
+        bc, bs = torch.empty((A, NB), device=dev()), torch.empty((A, NB), device=dev())
+        B.sop_pair_search(L.W, c, fmt, atoms, pt, st, res, B.alloc_workspace(B.pair_search_workspace(M, K, A), dev()), block_cos=bc, block_sse=bs,
+                          select_mse=by_error)
+        P, S = B.read_pair_table(pt, A), B.read_pair_table(st, A)
+        pair, four = _expect(bc.cpu().numpy(), bs.cpu().numpy(), atoms, bool(fmt.sign_bits), by_error)
+        for table, want in ((P, pair), (S, four)):
+            for a in range(A):
+                for b in range(A):
+                    if (a, b) not in want:
+                        assert table[a, b]["n_sel1"] == -1
+                        continue
+                    wc, we, n1, nn = want[a, b]
+                    got = table[a, b]
+                    assert (got["n_sel1"], got["n_neg"]) == (n1, nn), (a, b)
+                    gap = 1.0 - wc.astype(np.float64)
+                    assert abs((1.0 - got["acos"]) - gap.mean()) <= TOL * np.abs(gap).mean() + 4e-16, (a, b)
+                    assert got["mse"] == pytest.approx(we.astype(np.float64).sum() / (M * K), rel=TOL), (a, b)
