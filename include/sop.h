@@ -287,12 +287,11 @@ int sop_dd4_lloyd_workspace(long long M, long long K, size_t* bytes);
 int sop_dd4_lloyd_launches(long long M, long long K, int iters, int flags, int* launches);
 /* Launch-shape parameters of sop_dd4_lloyd for this process (test aid, no counterpart in the paper; results do
  * not depend on them).  cell_spill_tiles in [1, 128]: cache tiles a CTA sorts between two transfers of its
- * per-cell partial sums to the global sums (default 128, the most the 32-bit limbs allow);
- * cache_ctas >= 0: largest grid of the cache kernel (0 = default, three CTAs per SM);
- * tiles_per_warp in [1, 4]: cache tiles one warp of an iteration CTA walks between two folds of its 32-bit partial
- *   sums into 64-bit ones (default 4, the most the partial sums hold).
- * iter_ctas >= 0: largest grid of the iteration kernels (0 = default: one warp per cache tile of the expected pool,
- *   at most eight CTAs per SM and, in one cooperative launch, what is resident at once).
+ * per-cell partial sums to the global sums (default 128);
+ * cache_ctas >= 0: largest grid of the cache kernel (0 = default, two CTAs per SM);
+ * tiles_per_warp in [1, 4]: accepted, without effect;
+ * iter_ctas >= 0: largest grid of the iteration kernels (0 = default: a CTA per four cache tiles of the expected pool,
+ *   at most one per SM).
  * SOP_ERR_RANGE outside these ranges. */
 int sop_dd4_lloyd_tuning(int cell_spill_tiles, int cache_ctas, int tiles_per_warp, int iter_ctas);
 int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, const float* c_dev, int g,

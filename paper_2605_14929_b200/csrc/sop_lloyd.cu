@@ -12,24 +12,20 @@
 //   pool_list_kernel      compacts the indices of the pool blocks into a dense list.
 //   pool_cache_kernel     the pool elements never change between iterations, only the table does:
 //                         (u, omega) of every pool element is computed once (u = w / scale) and kept
-//                         in tiles of 4096 elements, each counting-sorted by the cell of u on a
+//                         in tiles of 6144 elements, each counting-sorted by the cell of u on a
 //                         uniform grid (641 cells of width 2^-8); the start of every cell inside
 //                         every tile is kept too, and per cell, over the whole pool, the int64
-//                         fixed-point sums of omega and omega u and the moments
-//                         sum omega, sum omega u, sum omega u^2.
-//   lloyd_iteration       one iteration (device function).  A cell that holds no decision threshold of
+//                         fixed-point sums of omega and omega u and the moments of omega
+//                         about the cell's centre.
+//   lloyd_iter_kernel     the iterations.  A cell that holds no decision threshold of
 //                         the current table lies inside one entry's interval: its elements are
 //                         accounted for by the cell's sums and moments, without touching them.  Only
-//                         the cells that hold a threshold are walked element by element, exactly: one
-//                         warp per tile, the lanes taking contiguous shares of those cells' elements.
+//                         the cells that hold a threshold are walked element by element, exactly.
 //                         Per-entry sums are int64 fixed point (exactly associative: the table is the
 //                         same bit for bit as a sequential sum over all elements gives), distortion
-//                         FP64.  The CTA that finishes last turns the sums into centroids, snaps them to
-//                         bf16, sorts, publishes the next iteration's descriptor and clears the
-//                         accumulators.
-//   lloyd_persistent_kernel  all iterations in one cooperative launch; between iterations the CTAs wait,
-//                         bounded, for the flag of the CTA that finished last.
-//   lloyd_split_kernel    one iteration per launch: used where the grid cannot be resident at once.
+//                         FP64.  All iterations run in one cooperative launch, with a bounded wait for
+//                         everybody's sums between them, or one per launch where the grid cannot be
+//                         resident at once.
 #include <math.h>
 #include <stddef.h>
 #include <string.h>
@@ -63,18 +59,14 @@ struct LloydWs {
   // radix select state
   unsigned hist[3][2048];
   // iteration state
-  unsigned long long accN[SOP_MAX_ENTRIES];
-  long long accS[SOP_MAX_ENTRIES];
-  double accD;
+  unsigned long long accN[SOP_MAX_LLOYD_ITERS + 1][SOP_MAX_ENTRIES];
+  long long accS[SOP_MAX_LLOYD_ITERS + 1][SOP_MAX_ENTRIES];
+  double accD[SOP_MAX_LLOYD_ITERS + 1];
   unsigned tau_key;  // pool threshold as a ranking key: the pool is every block whose key is not above it
   float cmax;
   int k;
   int fmta;
-  unsigned done;         // CTAs of the running iteration that have added their sums (one launch per iteration)
-  // one launch for all iterations: CTAs that have added their sums in iteration i, and the flag that the
-  // table of iteration i + 1 is published; never reset (the header is cleared before every call)
-  unsigned arrive[SOP_MAX_LLOYD_ITERS + 1];
-  unsigned ready[SOP_MAX_LLOYD_ITERS + 1];
+  unsigned arrive[SOP_MAX_LLOYD_ITERS + 1];      // CTAs that have added their sums of an iteration
   unsigned error;        // a CTA gave up waiting for a flag
   unsigned list_count;   // blocks appended to the pool list
   int pad;
@@ -83,7 +75,7 @@ struct LloydWs {
   // per cell, over the whole pool (filled once by pool_cache_kernel)
   unsigned long long cellN[SORT_ROWS];     // sum fix(omega)
   long long cellS[SORT_ROWS];              // sum fix(omega u)
-  double cellA[3][SORT_ROWS];              // sum omega, sum omega u, sum omega u^2
+  double cellA[3][SORT_ROWS];              // sum omega, sum omega d, sum omega d^2, d = 256 u - (number of the cell's centre)
   long long cellQ[SORT_ROWS];              // sum fix((omega u) u): the exact second moment the grid-constrained construction needs
   // not cleared per call: scratch of the dynamic programme, and where the last run starts per (number of runs, last cell)
   short dp_cut[SOP_MAX_ENTRIES][SORT_ROWS];
@@ -102,20 +94,22 @@ struct LloydArgs {
   float* omega;               // workspace: K floats, c / max(c)
   unsigned* pool_idx;         // workspace: NB words, indices of the pool blocks
   uint2* cache;               // workspace: pairs (u, omega) as bit patterns, tiles of TILE_ELEMS sorted by cell
-  unsigned short* tile_start; // workspace: [tiles][SORT_ROWS + 1] first sorted position of every cell in every tile
+  unsigned short* tile_start; // workspace: [tiles][TS_PITCH] first sorted position of every cell in every tile
 };
 
 static size_t lloyd_off_omega() { return (sizeof(LloydWs) + 255) & ~(size_t)255; }
 static size_t lloyd_off_idx(long long K) { return lloyd_off_omega() + (((size_t)K * 4 + 255) & ~(size_t)255); }
 static size_t lloyd_off_cache(long long M, long long K) { return lloyd_off_idx(K) + ((((size_t)M * (size_t)(K / SOP_G)) * 4 + 255) & ~(size_t)255); }
-constexpr int TILE_ELEMS = LTB * SOP_G;   // pool elements per cache tile: one block per thread of a CTA
+constexpr int CTB = 384;                        // threads of a cache CTA = pool blocks of a cache tile
+constexpr int TILE_ELEMS = CTB * SOP_G;         // pool elements per cache tile
+constexpr int TS_PITCH = (SORT_ROWS + 1 + 7) / 8 * 8;     // cell starts of a tile, whole 16-byte groups
 static size_t lloyd_off_tiles(long long M, long long K) {
   const size_t nb = (size_t)M * (size_t)(K / SOP_G);
-  return lloyd_off_cache(M, K) + ((nb + LTB - 1) / LTB) * TILE_ELEMS * sizeof(uint2);   // whole tiles
+  return lloyd_off_cache(M, K) + ((nb + CTB - 1) / CTB) * TILE_ELEMS * sizeof(uint2);   // whole tiles
 }
 static size_t lloyd_ws_bytes(long long M, long long K) {
   const size_t nb = (size_t)M * (size_t)(K / SOP_G);
-  return lloyd_off_tiles(M, K) + ((((nb + LTB - 1) / LTB) * (SORT_ROWS + 1) * sizeof(unsigned short) + 255) & ~(size_t)255);
+  return lloyd_off_tiles(M, K) + ((((nb + CTB - 1) / CTB) * TS_PITCH * sizeof(unsigned short) + 255) & ~(size_t)255);
 }
 
 __device__ __forceinline__ unsigned cos_key(float x) {
@@ -236,23 +230,7 @@ __device__ __forceinline__ int sort_cell(float u) {
   return (int)(__float_as_uint(t) - __float_as_uint(SORT_MAGIC));
 }
 
-// Threads 0..31 of a CTA; s_lut holds the sorted table padded to 32 entries with its last value.
-// Thread j writes entry j, its decision threshold (the same rule as build_thresholds: the largest
-// fp32 <= the midpoint, a repeated entry takes the threshold above it, +inf from n_entries - 1 on)
-// and the lookup cell of that threshold.  sort_cell is monotone, so an element in a lower cell than a
-// threshold's is below the threshold and one in a higher cell is above it: only the elements of the
-// cells listed here need the comparison itself.
-__device__ void lloyd_publish_desc(LloydWs* ws, const float* s_lut, int ne) {
-  const int j = threadIdx.x;
-  if (j >= SOP_MAX_ENTRIES) return;
-  int jj = j;
-  while (jj < ne - 1 && s_lut[jj] == s_lut[jj + 1]) ++jj;
-  const float t = jj < ne - 1 ? __double2float_rd(0.5 * ((double)s_lut[jj] + (double)s_lut[jj + 1])) : __int_as_float(0x7F800000);
-  ws->desc.lut[j] = s_lut[j];
-  ws->desc.tau[j] = t;
-  ws->desc.thr_cell[j] = j < ne - 1 ? sort_cell(t) : SORT_ROWS;
-  if (j == 0) ws->desc.n_entries = ne;
-}
+__device__ void make_desc(IterDesc* d, const float* table, int ne);
 
 __global__ void __launch_bounds__(SETUP_TB) lloyd_setup_kernel(LloydArgs a, AtomsDev A, const sop_search_result* __restrict__ res,
                                                                LloydWs* __restrict__ ws, double* __restrict__ distortion, int iters) {
@@ -296,18 +274,11 @@ __global__ void __launch_bounds__(SETUP_TB) lloyd_setup_kernel(LloydArgs a, Atom
       if (at.negated) v = -v;
       s_lut[j] = v;
     }
-    for (int j = 0; j < SOP_MAX_ENTRIES; ++j) { ws->accN[j] = 0; ws->accS[j] = 0; }
-    ws->accD = 0.0;
-    ws->done = 0;
-    ws->list_count = 0;
     // "not finished": the closing iteration overwrites it with the final distortion (never negative)
     distortion[iters] = -1.0;
   }
-  for (int r = threadIdx.x; r < SORT_ROWS; r += SETUP_TB) {
-    ws->cellN[r] = 0; ws->cellS[r] = 0; ws->cellQ[r] = 0; ws->cellA[0][r] = 0.0; ws->cellA[1][r] = 0.0; ws->cellA[2][r] = 0.0;
-  }
   __syncthreads();
-  lloyd_publish_desc(ws, s_lut, s_ne);
+  if (threadIdx.x < 32) make_desc(&ws->desc, s_lut, s_ne);
 }
 
 // Dense list of the pool blocks.  A thread takes sixteen consecutive blocks per round (four 128-bit loads in flight
@@ -363,27 +334,7 @@ __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __
   }
 }
 
-
-// u of the 16 elements of pool block `blk`
-__device__ __forceinline__ void pool_block_u(const LloydArgs& a, const FmtDev& F, int k, unsigned blk, float (&u)[16], unsigned& j_out) {
-  const unsigned nbk = (unsigned)a.nbk;
-  const unsigned m = blk / nbk, j = blk - m * nbk;
-  j_out = j;
-  const uint4* p = reinterpret_cast<const uint4*>(a.W + (long long)m * a.ldw + (long long)j * SOP_G);
-  const uint4 v0 = __ldg(p), v1 = __ldg(p + 1);
-  const uint32_t wb[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-  uint32_t mb = 0;       // the maximum of the sixteen 15-bit magnitude patterns, two per word at a time
-#pragma unroll
-  for (int q = 0; q < 8; ++q) mb = __vmaxu2(mb, wb[q] & 0x7FFF7FFFu);
-  mb = max(mb & 0xFFFFu, mb >> 16);
-  const float amax = __uint_as_float(mb << 16);
-  const float s_hat = scale_quantize(amax, k, F).s_hat;    // a DD table declares tmax = 1
-  const float rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
-#pragma unroll
-  for (int e = 0; e < 16; ++e) u[e] = __fmul_rn((e & 1) ? bf16hi(wb[e >> 1]) : bf16lo(wb[e >> 1]), rcp);
-}
-
-// One tile = the 256 pool blocks (4096 elements) of one CTA pass.  The tile is counting-sorted by
+// One tile = the CTB pool blocks (TILE_ELEMS elements) of one CTA pass.  The tile is counting-sorted by
 // cell in shared memory.  Sorted position p is stored at slot (p & ~15) | ((p ^ (p >> 4)) & 15): the elements of a
 // cell stay next to each other in memory (an iteration reads the split cells' runs, a few 32-byte sectors each,
 // instead of one sector per element), and the thread that sums positions 16 t .. 16 t + 15 of the tile in shared
@@ -396,96 +347,96 @@ __device__ __forceinline__ long long fix24(float v) {   // llrint(v * 2^24): exa
   return fabsf(s) < 2147483648.0f ? (long long)__float2int_rn(s) : __float2ll_rn(s);
 }
 
-constexpr int CELL_LIMBS = 14;            // Lloyd: counts (2), sum omega u (3), three moments (3 each)
-constexpr int CELL_LIMBS_DP = 8;          // dynamic programme: counts (2), sum omega u (3), sum omega u u (3)
-constexpr int CELL_SPILL_TILES_MAX = 128;     // a low limb takes at most 258 * (2^16 - 1) per tile: 128 tiles stay below 2^32
-constexpr int TILES_PER_WARP_MAX = 4;         // tiles a warp of an iteration CTA walks between two folds of its limb sums (see flush_limbs)
+constexpr int CELL_SPILL_TILES_MAX = 128;     // cache tiles a CTA sorts between two transfers of its per-cell sums to the global ones (any number is safe)
+constexpr int TILES_PER_WARP_MAX = 4;         // range of a tuning argument that has no effect any more
 
-// Launch-shape parameters of the pool cache and of the iteration grid.  The defaults are the largest values the
-// limb arithmetic allows; sop_dd4_lloyd_tuning lowers them (tests reach the mid-loop spill and a multi-tile warp
-// share on small layers that way).  Results do not depend on them.
-struct LloydTune { int spill_tiles, cache_ctas, tiles_per_warp, iter_ctas; };
-static LloydTune g_tune = {CELL_SPILL_TILES_MAX, 0, TILES_PER_WARP_MAX, 0};
-constexpr double MOMENT_UNIT = 1099511627776.0;   // 2^40
+// Launch-shape parameters of the pool cache and of the iteration grid; sop_dd4_lloyd_tuning lowers them (tests reach the
+// mid-loop transfer and CTAs with many tiles on small layers that way).  Results do not depend on them.
+struct LloydTune { int spill_tiles, cache_ctas, iter_ctas; };
+static LloydTune g_tune = {CELL_SPILL_TILES_MAX, 0, 0};
 
-__device__ __forceinline__ void add_limbs3(unsigned (*cL)[SORT_ROWS], int first, int cell, long long v) {
-  atomicAdd(&cL[first][cell], (unsigned)(v & 0xFFFFll));
-  atomicAdd(&cL[first + 1][cell], (unsigned)((v >> 16) & 0xFFFFll));
-  atomicAdd(&cL[first + 2][cell], (unsigned)(int)(v >> 32));
-}
+// Sums of a run (at most 16 elements of one cell, |u| <= WIDE_U): fix(omega) below 2^29, fix(omega u) below 2^30 in magnitude, and
+//   Lloyd: the moments sum omega, sum omega d, sum omega d^2 of the distance d = 256 u - (number of the cell's centre);
+//   DP: fix(omega u u), exact, in the bits of m0.
+// Kept as arrays: the runs that neighbouring threads store go to neighbouring cells.
+template <int N> struct RunArrays { int2 ns[N]; double m0[N], m1[N], m2[N]; };
+constexpr float WIDE_U = 2.0f;                   // blocks with a larger |u| (a scale that saturated) make their tile a wide one
 
-// One run of elements of one cell (at most 16): fix(omega) sums below 2^28, fix(omega u) and fix(omega u u) sums below
-// 2^37 in magnitude, moments below 2^6 in magnitude (so below 2^46 in units of 2^-40).
-// DP: the sums that the grid-constrained construction reads (fix(omega), fix(omega u), fix(omega u u)); otherwise those of
-// the Lloyd iterations (fix(omega), fix(omega u) and the three moments).
+struct CacheSmem {
+  uint2 stage[TILE_ELEMS];
+  unsigned hist[2][SORT_ROWS + 3];               // per cell: count, then first sorted position; of this tile and the next
+  // runs: [0, CTB) the threads' first ones, then by cell a thread's other ones (no two threads have the same cell among them)
+  RunArrays<CTB + SORT_ROWS> run;
+  unsigned long long accN[SORT_ROWS];            // this CTA's per-cell sums
+  long long accS[SORT_ROWS];
+  double accA[3][SORT_ROWS];
+  unsigned warp_tot[CTB / 32];
+};
+
+// Whole CTA, after a barrier: the CTA's sums are added to the per-cell sums of the pool and cleared.
 template <bool DP>
-__device__ __forceinline__ void flush_cell(unsigned (*cL)[SORT_ROWS], int cell, unsigned long long n, unsigned long long sv,
-                                           unsigned long long sq, double a0, double a1, double a2) {
-  atomicAdd(&cL[0][cell], (unsigned)(n & 0xFFFFull));
-  atomicAdd(&cL[1][cell], (unsigned)(n >> 16));
-  add_limbs3(cL, 2, cell, (long long)sv);
-  if (DP) {
-    add_limbs3(cL, 5, cell, (long long)sq);
-  } else {
-    add_limbs3(cL, 5, cell, __double2ll_rn(a0 * MOMENT_UNIT));
-    add_limbs3(cL, 8, cell, __double2ll_rn(a1 * MOMENT_UNIT));
-    add_limbs3(cL, 11, cell, __double2ll_rn(a2 * MOMENT_UNIT));
-  }
-}
-
-__device__ __forceinline__ long long join_limbs3(unsigned (*cL)[SORT_ROWS], int first, int cell) {
-  return (long long)cL[first][cell] + ((long long)cL[first + 1][cell] << 16) + ((long long)(int)cL[first + 2][cell] << 32);
-}
-
-// Whole CTA, after a barrier: the CTA's limbs are added to the per-cell sums of the pool and cleared.
-template <bool DP>
-__device__ void spill_cells(unsigned (*cL)[SORT_ROWS], LloydWs* ws) {
-  for (int r = threadIdx.x; r < SORT_ROWS; r += blockDim.x) {
-    const unsigned long long n = (unsigned long long)cL[0][r] + ((unsigned long long)cL[1][r] << 16);
-    const long long sv = join_limbs3(cL, 2, r);
-    if (n) atomicAdd(&ws->cellN[r], n);
-    if (sv) atomicAdd(reinterpret_cast<unsigned long long*>(&ws->cellS[r]), (unsigned long long)sv);
+__device__ void spill_cells(CacheSmem& S, LloydWs* ws) {
+  for (int r = threadIdx.x; r < SORT_ROWS; r += CTB) {
+    if (S.accN[r]) atomicAdd(&ws->cellN[r], S.accN[r]);
+    if (S.accS[r]) atomicAdd(reinterpret_cast<unsigned long long*>(&ws->cellS[r]), (unsigned long long)S.accS[r]);
+    S.accN[r] = 0; S.accS[r] = 0;
     if (DP) {
-      const long long sq = join_limbs3(cL, 5, r);
-      if (sq) atomicAdd(reinterpret_cast<unsigned long long*>(&ws->cellQ[r]), (unsigned long long)sq);
+      const long long q = __double_as_longlong(S.accA[0][r]);
+      if (q) atomicAdd(reinterpret_cast<unsigned long long*>(&ws->cellQ[r]), (unsigned long long)q);
+      S.accA[0][r] = 0.0;
     } else {
-      const long long m0 = join_limbs3(cL, 5, r), m1 = join_limbs3(cL, 8, r), m2 = join_limbs3(cL, 11, r);
-      if (m0) atomicAdd(&ws->cellA[0][r], (double)m0 * (1.0 / MOMENT_UNIT));
-      if (m1) atomicAdd(&ws->cellA[1][r], (double)m1 * (1.0 / MOMENT_UNIT));
-      if (m2) atomicAdd(&ws->cellA[2][r], (double)m2 * (1.0 / MOMENT_UNIT));
-    }
 #pragma unroll
-    for (int l = 0; l < (DP ? CELL_LIMBS_DP : CELL_LIMBS); ++l) cL[l][r] = 0;
+      for (int x = 0; x < 3; ++x) {
+        if (S.accA[x][r] != 0.0) atomicAdd(&ws->cellA[x][r], S.accA[x][r]);
+        S.accA[x][r] = 0.0;
+      }
+    }
   }
 }
 
+// What bounds it: shared-memory wavefronts (80 % busy): the sort's scattered accesses and the runs' sums.  A tile's weights are loaded
+// while the tile before it is summed (the kernel waited for them for a third of its time), the sums run without divergence -- a run is
+// stored when the next one begins, and the owner of a cell collects its runs afterwards -- and the sorted tile leaves by one
+// asynchronous bulk copy.  8192 x 8192, half the blocks in the pool: 167 us (228 us with limb atomics per run, executed for one lane
+// at a time); 28672 x 8192: 563 us (772 us).
 template <bool DP>
-__global__ void __launch_bounds__(LTB) pool_cache_kernel(LloydArgs a, FmtDev F, LloydWs* __restrict__ ws, long long* __restrict__ pool_count_out,
+__global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev F, LloydWs* __restrict__ ws, long long* __restrict__ pool_count_out,
                                                          unsigned spill_tiles) {
-  __shared__ unsigned hist[SORT_ROWS + 3];
-  __shared__ unsigned warp_tot[LTB / 32];
-  extern __shared__ __align__(16) uint2 stage[];                  // TILE_ELEMS pairs (dynamic: the kernel needs 60 KB in all)
-  // this CTA's share of the per-cell sums, as 32-bit limbs that native shared-memory atomics add:
-  // [0..1] sum fix(omega), [2..4] sum fix(omega u), then either [5..7], [8..10], [11..13] the three moments in units
-  // of 2^-40 or (DP) [5..7] sum fix(omega u u).  Low limbs hold 16 bits, the top limb the signed rest.
-  constexpr int NL = DP ? CELL_LIMBS_DP : CELL_LIMBS;
-  __shared__ unsigned cL[NL][SORT_ROWS];
+  extern __shared__ __align__(128) unsigned char cache_smem[];
+  CacheSmem& S = *reinterpret_cast<CacheSmem*>(cache_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < NL * SORT_ROWS; i += LTB) (&cL[0][0])[i] = 0;
-  unsigned tiles_since_spill = 0;
+  for (int r = tid; r < SORT_ROWS; r += CTB) { S.accN[r] = 0; S.accS[r] = 0; S.accA[0][r] = S.accA[1][r] = S.accA[2][r] = 0.0; }
+  for (int i = tid; i < SORT_ROWS + 3; i += CTB) S.hist[0][i] = 0;
   const unsigned count = ws->list_count;
-  const unsigned n_tiles = (count + LTB - 1) / LTB;
+  const unsigned n_tiles = (count + CTB - 1) / CTB;
   const int k = ws->k;
   if (blockIdx.x == 0 && tid == 0) *pool_count_out = (long long)count;   // the list is complete: its length is the pool size
-  for (unsigned tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    for (int i = tid; i < SORT_ROWS + 3; i += LTB) hist[i] = 0;
-    __syncthreads();
-    const unsigned i = tile * LTB + tid;
-    float u[16], om[16];
-    if (i < count) {
-      unsigned j;
-      pool_block_u(a, F, k, a.pool_idx[i], u, j);
-      const float4* op = reinterpret_cast<const float4*>(a.omega + (size_t)j * SOP_G);
+  const unsigned nbk = (unsigned)a.nbk;
+  unsigned tiles_since_spill = 0;
+  int cur = 0;
+  // the weights of a tile are loaded one tile ahead, the list entries two
+  uint4 wn0 = make_uint4(0u, 0u, 0u, 0u), wn1 = wn0;
+  unsigned jn = 0, idx2 = 0;
+  auto load_idx = [&](unsigned tile) { const unsigned i = tile * CTB + tid; return tile < n_tiles && i < count ? a.pool_idx[i] : 0xFFFFFFFFu; };
+  auto load_w = [&](unsigned blk) {
+    wn0 = wn1 = make_uint4(0u, 0u, 0u, 0u);
+    jn = 0xFFFFFFFFu;
+    if (blk != 0xFFFFFFFFu) {
+      const unsigned m = blk / nbk;
+      jn = blk - m * nbk;
+      const uint4* p = reinterpret_cast<const uint4*>(a.W + (long long)m * a.ldw + (long long)jn * SOP_G);
+      wn0 = __ldg(p); wn1 = __ldg(p + 1);
+    }
+  };
+  load_w(load_idx(blockIdx.x));
+  idx2 = load_idx(blockIdx.x + gridDim.x);
+  __syncthreads();
+  for (unsigned tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, cur ^= 1) {
+    unsigned* hist = S.hist[cur];
+    const uint32_t wb[8] = {wn0.x, wn0.y, wn0.z, wn0.w, wn1.x, wn1.y, wn1.z, wn1.w};
+    float om[16];
+    if (jn != 0xFFFFFFFFu) {
+      const float4* op = reinterpret_cast<const float4*>(a.omega + (size_t)jn * SOP_G);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const float4 o = __ldg(op + q);
@@ -493,362 +444,492 @@ __global__ void __launch_bounds__(LTB) pool_cache_kernel(LloydArgs a, FmtDev F, 
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < 16; ++e) { u[e] = 0.0f; om[e] = 0.0f; }
+      for (int e = 0; e < 16; ++e) om[e] = 0.0f;
     }
+    uint32_t mb = 0;       // the maximum of the sixteen 15-bit magnitude patterns, two per word at a time
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mb = __vmaxu2(mb, wb[q] & 0x7FFF7FFFu);
+    mb = max(mb & 0xFFFFu, mb >> 16);
+    const float amax = __uint_as_float(mb << 16);
+    const float s_hat = scale_quantize(amax, k, F).s_hat;    // a DD table declares tmax = 1
+    const float rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
     unsigned where[16];   // cell << 16 | arrival number inside the cell
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
-      const unsigned c = (unsigned)sort_cell(u[e]);
+      const float u = __fmul_rn((e & 1) ? bf16hi(wb[e >> 1]) : bf16lo(wb[e >> 1]), rcp);
+      const unsigned c = (unsigned)sort_cell(u);
       where[e] = (c << 16) | atomicAdd(&hist[c], 1u);
     }
-    __syncthreads();
-    // exclusive scan of the 641 counts: three bins per thread
+    const bool wide = __syncthreads_or(!(__fmul_rn(amax, rcp) <= WIDE_U)) != 0;
+    // exclusive scan of the counts: two bins per thread
     {
-      const int b0 = 3 * tid;
-      unsigned c0 = 0, c1 = 0, c2 = 0;
-      if (b0 < SORT_ROWS) { c0 = hist[b0]; c1 = hist[b0 + 1]; c2 = hist[b0 + 2]; }
-      const unsigned local = c0 + c1 + c2;
+      static_assert(2 * CTB >= SORT_ROWS + 1, "two bins per thread");
+      const int b0 = 2 * tid;
+      unsigned c0 = 0, c1 = 0;
+      if (b0 < SORT_ROWS) { c0 = hist[b0]; c1 = hist[b0 + 1]; }        // (hist[SORT_ROWS] is zero)
+      const unsigned local = c0 + c1;
       unsigned incl = local;
       for (int o = 1; o < 32; o <<= 1) {
         const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
         if (lane >= o) incl += v;
       }
-      if (lane == 31) warp_tot[warp] = incl;
+      if (lane == 31) S.warp_tot[warp] = incl;
+      if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");       // the tile before this one has left the stage
       __syncthreads();
       unsigned base = 0;
-      for (int w = 0; w < warp; ++w) base += warp_tot[w];
+      for (int w = 0; w < warp; ++w) base += S.warp_tot[w];
       const unsigned excl = base + incl - local;
-      if (b0 < SORT_ROWS) { hist[b0] = excl; hist[b0 + 1] = excl + c0; hist[b0 + 2] = excl + c0 + c1; }
+      if (b0 <= SORT_ROWS) { hist[b0] = excl; hist[b0 + 1] = excl + c0; }      // hist[SORT_ROWS] = TILE_ELEMS: the end of the last cell
     }
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
+      const float u = __fmul_rn((e & 1) ? bf16hi(wb[e >> 1]) : bf16lo(wb[e >> 1]), rcp);
       const unsigned p = hist[where[e] >> 16] + (where[e] & 0xFFFFu);
-      stage[tile_slot(p)] = make_uint2(__float_as_uint(u[e]), __float_as_uint(om[e]));
+      S.stage[tile_slot(p)] = make_uint2(__float_as_uint(u), __float_as_uint(om[e]));
     }
+    load_w(idx2);
+    idx2 = load_idx(tile + 2 * gridDim.x);
+    if (!DP) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (!DP) {      // the dynamic programme reads the per-cell sums only: no iteration walks the elements again
-      uint4* dst = reinterpret_cast<uint4*>(a.cache + (size_t)tile * TILE_ELEMS);
-      const uint4* src = reinterpret_cast<const uint4*>(stage);
-#pragma unroll
-      for (int q = 0; q < TILE_ELEMS / 2 / LTB; ++q) dst[q * LTB + tid] = src[q * LTB + tid];
-      unsigned short* ts = a.tile_start + (size_t)tile * (SORT_ROWS + 1);
-      for (int r = tid; r <= SORT_ROWS; r += LTB) ts[r] = (unsigned short)hist[r];      // hist[SORT_ROWS] = 4096: the end of the last cell
+      if (tid == 0) {
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                     ::"l"(a.cache + (size_t)tile * TILE_ELEMS), "r"((unsigned)__cvta_generic_to_shared(S.stage)), "r"((unsigned)(TILE_ELEMS * sizeof(uint2))) : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      }
+      unsigned* ts = reinterpret_cast<unsigned*>(a.tile_start + (size_t)tile * TS_PITCH);
+      if (2 * tid <= SORT_ROWS) ts[tid] = hist[2 * tid] | (hist[2 * tid + 1] << 16);
     }
-    // per-cell sums: thread t owns the sorted positions 16 t .. 16 t + 15 (ascending cells), keeps the
-    // current cell's sums in registers and adds them to the CTA's limbs when the cell changes
-    {
-      int cur = -1;
-      unsigned long long n = 0, sv = 0, sq = 0;
-      double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-#pragma unroll 4
-      for (int i2 = 0; i2 < 16; ++i2) {
-        const uint2 v = stage[tile_slot(16u * (unsigned)tid + (unsigned)i2)];
-        const float u = __uint_as_float(v.x), om = __uint_as_float(v.y);
-        const int c = sort_cell(u);
-        if (c != cur) {
-          if (cur >= 0) flush_cell<DP>(cL, cur, n, sv, sq, a0, a1, a2);
-          cur = c; n = 0; sv = 0; sq = 0; a0 = a1 = a2 = 0.0;
+    for (int i = tid; i < SORT_ROWS + 3; i += CTB) S.hist[cur ^ 1][i] = 0;
+    if (!wide) {
+      // thread t owns the sorted positions 16 t .. 16 t + 15 (ascending cells): run after run in registers
+      int n = 0, s = 0, c_now = -1, q_sum = 0;
+      double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+      int dst = tid;
+      auto store = [&]() {
+        S.run.ns[dst] = make_int2(n, s);
+        if (DP) { S.run.m0[dst] = __longlong_as_double((long long)q_sum); }
+        else { S.run.m0[dst] = m0; S.run.m1[dst] = m1; S.run.m2[dst] = m2; }
+      };
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const uint2 v = S.stage[(unsigned)(16 * tid) + (unsigned)(i ^ (tid & 15))];
+        const float u = __uint_as_float(v.x), w = __uint_as_float(v.y);
+        const float t = fminf(fmaxf(__fmaf_rn(u, SORT_INVH, SORT_MAGIC + (float)SORT_CHALF), SORT_MAGIC), SORT_MAGIC + (float)(2 * SORT_CHALF));
+        const int c = (int)(__float_as_uint(t) - __float_as_uint(SORT_MAGIC));
+        const bool next = i > 0 && c != c_now;
+        if (next) {
+          store();
+          dst = CTB + c;
         }
-        const float ou = fminf(fmaxf(__fmul_rn(om, u), -256.0f), 256.0f);
-        n += (unsigned long long)__float2uint_rn(__fmul_rn(om, 16777216.0f));   // omega in [0, 1]
-        sv += (unsigned long long)fix24(ou);
+        c_now = c;
+        const float w24 = __fmul_rn(w, 16777216.0f), ou24 = __fmul_rn(w24, u);   // omega u, rounded once, times 2^24
+        n = (next ? 0 : n) + __float2int_rn(w24);                                // omega in [0, 1]
+        s = (next ? 0 : s) + __float2int_rn(ou24);
         if (DP) {
-          sq += (unsigned long long)fix24(__fmul_rn(ou, u));
+          q_sum = (next ? 0 : q_sum) + __float2int_rn(__fmul_rn(ou24, u));
         } else {
-          const double dou = (double)om * (double)u;
-          a0 += (double)om; a1 += dou; a2 += dou * (double)u;
+          const double keep = next ? 0.0 : 1.0, wd = (double)w;
+          const double d = (double)__fmaf_rn(u, SORT_INVH, __fsub_rn(SORT_MAGIC + (float)SORT_CHALF, t));      // 256 u - (c - 320): exact in a cell
+          const double x = __dmul_rn(wd, d);
+          m0 = __fma_rn(m0, keep, wd);
+          m1 = __fma_rn(m1, keep, x);
+          m2 = __fma_rn(m2, keep, __dmul_rn(x, d));
         }
       }
-      flush_cell<DP>(cL, cur, n, sv, sq, a0, a1, a2);
+      store();
     }
     __syncthreads();
-    // a cell takes at most 258 flushes per tile and a low limb 2^16 - 1 per flush: the limbs go to the
-    // global sums before they can wrap
-    if (++tiles_since_spill == spill_tiles) {
-      spill_cells<DP>(cL, ws);
-      tiles_since_spill = 0;
-      __syncthreads();
-    }
-  }
-  if (tiles_since_spill) spill_cells<DP>(cL, ws);
-}
-
-// One warp per tile.  The elements of the tile that lie in cells holding a threshold (sorted positions
-// [start[c], start[c + 1]) for every such cell c) are dealt to the 32 lanes in contiguous shares, four
-// loads in flight per lane: entry lo or hi by the exact threshold.  Sums go to the CTA's per-entry
-// accumulators with shared-memory atomics (a few hundred elements per tile).
-constexpr int MAX_SPLIT = 32;   // a table has at most 31 thresholds, so at most 31 cells hold one
-
-// Between two folds a CTA walks at most 2^17 elements (8 warps, at most four tiles each), every element adds at most
-// 2^24 to n and 2^32 in magnitude to sv, and there is at most one flush per element.  With 12-bit low
-// limbs every limb sum stays below 2^31: n = 12 bits + the rest, sv = 12 + 12 bits + the signed rest.
-__device__ __forceinline__ void flush_limbs(unsigned* n0, unsigned* n1, unsigned* s0, unsigned* s1, int* s2, int code,
-                                            unsigned long long n, unsigned long long sv) {
-  atomicAdd(&n0[code], (unsigned)(n & 0xFFFull));
-  atomicAdd(&n1[code], (unsigned)(n >> 12));
-  atomicAdd(&s0[code], (unsigned)(sv & 0xFFFull));
-  atomicAdd(&s1[code], (unsigned)((sv >> 12) & 0xFFFull));
-  atomicAdd(&s2[code], (int)((long long)sv >> 24));
-}
-
-// One iteration, by a whole CTA.  `counter` counts the CTAs that have added their sums; the CTA that arrives
-// last updates the table and returns true.  FRESH: the descriptor was written during this launch by another
-// CTA, so it is read past the L1.
-template <bool FRESH>
-__device__ __forceinline__ bool lloyd_iteration(const LloydArgs& a, LloydWs* __restrict__ ws, double* __restrict__ distortion,
-                                                int it, int last, float* __restrict__ out_lut, unsigned* counter, bool reset_counter,
-                                                unsigned fold_period) {
-  __shared__ __align__(16) IterDesc d;
-  __shared__ unsigned long long sN[SOP_MAX_ENTRIES], sS[SOP_MAX_ENTRIES];
-  // flushes of the element walk: native 32-bit atomics on limbs, combined into sN / sS afterwards
-  __shared__ unsigned lN[2][SOP_MAX_ENTRIES], lS0[SOP_MAX_ENTRIES], lS1[SOP_MAX_ENTRIES];
-  __shared__ int lS2[SOP_MAX_ENTRIES];
-  __shared__ double sD;
-  __shared__ int s_is_last;
-  __shared__ unsigned s_list_count;
-  __shared__ CellEntry s_entry[MAX_SPLIT];
-  __shared__ unsigned short s_cell[MAX_SPLIT];
-  __shared__ unsigned short s_off[LTB / 32][MAX_SPLIT + 1];   // per warp: first item of every split cell in the tile
-  __shared__ unsigned short s_p0[LTB / 32][MAX_SPLIT];
-  __shared__ float s_new[SOP_MAX_ENTRIES];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  {
-    constexpr int DW = (int)(sizeof(IterDesc) / sizeof(unsigned));
-    static_assert(DW <= LTB, "one descriptor word per thread");
-    if (tid < DW) {
-      const unsigned* src = reinterpret_cast<const unsigned*>(&ws->desc) + tid;
-      reinterpret_cast<unsigned*>(&d)[tid] = FRESH ? __ldcg(src) : *src;
-    }
-    if (tid == LTB - 1) s_list_count = ws->list_count;
-    if (tid < 32) { sN[tid] = 0; sS[tid] = 0; lN[0][tid] = lN[1][tid] = lS0[tid] = lS1[tid] = 0; lS2[tid] = 0; }
-    if (tid == 0) sD = 0.0;
-  }
-  __syncthreads();
-  const int ne = d.n_entries;
-  const unsigned n_tiles = (s_list_count + LTB - 1) / LTB;
-  const float* lutv = d.lut;
-  const float* tau = d.tau;
-  // the cells that hold thresholds: thresholds ascend, so those of one cell are neighbours.  Every warp
-  // derives the same list and writes the same values.
-  int n_split;
-  {
-    const bool on = lane < ne - 1;
-    const int c = d.thr_cell[lane];
-    const int cp = __shfl_up_sync(0xFFFFFFFFu, c, 1), cn = __shfl_down_sync(0xFFFFFFFFu, c, 1);
-    const bool first = on && (lane == 0 || cp != c);
-    const bool single = lane == ne - 2 || cn != c;
-    const unsigned fm = __ballot_sync(0xFFFFFFFFu, first);
-    n_split = __popc(fm);
-    if (first) {
-      const int idx = __popc(fm & ((1u << lane) - 1u));
-      CellEntry e;
-      e.thr = tau[lane];
-      e.codes = single ? ((unsigned)lane | ((unsigned)(lane + 1) << 8)) : 0xFFFFu;
-      s_cell[idx] = (unsigned short)c;
-      s_entry[idx] = e;
-    }
-    __syncwarp();
-  }
-  double D = 0.0;
-  {
-    // every cell without a threshold through its sums and moments, spread over the grid (a thread takes
-    // one cell): its entry is the number of thresholds in lower cells, and
-    // sum omega (u - q)^2 = A2 - 2 q A1 + q^2 A0 for the entry's value q
-    for (int r = (int)blockIdx.x + (int)gridDim.x * (LTB - 1 - tid); r < SORT_ROWS; r += (int)gridDim.x * LTB) {
-      const unsigned long long cn = ws->cellN[r];
-      const long long cs = ws->cellS[r];
-      const double a0 = ws->cellA[0][r], a1 = ws->cellA[1][r], a2 = ws->cellA[2][r];
-      int j = 0;
-      bool split = false;
-      for (int k = 0; k < ne - 1; ++k) { const int c = d.thr_cell[k]; j += c < r ? 1 : 0; split |= c == r; }
-      if (!split && (cn || a0 != 0.0)) {
-        if (!last) { atomicAdd(&sN[j], cn); atomicAdd(&sS[j], (unsigned long long)cs); }
-        const double q = (double)lutv[j];
-        D += a2 - 2.0 * q * a1 + q * q * a0;
+    // the owner of a cell adds up its runs: the run of the thread where it begins (its first one when the cell begins at the
+    // thread's first position) and the first runs of the threads after that up to the one where it ends
+    if (!wide) {
+      for (int c = tid; c < SORT_ROWS; c += CTB) {
+        const unsigned p0 = hist[c], p1 = hist[c + 1];
+        if (p0 == p1) continue;
+        const unsigned t0 = p0 >> 4, t1 = (p1 - 1) >> 4;
+        const unsigned r = (p0 & 15u) == 0u ? t0 : (unsigned)(CTB + c);
+        unsigned long long n = (unsigned)S.run.ns[r].x;
+        long long s = S.run.ns[r].y, q = DP ? __double_as_longlong(S.run.m0[r]) : 0;
+        double m0 = S.run.m0[r], m1 = DP ? 0.0 : S.run.m1[r], m2 = DP ? 0.0 : S.run.m2[r];
+        for (unsigned t = t0 + 1; t <= t1; ++t) {
+          n += (unsigned)S.run.ns[t].x; s += S.run.ns[t].y;
+          if (DP) q += __double_as_longlong(S.run.m0[t]);
+          else { m0 += S.run.m0[t]; m1 += S.run.m1[t]; m2 += S.run.m2[t]; }
+        }
+        S.accN[c] += n; S.accS[c] += s;
+        if (DP) S.accA[0][c] = __longlong_as_double(__double_as_longlong(S.accA[0][c]) + q);
+        else { S.accA[0][c] += m0; S.accA[1][c] += m1; S.accA[2][c] += m2; }
       }
-    }
-  }
-  // Round k of the CTA covers tiles (k gridDim + blockIdx) 8 .. + 7, one per warp.  The limb accumulators hold what a
-  // warp adds in at most four rounds (flush_limbs), so every fold_period <= 4 rounds the CTA folds them into its
-  // 64-bit sums: a CTA may then walk any number of tiles, and a grid that is resident at once serves any pool.
-  for (unsigned k = 0;; ++k) {
-    const unsigned tile0 = (k * gridDim.x + blockIdx.x) * (LTB / 32);
-    if (tile0 >= n_tiles) break;                       // the same for every warp of the CTA
-    if (k != 0 && k % fold_period == 0) {
-      __syncthreads();
-      if (tid < 32 && !last) {
-        sN[tid] += (unsigned long long)lN[0][tid] + ((unsigned long long)lN[1][tid] << 12);
-        sS[tid] += (unsigned long long)lS0[tid] + ((unsigned long long)lS1[tid] << 12) + ((unsigned long long)(long long)lS2[tid] << 24);
-        lN[0][tid] = lN[1][tid] = lS0[tid] = lS1[tid] = 0; lS2[tid] = 0;
-      }
-      __syncthreads();
-    }
-    const unsigned tile = tile0 + warp;
-    if (tile >= n_tiles) continue;
-    const unsigned short* ts = a.tile_start + (size_t)tile * (SORT_ROWS + 1);
-    const uint2* src = a.cache + (size_t)tile * TILE_ELEMS;
-    // segment lengths -> exclusive offsets (one cell per lane)
-    unsigned len0 = 0, q0 = 0;
-    if (lane < n_split) { const int c = s_cell[lane]; q0 = ts[c]; len0 = ts[c + 1] - q0; }
-    unsigned inc0 = len0;
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v0 = __shfl_up_sync(0xFFFFFFFFu, inc0, o);
-      if (lane >= o) inc0 += v0;
-    }
-    const unsigned total = __shfl_sync(0xFFFFFFFFu, inc0, 31);
-    __syncwarp();
-    s_off[warp][lane] = (unsigned short)(inc0 - len0); s_p0[warp][lane] = (unsigned short)q0;
-    if (lane == 0) s_off[warp][MAX_SPLIT] = (unsigned short)total;
-    __syncwarp();
-    // every lane takes a contiguous share of the items: its entry changes a few times at most, so the
-    // sums of the current entry stay in registers and reach the CTA's accumulators on a change
-    const unsigned share = (total + 31u) / 32u;
-    const unsigned i_lo = min(total, lane * share), i_hi = min(total, i_lo + share);
-    int cur = -1;
-    unsigned long long n = 0, sv = 0;
-    for (unsigned base = i_lo; base < i_hi; base += 4) {
-      uint2 v[4];
-      int cell_l[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const unsigned item = base + k;
-        cell_l[k] = -1;
-        v[k] = make_uint2(0u, 0u);
-        if (item < i_hi) {
-          int l = 0;                       // the split cell whose item range holds `item`: binary search over <= 32 offsets
-#pragma unroll
-          for (int step = 16; step >= 1; step >>= 1) {     // branch-free: s_off has MAX_SPLIT + 1 entries
-            const int t = l + step;
-            const bool ok = (t < n_split) & (s_off[warp][min(t, MAX_SPLIT)] <= item);
-            l = ok ? t : l;
-          }
-          cell_l[k] = l;
-          const unsigned pp = s_p0[warp][l] + (item - s_off[warp][l]);
-          v[k] = __ldg(src + tile_slot(pp));
+    } else {
+      // a wide tile: element by element in 64 bits, straight to the global sums
+#pragma unroll 1
+      for (int i = 0; i < 16; ++i) {
+        const uint2 v = S.stage[(unsigned)(16 * tid) + (unsigned)(i ^ (tid & 15))];
+        const float u = __uint_as_float(v.x), w = __uint_as_float(v.y);
+        if (w == 0.0f) continue;
+        const int c = sort_cell(u);
+        const float ou = fminf(fmaxf(__fmul_rn(w, u), -256.0f), 256.0f);
+        atomicAdd(&ws->cellN[c], (unsigned long long)fix24(w));
+        atomicAdd(reinterpret_cast<unsigned long long*>(&ws->cellS[c]), (unsigned long long)fix24(ou));
+        if (DP) {
+          atomicAdd(reinterpret_cast<unsigned long long*>(&ws->cellQ[c]), (unsigned long long)fix24(__fmul_rn(ou, u)));
+        } else {
+          const double d = (double)u * 256.0 - (double)(c - SORT_CHALF);
+          atomicAdd(&ws->cellA[0][c], (double)w);
+          atomicAdd(&ws->cellA[1][c], (double)w * d);
+          atomicAdd(&ws->cellA[2][c], (double)w * d * d);
         }
       }
+    }
+    if (++tiles_since_spill == spill_tiles) {
+      spill_cells<DP>(S, ws);               // (a thread clears the cells it owns)
+      tiles_since_spill = 0;
+    }
+  }
+  if (tiles_since_spill) spill_cells<DP>(S, ws);
+  if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------------------------
+// The iterations.  A cell that holds a threshold of the current table ("split cell") is walked element by element; every other
+// cell lies inside one entry's interval and is accounted for by its sums.
+//   A CTA owns a contiguous range of cache tiles and keeps their cell starts in shared memory over all iterations.  A run is the
+//   elements of one split cell in one tile; eight lanes take a run (neighbouring 8-byte elements), four tiles per warp and step,
+//   the next step's elements are loaded ahead.  The warps take the runs cell by cell: the sums of a cell (all of it, and the part
+//   above its threshold) stay in registers until the warp moves to the next cell, one to three times per iteration.
+//   The cells without a threshold are a matter of CTA 0: prefix sums over all cells, built once, make an entry's share the
+//   difference of two of them.  (About the origin, in FP64: the distortion is a few thousandths of the second moment, so 1e-16 of
+//   that leaves it 1e-13.)
+//   Every CTA adds its sums to the iteration's global ones, arrives at a counter, waits (bounded) until all have arrived and then
+//   works out the next table for itself: the sums are integers, so all get the same one and nobody has to hand it on.
+// What bounds it: the chain of one iteration (the first elements, global additions, their fence, arrival, sums, table: about 4.5 us;
+// 9 us when the last CTA worked out the table and handed it on) and, for a large pool, the latency of the split cells' elements.
+// Nine iterations on 25 thousand pool blocks 44 us (82 us with a warp per tile), on 2 million 102 us (150 us), on 7.3 million
+// 241 us (341 us).  Every warp must have its share of every cell: dealt cell by cell, the warps of the outer thresholds waited
+// for those of the inner ones and the 7.3 million took 685 us.
+// ---------------------------------------------------------------------------------------------
+constexpr int ITB = 768;            // threads of an iteration CTA (one per SM)
+constexpr int PRE = 4;              // elements of a run that a lane loads one step ahead
+constexpr int MAX_SPLIT = 32;       // a table has at most 31 thresholds, so at most 31 cells hold one
+constexpr int LIMBS = 3;            // 64-bit sums modulo 2^64 as 20 + 20 + 24 bits, which native 32-bit shared-memory additions take
+constexpr unsigned WAIT_POLLS = 1u << 21;      // polls of a few hundred ns: about half a second
+
+struct IterSmem {
+  IterDesc d;
+  unsigned limb[2][LIMBS][SOP_MAX_ENTRIES];    // this CTA's sums per entry: fix(omega), fix(omega u)
+  unsigned long long sum[2][SOP_MAX_ENTRIES];  // the same of cells with several thresholds
+  double warp_D[ITB / 32];
+  CellEntry entry[MAX_SPLIT];
+  unsigned short cell[MAX_SPLIT];
+  int n_split, stop, is_last;
+  float table[SOP_MAX_ENTRIES];
+  // CTA 0: sums over the cells before r
+  unsigned long long preN[SORT_ROWS + 1];
+  long long preS[SORT_ROWS + 1];
+  double preA[3][SORT_ROWS + 1];
+};
+
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v, unsigned lanes = 0xFFFFFFFFu) {      // modulo 2^64, by 32-bit sums of 27-bit limbs
+  const unsigned a = __reduce_add_sync(lanes, (unsigned)v & 0x7FFFFFFu), b = __reduce_add_sync(lanes, (unsigned)(v >> 27) & 0x7FFFFFFu),
+                 c = __reduce_add_sync(lanes, (unsigned)(v >> 54));
+  return (unsigned long long)a + ((unsigned long long)b << 27) + ((unsigned long long)c << 54);
+}
+__device__ __forceinline__ unsigned limb_of(unsigned long long v, int i) {
+  return i == 0 ? (unsigned)v & 0xFFFFFu : i == 1 ? (unsigned)(v >> 20) & 0xFFFFFu : (unsigned)(v >> 40);
+}
+__device__ __forceinline__ unsigned long long join_limbs(IterSmem& S, int w, int code) {
+  return (unsigned long long)S.limb[w][0][code] + ((unsigned long long)S.limb[w][1][code] << 20) + ((unsigned long long)S.limb[w][2][code] << 40);
+}
+
+// One warp: the cells that hold thresholds (thresholds ascend, so those of one cell are neighbours).
+__device__ void split_cells(IterSmem& S) {
+  const int lane = threadIdx.x & 31, ne = S.d.n_entries;
+  const bool on = lane < ne - 1;
+  const int c = S.d.thr_cell[lane];
+  const int cp = __shfl_up_sync(0xFFFFFFFFu, c, 1), cn = __shfl_down_sync(0xFFFFFFFFu, c, 1);
+  const bool first = on && (lane == 0 || cp != c);
+  const bool single = lane == ne - 2 || cn != c;
+  const unsigned fm = __ballot_sync(0xFFFFFFFFu, first);
+  if (first) {
+    const int idx = __popc(fm & ((1u << lane) - 1u));
+    CellEntry e;
+    e.thr = S.d.tau[lane];
+    e.codes = single ? ((unsigned)lane | ((unsigned)(lane + 1) << 8)) : 0xFFFFu;
+    S.cell[idx] = (unsigned short)c;
+    S.entry[idx] = e;
+  }
+  if (lane == 0) S.n_split = __popc(fm);
+}
+
+// One warp: the descriptor of a table (entry j of the sorted table, padded with its last value, in lane j): the decision
+// thresholds (the same rule as build_thresholds: the largest fp32 <= the midpoint, a repeated entry takes the threshold above
+// it, +inf from n_entries - 1 on) and their lookup cells.  sort_cell is monotone, so an element in a lower cell than a
+// threshold's is below the threshold and one in a higher cell is above it: only the elements of the cells listed here need the
+// comparison itself.
+__device__ void make_desc(IterDesc* d, const float* table, int ne) {
+  const int j = threadIdx.x & 31;
+  int jj = j;
+  while (jj < ne - 1 && table[jj] == table[jj + 1]) ++jj;
+  const float t = jj < ne - 1 ? __double2float_rd(0.5 * ((double)table[jj] + (double)table[jj + 1])) : __int_as_float(0x7F800000);
+  d->lut[j] = table[j];
+  d->tau[j] = t;
+  d->thr_cell[j] = j < ne - 1 ? sort_cell(t) : SORT_ROWS;
+  if (j == 0) d->n_entries = ne;
+}
+
+// One warp: centroids one lane per entry, snapped to bf16, ascending (ties by index); leaves the new table in S.table.
+__device__ void new_table(IterSmem& S, unsigned long long n, long long sv) {
+  const int j = threadIdx.x & 31, ne = S.d.n_entries;
+  float t = S.d.lut[j];                      // lanes from n_entries on hold the last entry's value
+  if (j < ne && n) {
+    const float cen = __double2float_rn(__ddiv_rn(__ll2double_rn(sv), __ull2double_rn(n)));
+    uint32_t b = __float_as_uint(cen);
+    b += 0x7FFFu + ((b >> 16) & 1u);
+    b &= 0xFFFF0000u;                        // nearest bf16, ties to even
+    t = __uint_as_float(b);
+  }
+  int rank = j;
+  const float before = __shfl_up_sync(0xFFFFFFFFu, t, 1);
+  if (__any_sync(0xFFFFFFFFu, j > 0 && j < ne && !(before <= t))) {      // (hardly ever: centroids of neighbouring intervals ascend)
+    rank = 0;
+#pragma unroll 1
+    for (int k = 0; k < ne; ++k) {
+      const float o = __shfl_sync(0xFFFFFFFFu, t, k);
+      rank += o < t || (o == t && k < j) ? 1 : 0;
+    }
+  }
+  if (j < ne) S.table[rank] = t;
+  __syncwarp();
+  const float top = S.table[ne - 1];
+  if (j >= ne) S.table[j] = top;             // padded with the last entry
+  __syncwarp();
+}
+
+// The whole CTA: adds its share of one iteration to the sums of that iteration and arrives.
+template <bool ALL>
+__device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __restrict__ ws, IterSmem& S, const unsigned short* __restrict__ ts,
+                                                unsigned tile0, int T, int it, bool last) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, sub = lane >> 3, ln = lane & 7;
+  constexpr int NW = ITB / 32;
+  const int n_split = S.n_split, Tc = (T + 3) / 4, total = n_split * Tc;
+  double D = 0.0;
+  // step x: cell x / Tc, tiles 4 (x % Tc) .. + 3; a warp takes every NW-th, so that each has its share of the cells with long runs
+  int l = Tc ? warp / Tc : 0, ch = warp - l * Tc;
+  unsigned p0 = 0, p1 = 0;
+  uint2 v[PRE];
+  const uint2* src = a.cache;
+  auto open_run = [&](int x, int lx, int cx) {
+    p0 = p1 = 0;
+    const int t = 4 * cx + sub;
+    if (x < total && t < T) {
+      const unsigned short* row = ts + (size_t)t * TS_PITCH + S.cell[lx];
+      p0 = row[0] + (unsigned)ln; p1 = row[1];
+      src = a.cache + (size_t)(tile0 + (unsigned)t) * TILE_ELEMS;
+    }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (cell_l[k] < 0) continue;
-        const CellEntry e = s_entry[cell_l[k]];
-        const float u = __uint_as_float(v[k].x), om = __uint_as_float(v[k].y);
-        int code;
-        if (e.codes == 0xFFFFu) code = count_below(tau, u);   // several thresholds in one cell: the general search
-        else code = (int)((u > e.thr ? e.codes >> 8 : e.codes) & 0xFFu);
-        const float dd = __fsub_rn(u, lutv[code]);
+    for (int i = 0; i < PRE; ++i) v[i] = p0 + 8u * i < p1 ? __ldg(src + tile_slot(p0 + 8u * i)) : make_uint2(0u, 0u);
+  };
+  open_run(warp, l, ch);
+  unsigned long long nA = 0, nH = 0;
+  long long sA = 0, sH = 0;
+#pragma unroll 1
+  for (int x = warp; x < total; x += NW) {
+    const CellEntry e = S.entry[l];
+    const int c_now = S.cell[l], l_now = l;
+    unsigned q = p0;
+    const unsigned q1 = p1;
+    uint2 w[PRE];
+#pragma unroll
+    for (int i = 0; i < PRE; ++i) w[i] = v[i];
+    const uint2* from = src;
+    ch += NW;
+    while (ch >= Tc) { ch -= Tc; ++l; }
+    open_run(x + NW, l, ch);
+    // The end cells hold everything beyond the grid (any u), and a cell with several thresholds needs the general search.
+    if (e.codes != 0xFFFFu && c_now != 0 && c_now != SORT_ROWS - 1) {
+      const float qlo = S.d.lut[e.codes & 0xFFu], qhi = S.d.lut[e.codes >> 8];
+#pragma unroll 1
+      for (;;) {
+        unsigned n = 0, nh = 0;
+        int s = 0, sh = 0;
+        // |u| <= 1.26: the four terms of a lane stay below 2^31.  An element that is not there reads as (0, 0): its omega is zero.
+#pragma unroll
+        for (int i = 0; i < PRE; ++i) {
+          const float u = __uint_as_float(w[i].x), om = __uint_as_float(w[i].y);
+          const bool hi = u > e.thr;
+          const float dd = __fsub_rn(u, hi ? qhi : qlo);
+          D += (double)__fmul_rn(__fmul_rn(om, dd), dd);
+          const float om24 = __fmul_rn(om, 16777216.0f);
+          const unsigned ni = __float2uint_rn(om24);             // omega in [0, 1]
+          const int si = __float2int_rn(__fmul_rn(om24, u));     // omega u, rounded once, times 2^24
+          n += ni; s += si;
+          if (hi) { nh += ni; sh += si; }
+        }
+        nA += n; nH += nh; sA += s; sH += sh;
+        q += 8u * PRE;
+        if (!__any_sync(0xFFFFFFFFu, q < q1)) break;
+#pragma unroll
+        for (int i = 0; i < PRE; ++i) w[i] = q + 8u * i < q1 ? __ldg(from + tile_slot(q + 8u * i)) : make_uint2(0u, 0u);
+      }
+      if ((l != l_now || x + NW >= total) && !last) {
+        const unsigned long long ta = warp_sum64(nA), th = warp_sum64(nH), ua = warp_sum64((unsigned long long)sA), uh = warp_sum64((unsigned long long)sH);
+        if (lane < 4 * LIMBS) {
+          const int side = lane / (2 * LIMBS), w2 = lane / LIMBS & 1, i = lane % LIMBS;      // below / above the threshold; n / s; limb
+          const unsigned long long y = side ? (w2 ? uh : th) : (w2 ? ua - uh : ta - th);
+          atomicAdd(&S.limb[w2][i][side ? e.codes >> 8 : e.codes & 0xFFu], limb_of(y, i));
+        }
+        nA = nH = 0; sA = sH = 0;
+      }
+    } else {
+#pragma unroll 1
+      for (; q < q1; q += 8u) {
+        const uint2 y = __ldg(from + tile_slot(q));
+        const float u = __uint_as_float(y.x), om = __uint_as_float(y.y);
+        const int code = count_below(S.d.tau, u);
+        const float dd = __fsub_rn(u, S.d.lut[code]);
         D += (double)__fmul_rn(__fmul_rn(om, dd), dd);
         if (!last) {
-          if (code != cur) {
-            if (cur >= 0) flush_limbs(lN[0], lN[1], lS0, lS1, lS2, cur, n, sv);
-            cur = code; n = 0; sv = 0;
-          }
-          const float ou = fminf(fmaxf(__fmul_rn(om, u), -256.0f), 256.0f);
-          n += (unsigned long long)__float2uint_rn(__fmul_rn(om, 16777216.0f));   // omega in [0, 1]
-          sv += (unsigned long long)fix24(ou);
+          const unsigned same = __match_any_sync(__activemask(), code);
+          const unsigned long long tn = warp_sum64((unsigned long long)fix24(om), same);
+          const unsigned long long ts = warp_sum64((unsigned long long)fix24(fminf(fmaxf(__fmul_rn(om, u), -256.0f), 256.0f)), same);
+          if (lane == __ffs((int)same) - 1) { atomicAdd(&S.sum[0][code], tn); atomicAdd(&S.sum[1][code], ts); }
         }
       }
+      __syncwarp();
     }
-    if (cur >= 0) flush_limbs(lN[0], lN[1], lS0, lS1, lS2, cur, n, sv);
   }
+#pragma unroll
   for (int o = 16; o; o >>= 1) D += __shfl_xor_sync(0xFFFFFFFFu, D, o);
-  if (lane == 0 && D != 0.0) atomicAdd(&sD, D);
+  if (lane == 0) S.warp_D[warp] = D;
   __syncthreads();
-  if (tid < ne && !last) {
-    sN[tid] += (unsigned long long)lN[0][tid] + ((unsigned long long)lN[1][tid] << 12);
-    sS[tid] += (unsigned long long)lS0[tid] + ((unsigned long long)lS1[tid] << 12) + ((unsigned long long)(long long)lS2[tid] << 24);
-    if (sN[tid]) atomicAdd(&ws->accN[tid], sN[tid]);
-    if (sS[tid]) atomicAdd(reinterpret_cast<unsigned long long*>(&ws->accS[tid]), sS[tid]);
-  }
-  if (tid == 0 && sD != 0.0) atomicAdd(&ws->accD, sD);
-  // the CTA that arrives last owns the update; no CTA waits for another
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_is_last = atomicAdd(counter, 1u) == gridDim.x - 1 ? 1 : 0;
-  __syncthreads();
-  const bool is_last = s_is_last != 0;
-  if (is_last && tid < 32) {
-    // one warp: every CTA has added its share (cells with a threshold element by element, the others by
-    // their sums).  Centroids one lane per entry, a rank sort, and the next iteration's descriptor.
+  if (warp == 0) {
+    const int ne = S.d.n_entries;
+    unsigned long long n = join_limbs(S, 0, lane) + S.sum[0][lane], s = join_limbs(S, 1, lane) + S.sum[1][lane];
+    S.sum[0][lane] = S.sum[1][lane] = 0ull;
+#pragma unroll
+    for (int i = 0; i < LIMBS; ++i) S.limb[0][i][lane] = S.limb[1][i][lane] = 0u;
+    double dsum = lane < ITB / 32 ? S.warp_D[lane] : 0.0;
+    if (blockIdx.x == 0 && lane < ne) {
+      // cells without a threshold between this entry's two
+      const int lo = lane ? S.d.thr_cell[lane - 1] + 1 : 0, hi = lane < ne - 1 ? S.d.thr_cell[lane] : SORT_ROWS;
+      if (lo < hi) {
+        n += S.preN[hi] - S.preN[lo];
+        s += (unsigned long long)(S.preS[hi] - S.preS[lo]);
+        const double q = 256.0 * (double)S.d.lut[lane];
+        const double b0 = S.preA[0][hi] - S.preA[0][lo], b1 = S.preA[1][hi] - S.preA[1][lo], b2 = S.preA[2][hi] - S.preA[2][lo];
+        dsum += (b2 - q * (2.0 * b1 - q * b0)) * (1.0 / 65536.0);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) dsum += __shfl_xor_sync(0xFFFFFFFFu, dsum, o);
+    if (!last && lane < ne) {
+      if (n) atomicAdd(&ws->accN[it][lane], n);
+      if (s) atomicAdd(reinterpret_cast<unsigned long long*>(&ws->accS[it][lane]), s);
+    }
+    if (lane == 0 && dsum != 0.0) atomicAdd(&ws->accD[it], dsum);
     __threadfence();
-    const unsigned long long n = __ldcg(&ws->accN[tid]);
-    const long long sv = __ldcg(&ws->accS[tid]);
-    if (tid == 0) distortion[it] = __ldcg(&ws->accD);
-    ws->accN[tid] = 0; ws->accS[tid] = 0;
-    if (tid == 0) { ws->accD = 0.0; if (reset_counter) *counter = 0; }
-    if (last) {
-      out_lut[tid] = tid < ne ? lutv[tid] : 0.0f;
+    __syncwarp();
+    if (ALL) {
+      if (lane == 0) atomicAdd(&ws->arrive[it], 1u);           // (no value back: nobody waits for it)
     } else {
-      float t = lutv[tid];                       // lanes from n_entries on hold the last entry's value
-      if (tid < ne && n) {
-        const float cen = __double2float_rn(__ddiv_rn(__ll2double_rn(sv), __ull2double_rn(n)));
-        uint32_t b = __float_as_uint(cen);
-        b += 0x7FFFu + ((b >> 16) & 1u);
-        b &= 0xFFFF0000u;                        // nearest bf16, ties to even
-        t = __uint_as_float(b);
-      }
-      // ascending order: the rank of an entry is the number of entries before it (ties by index)
-      int rank = 0;
-      for (int k = 0; k < 32; ++k) {
-        const float o = __shfl_sync(0xFFFFFFFFu, t, k);
-        rank += (k < ne && (o < t || (o == t && k < tid))) ? 1 : 0;
-      }
-      if (tid < ne) s_new[rank] = t;
+      if (lane == 0) S.is_last = atomicAdd(&ws->arrive[it], 1u) == gridDim.x - 1 ? 1 : 0;
       __syncwarp();
-      if (tid >= ne) s_new[tid] = 0.0f;
-      __syncwarp();
-      const float top = s_new[ne - 1];
-      __syncwarp();
-      if (tid >= ne) s_new[tid] = top;           // padded with the last entry
-      __syncwarp();
-      lloyd_publish_desc(ws, s_new, ne);
     }
   }
-  return is_last;
 }
 
-// One launch per iteration (the stream orders the iterations).
-__global__ void __launch_bounds__(LTB) lloyd_split_kernel(LloydArgs a, LloydWs* __restrict__ ws, double* __restrict__ distortion,
-                                                          int it, int last, float* __restrict__ out_lut, unsigned fold_period) {
-  lloyd_iteration<false>(a, ws, distortion, it, last, out_lut, &ws->done, true, fold_period);
-}
-
-// All iterations in one launch (launched cooperatively: every CTA is resident).  Between two iterations the
-// CTAs wait for the flag that the CTA which arrived last sets after it has published the next table.  The
-// wait is bounded: a CTA that gives up raises ws->error, every CTA then leaves, and the last distortion entry
-// is set to -1 (a distortion is never negative) so that the caller can tell.
-constexpr unsigned WAIT_POLLS = 1u << 22;     // times ~100 ns: about half a second
-
-__global__ void __launch_bounds__(LTB) lloyd_persistent_kernel(LloydArgs a, LloydWs* __restrict__ ws, double* __restrict__ distortion,
-                                                               int iters, float* __restrict__ out_lut, unsigned fold_period) {
-  __shared__ int s_stop;
-  for (int it = 0; it <= iters; ++it) {
-    const int last = it == iters;
-    const bool updater = lloyd_iteration<true>(a, ws, distortion, it, last, out_lut, &ws->arrive[it], false, fold_period);
-    if (last) break;
-    __syncthreads();                       // the updater's first warp has written the descriptor
-    if (threadIdx.x == 0) {
-      int stop = 0;
-      if (updater) {
-        __threadfence();
-        atomicExch(&ws->ready[it], 1u);
-      } else {
-        unsigned polls = 0;
-        while (*(volatile unsigned*)&ws->ready[it] == 0u) {
-          if (*(volatile unsigned*)&ws->error != 0u || ++polls > WAIT_POLLS) { atomicExch(&ws->error, 1u); stop = 1; break; }
-          __nanosleep(100);
+// ALL: every iteration in this launch (launched cooperatively: every CTA is resident); else iteration `it0` alone, whose last CTA
+// leaves the next table in ws->desc for the next launch.
+// The wait is bounded: a CTA that gives up raises ws->error, every CTA then leaves, and the last distortion entry stays -1 (a
+// distortion is never negative) so that the caller can tell.
+template <bool ALL>
+__global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs* __restrict__ ws, double* __restrict__ distortion, int it0, int iters,
+                                                           float* __restrict__ out_lut, int smem_tiles) {
+  extern __shared__ __align__(16) unsigned char iter_smem[];
+  IterSmem& S = *reinterpret_cast<IterSmem*>(iter_smem);
+  unsigned short* s_ts = reinterpret_cast<unsigned short*>(iter_smem + ((sizeof(IterSmem) + 15) & ~(size_t)15));
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const unsigned n_tiles = (ws->list_count + CTB - 1) / CTB;
+  const unsigned tile0 = (unsigned)((unsigned long long)blockIdx.x * n_tiles / gridDim.x);
+  const int T = (int)((unsigned)((unsigned long long)(blockIdx.x + 1) * n_tiles / gridDim.x) - tile0);
+  const unsigned short* ts = a.tile_start + (size_t)tile0 * TS_PITCH;
+  if (T <= smem_tiles) {                  // the cell starts of this CTA's tiles, kept over the iterations
+    const uint4* from = reinterpret_cast<const uint4*>(ts);
+    for (int i = tid; i < T * (TS_PITCH / 8); i += ITB) reinterpret_cast<uint4*>(s_ts)[i] = __ldg(from + i);
+    ts = s_ts;
+  }
+  {
+    constexpr int DW = (int)(sizeof(IterDesc) / sizeof(unsigned));
+    if (tid < DW) reinterpret_cast<unsigned*>(&S.d)[tid] = reinterpret_cast<const unsigned*>(&ws->desc)[tid];
+  }
+  if (tid < 2 * LIMBS * SOP_MAX_ENTRIES) (&S.limb[0][0][0])[tid] = 0u;
+  if (tid < 2 * SOP_MAX_ENTRIES) (&S.sum[0][0])[tid] = 0ull;
+  if (blockIdx.x == 0) {
+    // prefix sums over the cells, one cell per thread: inside the warps, then the warps' totals
+    __shared__ unsigned long long t_n[32];
+    __shared__ long long t_s[32];
+    __shared__ double t_a[3][32];
+    static_assert(SORT_ROWS <= ITB, "one cell per thread");
+    const bool in = tid < SORT_ROWS;
+    unsigned long long n = in ? ws->cellN[tid] : 0ull;
+    long long s = in ? ws->cellS[tid] : 0ll;
+    const double a0 = in ? ws->cellA[0][tid] : 0.0, a1 = in ? ws->cellA[1][tid] : 0.0, a2 = in ? ws->cellA[2][tid] : 0.0;
+    const double r = (double)(tid - SORT_CHALF);
+    double b[3] = {a0, a1 + r * a0, a2 + r * (2.0 * a1 + r * a0)};              // about the origin, in units of a cell
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long un = __shfl_up_sync(0xFFFFFFFFu, n, o);
+      const long long us = __shfl_up_sync(0xFFFFFFFFu, s, o);
+      double ub[3];
+#pragma unroll
+      for (int x = 0; x < 3; ++x) ub[x] = __shfl_up_sync(0xFFFFFFFFu, b[x], o);
+      if (lane >= o) { n += un; s += us; b[0] += ub[0]; b[1] += ub[1]; b[2] += ub[2]; }
+    }
+    if (lane == 31) { t_n[warp] = n; t_s[warp] = s; t_a[0][warp] = b[0]; t_a[1][warp] = b[1]; t_a[2][warp] = b[2]; }
+    __syncthreads();
+    for (int w = 0; w < warp && w < 32; ++w) { n += t_n[w]; s += t_s[w]; b[0] += t_a[0][w]; b[1] += t_a[1][w]; b[2] += t_a[2][w]; }
+    if (in) { S.preN[tid + 1] = n; S.preS[tid + 1] = s; S.preA[0][tid + 1] = b[0]; S.preA[1][tid + 1] = b[1]; S.preA[2][tid + 1] = b[2]; }
+    if (tid == 0) { S.preN[0] = 0; S.preS[0] = 0; S.preA[0][0] = S.preA[1][0] = S.preA[2][0] = 0.0; }
+  }
+  __syncthreads();
+  for (int it = it0;; ++it) {
+    const bool last = it == iters;
+    if (warp == 0) split_cells(S);
+    __syncthreads();
+    iteration_share<ALL>(a, ws, S, ts, tile0, T, it, last);
+    if (warp == 0) {
+      bool go = true;
+      if (ALL) {
+        // CTA 0 waits for the closing iteration too: it reports the result
+        if (lane == 0 && (!last || blockIdx.x == 0)) {
+          unsigned polls = 0, seen;
+          for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&ws->arrive[it]) : "memory");
+            if (seen >= gridDim.x) break;
+            if (++polls > WAIT_POLLS || ((polls & 63u) == 0u && *(volatile unsigned*)&ws->error != 0u)) { atomicExch(&ws->error, 1u); go = false; break; }
+          }
         }
+        go = __shfl_sync(0xFFFFFFFFu, go ? 1 : 0, 0) != 0;
+      } else {
+        go = S.is_last != 0;
         __threadfence();
       }
-      s_stop = stop;
+      if (go && (!ALL || blockIdx.x == 0)) {
+        if (lane == 0) distortion[it] = __ldcg(&ws->accD[it]);
+        if (last) out_lut[lane] = lane < S.d.n_entries ? S.d.lut[lane] : 0.0f;
+      }
+      if (go && !last) {
+        const unsigned long long n = __ldcg(&ws->accN[it][lane]);
+        const long long s = __ldcg(&ws->accS[it][lane]);
+        new_table(S, n, s);
+        make_desc(ALL ? &S.d : &ws->desc, S.table, S.d.n_entries);
+      }
+      if (lane == 0) S.stop = !ALL || last || !go ? 1 : 0;
     }
     __syncthreads();
-    if (s_stop) break;
+    if (S.stop) return;
   }
-  // Whoever leaves with the error flag up marks the result as invalid, whichever CTA gave up and whenever: a CTA
-  // that arrived late can still run the remaining iterations alone (nobody else arrives, so it never closes
-  // the last one), and it must not leave a valid-looking trace behind.
-  if (threadIdx.x == 0 && *(volatile unsigned*)&ws->error != 0u) distortion[iters] = -1.0;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -960,35 +1041,33 @@ __global__ void grid_dp_last_kernel(const DpScratch* __restrict__ dp, int n_entr
 
 int num_sms();
 
-// Grid of the iteration kernels and whether all iterations run in one cooperative launch: they do wherever the device
-// launches cooperatively (the CTAs wait for one another between iterations, so the whole grid has to be resident:
-// the grid is cut to what is, and a CTA walks as many tiles as that takes); otherwise there is one launch per iteration.
-static bool lloyd_iteration_plan(long long NB, long long pool_blocks, int iters, int flags, long long* grid_out) {
+// Grid of the iteration kernels and whether all iterations run in one cooperative launch: they do wherever the device launches
+// cooperatively (the CTAs wait for one another between iterations, so the whole grid has to be resident: at most one per SM);
+// otherwise there is one launch per iteration.  Four tiles per CTA at least: their split cells' runs keep its 128 groups of eight
+// lanes busy for half a step to a step, and a CTA less is an arrival less.
+static size_t iter_smem_bytes(int tiles) { return ((sizeof(IterSmem) + 15) & ~(size_t)15) + (size_t)tiles * TS_PITCH * sizeof(unsigned short); }
+constexpr size_t ITER_SMEM_MAX = 225 * 1024;
+
+static bool lloyd_iteration_plan(long long pool_blocks, int iters, int flags, long long* grid_out) {
   const int sms = num_sms();
-  const long long likely = (pool_blocks + LTB - 1) / LTB;           // cache tiles of the pool without ties at its threshold
-  long long grid = (likely + LTB / 32 - 1) / (LTB / 32);            // one warp per cache tile
-  if (grid > (long long)sms * 8) grid = (long long)sms * 8;
+  const long long likely = (pool_blocks + CTB - 1) / CTB;           // cache tiles of the pool without ties at its threshold
+  long long grid = (likely + 3) / 4;
+  if (grid > sms) grid = sms;
   if (g_tune.iter_ctas > 0 && grid > g_tune.iter_ctas) grid = g_tune.iter_ctas;
   if (grid < 1) grid = 1;
-  (void)NB;
   DeviceFacts* facts = device_facts();
   if (facts->coop_blocks_per_sm < 0) {
     int dev = 0, coop = 0, nb = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, lloyd_persistent_kernel, LTB, 0) == cudaSuccess)
+        cudaFuncSetAttribute(lloyd_iter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ITER_SMEM_MAX) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, lloyd_iter_kernel<true>, ITB, ITER_SMEM_MAX) == cudaSuccess)
       facts->coop_blocks_per_sm = nb;
     else
       facts->coop_blocks_per_sm = 0;
     cudaGetLastError();
   }
-  const long long resident = (long long)facts->coop_blocks_per_sm * sms;
-  bool persistent = false;
-  if (iters >= 1 && resident >= 1 && !(flags & SOP_LLOYD_LAUNCH_PER_ITERATION)) {
-    persistent = true;
-    if (grid > resident) grid = resident;
-  }
   *grid_out = grid;
-  return persistent;
+  return iters >= 1 && facts->coop_blocks_per_sm >= 1 && !(flags & SOP_LLOYD_LAUNCH_PER_ITERATION);
 }
 
 }  // namespace sop
@@ -1000,7 +1079,7 @@ int sop_dd4_lloyd_launches(long long M, long long K, int iters, int flags, int* 
   const int dp_entries = iters > 1 ? iters : 2;      // with SOP_LLOYD_GRID_DP the caller passes the number of table entries here
   if (M < 1 || K < 1 || (K % SOP_G) != 0 || iters < 0 || iters > sop::SOP_MAX_LLOYD_ITERS) return SOP_ERR_RANGE;
   long long grid = 1;
-  const bool persistent = sop::lloyd_iteration_plan(M * (K / SOP_G), M * (K / SOP_G), iters, flags, &grid);
+  const bool persistent = sop::lloyd_iteration_plan(M * (K / SOP_G), iters, flags, &grid);
   // radix select (three passes, unless the pool is cut by a threshold), set-up, pool list, pool cache, iterations
   // the dynamic programme: first row, one launch per further row (callers with a 16-entry table: 15), the backtrack
   *launches = ((flags & SOP_LLOYD_POOL_THRESHOLD) ? 0 : 3) + 3 + ((flags & SOP_LLOYD_GRID_DP) ? 2 + (dp_entries - 1) : (persistent ? 1 : iters + 1));
@@ -1013,7 +1092,6 @@ int sop_dd4_lloyd_tuning(int cell_spill_tiles, int cache_ctas, int tiles_per_war
       tiles_per_warp > TILES_PER_WARP_MAX || iter_ctas < 0) return SOP_ERR_RANGE;
   g_tune.spill_tiles = cell_spill_tiles;
   g_tune.cache_ctas = cache_ctas;
-  g_tune.tiles_per_warp = tiles_per_warp;
   g_tune.iter_ctas = iter_ctas;
   return SOP_OK;
 }
@@ -1100,18 +1178,19 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
 
   // (u, omega) of every pool element, once: sorted tiles, cell starts, per-cell sums and moments
   {
-    long long cg = (NB + LTB - 1) / LTB;      // one tile per CTA pass
-    const long long cg_max = g_tune.cache_ctas > 0 ? g_tune.cache_ctas : (long long)sms * 3;
+    long long cg = (NB + CTB - 1) / CTB;      // one tile per CTA pass
+    const long long cg_max = g_tune.cache_ctas > 0 ? g_tune.cache_ctas : (long long)sms * 2;
     if (cg > cg_max) cg = cg_max;
-    const size_t stage_bytes = (size_t)TILE_ELEMS * sizeof(uint2);
+    const size_t stage_bytes = sizeof(CacheSmem);
     DeviceFacts* facts = device_facts();
     if (!facts->lloyd_attr_set) {
       SOP_CUDA_TRY(cudaFuncSetAttribute(pool_cache_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage_bytes));
       SOP_CUDA_TRY(cudaFuncSetAttribute(pool_cache_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage_bytes));
+      SOP_CUDA_TRY(cudaFuncSetAttribute(lloyd_iter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ITER_SMEM_MAX));
       facts->lloyd_attr_set = true;
     }
-    if (grid_dp) pool_cache_kernel<true><<<(int)cg, LTB, stage_bytes, st>>>(a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles);
-    else pool_cache_kernel<false><<<(int)cg, LTB, stage_bytes, st>>>(a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles);
+    if (grid_dp) pool_cache_kernel<true><<<(int)cg, CTB, stage_bytes, st>>>(a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles);
+    else pool_cache_kernel<false><<<(int)cg, CTB, stage_bytes, st>>>(a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles);
     SOP_CUDA_TRY(cudaGetLastError());
   }
   if ((rc = profile_mark(SOP_PROFILE_POOL, 1, st))) return rc;
@@ -1128,17 +1207,20 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
     return SOP_OK;
   }
   long long grid = 1;
-  const bool persistent = lloyd_iteration_plan(NB, by_threshold ? NB : pool_rank, iters, flags, &grid);
-  unsigned fold_period = (unsigned)g_tune.tiles_per_warp;
+  const long long expected = by_threshold ? NB : pool_rank;
+  const bool persistent = lloyd_iteration_plan(expected, iters, flags, &grid);
+  // room for the cell starts of the tiles that a CTA is likely to have (and a few more, for ties); more tiles are read from memory
+  int smem_tiles = (int)(((expected + CTB - 1) / CTB + grid - 1) / grid + 4);
+  while (smem_tiles > 0 && iter_smem_bytes(smem_tiles) > ITER_SMEM_MAX) --smem_tiles;
+  const size_t iter_smem = iter_smem_bytes(smem_tiles);
   if ((rc = profile_mark(SOP_PROFILE_LLOYD, 0, st))) return rc;
   if (persistent) {
-    void* kargs[] = {(void*)&a, (void*)&ws, (void*)&distortion_dev, (void*)&iters, (void*)&out_lut_dev, (void*)&fold_period};
-    SOP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)lloyd_persistent_kernel, dim3((unsigned)grid), dim3(LTB), kargs, 0, st));
+    int it0 = 0;
+    void* kargs[] = {(void*)&a, (void*)&ws, (void*)&distortion_dev, (void*)&it0, (void*)&iters, (void*)&out_lut_dev, (void*)&smem_tiles};
+    SOP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)lloyd_iter_kernel<true>, dim3((unsigned)grid), dim3(ITB), kargs, iter_smem, st));
   } else {
-    for (int it = 0; it <= iters; ++it) {
-      const int last = it == iters;
-      lloyd_split_kernel<<<(int)grid, LTB, 0, st>>>(a, ws, distortion_dev, it, last, out_lut_dev, fold_period);
-    }
+    for (int it = 0; it <= iters; ++it)
+      lloyd_iter_kernel<false><<<(int)grid, ITB, iter_smem, st>>>(a, ws, distortion_dev, it, iters, out_lut_dev, smem_tiles);
   }
   if ((rc = profile_mark(SOP_PROFILE_LLOYD, 1, st))) return rc;
   SOP_CUDA_TRY(cudaGetLastError());
