@@ -146,6 +146,8 @@ int validate_layer(const void* W, long long M, long long K, long long ldw, const
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) norms_partial_kernel(const float* __restrict__ X, long long T, long long K,
                                                             long long ldx, double* __restrict__ part) {
+  pdl_trigger();
+  pdl_wait();
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long chunk = blockIdx.y;
   if (k >= K) return;
@@ -171,6 +173,8 @@ __global__ void __launch_bounds__(256) norms_partial_kernel(const float* __restr
 
 __global__ void __launch_bounds__(256) norms_final_kernel(const double* __restrict__ part, long long n_chunks, long long K,
                                                           long long T, float* __restrict__ c) {
+  pdl_trigger();
+  pdl_wait();
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= K) return;
   double total = 0.0;
@@ -239,10 +243,8 @@ int sop_channel_norms(const float* X_dev, long long T, long long K, long long ld
   dim3 grid((unsigned)((K + 255) / 256), (unsigned)n_chunks);
   int rc;
   if ((rc = sop::profile_mark(SOP_PROFILE_NORMS, 0, st))) return rc;
-  sop::norms_partial_kernel<<<grid, 256, 0, st>>>(X_dev, T, K, ldx, (double*)workspace_dev);
-  SOP_CUDA_TRY(cudaGetLastError());
-  sop::norms_final_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>((const double*)workspace_dev, n_chunks, K, T, c_dev);
-  SOP_CUDA_TRY(cudaGetLastError());
+  SOP_CUDA_TRY(sop::launch(sop::norms_partial_kernel, grid, 256, 0, st, X_dev, T, K, ldx, (double*)workspace_dev));
+  SOP_CUDA_TRY(sop::launch(sop::norms_final_kernel, dim3((unsigned)((K + 255) / 256)), 256, 0, st, (const double*)workspace_dev, n_chunks, K, T, c_dev));
   if ((rc = sop::profile_mark(SOP_PROFILE_NORMS, 1, st))) return rc;
   return SOP_OK;
 }
@@ -290,10 +292,8 @@ int sop_channel_norms_static(const float* X_dev, long long T, long long K, long 
   // every partial that the second kernel reads is written by the first one in this call: nothing has
   // to be cleared, whatever an earlier call left in the array
   dim3 grid((unsigned)((K + 255) / 256), (unsigned)n_chunks);
-  sop::norms_partial_kernel<<<grid, 256, 0, st>>>(X_dev, T, K, ldx, scratch);
-  SOP_CUDA_TRY(cudaGetLastError());
-  sop::norms_final_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(scratch, n_chunks, K, T, c_dev);
-  SOP_CUDA_TRY(cudaGetLastError());
+  SOP_CUDA_TRY(sop::launch(sop::norms_partial_kernel, grid, 256, 0, st, X_dev, T, K, ldx, scratch));
+  SOP_CUDA_TRY(sop::launch(sop::norms_final_kernel, dim3((unsigned)((K + 255) / 256)), 256, 0, st, (const double*)scratch, n_chunks, K, T, c_dev));
   return SOP_OK;
 }
 

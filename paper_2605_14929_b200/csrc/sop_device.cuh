@@ -43,6 +43,29 @@ int num_sms();
 // the first launch, edge 1 after the last.  No-op unless profiling is enabled.
 int profile_mark(int which, int edge, cudaStream_t st);
 
+// ---- launches ------------------------------------------------------------------------------
+// Every kernel of the library is launched so that it may start while the one before it on the stream still runs (programmatic
+// dependent launch): a pass is a chain of twenty short kernels, and the time from the end of one to the start of the next was a
+// sixth of a small layer's pass.  Rules that each kernel keeps: pdl_trigger() first (its successor may then be scheduled as its CTAs
+// leave), and pdl_wait() -- which returns when the kernels before it have completed and their writes are visible -- before the
+// first access to global memory; only what depends on the parameters alone comes before the wait.
+template <typename... P, typename... A>
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- kernel parameter blocks ---------------------------------------------------------------
 struct FmtDev {
   int y;                // mantissa bits

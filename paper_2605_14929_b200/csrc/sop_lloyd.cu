@@ -183,6 +183,8 @@ __device__ void derive_prefix(const LloydWs* ws, long long pool_rank, int passes
 
 template <int PASS>
 __global__ void __launch_bounds__(LTB) select_kernel(LloydArgs a, const sop_search_result* __restrict__ res, LloydWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned sh[2048];
   for (int i = threadIdx.x; i < 2048; i += LTB) sh[i] = 0;
   unsigned prefix = 0, cnt;
@@ -234,6 +236,8 @@ __device__ void make_desc(IterDesc* d, const float* table, int ne);
 
 __global__ void __launch_bounds__(SETUP_TB) lloyd_setup_kernel(LloydArgs a, AtomsDev A, const sop_search_result* __restrict__ res,
                                                                LloydWs* __restrict__ ws, double* __restrict__ distortion, int iters) {
+  pdl_trigger();
+  pdl_wait();
   unsigned prefix = 0, cnt = 0;
   long long rank = 0, below = 0;
   if (a.flags & SOP_LLOYD_POOL_THRESHOLD) prefix = pool_key(a.pool_threshold, a.flags);   // the caller fixes the threshold
@@ -287,6 +291,8 @@ __global__ void __launch_bounds__(SETUP_TB) lloyd_setup_kernel(LloydArgs a, Atom
 // CTAs; nothing downstream depends on it (integer sums, and an FP64 sum compared with a tolerance).
 constexpr int LIST_PER_THREAD = 16;
 __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned s_cnt[LTB / 32];
   __shared__ unsigned s_base;
   const unsigned tau_key = ws->tau_key;
@@ -402,6 +408,8 @@ __device__ void spill_cells(CacheSmem& S, LloydWs* ws) {
 template <bool DP>
 __global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev F, LloydWs* __restrict__ ws, long long* __restrict__ pool_count_out,
                                                          unsigned spill_tiles) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char cache_smem[];
   CacheSmem& S = *reinterpret_cast<CacheSmem*>(cache_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -846,6 +854,8 @@ __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __r
 template <bool ALL>
 __global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs* __restrict__ ws, double* __restrict__ distortion, int it0, int iters,
                                                            float* __restrict__ out_lut, int smem_tiles) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char iter_smem[];
   IterSmem& S = *reinterpret_cast<IterSmem*>(iter_smem);
   unsigned short* s_ts = reinterpret_cast<unsigned short*>(iter_smem + ((sizeof(IterSmem) + 15) & ~(size_t)15));
@@ -968,6 +978,8 @@ struct DpScratch {
 
 // One CTA: the non-empty cells, their prefix sums, and row 0 (cells 0..j as one run).
 __global__ void __launch_bounds__(DP_TB) grid_dp_first_kernel(const LloydWs* __restrict__ ws, DpScratch* __restrict__ dp) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int s_B;
   if (threadIdx.x == 0) {
     int B = 0;
@@ -986,6 +998,8 @@ __global__ void __launch_bounds__(DP_TB) grid_dp_first_kernel(const LloydWs* __r
 // Row r of the programme: one warp per last cell j, the lanes share the starts i of the last run; the least value wins,
 // a tie goes to the smallest i (what a sequential scan from the first start on keeps).
 __global__ void __launch_bounds__(DP_TB) grid_dp_row_kernel(DpScratch* __restrict__ dp, int r, short* __restrict__ cut) {
+  pdl_trigger();
+  pdl_wait();
   const int B = dp->B;
   const int lane = threadIdx.x & 31;
   const int j = blockIdx.x * (DP_TB / 32) + (threadIdx.x >> 5);
@@ -1012,6 +1026,8 @@ __global__ void __launch_bounds__(DP_TB) grid_dp_row_kernel(DpScratch* __restric
 // (n_entries - 1 at most); with fewer cells than entries the programme stops at the last row that has a cell.
 __global__ void grid_dp_last_kernel(const DpScratch* __restrict__ dp, int n_entries, const short* __restrict__ cut, float* __restrict__ out_lut,
                                     double* __restrict__ cost_out) {
+  pdl_trigger();
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int B = dp->B;
   if (B == 0) {
@@ -1166,14 +1182,14 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
   if (sg > sms * 4) sg = sms * 4;
   if (sg < 1) sg = 1;
   if (!by_threshold) {     // radix select of the pool_rank-th worst block (three passes over the ranking keys)
-    select_kernel<0><<<(int)sg, LTB, 0, st>>>(a, search_dev, ws);
-    select_kernel<1><<<(int)sg, LTB, 0, st>>>(a, search_dev, ws);
-    select_kernel<2><<<(int)sg, LTB, 0, st>>>(a, search_dev, ws);
+    SOP_CUDA_TRY(launch(select_kernel<0>, sg, LTB, 0, st, a, search_dev, ws));
+    SOP_CUDA_TRY(launch(select_kernel<1>, sg, LTB, 0, st, a, search_dev, ws));
+    SOP_CUDA_TRY(launch(select_kernel<2>, sg, LTB, 0, st, a, search_dev, ws));
     SOP_CUDA_TRY(cudaGetLastError());
   }
-  lloyd_setup_kernel<<<1, SETUP_TB, 0, st>>>(a, A, search_dev, ws, distortion_dev, iters);
+  SOP_CUDA_TRY(launch(lloyd_setup_kernel, 1, SETUP_TB, 0, st, a, A, search_dev, ws, distortion_dev, iters));
   SOP_CUDA_TRY(cudaGetLastError());
-  pool_list_kernel<<<(int)sg, LTB, 0, st>>>(a, ws);
+  SOP_CUDA_TRY(launch(pool_list_kernel, sg, LTB, 0, st, a, ws));
   SOP_CUDA_TRY(cudaGetLastError());
 
   // (u, omega) of every pool element, once: sorted tiles, cell starts, per-cell sums and moments
@@ -1189,8 +1205,8 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
       SOP_CUDA_TRY(cudaFuncSetAttribute(lloyd_iter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ITER_SMEM_MAX));
       facts->lloyd_attr_set = true;
     }
-    if (grid_dp) pool_cache_kernel<true><<<(int)cg, CTB, stage_bytes, st>>>(a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles);
-    else pool_cache_kernel<false><<<(int)cg, CTB, stage_bytes, st>>>(a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles);
+    if (grid_dp) SOP_CUDA_TRY(launch(pool_cache_kernel<true>, cg, CTB, stage_bytes, st, a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles));
+    else SOP_CUDA_TRY(launch(pool_cache_kernel<false>, cg, CTB, stage_bytes, st, a, F, ws, pool_count_dev, (unsigned)g_tune.spill_tiles));
     SOP_CUDA_TRY(cudaGetLastError());
   }
   if ((rc = profile_mark(SOP_PROFILE_POOL, 1, st))) return rc;
@@ -1198,10 +1214,10 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
     if ((rc = profile_mark(SOP_PROFILE_LLOYD, 0, st))) return rc;
     static_assert(sizeof(DpScratch) <= sizeof(((LloydWs*)nullptr)->dp_scratch), "scratch of the dynamic programme");
     DpScratch* dp = reinterpret_cast<DpScratch*>(ws->dp_scratch);
-    grid_dp_first_kernel<<<1, DP_TB, 0, st>>>(ws, dp);
+    SOP_CUDA_TRY(launch(grid_dp_first_kernel, 1, DP_TB, 0, st, ws, dp));
     for (int r = 1; r < ne; ++r)      // a row without a cell (fewer cells than entries) returns at once
-      grid_dp_row_kernel<<<(SORT_ROWS + DP_TB / 32 - 1) / (DP_TB / 32), DP_TB, 0, st>>>(dp, r, &ws->dp_cut[0][0]);
-    grid_dp_last_kernel<<<1, 32, 0, st>>>(dp, ne, &ws->dp_cut[0][0], out_lut_dev, distortion_dev);
+      SOP_CUDA_TRY(launch(grid_dp_row_kernel, (SORT_ROWS + DP_TB / 32 - 1) / (DP_TB / 32), DP_TB, 0, st, dp, r, &ws->dp_cut[0][0]));
+    SOP_CUDA_TRY(launch(grid_dp_last_kernel, 1, 32, 0, st, dp, ne, &ws->dp_cut[0][0], out_lut_dev, distortion_dev));
     SOP_CUDA_TRY(cudaGetLastError());
     if ((rc = profile_mark(SOP_PROFILE_LLOYD, 1, st))) return rc;
     return SOP_OK;
@@ -1220,7 +1236,7 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
     SOP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)lloyd_iter_kernel<true>, dim3((unsigned)grid), dim3(ITB), kargs, iter_smem, st));
   } else {
     for (int it = 0; it <= iters; ++it)
-      lloyd_iter_kernel<false><<<(int)grid, ITB, iter_smem, st>>>(a, ws, distortion_dev, it, iters, out_lut_dev, smem_tiles);
+      SOP_CUDA_TRY(launch(lloyd_iter_kernel<false>, grid, ITB, iter_smem, st, a, ws, distortion_dev, it, iters, out_lut_dev, smem_tiles));
   }
   if ((rc = profile_mark(SOP_PROFILE_LLOYD, 1, st))) return rc;
   SOP_CUDA_TRY(cudaGetLastError());

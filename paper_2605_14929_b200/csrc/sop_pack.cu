@@ -110,6 +110,8 @@ __device__ __forceinline__ void eval_block_regs(const float (&w)[16], const floa
 // (no channel norms needed); otherwise every candidate of the choice is evaluated here.
 template <bool USE_COS>
 __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ float lutv[2][32], tau[2][32];
   __shared__ uint2 cells[2][CELL_ROWS_MAX];       // per table and cell: {the cell's threshold (+inf: none), thresholds below the cell}
   __shared__ PackCand base[2];
@@ -477,8 +479,8 @@ int sop_pack(const void* W_dev, long long M, long long K, long long ldw, const f
   if (grid > (long long)sms * 4) grid = (long long)sms * 4;      // one wave of resident CTAs: the table set-up runs once per CTA
   if ((rc = profile_mark(SOP_PROFILE_PACK, 0, st))) return rc;
   const bool negs_known = !use_sign || from_result || (a.cos_neg_a >= 0 && (!pair || a.cos_neg_b >= 0));
-  if (block_cos_dev && negs_known) pack_kernel<true><<<(int)grid, PTB, 0, st>>>(a, A, F, search_dev);
-  else pack_kernel<false><<<(int)grid, PTB, 0, st>>>(a, A, F, search_dev);
+  if (block_cos_dev && negs_known) SOP_CUDA_TRY(launch(pack_kernel<true>, grid, PTB, 0, st, a, A, F, search_dev));
+  else SOP_CUDA_TRY(launch(pack_kernel<false>, grid, PTB, 0, st, a, A, F, search_dev));
   if ((rc = profile_mark(SOP_PROFILE_PACK, 1, st))) return rc;
   SOP_CUDA_TRY(cudaGetLastError());
   return SOP_OK;

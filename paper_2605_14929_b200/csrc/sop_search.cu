@@ -141,6 +141,8 @@ __device__ __forceinline__ float absmax_bits(const uint32_t (&v)[8]) {
 __device__ void kselect_body(const Plan& P, const FmtDev& F, const unsigned* hist, WsHeader* hdr);
 
 __global__ void __launch_bounds__(256) prepass_kernel(LayerArgs L, Plan P, FmtDev F, unsigned* __restrict__ hist, WsHeader* __restrict__ hdr) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned sh[SOP_MAX_CLASSES * SOP_HIST_BINS];
   for (int i = threadIdx.x; i < P.n_classes * SOP_HIST_BINS; i += blockDim.x) sh[i] = 0;
   __syncthreads();
@@ -180,6 +182,8 @@ __global__ void __launch_bounds__(256) prepass_kernel(LayerArgs L, Plan P, FmtDe
 
 // The shifts of another scale format from the histograms that an earlier prepass of the same layer left in the workspace.
 __global__ void __launch_bounds__(256) kselect_kernel(Plan P, FmtDev F, const unsigned* __restrict__ hist, WsHeader* __restrict__ hdr) {
+  pdl_trigger();
+  pdl_wait();
   if (threadIdx.x == 0) hdr->wmax_bits = hist[SOP_MAX_CLASSES * SOP_HIST_BINS];
   __threadfence();
   __syncthreads();
@@ -745,15 +749,22 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
 // Evaluates the candidates of eval_mask on every block and writes their columns of block_cos / block_sse: group by group, then
 // format by format (W is read again for each: it is a tenth of the time of one).
 template <int MAX_NP>
-__global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArgs L, Plan P, AtomsDev A, FmtDev F, const WsHeader* __restrict__ hdr,
+__global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArgs L, Plan P, AtomsDev A, FmtDev F, WsHeader* __restrict__ hdr,
                                                       float* __restrict__ block_cos, float* __restrict__ block_sse,
                                                       const sop_search_result* __restrict__ prev, unsigned c_off, unsigned tba) {
+  pdl_trigger();
   extern __shared__ __align__(128) unsigned char smem[];
   GroupScratch& S = *reinterpret_cast<GroupScratch*>(smem);
   __shared__ int cls_k[SOP_MAX_CLASSES];
   __shared__ float cls_pot[SOP_MAX_CLASSES];
 
   const int tid = threadIdx.x;
+  // the tables of fixed candidates come from the parameters: they are built while the kernel before this one ends
+  const bool early = (A.dd_mask & P.eval_mask) == 0u;
+  if (early)
+    for (int g = 0; g < P.n_groups; ++g) build_group(P, A, g, smem, S);
+  pdl_wait();
+  if (blockIdx.x == 0 && tid == 0) { hdr->done_reduce = 0u; hdr->reduce_error = 0u; }      // for the reduction that follows
   // thread -> fixed column block j, rows m = r0, r0 + R, ...; its sixteen channel norms stay in shared memory.  Control flow is
   // uniform: a thread with fewer rows evaluates its last block once more and stores nothing.
   const unsigned nbk = (unsigned)L.nbk, M = (unsigned)L.M;       // the block count fits 31 bits
@@ -798,7 +809,8 @@ __global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArg
     }
   }
 
-  for (int g = 0; g < P.n_groups; ++g) build_group(P, A, g, smem, S);
+  if (!early)
+    for (int g = 0; g < P.n_groups; ++g) build_group(P, A, g, smem, S);
   __syncthreads();
   if ((unsigned)tid >= tba) return;                              // (whole warps: they only helped with the tables)
 
@@ -1088,6 +1100,7 @@ __global__ void __launch_bounds__(RTB, 1) reduce_kernel(LayerArgs L, RedPlan P, 
                                                         WsHeader* __restrict__ hdr, PartialSums partials, const float* __restrict__ block_cos,
                                                         const float* __restrict__ block_sse, sop_pair_stat* pair_table, sop_pair_stat* signed_table,
                                                         sop_search_result* __restrict__ res, const sop_search_result* __restrict__ prev) {
+  pdl_trigger();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ BundleSums s_part[RED_WARPS];
   __shared__ unsigned long long s_row[2 * SOP_MAX_ATOMS];      // address of every fetched row: a column's cosines, its errors
@@ -1116,6 +1129,7 @@ __global__ void __launch_bounds__(RTB, 1) reduce_kernel(LayerArgs L, RedPlan P, 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  pdl_wait();
   __syncthreads();
   BundleSums* mine = s_part + (warp < RED_WARPS ? warp : 0);
   if (warp == RED_WARPS) {
@@ -1652,17 +1666,18 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   // a lane counts its blocks in 12 bits: at most 4095 of them even where a bundle has one warp only
   while (((n_tiles + rgrid - 1) / rgrid) * units * (RUNIT / 32) > 4095) ++rgrid;
 
-  // the header always starts from zero; the histograms (and max|W| behind them) only when this call fills them
-  SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, (k_from_result || reuse_prepass) ? ws_hist_off() : ws_part_off(), st));
+  // the prepass adds to its histograms; the reduction's counters are cleared by the sweep where there is one
+  if (!k_from_result && !reuse_prepass) SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, ws_part_off(), st));
+  else if (!eval_mask) SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, ws_hist_off(), st));
   if ((rc = profile_mark(SOP_PROFILE_PREPASS, 0, st))) return rc;
   if (reuse_prepass) {
-    kselect_kernel<<<1, 256, 0, st>>>(P, F, hist, hdr);
+    SOP_CUDA_TRY(launch(kselect_kernel, 1, 256, 0, st, P, F, hist, hdr));
     SOP_CUDA_TRY(cudaGetLastError());
   } else if (!k_from_result) {
     // one read of W: block scales' exponent histogram, max|W|, then the shifts (last CTA)
     long long want = (L.NB + 255) / 256;
     const int pgrid = (int)(want < (long long)sms * 8 ? want : (long long)sms * 8);
-    prepass_kernel<<<pgrid, 256, 0, st>>>(L, P, F, hist, hdr);
+    SOP_CUDA_TRY(launch(prepass_kernel, pgrid, 256, 0, st, L, P, F, hist, hdr));
     SOP_CUDA_TRY(cudaGetLastError());
   }
   if ((rc = profile_mark(SOP_PROFILE_PREPASS, 1, st))) return rc;
@@ -1682,7 +1697,7 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   if ((rc = profile_mark(SOP_PROFILE_SWEEP, 0, st))) return rc;
   if (eval_mask) {
     const unsigned c_off = (unsigned)(smem - SWEEP_C_BYTES);
-#define SOP_LAUNCH_SWEEP(NP) sweep_kernel<NP><<<(int)grid, TB, smem, st>>>(L, P, A, F, hdr, cos_cols, sse_cols, prev_result_dev, c_off, (unsigned)tba)
+#define SOP_LAUNCH_SWEEP(NP) SOP_CUDA_TRY(launch(sweep_kernel<NP>, grid, TB, smem, st, L, P, A, F, hdr, cos_cols, sse_cols, prev_result_dev, c_off, (unsigned)tba))
     if (max_np == 0) SOP_LAUNCH_SWEEP(0);
     else if (max_np == 1) SOP_LAUNCH_SWEEP(1);
     else if (max_np == 2) SOP_LAUNCH_SWEEP(2);
@@ -1703,8 +1718,8 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
     const size_t rs = reduce_smem_bytes(Q.n_cols, units, n_stage);
     const int fin = l == n_launch - 1 ? 1 : 0;
 #define SOP_LAUNCH_REDUCE(SE, VC)                                                                                                   \
-  reduce_kernel<SE, VC><<<(int)rgrid, RTB, rs, st>>>(L, Rp, Q, units, n_stage, fin, hdr, partials, cos_cols, sse_cols, pair_table_dev, \
-                                                     signed_table_dev, result_dev, prev_result_dev)
+  SOP_CUDA_TRY(launch(reduce_kernel<SE, VC>, rgrid, RTB, rs, st, L, Rp, Q, units, n_stage, fin, hdr, partials, cos_cols, sse_cols, pair_table_dev, \
+                                                     signed_table_dev, result_dev, prev_result_dev))
     if (sel_err) { if (vec) SOP_LAUNCH_REDUCE(true, true); else SOP_LAUNCH_REDUCE(true, false); }
     else { if (vec) SOP_LAUNCH_REDUCE(false, true); else SOP_LAUNCH_REDUCE(false, false); }
 #undef SOP_LAUNCH_REDUCE

@@ -88,6 +88,8 @@ __device__ __forceinline__ unsigned cta_excl_scan(unsigned v, unsigned* s_warp, 
 __global__ void __launch_bounds__(1024) tile_scan_kernel(unsigned* __restrict__ tile_sums, long long n_tiles, unsigned* __restrict__ row_start,
                                                          long long M, long long* __restrict__ count, SparseWs* __restrict__ ws, int wr,
                                                          int* __restrict__ scale_exp_out, float* __restrict__ tau_out) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned s_warp[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long per = ((n_tiles + 31) / 32 + 31) / 32 * 32;            // tiles per warp, a multiple of 32
@@ -142,6 +144,8 @@ struct OpqArgs {
 };
 
 __global__ void __launch_bounds__(STB) opq_mask_kernel(OpqArgs a) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned s_cnt;
   const int tid = threadIdx.x;
   const long long n_tiles = (a.NB + STB - 1) / STB;
@@ -185,6 +189,8 @@ __global__ void __launch_bounds__(STB) opq_mask_kernel(OpqArgs a) {
 }
 
 __global__ void __launch_bounds__(STB) opq_write_kernel(OpqArgs a) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned s_warp[STB / 32];
   const int tid = threadIdx.x;
   const long long n_tiles = (a.NB + STB - 1) / STB;
@@ -385,6 +391,8 @@ __device__ __forceinline__ unsigned wr_key(float met) {
 template <int PASS, bool LUT4>
 __global__ void __launch_bounds__(STB) wr_hist_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
                                                       SparseWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ WrShared sh;
   __shared__ unsigned hist[2048];
   const int tid = threadIdx.x;
@@ -435,6 +443,8 @@ __global__ void __launch_bounds__(STB) wr_hist_kernel(WrArgs a, AtomsDev A, FmtD
 // beyond the histogram's total (no pair to correct, so the histogram is empty) leaves a NaN threshold: nothing
 // compares >= to it.
 __global__ void __launch_bounds__(1024) wr_pick_kernel(SparseWs* __restrict__ ws, int pass, long long n_keep) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned long long s_warp[32];
   __shared__ int s_bin;
   __shared__ unsigned long long s_before;
@@ -502,6 +512,8 @@ struct WrValue {
 template <bool LUT4>
 __global__ void __launch_bounds__(STB) wr_collect_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
                                                          SparseWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ WrShared sh;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) wr_setup(a, A, res, sh);
@@ -553,12 +565,16 @@ __global__ void __launch_bounds__(STB) wr_collect_kernel(WrArgs a, AtomsDev A, F
 }
 
 __global__ void wr_mode_kernel(SparseWs* __restrict__ ws, unsigned cand_cap) {
+  pdl_trigger();
+  pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) ws->overflow = ws->n_cand > cand_cap ? 1u : 0u;
 }
 
 // The selection passes over the candidate list instead of the layer.
 template <int PASS>
 __global__ void __launch_bounds__(STB) wr_cand_hist_kernel(WrArgs a, SparseWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ unsigned hist[2048];
   if (ws->overflow) return;
   const int tid = threadIdx.x;
@@ -579,6 +595,8 @@ __global__ void __launch_bounds__(STB) wr_cand_hist_kernel(WrArgs a, SparseWs* _
 // The kept candidates: their bit in the per-block masks (two blocks per 32-bit word), their tile's record count (cleared
 // by the host call), the largest |E| among them.
 __global__ void __launch_bounds__(STB) wr_mark_kernel(WrArgs a, SparseWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   if (ws->overflow) return;
   const float tau = __uint_as_float(ws->tau_bits);
   const unsigned n = ws->n_cand;
@@ -599,6 +617,8 @@ __global__ void __launch_bounds__(STB) wr_mark_kernel(WrArgs a, SparseWs* __rest
 template <bool LUT4>
 __global__ void __launch_bounds__(STB) wr_count_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
                                                        SparseWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ WrShared sh;
   __shared__ unsigned s_cnt;
   const int tid = threadIdx.x;
@@ -637,6 +657,8 @@ __global__ void __launch_bounds__(STB) wr_count_kernel(WrArgs a, AtomsDev A, Fmt
 template <bool LUT4>
 __global__ void __launch_bounds__(STB) wr_write_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
                                                        const SparseWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ WrShared sh;
   __shared__ unsigned s_warp[STB / 32];
   const int tid = threadIdx.x;
@@ -680,6 +702,8 @@ __global__ void __launch_bounds__(STB) wr_write_kernel(WrArgs a, AtomsDev A, Fmt
 template <bool LUT4>
 __global__ void __launch_bounds__(STB) wr_map_write_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
                                                            const SparseWs* __restrict__ ws) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ WrShared sh;
   __shared__ unsigned s_warp[STB / 32];
   __shared__ unsigned s_n;
@@ -779,9 +803,9 @@ int sop_opq_extract(const void* W_dev, long long M, long long K, long long ldw, 
   const int grid = (int)(n_tiles < cap ? n_tiles : cap);
   int rc;
   if ((rc = profile_mark(SOP_PROFILE_OPQ, 0, st))) return rc;
-  opq_mask_kernel<<<grid, STB, 0, st>>>(a);
-  tile_scan_kernel<<<1, 1024, 0, st>>>(a.tile_sums, n_tiles, row_start_dev, M, count_dev, (SparseWs*)workspace_dev, 0, nullptr, nullptr);
-  opq_write_kernel<<<grid, STB, 0, st>>>(a);
+  SOP_CUDA_TRY(launch(opq_mask_kernel, grid, STB, 0, st, a));
+  SOP_CUDA_TRY(launch(tile_scan_kernel, 1, 1024, 0, st, a.tile_sums, n_tiles, row_start_dev, M, count_dev, (SparseWs*)workspace_dev, 0, nullptr, nullptr));
+  SOP_CUDA_TRY(launch(opq_write_kernel, grid, STB, 0, st, a));
   SOP_CUDA_TRY(cudaGetLastError());
   if ((rc = profile_mark(SOP_PROFILE_OPQ, 1, st))) return rc;
   return SOP_OK;
@@ -885,24 +909,24 @@ int sop_wr_extract(const void* W_dev, long long M, long long K, long long ldw, c
   }
 #define SOP_WR_LAUNCHES(L4)                                                          \
   do {                                                                               \
-    wr_hist_kernel<-1, L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);           \
-    wr_pick_kernel<<<1, 1024, 0, st>>>(ws, -1, n_keep);                              \
-    wr_collect_kernel<L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);            \
-    wr_mode_kernel<<<1, 32, 0, st>>>(ws, a.cand_cap);                                \
-    wr_cand_hist_kernel<0><<<lgrid, STB, 0, st>>>(a, ws);                            \
-    wr_hist_kernel<0, L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);            \
-    wr_pick_kernel<<<1, 1024, 0, st>>>(ws, 0, n_keep);                               \
-    wr_cand_hist_kernel<1><<<lgrid, STB, 0, st>>>(a, ws);                            \
-    wr_hist_kernel<1, L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);            \
-    wr_pick_kernel<<<1, 1024, 0, st>>>(ws, 1, n_keep);                               \
-    wr_cand_hist_kernel<2><<<lgrid, STB, 0, st>>>(a, ws);                            \
-    wr_hist_kernel<2, L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);            \
-    wr_pick_kernel<<<1, 1024, 0, st>>>(ws, 2, n_keep);                               \
-    wr_mark_kernel<<<lgrid, STB, 0, st>>>(a, ws);                                    \
-    wr_count_kernel<L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);              \
-    tile_scan_kernel<<<1, 1024, 0, st>>>(a.tile_sums, n_tiles, row_start_dev, M, count_dev, ws, 1, scale_exp_dev, tau_dev); \
-    wr_map_write_kernel<L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);          \
-    wr_write_kernel<L4><<<grid, STB, 0, st>>>(a, A, F, search_dev, ws);              \
+    SOP_CUDA_TRY(launch(wr_hist_kernel<-1, L4>, grid, STB, 0, st, a, A, F, search_dev, ws));           \
+    SOP_CUDA_TRY(launch(wr_pick_kernel, 1, 1024, 0, st, ws, -1, n_keep));                              \
+    SOP_CUDA_TRY(launch(wr_collect_kernel<L4>, grid, STB, 0, st, a, A, F, search_dev, ws));            \
+    SOP_CUDA_TRY(launch(wr_mode_kernel, 1, 32, 0, st, ws, a.cand_cap));                                \
+    SOP_CUDA_TRY(launch(wr_cand_hist_kernel<0>, lgrid, STB, 0, st, a, ws));                            \
+    SOP_CUDA_TRY(launch(wr_hist_kernel<0, L4>, grid, STB, 0, st, a, A, F, search_dev, ws));            \
+    SOP_CUDA_TRY(launch(wr_pick_kernel, 1, 1024, 0, st, ws, 0, n_keep));                               \
+    SOP_CUDA_TRY(launch(wr_cand_hist_kernel<1>, lgrid, STB, 0, st, a, ws));                            \
+    SOP_CUDA_TRY(launch(wr_hist_kernel<1, L4>, grid, STB, 0, st, a, A, F, search_dev, ws));            \
+    SOP_CUDA_TRY(launch(wr_pick_kernel, 1, 1024, 0, st, ws, 1, n_keep));                               \
+    SOP_CUDA_TRY(launch(wr_cand_hist_kernel<2>, lgrid, STB, 0, st, a, ws));                            \
+    SOP_CUDA_TRY(launch(wr_hist_kernel<2, L4>, grid, STB, 0, st, a, A, F, search_dev, ws));            \
+    SOP_CUDA_TRY(launch(wr_pick_kernel, 1, 1024, 0, st, ws, 2, n_keep));                               \
+    SOP_CUDA_TRY(launch(wr_mark_kernel, lgrid, STB, 0, st, a, ws));                                    \
+    SOP_CUDA_TRY(launch(wr_count_kernel<L4>, grid, STB, 0, st, a, A, F, search_dev, ws));              \
+    SOP_CUDA_TRY(launch(tile_scan_kernel, 1, 1024, 0, st, a.tile_sums, n_tiles, row_start_dev, M, count_dev, ws, 1, scale_exp_dev, tau_dev)); \
+    SOP_CUDA_TRY(launch(wr_map_write_kernel<L4>, grid, STB, 0, st, a, A, F, search_dev, ws));          \
+    SOP_CUDA_TRY(launch(wr_write_kernel<L4>, grid, STB, 0, st, a, A, F, search_dev, ws));              \
   } while (0)
   if (lut4) SOP_WR_LAUNCHES(true); else SOP_WR_LAUNCHES(false);
 #undef SOP_WR_LAUNCHES
