@@ -272,7 +272,7 @@ int sop_profile_last_sweep_ms(float* ms);   /* = sop_profile_last_ms(SOP_PROFILE
  *     A caller reads distortion_dev[iters] after synchronising and treats a negative value as a failed call.
  *   pool_count_dev: one long long, number of blocks in the pool.
  * Workspace: 8 bytes per weight element (u and omega of every pool element are kept across the
- *   iterations), 4 bytes per block (the pool list) and 4 bytes per channel, plus a fixed header. */
+ *   iterations), 4 bytes per block (the pool list) and 4 bytes per channel, plus a fixed header (2 MB). */
 #define SOP_LLOYD_POOL_BY_ERROR 1
 #define SOP_LLOYD_UNIFORM_WEIGHTS 2
 #define SOP_LLOYD_POOL_THRESHOLD 4
@@ -282,8 +282,8 @@ int sop_dd4_lloyd_workspace(long long M, long long K, size_t* bytes);
 /* Number of kernel launches one sop_dd4_lloyd call with these sizes and flags makes on the current device
  * (measurement aid, no counterpart in the paper).  All iterations run in one cooperative launch where the
  * device supports such launches (the grid is cut to what is resident at once); otherwise, or with
- * SOP_LLOYD_LAUNCH_PER_ITERATION, there is one launch per iteration.  With SOP_LLOYD_GRID_DP pass the number of
- * table entries as `iters`: the dynamic programme takes one launch per row plus two. */
+ * SOP_LLOYD_LAUNCH_PER_ITERATION, there is one launch per iteration.  With SOP_LLOYD_GRID_DP (any `iters`) the
+ * dynamic programme takes two launches in their place. */
 int sop_dd4_lloyd_launches(long long M, long long K, int iters, int flags, int* launches);
 /* Launch-shape parameters of sop_dd4_lloyd for this process (test aid, no counterpart in the paper; results do
  * not depend on them).  cell_spill_tiles in [1, 128]: cache tiles a CTA sorts between two transfers of its

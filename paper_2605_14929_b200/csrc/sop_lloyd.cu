@@ -77,9 +77,8 @@ struct LloydWs {
   long long cellS[SORT_ROWS];              // sum fix(omega u)
   double cellA[3][SORT_ROWS];              // sum omega, sum omega d, sum omega d^2, d = 256 u - (number of the cell's centre)
   long long cellQ[SORT_ROWS];              // sum fix((omega u) u): the exact second moment the grid-constrained construction needs
-  // not cleared per call: scratch of the dynamic programme, and where the last run starts per (number of runs, last cell)
+  // not cleared per call: where the last run starts per (number of runs, last cell) of the dynamic programme
   short dp_cut[SOP_MAX_ENTRIES][SORT_ROWS];
-  long long dp_scratch[4 * (SORT_ROWS + 1) + 2 * SORT_ROWS];
 };
 
 struct LloydArgs {
@@ -97,7 +96,9 @@ struct LloydArgs {
   unsigned short* tile_start; // workspace: [tiles][TS_PITCH] first sorted position of every cell in every tile
 };
 
-static size_t lloyd_off_omega() { return (sizeof(LloydWs) + 255) & ~(size_t)255; }
+static size_t lloyd_off_dp() { return (sizeof(LloydWs) + 255) & ~(size_t)255; }
+static size_t lloyd_dp_bytes();
+static size_t lloyd_off_omega() { return lloyd_off_dp() + lloyd_dp_bytes(); }
 static size_t lloyd_off_idx(long long K) { return lloyd_off_omega() + (((size_t)K * 4 + 255) & ~(size_t)255); }
 static size_t lloyd_off_cache(long long M, long long K) { return lloyd_off_idx(K) + ((((size_t)M * (size_t)(K / SOP_G)) * 4 + 255) & ~(size_t)255); }
 constexpr int CTB = 384;                        // threads of a cache CTA = pool blocks of a cache tile
@@ -948,10 +949,35 @@ __global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs
 // S = sum fix(omega u), Q = sum fix((omega u) u), integers, so independent of any order.  The cells with H > 0, in
 // ascending order, are cut into min(n_entries, cells) runs; a run's code point is the bf16 value nearest to S / H
 // (clamped to +-1.25) and it costs Q - 2 q S + q^2 H; the least total cost wins, a tie between cuts goes to the earliest.
-// One launch per row of the programme (number of runs), one warp per last cell; the FP64 operations are written one by
-// one (no contraction), so every comparison sees the same numbers as a sequential evaluation.
+//   grid_dp_cost_kernel   the costs of all runs i .. j, which no row of the programme changes: every CTA works out the prefix sums
+//                         for itself and takes its share of the 205 thousand divisions
+//   grid_dp_rows_kernel   the rows (number of runs) in one cluster of eight CTAs: a CTA keeps the costs of every eighth last cell
+//                         in shared memory, a warp takes a last cell, the row's least costs go to all eight CTAs' shared memory
+//                         and a cluster barrier ends the row; then the backtrack
+// The FP64 operations are written one by one (no contraction), so every comparison sees the same numbers as a sequential evaluation.
+// What bounds it: the latency of the rows (about 3 us each).  2048 x 4096, 16 entries: 223 us with one launch per row that worked the
+// costs out again and a serial first and last step, 75 us now.
 // ---------------------------------------------------------------------------------------------
-constexpr int DP_TB = 256;
+constexpr int DP_TB = 1024;
+constexpr int DP_CL = 8;                                                             // CTAs of the cluster
+constexpr int DP_COLS = (SORT_ROWS + DP_CL - 1) / DP_CL;                             // last cells of a CTA
+constexpr int DP_SLICE = DP_CL / 2 * DP_COLS * (DP_COLS - 1) + DP_CL * DP_COLS;      // costs of a CTA, at most
+
+// Scratch of the dynamic programme in the workspace: prefix sums of the non-empty cells, the costs by CTA of the cluster.
+struct DpScratch {
+  int B;
+  int pad;
+  long long pH[SORT_ROWS + 1], pS[SORT_ROWS + 1], pQ[SORT_ROWS + 1];
+  double cost[DP_CL][DP_SLICE];
+};
+
+static size_t lloyd_dp_bytes() { return (sizeof(DpScratch) + 255) & ~(size_t)255; }
+
+// the costs of last cell j (starts 0 .. j) in the slice of CTA j % DP_CL: the cells j % DP_CL, j % DP_CL + DP_CL, ... one after the other
+__device__ __forceinline__ int dp_column(int j) {
+  const int t = j / DP_CL, c = j % DP_CL;
+  return DP_CL / 2 * t * (t - 1) + (c + 1) * t;
+}
 
 __device__ __forceinline__ double dp_run_cost(const long long* pH, const long long* pS, const long long* pQ, int i, int j, float* q_out) {
   const double h = __ll2double_rn(pH[j + 1] - pH[i]), sm = __ll2double_rn(pS[j + 1] - pS[i]), qq = __ll2double_rn(pQ[j + 1] - pQ[i]);
@@ -968,91 +994,134 @@ __device__ __forceinline__ double dp_run_cost(const long long* pH, const long lo
   return __dadd_rn(__dsub_rn(qq, a), c);
 }
 
-// Scratch of the dynamic programme in the workspace: prefix sums of the non-empty cells, two rows of least costs.
-struct DpScratch {
-  int B;
-  int pad;
-  long long pH[SORT_ROWS + 1], pS[SORT_ROWS + 1], pQ[SORT_ROWS + 1];
+__global__ void __launch_bounds__(DP_TB) grid_dp_cost_kernel(const LloydWs* __restrict__ ws, DpScratch* __restrict__ dp) {
+  __shared__ long long pre[3][SORT_ROWS + 1];
+  __shared__ long long tot[4][32];
+  pdl_trigger();
+  pdl_wait();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  static_assert(SORT_ROWS <= DP_TB, "one cell per thread");
+  long long v[3] = {0, 0, 0};
+  if (tid < SORT_ROWS) { v[0] = (long long)ws->cellN[tid]; v[1] = ws->cellS[tid]; v[2] = ws->cellQ[tid]; }
+  const bool on = v[0] > 0;
+  if (!on) v[1] = v[2] = 0;
+  long long n = on ? 1 : 0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long a = __shfl_up_sync(0xFFFFFFFFu, v[0], o), b = __shfl_up_sync(0xFFFFFFFFu, v[1], o), c = __shfl_up_sync(0xFFFFFFFFu, v[2], o);
+    const long long m = __shfl_up_sync(0xFFFFFFFFu, n, o);
+    if (lane >= o) { v[0] += a; v[1] += b; v[2] += c; n += m; }
+  }
+  if (lane == 31) { tot[0][warp] = v[0]; tot[1][warp] = v[1]; tot[2][warp] = v[2]; tot[3][warp] = n; }
+  __syncthreads();
+  int B = 0;
+  for (int w = 0; w < DP_TB / 32; ++w) {
+    if (w < warp) { v[0] += tot[0][w]; v[1] += tot[1][w]; v[2] += tot[2][w]; n += tot[3][w]; }
+    B += (int)tot[3][w];
+  }
+  if (on) { pre[0][n] = v[0]; pre[1][n] = v[1]; pre[2][n] = v[2]; }
+  if (tid < 3) pre[tid][0] = 0;
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    for (int i = tid; i <= B; i += DP_TB) { dp->pH[i] = pre[0][i]; dp->pS[i] = pre[1][i]; dp->pQ[i] = pre[2][i]; }
+    if (tid == 0) dp->B = B;
+  }
+  // last cells j and B - 1 - j together have B + 1 starts: the CTAs take such pairs
+  for (int p = blockIdx.x; 2 * p < B; p += gridDim.x) {
+    const int ja = p, jb = B - 1 - p;
+    const int n_a = ja + 1, total = jb > ja ? n_a + jb + 1 : n_a;
+    for (int x = tid; x < total; x += DP_TB) {
+      const int j = x < n_a ? ja : jb, i = x < n_a ? x : x - n_a;
+      dp->cost[j % DP_CL][dp_column(j) + i] = dp_run_cost(pre[0], pre[1], pre[2], i, j, nullptr);
+    }
+  }
+}
+
+struct DpSmem {
   double best[2][SORT_ROWS];
+  float lut[SOP_MAX_ENTRIES];
+  double cost[DP_SLICE];          // CTA 0, after the last row: where the last run starts, [rows][SORT_ROWS] 16-bit numbers
 };
 
-// One CTA: the non-empty cells, their prefix sums, and row 0 (cells 0..j as one run).
-__global__ void __launch_bounds__(DP_TB) grid_dp_first_kernel(const LloydWs* __restrict__ ws, DpScratch* __restrict__ dp) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ int s_B;
-  if (threadIdx.x == 0) {
-    int B = 0;
-    dp->pH[0] = dp->pS[0] = dp->pQ[0] = 0;
-    for (int t = 0; t < SORT_ROWS; ++t) {
-      const long long h = (long long)ws->cellN[t];
-      if (h > 0) { dp->pH[B + 1] = dp->pH[B] + h; dp->pS[B + 1] = dp->pS[B] + ws->cellS[t]; dp->pQ[B + 1] = dp->pQ[B] + ws->cellQ[t]; ++B; }
-    }
-    dp->B = B;
-    s_B = B;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < s_B; j += DP_TB) dp->best[0][j] = dp_run_cost(dp->pH, dp->pS, dp->pQ, 0, j, nullptr);
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Row r of the programme: one warp per last cell j, the lanes share the starts i of the last run; the least value wins,
-// a tie goes to the smallest i (what a sequential scan from the first start on keeps).
-__global__ void __launch_bounds__(DP_TB) grid_dp_row_kernel(DpScratch* __restrict__ dp, int r, short* __restrict__ cut) {
+__global__ void __cluster_dims__(DP_CL, 1, 1) __launch_bounds__(DP_TB) grid_dp_rows_kernel(const DpScratch* __restrict__ dp, int n_entries,
+                                                                                         short* __restrict__ cut, float* __restrict__ out_lut,
+                                                                                         double* __restrict__ cost_out) {
+  extern __shared__ __align__(16) unsigned char dp_smem[];
+  DpSmem& S = *reinterpret_cast<DpSmem*>(dp_smem);
   pdl_trigger();
   pdl_wait();
-  const int B = dp->B;
-  const int lane = threadIdx.x & 31;
-  const int j = blockIdx.x * (DP_TB / 32) + (threadIdx.x >> 5);
-  if (j >= B || j < r) return;
-  const double* prev = dp->best[(r - 1) & 1];
-  double bv = 0.0;
-  int bi = -1;
-  for (int i = r + lane; i <= j; i += 32) {
-    const double v = __dadd_rn(prev[i - 1], dp_run_cost(dp->pH, dp->pS, dp->pQ, i, j, nullptr));
-    if (bi < 0 || v < bv) { bv = v; bi = i; }
-  }
-  for (int o = 16; o; o >>= 1) {
-    const double ov = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
-    const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
-    if (oi >= 0 && (bi < 0 || ov < bv || (ov == bv && oi < bi))) { bv = ov; bi = oi; }
-  }
-  if (lane == 0) {
-    dp->best[r & 1][j] = bv;
-    cut[(size_t)r * SORT_ROWS + j] = (short)bi;
-  }
-}
-
-// One thread: the backtrack, the code points in ascending order, the least total cost.  rows = rows the host launched
-// (n_entries - 1 at most); with fewer cells than entries the programme stops at the last row that has a cell.
-__global__ void grid_dp_last_kernel(const DpScratch* __restrict__ dp, int n_entries, const short* __restrict__ cut, float* __restrict__ out_lut,
-                                    double* __restrict__ cost_out) {
-  pdl_trigger();
-  pdl_wait();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int B = dp->B;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = (int)blockIdx.x;       // one cluster
+  const int B = dp->B, R = min(n_entries, B);
   if (B == 0) {
-    for (int e = 0; e < SOP_MAX_ENTRIES; ++e) out_lut[e] = 0.0f;
-    cost_out[0] = 0.0;
-    return;
+    if (rank == 0 && tid < SOP_MAX_ENTRIES) out_lut[tid] = 0.0f;
+    if (rank == 0 && tid == 0) cost_out[0] = 0.0;
+    return;                                            // (the same in every CTA)
   }
-  const int R = min(n_entries, B);
-  float lut[SOP_MAX_ENTRIES];
-  int j = B - 1, n = 0;
-  for (int r = R - 1; r >= 0; --r) {
-    const int i = r == 0 ? 0 : (int)cut[(size_t)r * SORT_ROWS + j];
-    float q;
-    dp_run_cost(dp->pH, dp->pS, dp->pQ, i, j, &q);
-    lut[n++] = q;
-    j = i - 1;
+  const int n_cols = rank < B ? (B - 1 - rank) / DP_CL + 1 : 0, j_end = rank + DP_CL * n_cols;
+  const int n_cost = dp_column(j_end);
+  for (int x = tid; x < n_cost; x += DP_TB) S.cost[x] = dp->cost[rank][x];
+  for (int j = tid; j < B; j += DP_TB) S.best[0][j] = dp->cost[j % DP_CL][dp_column(j)];        // one run: cells 0 .. j
+  cluster_sync();
+  for (int r = 1; r < R; ++r) {
+    const double* prev = S.best[(r - 1) & 1];
+    // a warp per last cell j, the lanes share the starts i of the last run; the least value wins, a tie goes to the smallest i (what
+    // a sequential scan from the first start on keeps)
+    for (int t = warp; t < n_cols; t += DP_TB / 32) {
+      const int j = rank + DP_CL * t;
+      if (j < r) continue;
+      const double* col = S.cost + dp_column(j);
+      double bv = 0.0;
+      int bi = -1;
+      for (int i = r + lane; i <= j; i += 32) {
+        const double v = __dadd_rn(prev[i - 1], col[i]);
+        if (bi < 0 || v < bv) { bv = v; bi = i; }
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
+        const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+        if (oi >= 0 && (bi < 0 || ov < bv || (ov == bv && oi < bi))) { bv = ov; bi = oi; }
+      }
+      if (lane < DP_CL) {                              // to the shared memory of every CTA of the cluster
+        unsigned at;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(&S.best[r & 1][j])), "r"(lane));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(bv) : "memory");
+      }
+      if (lane == 0) cut[(size_t)r * SORT_ROWS + j] = (short)bi;
+    }
+    cluster_sync();
   }
-  for (int a = 1; a < n; ++a) {                   // ascending: insertion sort of at most 32 values
-    const float v = lut[a];
-    int b = a - 1;
-    while (b >= 0 && lut[b] > v) { lut[b + 1] = lut[b]; --b; }
-    lut[b + 1] = v;
+  if (rank != 0) return;
+  // the backtrack, the code points in ascending order, the least total cost; with fewer cells than entries the programme stops at
+  // the last row that has a cell
+  short* s_cut = reinterpret_cast<short*>(S.cost);
+  for (int x = tid; x < R * SORT_ROWS; x += DP_TB) s_cut[x] = x < SORT_ROWS ? 0 : __ldcg(cut + x);
+  __syncthreads();
+  if (warp == 0) {
+    int j = B - 1, my_i = 0, my_j = 0;
+    for (int r = R - 1; r >= 0; --r) {
+      const int i = s_cut[r * SORT_ROWS + j];
+      if (lane == r) { my_i = i; my_j = j; }
+      j = i - 1;
+    }
+    float q = __int_as_float(0x7F800000);
+    if (lane < R) dp_run_cost(dp->pH, dp->pS, dp->pQ, my_i, my_j, &q);
+    int at = 0;                                        // ascending, ties by run
+#pragma unroll 1
+    for (int k = 0; k < R; ++k) {
+      const float o = __shfl_sync(0xFFFFFFFFu, q, k);
+      at += o < q || (o == q && k < lane) ? 1 : 0;
+    }
+    if (lane < R) S.lut[at] = q;
+    __syncwarp();
+    out_lut[lane] = lane < n_entries ? S.lut[min(lane, R - 1)] : 0.0f;
+    if (lane == 0) cost_out[0] = __ddiv_rn(S.best[(R - 1) & 1][B - 1], 16777216.0);
   }
-  for (int e = 0; e < SOP_MAX_ENTRIES; ++e) out_lut[e] = e < n ? lut[e] : (e < n_entries ? lut[n - 1] : 0.0f);
-  cost_out[0] = __ddiv_rn(dp->best[(R - 1) & 1][B - 1], 16777216.0);
 }
 
 int num_sms();
@@ -1092,13 +1161,12 @@ extern "C" {
 
 int sop_dd4_lloyd_launches(long long M, long long K, int iters, int flags, int* launches) {
   if (!launches) return SOP_ERR_NULL;
-  const int dp_entries = iters > 1 ? iters : 2;      // with SOP_LLOYD_GRID_DP the caller passes the number of table entries here
   if (M < 1 || K < 1 || (K % SOP_G) != 0 || iters < 0 || iters > sop::SOP_MAX_LLOYD_ITERS) return SOP_ERR_RANGE;
   long long grid = 1;
   const bool persistent = sop::lloyd_iteration_plan(M * (K / SOP_G), iters, flags, &grid);
   // radix select (three passes, unless the pool is cut by a threshold), set-up, pool list, pool cache, iterations
-  // the dynamic programme: first row, one launch per further row (callers with a 16-entry table: 15), the backtrack
-  *launches = ((flags & SOP_LLOYD_POOL_THRESHOLD) ? 0 : 3) + 3 + ((flags & SOP_LLOYD_GRID_DP) ? 2 + (dp_entries - 1) : (persistent ? 1 : iters + 1));
+  // the dynamic programme: the costs, the rows
+  *launches = ((flags & SOP_LLOYD_POOL_THRESHOLD) ? 0 : 3) + 3 + ((flags & SOP_LLOYD_GRID_DP) ? 2 : (persistent ? 1 : iters + 1));
   return SOP_OK;
 }
 
@@ -1202,6 +1270,7 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
     if (!facts->lloyd_attr_set) {
       SOP_CUDA_TRY(cudaFuncSetAttribute(pool_cache_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage_bytes));
       SOP_CUDA_TRY(cudaFuncSetAttribute(pool_cache_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage_bytes));
+      SOP_CUDA_TRY(cudaFuncSetAttribute(grid_dp_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DpSmem)));
       SOP_CUDA_TRY(cudaFuncSetAttribute(lloyd_iter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ITER_SMEM_MAX));
       facts->lloyd_attr_set = true;
     }
@@ -1212,13 +1281,9 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
   if ((rc = profile_mark(SOP_PROFILE_POOL, 1, st))) return rc;
   if (grid_dp) {
     if ((rc = profile_mark(SOP_PROFILE_LLOYD, 0, st))) return rc;
-    static_assert(sizeof(DpScratch) <= sizeof(((LloydWs*)nullptr)->dp_scratch), "scratch of the dynamic programme");
-    DpScratch* dp = reinterpret_cast<DpScratch*>(ws->dp_scratch);
-    SOP_CUDA_TRY(launch(grid_dp_first_kernel, 1, DP_TB, 0, st, ws, dp));
-    for (int r = 1; r < ne; ++r)      // a row without a cell (fewer cells than entries) returns at once
-      SOP_CUDA_TRY(launch(grid_dp_row_kernel, (SORT_ROWS + DP_TB / 32 - 1) / (DP_TB / 32), DP_TB, 0, st, dp, r, &ws->dp_cut[0][0]));
-    SOP_CUDA_TRY(launch(grid_dp_last_kernel, 1, 32, 0, st, dp, ne, &ws->dp_cut[0][0], out_lut_dev, distortion_dev));
-    SOP_CUDA_TRY(cudaGetLastError());
+    DpScratch* dp = reinterpret_cast<DpScratch*>(wsb + lloyd_off_dp());
+    SOP_CUDA_TRY(launch(grid_dp_cost_kernel, sms, DP_TB, 0, st, ws, dp));
+    SOP_CUDA_TRY(launch(grid_dp_rows_kernel, DP_CL, DP_TB, sizeof(DpSmem), st, dp, ne, &ws->dp_cut[0][0], out_lut_dev, distortion_dev));
     if ((rc = profile_mark(SOP_PROFILE_LLOYD, 1, st))) return rc;
     return SOP_OK;
   }
