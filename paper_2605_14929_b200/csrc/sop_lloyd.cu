@@ -1,15 +1,14 @@
 // sop_dd4_lloyd: per-layer data-derived codebook (DD-n) by Lloyd iteration on the pool of blocks
 // that the primary codebook reconstructs worst.
 //
+//   lloyd_init_kernel     clears the header, max(c), the shift k, the initial table (FMTa, reversed and negated if
+//                         FMTa is a negated atom) as the first iteration's descriptor.
 //   select_kernel<PASS>   three-pass radix select (11 + 11 + 10 bits) of the pool_rank-th worst block by
-//                         its ranking key (cosine ascending, or error descending); each pass re-derives
-//                         the prefix from the previous histograms with a CTA-wide scan.  Not run when the
+//                         its ranking key (cosine ascending, or error descending); each pass finds the bin
+//                         of the previous histogram with a CTA-wide scan.  Not run when the
 //                         caller fixes the pool threshold.
-//   lloyd_setup_kernel    threshold key from the last histogram (or from the given threshold), max(c),
-//                         the shift k, the initial table (FMTa, reversed and negated if FMTa is a negated
-//                         atom), the per-channel weight table omega = c / max(c) (or 1), and the first
-//                         iteration descriptor.
-//   pool_list_kernel      compacts the indices of the pool blocks into a dense list.
+//   pool_list_kernel      threshold key from the last histogram (or from the given threshold); compacts the indices of the pool
+//                         blocks into a dense list; the per-channel weight table omega = c / max(c) (or 1).
 //   pool_cache_kernel     the pool elements never change between iterations, only the table does:
 //                         (u, omega) of every pool element is computed once (u = w / scale) and kept
 //                         in tiles of 6144 elements, each counting-sorted by the cell of u on a
@@ -35,7 +34,7 @@
 namespace sop {
 
 constexpr int LTB = 256;
-constexpr int SETUP_TB = 1024;
+constexpr int INIT_TB = 1024;
 constexpr int SOP_MAX_LLOYD_ITERS = 64;
 constexpr int SORT_CHALF = 320;                 // lookup grid on u: cell width 2^-8, rows cover |u| <= 1.25,
 constexpr int SORT_ROWS = 2 * SORT_CHALF + 1;   // the first and last row take everything beyond
@@ -62,22 +61,24 @@ struct LloydWs {
   unsigned long long accN[SOP_MAX_LLOYD_ITERS + 1][SOP_MAX_ENTRIES];
   long long accS[SOP_MAX_LLOYD_ITERS + 1][SOP_MAX_ENTRIES];
   double accD[SOP_MAX_LLOYD_ITERS + 1];
-  unsigned tau_key;  // pool threshold as a ranking key: the pool is every block whose key is not above it
-  float cmax;
-  int k;
-  int fmta;
+  unsigned prefix[3];       // of the selected key after one, two passes
+  unsigned pad3;
+  long long rank[3];        // its rank inside that prefix
   unsigned arrive[SOP_MAX_LLOYD_ITERS + 1];      // CTAs that have added their sums of an iteration
   unsigned error;        // a CTA gave up waiting for a flag
   unsigned list_count;   // blocks appended to the pool list
-  int pad;
-  // the current codebook, rewritten by whoever changes it (set-up, then each update)
-  IterDesc desc;
   // per cell, over the whole pool (filled once by pool_cache_kernel)
   unsigned long long cellN[SORT_ROWS];     // sum fix(omega)
   long long cellS[SORT_ROWS];              // sum fix(omega u)
   double cellA[3][SORT_ROWS];              // sum omega, sum omega d, sum omega d^2, d = 256 u - (number of the cell's centre)
   long long cellQ[SORT_ROWS];              // sum fix((omega u) u): the exact second moment the grid-constrained construction needs
-  // not cleared per call: where the last run starts per (number of runs, last cell) of the dynamic programme
+  // from here on set by lloyd_init_kernel
+  alignas(16) float cmax;
+  int k;
+  int fmta;
+  // the current codebook, rewritten by whoever changes it (set-up, then each update)
+  IterDesc desc;
+  // neither: where the last run starts per (number of runs, last cell) of the dynamic programme
   short dp_cut[SOP_MAX_ENTRIES][SORT_ROWS];
 };
 
@@ -165,21 +166,19 @@ __device__ void find_bin(const unsigned* __restrict__ hist, int nb, long long ra
   __syncthreads();
 }
 
-// After pass p the selected element lies in one bin of hist[p]; the key prefix, the rank inside
-// that bin and the number of elements below it follow from the histograms of the passes so far.
-__device__ void derive_prefix(const LloydWs* ws, long long pool_rank, int passes, unsigned* prefix, long long* rank_out,
-                              long long* below_out, unsigned* last_count) {
-  long long rank = pool_rank, below = 0;
-  unsigned pre = 0, cnt = 0;
-  for (int p = 0; p < passes; ++p) {
-    int bin;
-    long long before;
-    find_bin(ws->hist[p], p < 2 ? 2048 : 1024, rank, &bin, &before, &cnt);
-    rank -= before;
-    below += before;
-    pre = (pre << (p < 2 ? 11 : 10)) | (unsigned)bin;
-  }
-  *prefix = pre; *rank_out = rank; *below_out = below; *last_count = cnt;
+// Whole CTA, after `passes` >= 1 passes: the prefix of the selected key from the histogram of the last pass; the passes before it
+// have left theirs in the workspace, and the first CTA leaves this one.
+__device__ unsigned derive_prefix(LloydWs* ws, long long pool_rank, int passes) {
+  const int p = passes - 1;
+  const unsigned pre = p ? __ldcg(&ws->prefix[p - 1]) : 0u;
+  const long long rank = p ? __ldcg(&ws->rank[p - 1]) : pool_rank;
+  int bin;
+  long long before;
+  unsigned cnt;
+  find_bin(ws->hist[p], p < 2 ? 2048 : 1024, rank, &bin, &before, &cnt);
+  const unsigned out = (pre << (p < 2 ? 11 : 10)) | (unsigned)bin;
+  if (blockIdx.x == 0 && threadIdx.x == 0) { ws->prefix[p] = out; ws->rank[p] = rank - before; }
+  return out;
 }
 
 template <int PASS>
@@ -188,9 +187,8 @@ __global__ void __launch_bounds__(LTB) select_kernel(LloydArgs a, const sop_sear
   pdl_wait();
   __shared__ unsigned sh[2048];
   for (int i = threadIdx.x; i < 2048; i += LTB) sh[i] = 0;
-  unsigned prefix = 0, cnt;
-  long long rank, below;
-  if (PASS > 0) derive_prefix(ws, a.pool_rank, PASS, &prefix, &rank, &below, &cnt);
+  unsigned prefix = 0;
+  if (PASS > 0) prefix = derive_prefix(ws, a.pool_rank, PASS);
   __syncthreads();
   const float* row = a.cosrow_base + (size_t)resolve_fmta(a, res) * a.NB;
   auto count = [&](float x) {
@@ -235,82 +233,78 @@ __device__ __forceinline__ int sort_cell(float u) {
 
 __device__ void make_desc(IterDesc* d, const float* table, int ne);
 
-__global__ void __launch_bounds__(SETUP_TB) lloyd_setup_kernel(LloydArgs a, AtomsDev A, const sop_search_result* __restrict__ res,
-                                                               LloydWs* __restrict__ ws, double* __restrict__ distortion, int iters) {
+// CTA 0: max(c) and what the first table needs; the others clear the header.
+__global__ void __launch_bounds__(INIT_TB) lloyd_init_kernel(LloydArgs a, AtomsDev A, const sop_search_result* __restrict__ res,
+                                                             LloydWs* __restrict__ ws, double* __restrict__ distortion, int iters) {
+  __shared__ float red[INIT_TB / 32];
+  __shared__ float s_lut[SOP_MAX_ENTRIES];
   pdl_trigger();
   pdl_wait();
-  unsigned prefix = 0, cnt = 0;
-  long long rank = 0, below = 0;
-  if (a.flags & SOP_LLOYD_POOL_THRESHOLD) prefix = pool_key(a.pool_threshold, a.flags);   // the caller fixes the threshold
-  else derive_prefix(ws, a.pool_rank, 3, &prefix, &rank, &below, &cnt);
-  __shared__ float red[SETUP_TB / 32];
-  __shared__ float s_cmax;
-  __shared__ float s_lut[SOP_MAX_ENTRIES];
-  __shared__ int s_ne;
+  const int tid = threadIdx.x;
+  if (blockIdx.x != 0) {
+    // everything that kernels add to, up to the values that CTA 0 writes
+    uint4* h = reinterpret_cast<uint4*>(ws);
+    const int n = (int)(offsetof(LloydWs, cmax) / sizeof(uint4));
+    for (int i = (int)(blockIdx.x - 1) * INIT_TB + tid; i < n; i += (int)(gridDim.x - 1) * INIT_TB) h[i] = make_uint4(0u, 0u, 0u, 0u);
+    return;
+  }
   float mx = 0.0f;
-  for (long long i = threadIdx.x; i < a.K; i += SETUP_TB) mx = fmaxf(mx, __ldg(a.c + i));
+  for (long long i = tid; i < a.K; i += INIT_TB) mx = fmaxf(mx, __ldg(a.c + i));
   for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = red[0];
-    for (int w = 1; w < SETUP_TB / 32; ++w) t = fmaxf(t, red[w]);
-    s_cmax = t;
+  if ((tid & 31) == 0) red[tid >> 5] = mx;
+  const int f = resolve_fmta(a, res), ne = A.atoms[f].n_entries;
+  if (tid < SOP_MAX_ENTRIES) {
+    const int j = min(tid, ne - 1), src = A.atoms[f].negated ? ne - 1 - j : j;       // padded with the last entry
+    float v = ((A.dd_mask >> f) & 1u) ? A.dd_lut[src] : A.atoms[f].lut[src];
+    if (A.atoms[f].negated) v = -v;
+    s_lut[tid] = v;
   }
   __syncthreads();
-  const float cmax = s_cmax;
-  for (long long i = threadIdx.x; i < a.K; i += SETUP_TB) {
-    const float om = (a.flags & SOP_LLOYD_UNIFORM_WEIGHTS) ? 1.0f : (cmax > 0.0f ? __fdiv_rn(__ldg(a.c + i), cmax) : 0.0f);
-    a.omega[i] = om;
-  }
-  if (threadIdx.x == 0) {
-    ws->tau_key = prefix;          // full 32-bit key after three passes (or the key of the given threshold)
-    ws->cmax = cmax;
-    const int f = resolve_fmta(a, res);
-    ws->fmta = f;
-    ws->k = a.k_mode == SOP_K_FROM_RESULT ? res->k[f] : a.k_mode;
-    const sop_atom& at = A.atoms[f];
-    const int ne = at.n_entries;
-    s_ne = ne;
-    const bool dd = (A.dd_mask >> f) & 1u;
-    for (int j = 0; j < SOP_MAX_ENTRIES; ++j) {
-      const int src = at.negated ? ne - 1 - min(j, ne - 1) : min(j, ne - 1);   // padded with the last entry
-      float v = dd ? A.dd_lut[src] : at.lut[src];
-      if (at.negated) v = -v;
-      s_lut[j] = v;
+  if (tid < 32) {
+    float t = red[tid];
+    for (int o = 16; o; o >>= 1) t = fmaxf(t, __shfl_xor_sync(0xFFFFFFFFu, t, o));
+    make_desc(&ws->desc, s_lut, ne);
+    if (tid == 0) {
+      ws->cmax = t;
+      ws->fmta = f;
+      ws->k = a.k_mode == SOP_K_FROM_RESULT ? res->k[f] : a.k_mode;
+      // "not finished": the closing iteration overwrites it with the final distortion (never negative)
+      distortion[iters] = -1.0;
     }
-    // "not finished": the closing iteration overwrites it with the final distortion (never negative)
-    distortion[iters] = -1.0;
   }
-  __syncthreads();
-  if (threadIdx.x < 32) make_desc(&ws->desc, s_lut, s_ne);
 }
 
-// Dense list of the pool blocks.  A thread takes sixteen consecutive blocks per round (four 128-bit loads in flight
-// where the row is 16-byte aligned); the CTA's count goes to the list's counter once per round (a warp scan of the
-// threads' counts, then a scan of the eight warp totals).  The order of the list depends on the scheduling of the
-// CTAs; nothing downstream depends on it (integer sums, and an FP64 sum compared with a tolerance).
-constexpr int LIST_PER_THREAD = 16;
+// Dense list of the pool blocks.  A warp takes 512 consecutive blocks per round (four 128-bit loads per lane in flight, each a
+// contiguous half kilobyte of the row, where it is 16-byte aligned); the counts of a lane's four groups of four are scanned
+// together as bytes of one word.  The CTA's count goes to the list's counter once per round; the indices are laid out in shared
+// memory and leave in whole lines.  The order of the list depends on the scheduling of the CTAs; nothing downstream depends on it
+// (integer sums, and FP64 sums compared with a tolerance).
+constexpr int LIST_ROUND = (LTB / 32) * 512;
 __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __restrict__ ws) {
+  __shared__ unsigned s_cnt[LTB / 32 + 1];
+  __shared__ unsigned s_base;
+  __shared__ unsigned s_idx[LIST_ROUND];
   pdl_trigger();
   pdl_wait();
-  __shared__ unsigned s_cnt[LTB / 32];
-  __shared__ unsigned s_base;
-  const unsigned tau_key = ws->tau_key;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned tau_key = (a.flags & SOP_LLOYD_POOL_THRESHOLD) ? pool_key(a.pool_threshold, a.flags)      // the caller fixes the threshold
+                                                                : derive_prefix(ws, a.pool_rank, 3);
+  {
+    const float cmax = ws->cmax;
+    for (long long i = (long long)blockIdx.x * LTB + tid; i < a.K; i += (long long)gridDim.x * LTB)
+      a.omega[i] = (a.flags & SOP_LLOYD_UNIFORM_WEIGHTS) ? 1.0f : (cmax > 0.0f ? __fdiv_rn(__ldg(a.c + i), cmax) : 0.0f);
+  }
   const float* row = a.cosrow_base + (size_t)ws->fmta * a.NB;
   const bool vec = (reinterpret_cast<uintptr_t>(row) & 15u) == 0;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long stride = (long long)gridDim.x * LTB * LIST_PER_THREAD;
-  const long long n_round = (a.NB + stride - 1) / stride;
-  long long i = ((long long)blockIdx.x * LTB + threadIdx.x) * LIST_PER_THREAD;
-  for (long long r = 0; r < n_round; ++r, i += stride) {
-    unsigned in = 0;
-    if (vec && i + LIST_PER_THREAD <= a.NB) {
-      float4 v[LIST_PER_THREAD / 4];
+  for (long long base = (long long)blockIdx.x * LIST_ROUND; base < a.NB; base += (long long)gridDim.x * LIST_ROUND) {
+    const long long i0 = base + warp * 512 + 4 * lane;
+    unsigned in = 0;                     // bit 4 q + b: block i0 + 128 q + b
+    if (vec && base + warp * 512 + 512 <= a.NB) {
+      float4 v[4];
 #pragma unroll
-      for (int q = 0; q < LIST_PER_THREAD / 4; ++q) v[q] = __ldg(reinterpret_cast<const float4*>(row + i) + q);
+      for (int q = 0; q < 4; ++q) v[q] = __ldg(reinterpret_cast<const float4*>(row + i0 + 128 * q));
 #pragma unroll
-      for (int q = 0; q < LIST_PER_THREAD / 4; ++q) {
+      for (int q = 0; q < 4; ++q) {
         in |= (pool_key(v[q].x, a.flags) <= tau_key ? 1u : 0u) << (4 * q);
         in |= (pool_key(v[q].y, a.flags) <= tau_key ? 1u : 0u) << (4 * q + 1);
         in |= (pool_key(v[q].z, a.flags) <= tau_key ? 1u : 0u) << (4 * q + 2);
@@ -318,26 +312,38 @@ __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __
       }
     } else {
 #pragma unroll 4
-      for (int q = 0; q < LIST_PER_THREAD; ++q)
-        if (i + q < a.NB && pool_key(__ldg(row + i + q), a.flags) <= tau_key) in |= 1u << q;
+      for (int x = 0; x < 16; ++x) {
+        const long long i = i0 + 128 * (x >> 2) + (x & 3);
+        if (i < a.NB && pool_key(__ldg(row + i), a.flags) <= tau_key) in |= 1u << x;
+      }
     }
-    const unsigned mine = (unsigned)__popc(in);
+    unsigned mine = 0;                   // a lane's four counts, a byte each (a warp's sum is at most 128)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mine |= (unsigned)__popc((in >> (4 * q)) & 15u) << (8 * q);
     unsigned incl = mine;
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
       if (lane >= o) incl += v;
     }
-    if (lane == 31) s_cnt[warp] = incl;
+    const unsigned tot = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - mine;
+    if (lane == 0) s_cnt[warp] = (tot & 255u) + ((tot >> 8) & 255u) + ((tot >> 16) & 255u) + (tot >> 24);
     __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned tot = 0;
-      for (int w = 0; w < LTB / 32; ++w) { const unsigned c = s_cnt[w]; s_cnt[w] = tot; tot += c; }
-      s_base = tot ? atomicAdd(&ws->list_count, tot) : 0u;
+    unsigned at = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < LTB / 32; ++w) { const unsigned c = s_cnt[w]; at += w < warp ? c : 0u; all += c; }
+    if (tid == 0) s_base = all ? atomicAdd(&ws->list_count, all) : 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      unsigned p = at + ((excl >> (8 * q)) & 255u);
+      at += (tot >> (8 * q)) & 255u;
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if ((in >> (4 * q + b)) & 1u) s_idx[p++] = (unsigned)(i0 + 128 * q + b);
     }
     __syncthreads();
-    unsigned at = s_base + s_cnt[warp] + incl - mine;
-    for (unsigned rest = in; rest; rest &= rest - 1u) a.pool_idx[at++] = (unsigned)(i + (__ffs((int)rest) - 1));
-    __syncthreads();             // s_cnt and s_base are rewritten in the next round
+    const unsigned to = s_base;
+    for (unsigned x = tid; x < all; x += LTB) a.pool_idx[to + x] = s_idx[x];
+    __syncthreads();             // s_cnt, s_base and s_idx are rewritten in the next round
   }
 }
 
@@ -1243,22 +1249,19 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
   a.tile_start = (unsigned short*)(wsb + lloyd_off_tiles(M, K));
   LloydWs* ws = (LloydWs*)workspace_dev;
   cudaStream_t st = (cudaStream_t)stream;
-  SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, offsetof(LloydWs, dp_cut), st));
   if ((rc = profile_mark(SOP_PROFILE_POOL, 0, st))) return rc;
   const int sms = num_sms();
   long long sg = (NB + LTB * 8 - 1) / (LTB * 8);
   if (sg > sms * 4) sg = sms * 4;
   if (sg < 1) sg = 1;
+  SOP_CUDA_TRY(launch(lloyd_init_kernel, 9, INIT_TB, 0, st, a, A, search_dev, ws, distortion_dev, iters));
   if (!by_threshold) {     // radix select of the pool_rank-th worst block (three passes over the ranking keys)
     SOP_CUDA_TRY(launch(select_kernel<0>, sg, LTB, 0, st, a, search_dev, ws));
     SOP_CUDA_TRY(launch(select_kernel<1>, sg, LTB, 0, st, a, search_dev, ws));
     SOP_CUDA_TRY(launch(select_kernel<2>, sg, LTB, 0, st, a, search_dev, ws));
-    SOP_CUDA_TRY(cudaGetLastError());
   }
-  SOP_CUDA_TRY(launch(lloyd_setup_kernel, 1, SETUP_TB, 0, st, a, A, search_dev, ws, distortion_dev, iters));
-  SOP_CUDA_TRY(cudaGetLastError());
-  SOP_CUDA_TRY(launch(pool_list_kernel, sg, LTB, 0, st, a, ws));
-  SOP_CUDA_TRY(cudaGetLastError());
+  const long long lg = (NB + LIST_ROUND - 1) / LIST_ROUND;
+  SOP_CUDA_TRY(launch(pool_list_kernel, (unsigned)(lg < sms * 6 ? lg : sms * 6), LTB, 0, st, a, ws));
 
   // (u, omega) of every pool element, once: sorted tiles, cell starts, per-cell sums and moments
   {
