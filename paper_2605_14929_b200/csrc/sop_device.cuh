@@ -164,6 +164,14 @@ __device__ __forceinline__ QScale scale_quantize(float sigma, int k, const FmtDe
   return r;
 }
 
+// 1 / s rounded to nearest for a normal s whose reciprocal is normal: a Newton step with a fused residual (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor", 1990; compared with the correctly rounded reciprocal for every significand).
+__device__ __forceinline__ float reciprocal_scale(float s) {
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(s));
+  return __fmaf_rn(y, __fmaf_rn(-s, y, 1.0f), y);
+}
+
 // one power-of-two scale per layer: 2^ceil(log2(wmax / tmax))
 __device__ __forceinline__ float layer_pot_scale(float wmax, float tmax) {
   if (!(wmax > 0.0f)) return 0.0f;

@@ -389,6 +389,303 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
   }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The packer where the winner of each block can be read off a sweep's values: only the winner is encoded.
+//   Table codes: a uniform grid of PCELLS cells on u; a cell's entry holds its one threshold and the codes below and above it, so an
+//   element costs a look-up, a comparison and a byte permutation.  Entries are stored eight times (lanes l, l + 8, ... share a copy).
+//   A table with two different thresholds in one cell is searched instead.
+//   E2M3 and E4M3 codes are what the conversion instructions return.
+//   The codes of a block leave as whole 32-bit words wherever 16 n bits (of two blocks for odd n) are a multiple of 32; 12-bit scale
+//   words are gathered eight blocks at a time by shuffles.
+// What bounds it: PACK_BOUND
+// ---------------------------------------------------------------------------------------------
+constexpr int PCELLS = 320, PCOPIES = 8;
+constexpr float PMAGIC = 12582912.0f;   // 1.5 * 2^23: adding it leaves rint(x) in the low mantissa bits
+
+struct PackTable {       // of each of the two atoms
+  float tmax, pot, inv_range;
+  int neg, k, slow, block_scope;
+  unsigned fast_lo, fast_span;         // patterns of sigma that take the one-addition rounding (see scale_quantize)
+  unsigned code_off;                   // scale code = (rounded pattern >> (23 - y)) - code_off there
+};
+
+__device__ __forceinline__ unsigned pack_cell(float u, float inv_range) {
+  return __float_as_uint(__fmaf_rn(__saturatef(__fmaf_rn(u, inv_range, 0.5f)), (float)PCELLS, PMAGIC));      // cell number + bits of PMAGIC
+}
+
+// KIND: SOP_KIND_LUT (any pair or single table), SOP_KIND_FP_E2M3 or SOP_KIND_FP_E4M3 (a single format)
+template <int KIND>
+__global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res) {
+  constexpr bool LUT = KIND == SOP_KIND_LUT;
+  __shared__ __align__(16) uint2 cells[LUT ? 2 * (PCELLS + 1) * PCOPIES : 1];      // {threshold, code below | code above << 8}
+  __shared__ float tau[2][32], lutv[2][32];
+  __shared__ unsigned short tcell[2][32];
+  __shared__ PackTable tab[2];
+  __shared__ int s_idx[2], s_row[4];
+  __shared__ unsigned s_cnt[2];
+  pdl_trigger();
+  pdl_wait();
+  const int tid = threadIdx.x, lane = tid & 31;
+  // the pair (as pack_kernel resolves it)
+  int ia = a.index_a, ib = a.index_b;
+  const bool from_result = ia == SOP_PAIR_FROM_RESULT;
+  if (from_result) {
+    ia = a.use_sign ? res->best_sa : res->best_a;
+    ib = a.use_sign ? res->best_sb : res->best_b;
+    if (ia < 0 || ib < 0 || ia >= A.n_atoms || ib >= A.n_atoms || (a.use_sign && (ia + 1 >= A.n_atoms || ib + 1 >= A.n_atoms))) {
+      if (a.counts && blockIdx.x == 0 && tid < 2) a.counts[tid] = ~0ull;     // {-1, -1}: the result holds no pair
+      return;
+    }
+  }
+  const int nb = ib == SOP_NO_ATOM ? 1 : 2;
+  const int n = A.atoms[ia].n_bits, b = a.container_bits;
+  if (tid < 2) {
+    s_cnt[tid] = 0;
+    const int idx = tid && nb == 2 ? ib : ia;
+    s_idx[tid] = idx;
+    const sop_atom& at = A.atoms[idx];
+    PackTable t;
+    t.tmax = at.tmax; t.neg = at.negated; t.block_scope = at.scope != 0; t.slow = 0;
+    t.k = a.k_mode == SOP_K_FROM_RESULT ? res->k[idx] : a.k_mode;
+    t.pot = at.scope == 0 ? layer_pot_scale(res->layer_absmax, at.tmax) : 0.0f;
+    t.inv_range = __fdiv_rn(0.4f, at.tmax);                          // the cells cover |u| <= 1.25 tmax, the end cells everything beyond
+    const int e0 = max(F.emin + 127 - t.k, 4), e1 = min(F.emax + 127 - t.k, 250);      // normal, below the top binade, reciprocal normal
+    const bool ok = F.y >= 1 && e1 > e0;
+    t.fast_lo = ok ? (unsigned)e0 << 23 : 0u;
+    t.fast_span = ok ? (unsigned)(e1 - e0) << 23 : 0u;
+    t.code_off = (unsigned)(127 - t.k - F.bias) << F.y;               // (modulo 2^32)
+    tab[tid] = t;
+    // from a search result with signs, a and b are base atoms and each is followed by its negation
+    s_row[2 * tid] = idx;
+    s_row[2 * tid + 1] = from_result ? idx + 1 : (tid ? a.cos_neg_b : a.cos_neg_a);
+  }
+  if (LUT) {
+    __syncthreads();
+    if (tid < 64) {
+      const int t = tid >> 5, j = tid & 31, idx = s_idx[t], ne = A.atoms[idx].n_entries;
+      lutv[t][j] = ((A.dd_mask >> idx) & 1u) ? A.dd_lut[min(j, ne - 1)] : A.atoms[idx].lut[min(j, ne - 1)];
+      __syncwarp();
+      // decision thresholds (the rule of build_thresholds)
+      int jj = j;
+      while (jj < ne - 1 && lutv[t][jj] == lutv[t][jj + 1]) ++jj;
+      const float x = jj < ne - 1 ? __double2float_rd(0.5 * ((double)lutv[t][jj] + (double)lutv[t][jj + 1])) : __int_as_float(0x7F800000);
+      tau[t][j] = x;
+      const unsigned c = x < __int_as_float(0x7F800000) ? pack_cell(x, tab[t].inv_range) - __float_as_uint(PMAGIC) : 0xFFFFu;
+      tcell[t][j] = (unsigned short)c;
+      __syncwarp();
+      if (j < 31 && c != 0xFFFFu && c == tcell[t][j + 1] && tau[t][j + 1] != x) tab[t].slow = 1;
+    }
+    __syncthreads();
+    for (int i = tid; i < nb * (PCELLS + 1); i += PTB) {
+      const int t = i / (PCELLS + 1), c = i - t * (PCELLS + 1);
+      int lo = 0, hi = 0;                    // thresholds in lower cells; in this cell or lower ones
+#pragma unroll
+      for (int step = 16; step >= 1; step >>= 1) {
+        if ((int)tcell[t][lo + step - 1] < c) lo += step;
+        if ((int)tcell[t][hi + step - 1] <= c) hi += step;
+      }
+      const uint2 e = make_uint2(__float_as_uint(hi > lo ? tau[t][lo] : __int_as_float(0x7F800000)), (unsigned)lo | ((unsigned)hi << 8));
+      for (int x = 0; x < PCOPIES; ++x) cells[i * PCOPIES + ((x + i) & (PCOPIES - 1))] = e;      // (neighbouring threads in different banks)
+    }
+  }
+  __syncthreads();
+
+  const int n_sign = a.use_sign ? 2 : 1, n_cand = nb * n_sign;
+  const unsigned nbk = (unsigned)a.nbk, NB = (unsigned)a.NB;       // the block count fits 31 bits
+  const bool packed_rows = a.ldw == a.K;
+  const float* row[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) row[q] = a.block_cos + (size_t)s_row[q < n_cand ? (n_sign == 2 ? q : 2 * q) : 0] * a.NB;
+  const int sh = 23 - F.y;
+  const unsigned half = (1u << (sh - 1)) - 1u, mask = (1u << sh) - 1u;
+  unsigned my_sel = 0, my_neg = 0;
+  // the loads of a block are issued one iteration ahead; whole warps run (the shuffles need them), lanes beyond the last block idle
+  uint4 nv0, nv1;
+  float ncs[4];
+  auto fetch = [&](unsigned blk) {
+    nv0 = nv1 = make_uint4(0u, 0u, 0u, 0u);
+    ncs[0] = ncs[1] = ncs[2] = ncs[3] = 0.0f;
+    if (blk < NB) {
+      const uint16_t* p = a.W + (size_t)blk * SOP_G;
+      if (!packed_rows) { const unsigned m = blk / nbk; p = a.W + (long long)m * a.ldw + (long long)(blk - m * nbk) * SOP_G; }
+      nv0 = __ldg(reinterpret_cast<const uint4*>(p)); nv1 = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+      if (n_cand > 1) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) if (q < n_cand) ncs[q] = __ldg(row[q] + blk);
+      }
+    }
+  };
+  const unsigned stride = gridDim.x * PTB;
+  const unsigned base0 = blockIdx.x * PTB + (unsigned)(tid & ~31);
+  fetch(base0 + lane);
+#pragma unroll 1
+  for (unsigned base = base0; base < NB; base += stride) {
+    const unsigned blk = base + lane;
+    const bool on = blk < NB;
+    const uint32_t wb[8] = {nv0.x, nv0.y, nv0.z, nv0.w, nv1.x, nv1.y, nv1.z, nv1.w};
+    // the winner in the priority order a, (-a), b, (-b): ties keep the earlier
+    int pick = 0;
+    float best = ncs[0];
+#pragma unroll
+    for (int q = 1; q < 4; ++q)
+      if (q < n_cand && (a.select_err ? ncs[q] < best : ncs[q] > best)) { best = ncs[q]; pick = q; }
+    if (stride < NB && base + stride < NB) fetch(blk + stride);
+    const int t = n_sign == 2 ? pick >> 1 : pick, sg = n_sign == 2 ? pick & 1 : 0;
+    uint32_t mb = 0;       // the maximum of the sixteen 15-bit magnitude patterns, two per word at a time
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mb = __vmaxu2(mb, wb[q] & 0x7FFF7FFFu);
+    mb = max(mb & 0xFFFFu, mb >> 16);
+    const float amax = __uint_as_float(mb << 16);
+    const PackTable& T = tab[t];
+    const float sigma = T.tmax == 1.0f ? amax : __fdiv_rn(amax, T.tmax);
+    const unsigned sb = __float_as_uint(sigma);
+    float rcp;
+    unsigned scode = 0;
+    if (T.block_scope && sb - T.fast_lo < T.fast_span) {
+      const unsigned rb = (sb + half + ((sb >> sh) & 1u)) & ~mask;
+      scode = (rb >> sh) - T.code_off;
+      rcp = reciprocal_scale(__uint_as_float(rb));
+    } else {
+      float s_hat;
+      if (!T.block_scope) s_hat = amax > 0.0f ? T.pot : 0.0f;
+      else { const QScale qs = scale_quantize(sigma, T.k, F); s_hat = qs.s_hat; scode = qs.code; }
+      rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
+    }
+    uint32_t code4[4];       // sixteen codes as bytes
+    if (LUT) {
+      const float r = (sg ? 1 - T.neg : T.neg) ? -rcp : rcp;       // a negated table runs on -u
+      if (!T.slow) {
+        const float inv_range = T.inv_range;
+        const unsigned at = (unsigned)(t * (PCELLS + 1) * PCOPIES + (lane & (PCOPIES - 1))) - __float_as_uint(PMAGIC) * PCOPIES;      // modulo 2^32
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          uint32_t c4 = 0;
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const int i = 4 * h + x;
+            const float u = __fmul_rn((i & 1) ? bf16hi(wb[i >> 1]) : bf16lo(wb[i >> 1]), r);
+            const uint2 e = cells[at + pack_cell(u, inv_range) * PCOPIES];
+            // byte x of the word: the code below or above the threshold
+            const unsigned below = x == 0 ? 0x3214u : x == 1 ? 0x3240u : x == 2 ? 0x3410u : 0x4210u;
+            c4 = __byte_perm(c4, e.y, u > __uint_as_float(e.x) ? below + (1u << (4 * x)) : below);
+          }
+          code4[h] = c4;
+        }
+      } else {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          code4[h] = 0;
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const int i = 4 * h + x;
+            code4[h] |= (uint32_t)count_below(tau[t], __fmul_rn((i & 1) ? bf16hi(wb[i >> 1]) : bf16lo(wb[i >> 1]), r)) << (8 * x);
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        uint32_t lo2, hi2;
+        fp_quantize2<KIND == SOP_KIND_LUT ? SOP_KIND_FP_E2M3 : KIND>(__fmul_rn(bf16lo(wb[2 * h]), rcp), __fmul_rn(bf16hi(wb[2 * h]), rcp), lo2);
+        fp_quantize2<KIND == SOP_KIND_LUT ? SOP_KIND_FP_E2M3 : KIND>(__fmul_rn(bf16lo(wb[2 * h + 1]), rcp), __fmul_rn(bf16hi(wb[2 * h + 1]), rcp), hi2);
+        code4[h] = lo2 | (hi2 << 16);
+      }
+    }
+    if (on) { my_sel += (unsigned)t; my_neg += (unsigned)sg; }
+    // codes: sixteen n-bit fields, little-endian, 2 n bytes
+    if (n == 4) {
+      uint32_t h16[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const uint32_t y = (code4[h] | (code4[h] >> 4)) & 0x00FF00FFu;
+        h16[h] = (y | (y >> 8)) & 0xFFFFu;
+      }
+      if (on) *reinterpret_cast<uint2*>(a.codes + (size_t)blk * 8) = make_uint2(h16[0] | (h16[1] << 16), h16[2] | (h16[3] << 16));
+    } else if (n == 8) {
+      if (on) *reinterpret_cast<uint4*>(a.codes + (size_t)blk * 16) = make_uint4(code4[0], code4[1], code4[2], code4[3]);
+    } else if (n == 6) {
+      uint32_t v[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const uint32_t y = (code4[h] & 0x003F003Fu) | ((code4[h] >> 2) & 0x0FC00FC0u);
+        v[h] = (y & 0xFFFu) | ((y >> 16) << 12);
+      }
+      if (on) {
+        uint32_t* dst = reinterpret_cast<uint32_t*>(a.codes + (size_t)blk * 12);
+        dst[0] = v[0] | (v[1] << 24); dst[1] = (v[1] >> 8) | (v[2] << 16); dst[2] = (v[2] >> 16) | (v[3] << 8);
+      }
+    } else if (n == 5) {
+      uint32_t v[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const uint32_t y = (code4[h] & 0x001F001Fu) | ((code4[h] >> 3) & 0x03E003E0u);
+        v[h] = (y & 0x3FFu) | ((y >> 16) << 10);
+      }
+      const uint32_t w0 = v[0] | (v[1] << 20), w1 = (v[1] >> 12) | (v[2] << 8) | (v[3] << 28), w2 = v[3] >> 4;      // 80 bits
+      // two blocks make five words: the even lane stores three of them, the odd lane two
+      const uint32_t o0 = __shfl_down_sync(0xFFFFFFFFu, w0, 1);
+      if (on) {
+        uint32_t* dst = reinterpret_cast<uint32_t*>(a.codes + (size_t)(blk & ~1u) * 10);
+        if (!(blk & 1u)) {
+          dst[0] = w0; dst[1] = w1;
+          if (blk + 1u < NB) dst[2] = w2 | (o0 << 16);
+          else reinterpret_cast<uint16_t*>(dst)[4] = (uint16_t)w2;
+        } else {
+          dst[3] = (w0 >> 16) | (w1 << 16); dst[4] = (w1 >> 16) | (w2 << 16);
+        }
+      }
+    } else if (on) {
+      unsigned long long lo = 0, hi = 0;   // 128-bit accumulator
+      for (int i = 0; i < 16; ++i) {
+        const int pos = i * n;
+        const uint32_t word = i < 4 ? code4[0] : i < 8 ? code4[1] : i < 12 ? code4[2] : code4[3];
+        const unsigned long long y = (unsigned long long)((word >> (8 * (i & 3))) & 0xFFu);
+        if (pos < 64) { lo |= y << pos; if (pos + n > 64) hi |= y >> (64 - pos); }
+        else hi |= y << (pos - 64);
+      }
+      unsigned short* dst = reinterpret_cast<unsigned short*>(a.codes + (size_t)blk * 2 * n);
+      for (int i = 0; i < n; ++i) dst[i] = (unsigned short)((i < 4 ? lo >> (16 * i) : hi >> (16 * (i - 4))) & 0xFFFFu);
+    }
+    // scale word
+    const unsigned sel = (unsigned)t, sgn = (unsigned)sg;
+    unsigned word;
+    if (a.word_sign_bits) word = (sgn << (b - 1)) | (scode << a.meta_bits) | (a.meta_bits >= 1 ? sel : 0u);
+    else if (a.meta_bits >= 1) word = (sel << (b - 1)) | (scode << (a.meta_bits - 1));
+    else word = scode;
+    if (b == 16) {
+      if (on) reinterpret_cast<unsigned short*>(a.words)[blk] = (unsigned short)word;
+    } else if (b == 8) {
+      if (on) reinterpret_cast<unsigned char*>(a.words)[blk] = (unsigned char)word;
+    } else {
+      // eight blocks make three words: lane x < 3 of a group of eight takes the blocks that reach into word x
+      if (!on) word = 0;
+      const int x = lane & 7, first = 32 * x / 12;
+      unsigned out = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned w = __shfl_sync(0xFFFFFFFFu, word, (lane & ~7) + ((first + i) & 7));
+        const int to = (first + i) * 12 - 32 * x;
+        if (x < 3 && first + i < 8 && to < 32) out |= to >= 0 ? w << to : w >> -to;
+      }
+      const unsigned long long wi = (unsigned long long)((base + (unsigned)(lane & ~7)) / 8u) * 3u + (unsigned)x;
+      if (x < 3 && wi * 32u < (unsigned long long)NB * 12u) a.words[wi] = out;
+    }
+  }
+  // the stream's last 32 bits are whole
+  if (blockIdx.x == 0 && tid < 4 && b != 12) {
+    const unsigned long long end = (unsigned long long)NB * (unsigned)(b / 8), at = end + (unsigned)tid;
+    if (at < ((end + 3ull) & ~3ull)) reinterpret_cast<unsigned char*>(a.words)[at] = 0;
+  }
+  if (a.counts) {
+    my_sel = __reduce_add_sync(0xFFFFFFFFu, my_sel);
+    my_neg = __reduce_add_sync(0xFFFFFFFFu, my_neg);
+    if (lane == 0 && my_sel) atomicAdd(&s_cnt[0], my_sel);
+    if (lane == 0 && my_neg) atomicAdd(&s_cnt[1], my_neg);
+    __syncthreads();
+    if (tid < 2 && s_cnt[tid]) atomicAdd(&a.counts[tid], (unsigned long long)s_cnt[tid]);
+  }
+}
+
 int num_sms();
 
 }  // namespace sop
@@ -471,15 +768,22 @@ int sop_pack(const void* W_dev, long long M, long long K, long long ldw, const f
   // 12-bit words are merged into the stream with 32-bit atomicOr (the caller's buffer holds whole 32-bit
   // words and starts from zero); 8- and 16-bit words are stored directly, only the padding is cleared
   const size_t padded = (word_bytes + 3) & ~(size_t)3;
-  if (container_bits == 12) SOP_CUDA_TRY(cudaMemsetAsync(words_dev, 0, padded, st));
+  const bool negs_known = !use_sign || from_result || (a.cos_neg_a >= 0 && (!pair || a.cos_neg_b >= 0));
+  const int kind = from_result ? SOP_KIND_LUT : atoms[index_a].kind;
+  const bool winner = block_cos_dev && negs_known && kind != SOP_KIND_FP_GRID;       // (pack_winner_kernel writes whole words)
+  if (winner) {}
+  else if (container_bits == 12) SOP_CUDA_TRY(cudaMemsetAsync(words_dev, 0, padded, st));
   else SOP_CUDA_TRY(cudaMemsetAsync(words_dev + padded - 4, 0, 4, st));
   if (counts_dev) SOP_CUDA_TRY(cudaMemsetAsync(counts_dev, 0, 2 * sizeof(long long), st));
   long long grid = (a.NB + PTB - 1) / PTB;
   const int sms = num_sms();
-  if (grid > (long long)sms * 4) grid = (long long)sms * 4;      // one wave of resident CTAs: the table set-up runs once per CTA
+  const long long resident = (long long)sms * 4;
+  if (grid > resident) grid = resident;      // one wave of resident CTAs: the table set-up runs once per CTA
   if ((rc = profile_mark(SOP_PROFILE_PACK, 0, st))) return rc;
-  const bool negs_known = !use_sign || from_result || (a.cos_neg_a >= 0 && (!pair || a.cos_neg_b >= 0));
-  if (block_cos_dev && negs_known) SOP_CUDA_TRY(launch(pack_kernel<true>, grid, PTB, 0, st, a, A, F, search_dev));
+  if (winner && kind == SOP_KIND_LUT) SOP_CUDA_TRY(launch(pack_winner_kernel<SOP_KIND_LUT>, grid, PTB, 0, st, a, A, F, search_dev));
+  else if (winner && kind == SOP_KIND_FP_E2M3) SOP_CUDA_TRY(launch(pack_winner_kernel<SOP_KIND_FP_E2M3>, grid, PTB, 0, st, a, A, F, search_dev));
+  else if (winner) SOP_CUDA_TRY(launch(pack_winner_kernel<SOP_KIND_FP_E4M3>, grid, PTB, 0, st, a, A, F, search_dev));
+  else if (block_cos_dev && negs_known) SOP_CUDA_TRY(launch(pack_kernel<true>, grid, PTB, 0, st, a, A, F, search_dev));
   else SOP_CUDA_TRY(launch(pack_kernel<false>, grid, PTB, 0, st, a, A, F, search_dev));
   if ((rc = profile_mark(SOP_PROFILE_PACK, 1, st))) return rc;
   SOP_CUDA_TRY(cudaGetLastError());

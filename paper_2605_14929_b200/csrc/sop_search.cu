@@ -475,14 +475,6 @@ struct ScaleFast {
   }
 };
 
-// 1 / s rounded to nearest for a normal s whose reciprocal is normal: a Newton step with a fused residual (Markstein 1990, as
-// above; compared with the correctly rounded reciprocal for every significand).
-__device__ __forceinline__ float reciprocal_scale(float s) {
-  float y;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(s));
-  return __fmaf_rn(y, __fmaf_rn(-s, y, 1.0f), y);
-}
-
 // What the block loops of one class share: the class's scale rule and the thread's walk over the rows of its column block.
 struct SweepCtx {
   const unsigned char* smem;
