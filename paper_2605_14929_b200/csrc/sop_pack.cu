@@ -3,6 +3,8 @@
 // encoded: 2n bytes of codes plus one b-bit scale word (sign, exponent, mantissa, selector).  Reads W once,
 // writes ~n/8 + b/128 bytes per element; bound by instruction issue (the encode), not by bytes.  Table codes
 // come from a uniform cell grid on u where the table allows it, else from a binary search over the thresholds.
+// pack_winner_kernel serves winners whose cosines or errors a sweep has written (tables, E2M3, E4M3);
+// pack_kernel serves parametric grids and choices that have to be evaluated here.
 #include <string.h>
 
 #include "sop_device.cuh"
@@ -397,7 +399,10 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
 //   E2M3 and E4M3 codes are what the conversion instructions return.
 //   The codes of a block leave as whole 32-bit words wherever 16 n bits (of two blocks for odd n) are a multiple of 32; 12-bit scale
 //   words are gathered eight blocks at a time by shuffles.
-// What bounds it: PACK_BOUND
+// What bounds it: instruction issue (70 to 74 % of the slots) with the shared-memory wavefronts of the grid look-ups (63 %) close behind;
+// 230 MB of DRAM traffic would take 35 us at 8192 x 8192, where it takes 76 us (the general kernel: 95 us).  The whole
+// pass over 14336 x 4096 in E2M3 fell from 288 to 201 us with it, of which 10 us come from code width and candidate count being template
+// parameters.
 // ---------------------------------------------------------------------------------------------
 constexpr int PCELLS = 320, PCOPIES = 8;
 constexpr float PMAGIC = 12582912.0f;   // 1.5 * 2^23: adding it leaves rint(x) in the low mantissa bits
@@ -413,8 +418,9 @@ __device__ __forceinline__ unsigned pack_cell(float u, float inv_range) {
   return __float_as_uint(__fmaf_rn(__saturatef(__fmaf_rn(u, inv_range, 0.5f)), (float)PCELLS, PMAGIC));      // cell number + bits of PMAGIC
 }
 
-// KIND: SOP_KIND_LUT (any pair or single table), SOP_KIND_FP_E2M3 or SOP_KIND_FP_E4M3 (a single format)
-template <int KIND>
+// KIND: SOP_KIND_LUT (any pair or single table), SOP_KIND_FP_E2M3 or SOP_KIND_FP_E4M3 (a single format).  N: bits of a code (0: as the
+// atom says).  NC: candidates of the choice, 1, 2 (a pair, or a table and its negation) or 4.
+template <int KIND, int N, int NC>
 __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res) {
   constexpr bool LUT = KIND == SOP_KIND_LUT;
   __shared__ __align__(16) uint2 cells[LUT ? 2 * (PCELLS + 1) * PCOPIES : 1];      // {threshold, code below | code above << 8}
@@ -438,7 +444,7 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
     }
   }
   const int nb = ib == SOP_NO_ATOM ? 1 : 2;
-  const int n = A.atoms[ia].n_bits, b = a.container_bits;
+  const int n = N ? N : A.atoms[ia].n_bits, b = a.container_bits;
   if (tid < 2) {
     s_cnt[tid] = 0;
     const int idx = tid && nb == 2 ? ib : ia;
@@ -490,28 +496,30 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
   }
   __syncthreads();
 
-  const int n_sign = a.use_sign ? 2 : 1, n_cand = nb * n_sign;
+  const bool signs = NC == 4 || (NC == 2 && a.use_sign);      // the candidates are a table and its negation, once or twice
   const unsigned nbk = (unsigned)a.nbk, NB = (unsigned)a.NB;       // the block count fits 31 bits
   const bool packed_rows = a.ldw == a.K;
-  const float* row[4];
+  const unsigned flip = a.select_err ? 0x80000000u : 0u;      // errors are compared as their negatives
+  const float* row[NC];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) row[q] = a.block_cos + (size_t)s_row[q < n_cand ? (n_sign == 2 ? q : 2 * q) : 0] * a.NB;
+  for (int q = 0; q < NC; ++q) row[q] = a.block_cos + (size_t)s_row[signs ? q : 2 * q] * a.NB;
   const int sh = 23 - F.y;
   const unsigned half = (1u << (sh - 1)) - 1u, mask = (1u << sh) - 1u;
   unsigned my_sel = 0, my_neg = 0;
   // the loads of a block are issued one iteration ahead; whole warps run (the shuffles need them), lanes beyond the last block idle
   uint4 nv0, nv1;
-  float ncs[4];
+  float ncs[NC];
   auto fetch = [&](unsigned blk) {
     nv0 = nv1 = make_uint4(0u, 0u, 0u, 0u);
-    ncs[0] = ncs[1] = ncs[2] = ncs[3] = 0.0f;
+#pragma unroll
+    for (int q = 0; q < NC; ++q) ncs[q] = 0.0f;
     if (blk < NB) {
       const uint16_t* p = a.W + (size_t)blk * SOP_G;
       if (!packed_rows) { const unsigned m = blk / nbk; p = a.W + (long long)m * a.ldw + (long long)(blk - m * nbk) * SOP_G; }
       nv0 = __ldg(reinterpret_cast<const uint4*>(p)); nv1 = __ldg(reinterpret_cast<const uint4*>(p) + 1);
-      if (n_cand > 1) {
+      if (NC > 1) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) if (q < n_cand) ncs[q] = __ldg(row[q] + blk);
+        for (int q = 0; q < NC; ++q) ncs[q] = __uint_as_float(__float_as_uint(__ldg(row[q] + blk)) ^ flip);
       }
     }
   };
@@ -527,10 +535,10 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
     int pick = 0;
     float best = ncs[0];
 #pragma unroll
-    for (int q = 1; q < 4; ++q)
-      if (q < n_cand && (a.select_err ? ncs[q] < best : ncs[q] > best)) { best = ncs[q]; pick = q; }
-    if (stride < NB && base + stride < NB) fetch(blk + stride);
-    const int t = n_sign == 2 ? pick >> 1 : pick, sg = n_sign == 2 ? pick & 1 : 0;
+    for (int q = 1; q < NC; ++q)
+      if (ncs[q] > best) { best = ncs[q]; pick = q; }
+    if (stride < NB - base) fetch(blk + stride);
+    const int t = NC == 1 ? 0 : signs ? pick >> 1 : pick, sg = NC > 1 && signs ? pick & 1 : 0;
     uint32_t mb = 0;       // the maximum of the sixteen 15-bit magnitude patterns, two per word at a time
 #pragma unroll
     for (int q = 0; q < 8; ++q) mb = __vmaxu2(mb, wb[q] & 0x7FFF7FFFu);
@@ -780,9 +788,16 @@ int sop_pack(const void* W_dev, long long M, long long K, long long ldw, const f
   const long long resident = (long long)sms * 4;
   if (grid > resident) grid = resident;      // one wave of resident CTAs: the table set-up runs once per CTA
   if ((rc = profile_mark(SOP_PROFILE_PACK, 0, st))) return rc;
-  if (winner && kind == SOP_KIND_LUT) SOP_CUDA_TRY(launch(pack_winner_kernel<SOP_KIND_LUT>, grid, PTB, 0, st, a, A, F, search_dev));
-  else if (winner && kind == SOP_KIND_FP_E2M3) SOP_CUDA_TRY(launch(pack_winner_kernel<SOP_KIND_FP_E2M3>, grid, PTB, 0, st, a, A, F, search_dev));
-  else if (winner) SOP_CUDA_TRY(launch(pack_winner_kernel<SOP_KIND_FP_E4M3>, grid, PTB, 0, st, a, A, F, search_dev));
+#define SOP_PACK(KD, NN, C) SOP_CUDA_TRY(launch(pack_winner_kernel<KD, NN, C>, grid, PTB, 0, st, a, A, F, search_dev))
+#define SOP_PACK_LUT(NN) do { if (n_cand == 4) SOP_PACK(SOP_KIND_LUT, NN, 4); else if (n_cand == 2) SOP_PACK(SOP_KIND_LUT, NN, 2); else SOP_PACK(SOP_KIND_LUT, NN, 1); } while (0)
+  const int n_cand = (pair ? 2 : 1) * (use_sign ? 2 : 1);
+  if (winner && kind == SOP_KIND_FP_E2M3) SOP_PACK(SOP_KIND_FP_E2M3, 6, 1);
+  else if (winner && kind == SOP_KIND_FP_E4M3) SOP_PACK(SOP_KIND_FP_E4M3, 8, 1);
+  else if (winner && n_bits == 4) SOP_PACK_LUT(4);
+  else if (winner && n_bits == 5) SOP_PACK_LUT(5);
+  else if (winner) SOP_PACK_LUT(0);
+#undef SOP_PACK_LUT
+#undef SOP_PACK
   else if (block_cos_dev && negs_known) SOP_CUDA_TRY(launch(pack_kernel<true>, grid, PTB, 0, st, a, A, F, search_dev));
   else SOP_CUDA_TRY(launch(pack_kernel<false>, grid, PTB, 0, st, a, A, F, search_dev));
   if ((rc = profile_mark(SOP_PROFILE_PACK, 1, st))) return rc;
