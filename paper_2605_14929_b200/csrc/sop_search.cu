@@ -140,42 +140,125 @@ __device__ __forceinline__ float absmax_bits(const uint32_t (&v)[8]) {
 
 __device__ void kselect_body(const Plan& P, const FmtDev& F, const unsigned* hist, WsHeader* hdr);
 
-__global__ void __launch_bounds__(256) prepass_kernel(LayerArgs L, Plan P, FmtDev F, unsigned* __restrict__ hist, WsHeader* __restrict__ hdr) {
+// exponent of sigma = a / tmax (the division rounded as the sweep rounds it), for a > 0; below every bin when sigma is zero
+__device__ __forceinline__ int sigma_exponent(float a, float tmax) {
+  const float sigma = tmax == 1.0f ? a : __fdiv_rn(a, tmax);
+  return sigma > 0.0f ? ilogb_pos(sigma) : -1000;
+}
+
+// The exponent of a block's sigma in a class depends on the seven mantissa bits of the block maximum only through one cut
+// point: from some mantissa on the quotient reaches the next power of two.  So a block is counted once, by its exponent
+// and by the region between the classes' cut points that its mantissa lies in; the CTA's counts are spread to the classes
+// at the end.  Where a quotient may leave the normal range the classes are counted one by one.
+// A thread stays in its block column and steps down the rows (`rows` whole rows are covered by the grid's threads), four
+// blocks in flight.
+// What bounds it: DRAM on a large layer (28672 x 8192: 73 us, 470 MB; 106 us with a block per thread in storage order, a division and a
+// shared-memory addition per class and block, and max|W| added up by every warp), latency on a small one.
+constexpr int PPB = 256;                 // threads per CTA
+constexpr int PP_FLY = 4;                // blocks in flight per thread
+__global__ void __launch_bounds__(PPB) prepass_kernel(LayerArgs L, Plan P, FmtDev F, unsigned* __restrict__ hist, WsHeader* __restrict__ hdr, unsigned rows) {
   pdl_trigger();
-  pdl_wait();
-  __shared__ unsigned sh[SOP_MAX_CLASSES * SOP_HIST_BINS];
-  for (int i = threadIdx.x; i < P.n_classes * SOP_HIST_BINS; i += blockDim.x) sh[i] = 0;
+  __shared__ unsigned s_cnt[(SOP_MAX_CLASSES + 1) * 256];      // [region][exponent]
+  __shared__ unsigned s_mark[4];                               // mantissas that are a cut point
+  __shared__ int s_cut[SOP_MAX_CLASSES], s_e0[SOP_MAX_CLASSES];
+  __shared__ unsigned short s_reg[128];                        // 256 x region of a mantissa
+  __shared__ unsigned s_wmax;
+  __shared__ int s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < (SOP_MAX_CLASSES + 1) * 256; i += PPB) s_cnt[i] = 0;
+  if (tid < SOP_MAX_CLASSES) s_cut[tid] = 128;
+  if (tid == 0) s_wmax = 0;
   __syncthreads();
-  uint32_t wmax = 0;
-  const unsigned nbk32 = (unsigned)L.nbk, NB32 = (unsigned)L.NB;         // the block count fits 31 bits
-  for (unsigned b = blockIdx.x * blockDim.x + threadIdx.x; b < NB32; b += gridDim.x * blockDim.x) {
-    const unsigned m = b / nbk32, j = b - m * nbk32;
-    uint32_t v[8];
-    load_block_bits(L.W + (long long)m * L.ldw + (long long)j * SOP_G, v);
-    const float a = absmax_bits(v);
-    wmax = max(wmax, __float_as_uint(a));
-    if (a > 0.0f) {
-      for (int cl = 0; cl < P.n_classes; ++cl) {
-        if (!P.cls[cl].auto_k) continue;
-        const float sigma = P.cls[cl].tmax == 1.0f ? a : __fdiv_rn(a, P.cls[cl].tmax);
-        if (sigma > 0.0f) atomicAdd(&sh[cl * SOP_HIST_BINS + ilogb_pos(sigma) + SOP_HIST_OFF], 1u);
+  bool cut = false;
+  int e_lo = 1, e_hi = 254;              // exponent fields for which every quotient is a normal number
+  for (int cl = 0; cl < P.n_classes; ++cl) {
+    if (!P.cls[cl].auto_k) continue;
+    const float tmax = P.cls[cl].tmax;
+    const int e0 = sigma_exponent(1.0f, tmax);
+    e_lo = max(e_lo, 1 - e0);
+    e_hi = tmax >= 1e-30f && tmax <= 1e30f ? min(e_hi, 253 - e0) : 0;
+    if (tid < 128 && tmax != 1.0f) {
+      const int here = sigma_exponent(__uint_as_float((127u << 23) | ((unsigned)tid << 16)), tmax);
+      const int below = tid ? sigma_exponent(__uint_as_float((127u << 23) | ((unsigned)(tid - 1) << 16)), tmax) : e0;
+      if (here != below) { s_cut[cl] = tid; cut = true; }
+    }
+    if (tid == 0) s_e0[cl] = e0;
+  }
+  const unsigned marks = __ballot_sync(0xFFFFFFFFu, cut);
+  if (warp < 4 && lane == 0) s_mark[warp] = marks;
+  __syncthreads();
+  int n_cuts = 0;
+#pragma unroll
+  for (int w = 0; w < 4; ++w) n_cuts += __popc(s_mark[w]);
+  if (tid < 128) {
+    int r = __popc(s_mark[warp] & (0xFFFFFFFFu >> (31 - lane)));
+    for (int w = 0; w < warp; ++w) r += __popc(s_mark[w]);
+    s_reg[tid] = (unsigned short)(256 * r);
+  }
+  __syncthreads();
+  pdl_wait();
+  const unsigned nbk = (unsigned)L.nbk, S = rows * nbk, t = blockIdx.x * PPB + tid;
+  unsigned wmax = 0;                     // 15-bit patterns
+  if (t < S) {
+    const unsigned m0 = t / nbk, j = t - m0 * nbk;
+    const uint16_t* p = L.W + (long long)m0 * L.ldw + (long long)j * SOP_G;
+    const long long step = (long long)rows * L.ldw;
+    unsigned left = ((unsigned)L.M - m0 + rows - 1) / rows;      // blocks of this thread
+    while (left) {
+      uint4 v[PP_FLY][2];
+#pragma unroll
+      for (int q = 0; q < PP_FLY; ++q)
+        if (q < (int)left) {
+          v[q][0] = __ldg(reinterpret_cast<const uint4*>(p + q * step));
+          v[q][1] = __ldg(reinterpret_cast<const uint4*>(p + q * step) + 1);
+        } else {
+          v[q][0] = v[q][1] = make_uint4(0u, 0u, 0u, 0u);
+        }
+      p += PP_FLY * step;
+      left -= min(left, (unsigned)PP_FLY);
+#pragma unroll
+      for (int q = 0; q < PP_FLY; ++q) {
+        const uint32_t wb[8] = {v[q][0].x, v[q][0].y, v[q][0].z, v[q][0].w, v[q][1].x, v[q][1].y, v[q][1].z, v[q][1].w};
+        const unsigned pat = __float_as_uint(absmax_bits(wb)) >> 16;
+        wmax = max(wmax, pat);
+        if (pat) {
+          const int e = (int)(pat >> 7);
+          if (e >= e_lo && e <= e_hi) {
+            atomicAdd(&s_cnt[(n_cuts ? s_reg[pat & 127u] : 0) + e], 1u);
+          } else {
+            for (int cl = 0; cl < P.n_classes; ++cl) {
+              if (!P.cls[cl].auto_k) continue;
+              const int x = sigma_exponent(__uint_as_float(pat << 16), P.cls[cl].tmax);
+              if (x > -1000) atomicAdd(&hist[cl * SOP_HIST_BINS + x + SOP_HIST_OFF], 1u);
+            }
+          }
+        }
       }
     }
   }
-  for (int o = 16; o; o >>= 1) wmax = max(wmax, __shfl_xor_sync(0xFFFFFFFFu, wmax, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(&hdr->wmax_bits, wmax);
+  wmax = __reduce_max_sync(0xFFFFFFFFu, wmax);
+  if (lane == 0 && wmax) atomicMax(&s_wmax, wmax);
   __syncthreads();
-  for (int i = threadIdx.x; i < P.n_classes * SOP_HIST_BINS; i += blockDim.x)
-    if (sh[i]) atomicAdd(&hist[i], sh[i]);
+  for (int i = tid; i < (n_cuts + 1) * 256; i += PPB) {
+    const unsigned n = s_cnt[i];
+    if (!n) continue;
+    int first = 0;                       // first mantissa of the region: all of a region's mantissas compare alike with every cut
+    for (int r = i >> 8, w = 0; r; ++w) {
+      unsigned mk = s_mark[w];
+      while (mk && r) { first = 32 * w + __ffs((int)mk) - 1; mk &= mk - 1u; --r; }
+    }
+    for (int cl = 0; cl < P.n_classes; ++cl)
+      if (P.cls[cl].auto_k) atomicAdd(&hist[cl * SOP_HIST_BINS + (i & 255) - 127 + s_e0[cl] + (first >= s_cut[cl] ? 1 : 0) + SOP_HIST_OFF], n);
+  }
+  if (tid == 0 && s_wmax) atomicMax(&hdr->wmax_bits, s_wmax << 16);
   // the CTA that arrives last turns the histogram into shifts; nobody waits for anybody
-  __shared__ int s_last;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&hdr->done_prepass, 1u) == gridDim.x - 1 ? 1 : 0;
+  if (tid == 0) s_last = atomicAdd(&hdr->done_prepass, 1u) == gridDim.x - 1 ? 1 : 0;
   __syncthreads();
   if (s_last) {
     __threadfence();
-    if (threadIdx.x == 0) hist[SOP_MAX_CLASSES * SOP_HIST_BINS] = __ldcg(&hdr->wmax_bits);    // kept for later calls on this layer
+    if (tid == 0) hist[SOP_MAX_CLASSES * SOP_HIST_BINS] = __ldcg(&hdr->wmax_bits);    // kept for later calls on this layer
     kselect_body(P, F, hist, hdr);
   }
 }
@@ -190,66 +273,56 @@ __global__ void __launch_bounds__(256) kselect_kernel(Plan P, FmtDev F, const un
   kselect_body(P, F, hist, hdr);
 }
 
-// One CTA of 256 threads.  Reads the global histogram and max|W| through the L2 (they were written by
-// other CTAs' atomics).  Per class: prefix sums of the 320 bins, the count of every shift k in
-// [-64, 64] as a difference of two prefix values, then the largest count with ties to the smallest |k|
-// and then to k > 0 (preference order 0, +1, -1, +2, -2, ...).
+// One CTA of 256 threads, a warp per class.  Reads the global histogram and max|W| through the L2 (they were written by
+// other CTAs' atomics).  Prefix sums of the 320 bins, the count of every shift k in [-64, 64] as a difference of two
+// prefix values, then the largest count with ties to the smallest |k| and then to k > 0 (preference order 0, +1, -1,
+// +2, -2, ...).  (One class after the other with the whole CTA took 1.5 us per class.)
 __device__ void kselect_body(const Plan& P, const FmtDev& F, const unsigned* hist, WsHeader* hdr) {
-  __shared__ unsigned long long pre[SOP_HIST_BINS + 1];
-  __shared__ unsigned long long red_c[8];
-  __shared__ int red_o[8];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float wmax = __uint_as_float(__ldcg(&hdr->wmax_bits));
-  for (int cl = 0; cl < P.n_classes; ++cl) {
-    int kstar = P.k_mode == SOP_K_AUTO ? 0 : P.k_mode;
-    if (P.cls[cl].scope == 0) kstar = 0;
-    if (P.cls[cl].auto_k) {
-      // inclusive prefix of the bins: two bins per thread (320 <= 512), warp scan, warp totals
-      unsigned long long v0 = 0, v1 = 0;
-      if (2 * tid < SOP_HIST_BINS) v0 = __ldcg(&hist[cl * SOP_HIST_BINS + 2 * tid]);
-      if (2 * tid + 1 < SOP_HIST_BINS) v1 = __ldcg(&hist[cl * SOP_HIST_BINS + 2 * tid + 1]);
-      unsigned long long incl = v0 + v1;
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      __syncthreads();
-      if (lane == 31) red_c[warp] = incl;
-      __syncthreads();
-      unsigned long long base = 0;
-      for (int w = 0; w < warp; ++w) base += red_c[w];
-      if (tid == 0) pre[0] = 0;
-      if (2 * tid < SOP_HIST_BINS) pre[2 * tid + 1] = base + incl - v1;
-      if (2 * tid + 1 < SOP_HIST_BINS) pre[2 * tid + 2] = base + incl;
-      __syncthreads();
-      // shift k = tid - 64 keeps the exponents e with emin <= e + k <= emax; bin of e is e + SOP_HIST_OFF
-      unsigned long long c = 0;
-      int order = 1 << 30;
-      if (tid < 129) {
-        const int k = tid - 64;
-        const int lo = max(F.emin - k + SOP_HIST_OFF, 0), hi = min(F.emax - k + SOP_HIST_OFF, SOP_HIST_BINS - 1);
-        c = hi >= lo ? pre[hi + 1] - pre[lo] : 0ull;
-        order = k == 0 ? 0 : (k > 0 ? 2 * k - 1 : -2 * k);
-      }
-      for (int o = 16; o; o >>= 1) {
-        const unsigned long long oc = __shfl_xor_sync(0xFFFFFFFFu, c, o);
-        const int oo = __shfl_xor_sync(0xFFFFFFFFu, order, o);
-        if (oc > c || (oc == c && oo < order)) { c = oc; order = oo; }
-      }
-      __syncthreads();
-      if (lane == 0) { red_c[warp] = c; red_o[warp] = order; }
-      __syncthreads();
-      if (tid == 0) {
-        for (int w = 1; w < 8; ++w)
-          if (red_c[w] > c || (red_c[w] == c && red_o[w] < order)) { c = red_c[w]; order = red_o[w]; }
-        kstar = order == 0 ? 0 : ((order & 1) ? (order + 1) / 2 : -(order / 2));
-      }
-      __syncthreads();
+  static_assert(SOP_MAX_CLASSES <= 8, "a warp per class");
+  constexpr int PER = SOP_HIST_BINS / 32;
+  static_assert(SOP_HIST_BINS % 32 == 0, "whole bins per lane");
+  __shared__ unsigned pre[SOP_MAX_CLASSES][SOP_HIST_BINS + 1];      // (at most one count per block: 31 bits)
+  const int lane = threadIdx.x & 31, cl = threadIdx.x >> 5;
+  if (cl >= P.n_classes) return;
+  int kstar = P.k_mode == SOP_K_AUTO ? 0 : P.k_mode;
+  if (P.cls[cl].scope == 0) kstar = 0;
+  if (P.cls[cl].auto_k) {
+    unsigned v[PER], local = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) v[i] = __ldcg(&hist[cl * SOP_HIST_BINS + PER * lane + i]);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) local += v[i];
+    unsigned incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += t;
     }
-    if (tid == 0) {
-      hdr->cls_k[cl] = kstar;
-      hdr->cls_pot[cl] = P.cls[cl].scope == 0 ? layer_pot_scale(wmax, P.cls[cl].tmax) : 0.0f;
+    unsigned run = incl - local;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) { pre[cl][PER * lane + i] = run; run += v[i]; }
+    if (lane == 31) pre[cl][SOP_HIST_BINS] = run;
+    __syncwarp();
+    // shift k keeps the exponents e with emin <= e + k <= emax; bin of e is e + SOP_HIST_OFF
+    unsigned best = 0;
+    int order = 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const int o = 32 * i + lane;                           // preference order of the shift
+      if (o >= 129) break;
+      const int k = (o & 1) ? (o + 1) / 2 : -(o / 2);
+      const int lo = max(F.emin - k + SOP_HIST_OFF, 0), hi = min(F.emax - k + SOP_HIST_OFF, SOP_HIST_BINS - 1);
+      const unsigned c = hi >= lo ? pre[cl][hi + 1] - pre[cl][lo] : 0u;
+      if (i == 0 || c > best) { best = c; order = o; }
     }
+    const unsigned top = __reduce_max_sync(0xFFFFFFFFu, best);
+    order = (int)__reduce_min_sync(0xFFFFFFFFu, best == top ? (unsigned)order : 0xFFFFu);
+    kstar = (order & 1) ? (order + 1) / 2 : -(order / 2);
+  }
+  if (lane == 0) {
+    const float wmax = __uint_as_float(__ldcg(&hdr->wmax_bits));
+    hdr->cls_k[cl] = kstar;
+    hdr->cls_pot[cl] = P.cls[cl].scope == 0 ? layer_pot_scale(wmax, P.cls[cl].tmax) : 0.0f;
   }
 }
 
@@ -1667,9 +1740,11 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
     SOP_CUDA_TRY(cudaGetLastError());
   } else if (!k_from_result) {
     // one read of W: block scales' exponent histogram, max|W|, then the shifts (last CTA)
-    long long want = (L.NB + 255) / 256;
-    const int pgrid = (int)(want < (long long)sms * 8 ? want : (long long)sms * 8);
-    SOP_CUDA_TRY(launch(prepass_kernel, pgrid, 256, 0, st, L, P, F, hist, hdr));
+    // (as many whole rows as four CTAs per SM have threads for)
+    const long long fit = (long long)sms * 4 * PPB / L.nbk;
+    const unsigned prows = (unsigned)(fit < 1 ? 1 : fit < M ? fit : M);
+    const int pgrid = (int)((prows * L.nbk + PPB - 1) / PPB);
+    SOP_CUDA_TRY(launch(prepass_kernel, pgrid, PPB, 0, st, L, P, F, hist, hdr, prows));
     SOP_CUDA_TRY(cudaGetLastError());
   }
   if ((rc = profile_mark(SOP_PROFILE_PREPASS, 1, st))) return rc;
