@@ -75,9 +75,19 @@ def lib():
         if not os.path.exists(_build.LIB):
             raise ImportError(f"{_build.LIB} is missing: run `python -m paper_2605_14929_b200.build` "
                               "(nvcc, sm_100a).  There is no CPU fallback.")
-        _lib = C.CDLL(_build.LIB)
-        _lib.sop_strerror.restype = C.c_char_p
-        _lib.sop_last_cuda_error.restype = C.c_char_p
+        loaded = C.CDLL(_build.LIB)
+        loaded.sop_strerror.restype = C.c_char_p
+        loaded.sop_last_cuda_error.restype = C.c_char_p
+        # declared argument types: plain Python integers are converted in C, without an object per argument (a small
+        # layer's pass is bound by the host: 48 us of calls)
+        P, LL, I, U, Z = C.c_void_p, C.c_longlong, C.c_int, C.c_uint, C.c_size_t
+        loaded.sop_channel_norms.argtypes = [P, LL, LL, LL, P, P, Z, P]
+        loaded.sop_pair_search.argtypes = [P, LL, LL, LL, P, I, P, I, P, I, P, U, U, U, I, P, P, P, P, P, P, P, Z, P]
+        loaded.sop_dd4_lloyd.argtypes = [P, LL, LL, LL, P, I, P, I, P, P, LL, C.c_float, I, P, I, I, I, P, P, P, P, Z, P]
+        loaded.sop_pack.argtypes = [P, LL, LL, LL, P, I, P, P, I, P, U, I, I, I, P, I, I, I, P, P, P, P, I, P]
+        loaded.sop_opq_extract.argtypes = [P, LL, LL, LL, I, C.c_double, P, LL, P, P, LL, P, P, Z, P]
+        loaded.sop_wr_extract.argtypes = [P, LL, LL, LL, P, I, P, P, I, P, U, I, I, I, P, I, I, I, P, P, LL, P, P, LL, P, P, P, P, Z, P]
+        _lib = loaded
     return _lib
 
 
@@ -120,14 +130,12 @@ def make_atoms(atoms) -> C.Array:
     return arr
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return C.c_void_p(0 if t is None else t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> int:
+    return 0 if t is None else t.data_ptr()
 
 
-def _stream(stream) -> C.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+def _stream(stream) -> int:
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
 
 def _ll(v) -> C.c_longlong:
@@ -187,8 +195,8 @@ def sop_channel_norms(X: torch.Tensor, c_out: torch.Tensor, workspace: torch.Ten
     assert X.is_cuda and X.dtype == torch.float32 and X.dim() == 2 and X.stride(1) == 1
     assert c_out.is_cuda and c_out.dtype == torch.float32 and c_out.is_contiguous()
     T, K = X.shape
-    _check(lib().sop_channel_norms(_ptr(X), _ll(T), _ll(K), _ll(X.stride(0)), _ptr(c_out), _ptr(workspace),
-                                   C.c_size_t(workspace.numel()), _stream(stream)), "sop_channel_norms")
+    _check(lib().sop_channel_norms(_ptr(X), T, K, X.stride(0), _ptr(c_out), _ptr(workspace),
+                                   workspace.numel(), _stream(stream)), "sop_channel_norms")
 
 
 NORMS_STATIC_DOUBLES = 1 << 19
@@ -201,7 +209,7 @@ def sop_channel_norms_static(X: torch.Tensor, c_out: torch.Tensor, stream=None) 
     assert X.is_cuda and X.dtype == torch.float32 and X.dim() == 2 and X.stride(1) == 1
     assert c_out.is_cuda and c_out.dtype == torch.float32 and c_out.is_contiguous()
     T, K = X.shape
-    _check(lib().sop_channel_norms_static(_ptr(X), _ll(T), _ll(K), _ll(X.stride(0)), _ptr(c_out), _stream(stream)),
+    _check(lib().sop_channel_norms_static(C.c_void_p(_ptr(X)), _ll(T), _ll(K), _ll(X.stride(0)), C.c_void_p(_ptr(c_out)), C.c_void_p(_stream(stream))),
            "sop_channel_norms_static")
 
 
@@ -216,15 +224,15 @@ def sop_pair_search(W: torch.Tensor, c: torch.Tensor, fmt, atoms: Sequence, pair
     into ``pair_table`` / ``signed_table``; only the entries with a newly evaluated candidate are formed."""
     assert W.is_cuda and W.dtype == torch.bfloat16 and W.dim() == 2 and W.stride(1) == 1
     M, K = W.shape
-    _check(lib().sop_pair_search(_ptr(W), _ll(M), _ll(K), _ll(W.stride(0)), _ptr(c), g, C.byref(make_fmt(fmt)), k_mode,
-                                 make_atoms(atoms), len(atoms), _ptr(dd_lut), C.c_uint(dd_mask), C.c_uint(eval_mask),
-                                 C.c_uint(load_mask),
+    _check(lib().sop_pair_search(_ptr(W), M, K, W.stride(0), _ptr(c), g, C.byref(make_fmt(fmt)), k_mode,
+                                 make_atoms(atoms), len(atoms), _ptr(dd_lut), dd_mask, eval_mask,
+                                 load_mask,
                                  (SEARCH_SINGLES_ONLY if singles_only else 0) | (SEARCH_SELECT_MSE if select_mse else 0)
                                  | (SEARCH_KEEP_LOADED_ENTRIES if keep_loaded else 0) | (SEARCH_REUSE_PREPASS if reuse_prepass else 0),
                                  _ptr(prev_result),
                                  _ptr(pair_table),
                                  _ptr(signed_table), _ptr(result), _ptr(block_cos), _ptr(block_sse), _ptr(workspace),
-                                 C.c_size_t(workspace.numel()), _stream(stream)), "sop_pair_search")
+                                 workspace.numel(), _stream(stream)), "sop_pair_search")
 
 
 def sop_dd4_lloyd(W: torch.Tensor, c: torch.Tensor, fmt, atoms: Sequence, block_cos: torch.Tensor, pool_rank: int,
@@ -238,15 +246,15 @@ def sop_dd4_lloyd(W: torch.Tensor, c: torch.Tensor, fmt, atoms: Sequence, block_
     by dynamic programming instead of Lloyd iterations; ``distortion[0]`` is then its least total cost."""
     assert W.is_cuda and W.dtype == torch.bfloat16 and W.dim() == 2 and W.stride(1) == 1
     M, K = W.shape
-    _check(lib().sop_dd4_lloyd(_ptr(W), _ll(M), _ll(K), _ll(W.stride(0)), _ptr(c), g, C.byref(make_fmt(fmt)), k_mode,
-                               _ptr(search_result), _ptr(block_cos), _ll(pool_rank),
-                               C.c_float(0.0 if pool_threshold is None else pool_threshold),
+    _check(lib().sop_dd4_lloyd(_ptr(W), M, K, W.stride(0), _ptr(c), g, C.byref(make_fmt(fmt)), k_mode,
+                               _ptr(search_result), _ptr(block_cos), int(pool_rank),
+                               0.0 if pool_threshold is None else pool_threshold,
                                (LLOYD_POOL_BY_ERROR if pool_by_error else 0) | (LLOYD_UNIFORM_WEIGHTS if uniform_weights else 0)
                                | (LLOYD_POOL_THRESHOLD if pool_threshold is not None else 0)
                                | (LLOYD_LAUNCH_PER_ITERATION if launch_per_iteration else 0) | (LLOYD_GRID_DP if grid_dp else 0),
                                make_atoms(atoms), len(atoms),
                                fmta_index, iters, _ptr(out_lut), _ptr(distortion), _ptr(pool_count), _ptr(workspace),
-                               C.c_size_t(workspace.numel()), _stream(stream)), "sop_dd4_lloyd")
+                               workspace.numel(), _stream(stream)), "sop_dd4_lloyd")
 
 
 def sop_pack(W: torch.Tensor, c: torch.Tensor, fmt, atoms: Sequence, codes: torch.Tensor, words: torch.Tensor,
@@ -258,8 +266,8 @@ def sop_pack(W: torch.Tensor, c: torch.Tensor, fmt, atoms: Sequence, codes: torc
     """``block_cos``: per-block cosines of a sweep, or with ``select_mse`` its per-block errors."""
     assert W.is_cuda and W.dtype == torch.bfloat16 and W.dim() == 2 and W.stride(1) == 1
     M, K = W.shape
-    _check(lib().sop_pack(_ptr(W), _ll(M), _ll(K), _ll(W.stride(0)), _ptr(c), g, C.byref(make_fmt(fmt)),
-                          make_atoms(atoms), len(atoms), _ptr(dd_lut), C.c_uint(dd_mask), index_a, index_b, k_mode,
+    _check(lib().sop_pack(_ptr(W), M, K, W.stride(0), _ptr(c), g, C.byref(make_fmt(fmt)),
+                          make_atoms(atoms), len(atoms), _ptr(dd_lut), dd_mask, index_a, index_b, k_mode,
                           _ptr(search_result), use_sign, container_bits, word_sign_bits, _ptr(codes), _ptr(words),
                           _ptr(counts), _ptr(block_cos), PACK_SELECT_MSE if select_mse else 0, _stream(stream)), "sop_pack")
 
@@ -283,9 +291,9 @@ def sop_opq_extract(W: torch.Tensor, m: float, W_out: torch.Tensor, row_start: t
     ``count``: one int64."""
     assert W.is_cuda and W.dtype == torch.bfloat16 and W.dim() == 2 and W.stride(1) == 1 and W_out.stride(1) == 1
     M, K = W.shape
-    _check(lib().sop_opq_extract(_ptr(W), _ll(M), _ll(K), _ll(W.stride(0)), g, C.c_double(m), _ptr(W_out), _ll(W_out.stride(0)),
-                                 _ptr(row_start), _ptr(records), _ll(0 if records is None else records.numel()), _ptr(count),
-                                 _ptr(workspace), C.c_size_t(workspace.numel()), _stream(stream)), "sop_opq_extract")
+    _check(lib().sop_opq_extract(_ptr(W), M, K, W.stride(0), g, m, _ptr(W_out), W_out.stride(0),
+                                 _ptr(row_start), _ptr(records), 0 if records is None else records.numel(), _ptr(count),
+                                 _ptr(workspace), workspace.numel(), _stream(stream)), "sop_opq_extract")
 
 
 def wr_workspace(M: int, K: int, device) -> torch.Tensor:
@@ -303,11 +311,11 @@ def sop_wr_extract(W: torch.Tensor, c: torch.Tensor, fmt, atoms: Sequence, codes
     """The arguments from ``fmt`` to ``word_sign_bits`` are those given to ``sop_pack`` for this layer."""
     assert W.is_cuda and W.dtype == torch.bfloat16 and W.dim() == 2 and W.stride(1) == 1
     M, K = W.shape
-    _check(lib().sop_wr_extract(_ptr(W), _ll(M), _ll(K), _ll(W.stride(0)), _ptr(c), g, C.byref(make_fmt(fmt)), make_atoms(atoms),
-                                len(atoms), _ptr(dd_lut), C.c_uint(dd_mask), index_a, index_b, k_mode, _ptr(search_result), use_sign,
-                                container_bits, word_sign_bits, _ptr(codes), _ptr(words), _ll(n_keep), _ptr(row_start),
-                                _ptr(records), _ll(0 if records is None else records.numel()), _ptr(count), _ptr(scale_exp),
-                                _ptr(tau), _ptr(workspace), C.c_size_t(workspace.numel()), _stream(stream)), "sop_wr_extract")
+    _check(lib().sop_wr_extract(_ptr(W), M, K, W.stride(0), _ptr(c), g, C.byref(make_fmt(fmt)), make_atoms(atoms),
+                                len(atoms), _ptr(dd_lut), dd_mask, index_a, index_b, k_mode, _ptr(search_result), use_sign,
+                                container_bits, word_sign_bits, _ptr(codes), _ptr(words), int(n_keep), _ptr(row_start),
+                                _ptr(records), 0 if records is None else records.numel(), _ptr(count), _ptr(scale_exp),
+                                _ptr(tau), _ptr(workspace), workspace.numel(), _stream(stream)), "sop_wr_extract")
 
 
 def pair_search_tuning(reduce_tile_pairs: bool = True) -> None:
