@@ -58,13 +58,14 @@ struct LloydWs {
   // radix select state
   unsigned hist[3][2048];
   // iteration state
-  unsigned long long accN[SOP_MAX_LLOYD_ITERS + 1][SOP_MAX_ENTRIES];
-  long long accS[SOP_MAX_LLOYD_ITERS + 1][SOP_MAX_ENTRIES];
+  // per entry: sum fix(omega); sum of the low words of the CTAs' sums fix(omega u); of their high words.  Each with the number of
+  // CTAs that have added theirs in its top byte (persistent iterations)
+  unsigned long long acc[SOP_MAX_LLOYD_ITERS + 1][3][SOP_MAX_ENTRIES];
   double accD[SOP_MAX_LLOYD_ITERS + 1];
   unsigned prefix[3];       // of the selected key after one, two passes
   unsigned pad3;
   long long rank[3];        // its rank inside that prefix
-  unsigned arrive[SOP_MAX_LLOYD_ITERS + 1];      // CTAs that have added their sums of an iteration
+  unsigned arrive[SOP_MAX_LLOYD_ITERS + 1];      // CTAs that have added their sums of an iteration (persistent iterations: of all of them)
   unsigned error;        // a CTA gave up waiting for a flag
   unsigned list_count;   // blocks appended to the pool list
   // per cell, over the whole pool (filled once by pool_cache_kernel)
@@ -616,25 +617,27 @@ __global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev 
 //   The cells without a threshold are a matter of CTA 0: prefix sums over all cells, built once, make an entry's share the
 //   difference of two of them.  (About the origin, in FP64: the distortion is a few thousandths of the second moment, so 1e-16 of
 //   that leaves it 1e-13.)
-//   Every CTA adds its sums to the iteration's global ones, arrives at a counter, waits (bounded) until all have arrived and then
-//   works out the next table for itself: the sums are integers, so all get the same one and nobody has to hand it on.
-// What bounds it: the chain of one iteration (the first elements, global additions, their fence, arrival, sums, table: about 4.5 us;
-// 9 us when the last CTA worked out the table and handed it on) and, for a large pool, the latency of the split cells' elements.
-// Nine iterations on 25 thousand pool blocks 44 us (82 us with a warp per tile), on 2 million 102 us (150 us), on 7.3 million
-// 241 us (341 us).  Every warp must have its share of every cell: dealt cell by cell, the warps of the outer thresholds waited
-// for those of the inner ones and the 7.3 million took 685 us.
+//   Every CTA adds its sums to the iteration's global ones, waits (bounded) until all have and then works out the next table for
+//   itself: the sums are integers, so all get the same one and nobody has to hand it on.  A sum carries the number of CTAs that have
+//   added to it in its top byte, so that neither a fence nor an arrival stands between the additions and their readers.
+// What bounds it: the chain of one iteration (the first elements, the sums, global additions, reading them back, table: about 3.7 us;
+// 4.5 us with an arrival counter behind a fence, 9 us when the last CTA worked out the table and handed it on) and, for a large pool,
+// the latency of the split cells' elements.  Nine iterations on 25 thousand pool blocks 41 us (49 us with the arrival counter, 82 us
+// with a warp per tile), on 2 million 97 us (150 us), on 7.3 million 235 us (341 us).  Every warp must have its share of every cell:
+// dealt cell by cell, the warps of the outer thresholds waited for those of the inner ones and the 7.3 million took 685 us.
 // ---------------------------------------------------------------------------------------------
 constexpr int ITB = 768;            // threads of an iteration CTA (one per SM)
 constexpr int PRE = 4;              // elements of a run that a lane loads one step ahead
 constexpr int MAX_SPLIT = 32;       // a table has at most 31 thresholds, so at most 31 cells hold one
 constexpr int LIMBS = 3;            // 64-bit sums modulo 2^64 as 20 + 20 + 24 bits, which native 32-bit shared-memory additions take
+constexpr int CTA_COUNT_BIT = 56;   // fewer than 2^27 blocks: a sum of omega stays below 2^55 (see lloyd_iteration_plan)
 constexpr unsigned WAIT_POLLS = 1u << 21;      // polls of a few hundred ns: about half a second
 
 struct IterSmem {
   IterDesc d;
   unsigned limb[2][LIMBS][SOP_MAX_ENTRIES];    // this CTA's sums per entry: fix(omega), fix(omega u)
   unsigned long long sum[2][SOP_MAX_ENTRIES];  // the same of cells with several thresholds
-  double warp_D[ITB / 32];
+  double lane_D[ITB];
   CellEntry entry[MAX_SPLIT];
   unsigned short cell[MAX_SPLIT];
   int n_split, stop, is_last;
@@ -814,44 +817,59 @@ __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __r
       __syncwarp();
     }
   }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) D += __shfl_xor_sync(0xFFFFFFFFu, D, o);
-  if (lane == 0) S.warp_D[warp] = D;
+  S.lane_D[tid] = D;
   __syncthreads();
   if (warp == 0) {
     const int ne = S.d.n_entries;
     unsigned long long n = join_limbs(S, 0, lane) + S.sum[0][lane], s = join_limbs(S, 1, lane) + S.sum[1][lane];
+    // CTA 0: the cells without a threshold between this entry's two
+    const int lo = blockIdx.x == 0 && lane < ne ? (lane ? S.d.thr_cell[lane - 1] + 1 : 0) : 0;
+    const int hi = blockIdx.x == 0 && lane < ne ? (lane < ne - 1 ? S.d.thr_cell[lane] : SORT_ROWS) : 0;
+    if (lo < hi) {
+      n += S.preN[hi] - S.preN[lo];
+      s += (unsigned long long)(S.preS[hi] - S.preS[lo]);
+    }
+    if (!last && lane < ne) {
+      const unsigned long long one = ALL ? 1ull << CTA_COUNT_BIT : 0ull;
+      atomicAdd(&ws->acc[it][0][lane], n + one);
+      atomicAdd(&ws->acc[it][1][lane], (s & 0xFFFFFFFFull) + one);
+      atomicAdd(&ws->acc[it][2][lane], (unsigned long long)((long long)s >> 32) + one);
+    }
+    // the rest happens while those are on their way
     S.sum[0][lane] = S.sum[1][lane] = 0ull;
 #pragma unroll
     for (int i = 0; i < LIMBS; ++i) S.limb[0][i][lane] = S.limb[1][i][lane] = 0u;
-    double dsum = lane < ITB / 32 ? S.warp_D[lane] : 0.0;
-    if (blockIdx.x == 0 && lane < ne) {
-      // cells without a threshold between this entry's two
-      const int lo = lane ? S.d.thr_cell[lane - 1] + 1 : 0, hi = lane < ne - 1 ? S.d.thr_cell[lane] : SORT_ROWS;
-      if (lo < hi) {
-        n += S.preN[hi] - S.preN[lo];
-        s += (unsigned long long)(S.preS[hi] - S.preS[lo]);
-        const double q = 256.0 * (double)S.d.lut[lane];
-        const double b0 = S.preA[0][hi] - S.preA[0][lo], b1 = S.preA[1][hi] - S.preA[1][lo], b2 = S.preA[2][hi] - S.preA[2][lo];
-        dsum += (b2 - q * (2.0 * b1 - q * b0)) * (1.0 / 65536.0);
-      }
+    // (a shorter chain, four sums at a time, had the CTAs poll the sums while they were being added to: 1 us of a pass slower)
+    double dsum = 0.0;
+#pragma unroll 8
+    for (int i = lane; i < ITB; i += 32) dsum += S.lane_D[i];
+    if (lo < hi) {
+      const double q = 256.0 * (double)S.d.lut[lane];
+      const double b0 = S.preA[0][hi] - S.preA[0][lo], b1 = S.preA[1][hi] - S.preA[1][lo], b2 = S.preA[2][hi] - S.preA[2][lo];
+      dsum += (b2 - q * (2.0 * b1 - q * b0)) * (1.0 / 65536.0);
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) dsum += __shfl_xor_sync(0xFFFFFFFFu, dsum, o);
-    if (!last && lane < ne) {
-      if (n) atomicAdd(&ws->accN[it][lane], n);
-      if (s) atomicAdd(reinterpret_cast<unsigned long long*>(&ws->accS[it][lane]), s);
-    }
     if (lane == 0 && dsum != 0.0) atomicAdd(&ws->accD[it], dsum);
-    __threadfence();
-    __syncwarp();
-    if (ALL) {
-      if (lane == 0) atomicAdd(&ws->arrive[it], 1u);           // (no value back: nobody waits for it)
-    } else {
+    if (!ALL || last) {
+      __threadfence();
+      __syncwarp();
       if (lane == 0) S.is_last = atomicAdd(&ws->arrive[it], 1u) == gridDim.x - 1 ? 1 : 0;
       __syncwarp();
     }
   }
+}
+
+// The sums of one iteration where they count their CTAs (one lane per entry): false while some are missing.
+__device__ __forceinline__ bool read_sums(const unsigned long long (*acc)[SOP_MAX_ENTRIES], unsigned ctas, unsigned long long& n, long long& s) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long v[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[i]) : "l"(&acc[i][lane]) : "memory");
+  const unsigned long long c0 = v[0] >> CTA_COUNT_BIT, c1 = v[1] >> CTA_COUNT_BIT, c2 = (v[2] + (1ull << (CTA_COUNT_BIT - 1))) >> CTA_COUNT_BIT;
+  n = v[0] - (c0 << CTA_COUNT_BIT);
+  s = (long long)((v[1] - (c1 << CTA_COUNT_BIT)) + ((v[2] - (c2 << CTA_COUNT_BIT)) << 32));      // modulo 2^64
+  return c0 == ctas && c1 == ctas && c2 == ctas;
 }
 
 // ALL: every iteration in this launch (launched cooperatively: every CTA is resident); else iteration `it0` alone, whose last CTA
@@ -910,16 +928,27 @@ __global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs
     if (tid == 0) { S.preN[0] = 0; S.preS[0] = 0; S.preA[0][0] = S.preA[1][0] = S.preA[2][0] = 0.0; }
   }
   __syncthreads();
+  if (warp == 0) split_cells(S);
+  __syncthreads();
   for (int it = it0;; ++it) {
     const bool last = it == iters;
-    if (warp == 0) split_cells(S);
-    __syncthreads();
     iteration_share<ALL>(a, ws, S, ts, tile0, T, it, last);
     if (warp == 0) {
       bool go = true;
-      if (ALL) {
-        // CTA 0 waits for the closing iteration too: it reports the result
-        if (lane == 0 && (!last || blockIdx.x == 0)) {
+      unsigned long long n = 0;
+      long long s = 0;
+      if (ALL && !last) {
+        for (unsigned polls = 0;;) {
+          const bool there = lane >= S.d.n_entries || read_sums(ws->acc[it], gridDim.x, n, s);
+          if (__all_sync(0xFFFFFFFFu, there)) break;
+          ++polls;
+          const bool give_up = polls > WAIT_POLLS || ((polls & 63u) == 0u && *(volatile unsigned*)&ws->error != 0u);
+          if (__any_sync(0xFFFFFFFFu, give_up)) { go = false; break; }
+        }
+        if (!go && lane == 0) atomicExch(&ws->error, 1u);
+      } else if (ALL) {
+        // CTA 0 waits for everybody's distortions: it reports the result
+        if (blockIdx.x == 0 && lane == 0) {
           unsigned polls = 0, seen;
           for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&ws->arrive[it]) : "memory");
@@ -928,19 +957,23 @@ __global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs
           }
         }
         go = __shfl_sync(0xFFFFFFFFu, go ? 1 : 0, 0) != 0;
+        if (go && blockIdx.x == 0)
+          for (int i = lane; i <= iters; i += 32) distortion[i] = __ldcg(&ws->accD[i]);
       } else {
         go = S.is_last != 0;
         __threadfence();
+        if (go && lane == 0) distortion[it] = __ldcg(&ws->accD[it]);
+        if (go && !last) {
+          n = __ldcg(&ws->acc[it][0][lane]);
+          s = (long long)(__ldcg(&ws->acc[it][1][lane]) + (__ldcg(&ws->acc[it][2][lane]) << 32));
+        }
       }
-      if (go && (!ALL || blockIdx.x == 0)) {
-        if (lane == 0) distortion[it] = __ldcg(&ws->accD[it]);
-        if (last) out_lut[lane] = lane < S.d.n_entries ? S.d.lut[lane] : 0.0f;
-      }
+      if (go && last && (!ALL || blockIdx.x == 0)) out_lut[lane] = lane < S.d.n_entries ? S.d.lut[lane] : 0.0f;
       if (go && !last) {
-        const unsigned long long n = __ldcg(&ws->accN[it][lane]);
-        const long long s = __ldcg(&ws->accS[it][lane]);
         new_table(S, n, s);
         make_desc(ALL ? &S.d : &ws->desc, S.table, S.d.n_entries);
+        __syncwarp();
+        if (ALL) split_cells(S);
       }
       if (lane == 0) S.stop = !ALL || last || !go ? 1 : 0;
     }
@@ -1139,11 +1172,12 @@ int num_sms();
 static size_t iter_smem_bytes(int tiles) { return ((sizeof(IterSmem) + 15) & ~(size_t)15) + (size_t)tiles * TS_PITCH * sizeof(unsigned short); }
 constexpr size_t ITER_SMEM_MAX = 225 * 1024;
 
-static bool lloyd_iteration_plan(long long pool_blocks, int iters, int flags, long long* grid_out) {
+static bool lloyd_iteration_plan(long long NB, long long pool_blocks, int iters, int flags, long long* grid_out) {
   const int sms = num_sms();
   const long long likely = (pool_blocks + CTB - 1) / CTB;           // cache tiles of the pool without ties at its threshold
   long long grid = (likely + 3) / 4;
   if (grid > sms) grid = sms;
+  if (grid > 255) grid = 255;                                       // (a byte counts them)
   if (g_tune.iter_ctas > 0 && grid > g_tune.iter_ctas) grid = g_tune.iter_ctas;
   if (grid < 1) grid = 1;
   DeviceFacts* facts = device_facts();
@@ -1158,7 +1192,7 @@ static bool lloyd_iteration_plan(long long pool_blocks, int iters, int flags, lo
     cudaGetLastError();
   }
   *grid_out = grid;
-  return iters >= 1 && facts->coop_blocks_per_sm >= 1 && !(flags & SOP_LLOYD_LAUNCH_PER_ITERATION);
+  return iters >= 1 && NB < (1ll << 27) && facts->coop_blocks_per_sm >= 1 && !(flags & SOP_LLOYD_LAUNCH_PER_ITERATION);
 }
 
 }  // namespace sop
@@ -1169,7 +1203,7 @@ int sop_dd4_lloyd_launches(long long M, long long K, int iters, int flags, int* 
   if (!launches) return SOP_ERR_NULL;
   if (M < 1 || K < 1 || (K % SOP_G) != 0 || iters < 0 || iters > sop::SOP_MAX_LLOYD_ITERS) return SOP_ERR_RANGE;
   long long grid = 1;
-  const bool persistent = sop::lloyd_iteration_plan(M * (K / SOP_G), iters, flags, &grid);
+  const bool persistent = sop::lloyd_iteration_plan(M * (K / SOP_G), M * (K / SOP_G), iters, flags, &grid);
   // radix select (three passes, unless the pool is cut by a threshold), set-up, pool list, pool cache, iterations
   // the dynamic programme: the costs, the rows
   *launches = ((flags & SOP_LLOYD_POOL_THRESHOLD) ? 0 : 3) + 3 + ((flags & SOP_LLOYD_GRID_DP) ? 2 : (persistent ? 1 : iters + 1));
@@ -1292,7 +1326,7 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
   }
   long long grid = 1;
   const long long expected = by_threshold ? NB : pool_rank;
-  const bool persistent = lloyd_iteration_plan(expected, iters, flags, &grid);
+  const bool persistent = lloyd_iteration_plan(NB, expected, iters, flags, &grid);
   // room for the cell starts of the tiles that a CTA is likely to have (and a few more, for ties); more tiles are read from memory
   int smem_tiles = (int)(((expected + CTB - 1) / CTB + grid - 1) / grid + 4);
   while (smem_tiles > 0 && iter_smem_bytes(smem_tiles) > ITER_SMEM_MAX) --smem_tiles;
