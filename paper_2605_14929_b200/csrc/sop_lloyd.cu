@@ -131,39 +131,43 @@ __device__ __forceinline__ int resolve_fmta(const LloydArgs& a, const sop_search
   return max(0, min(a.n_atoms - 1, f));
 }
 
-// CTA-wide (a multiple of 32 threads, at most 1024): the bin of `hist` (nb <= 2048 bins) holding the
-// element of 1-based rank `rank`; *before = elements in lower bins, *count = elements in that bin.
-__device__ void find_bin(const unsigned* __restrict__ hist, int nb, long long rank, int* bin, long long* before, unsigned* count) {
-  __shared__ long long s_warp[32];
+// CTA of LTB threads: the bin of `hist` (LTB PER bins) holding the element of 1-based rank `rank`; *before = elements in lower bins.
+// Every CTA of the pass that follows does this before it can start, so a thread's bins are loaded together.
+template <int PER>
+__device__ void find_bin(const unsigned* __restrict__ hist, long long rank, int* bin, long long* before) {
+  __shared__ unsigned s_warp[LTB / 32];
   __shared__ int s_bin;
-  __shared__ long long s_before;
-  __shared__ unsigned s_cnt;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int per = (nb + nt - 1) / nt;
-  const int b0 = tid * per;
-  long long local = 0;
-  for (int i = 0; i < per; ++i)
-    if (b0 + i < nb) local += hist[b0 + i];
-  long long incl = local;
+  __shared__ unsigned s_before;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned h[PER], local = 0;                        // (at most 2^27 blocks)
+#pragma unroll
+  for (int i = 0; i < PER; i += 4) {
+    const uint4 v = __ldcg(reinterpret_cast<const uint4*>(hist + tid * PER + i));
+    h[i] = v.x; h[i + 1] = v.y; h[i + 2] = v.z; h[i + 3] = v.w;
+  }
+#pragma unroll
+  for (int i = 0; i < PER; ++i) local += h[i];
+  unsigned incl = local;
+#pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const long long v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += v;
   }
   if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
-  long long base = 0;
-  for (int w = 0; w < warp; ++w) base += s_warp[w];
-  const long long excl = base + incl - local;
-  if (local > 0 && excl < rank && rank <= excl + local) {
-    long long run = excl;
-    for (int i = 0; i < per; ++i) {
-      const unsigned h = hist[b0 + i];
-      if (run + h >= rank) { s_bin = b0 + i; s_before = run; s_cnt = h; break; }
-      run += h;
+  unsigned run = incl - local;
+#pragma unroll
+  for (int w = 0; w < LTB / 32; ++w) run += w < warp ? s_warp[w] : 0u;
+  const unsigned want = (unsigned)rank;
+  if (run < want && want <= run + local) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      if (run < want && want <= run + h[i]) { s_bin = tid * PER + i; s_before = run; }
+      run += h[i];
     }
   }
   __syncthreads();
-  *bin = s_bin; *before = s_before; *count = s_cnt;
+  *bin = s_bin; *before = s_before;
   __syncthreads();
 }
 
@@ -175,8 +179,8 @@ __device__ unsigned derive_prefix(LloydWs* ws, long long pool_rank, int passes) 
   const long long rank = p ? __ldcg(&ws->rank[p - 1]) : pool_rank;
   int bin;
   long long before;
-  unsigned cnt;
-  find_bin(ws->hist[p], p < 2 ? 2048 : 1024, rank, &bin, &before, &cnt);
+  if (p < 2) find_bin<2048 / LTB>(ws->hist[p], rank, &bin, &before);
+  else find_bin<1024 / LTB>(ws->hist[p], rank, &bin, &before);
   const unsigned out = (pre << (p < 2 ? 11 : 10)) | (unsigned)bin;
   if (blockIdx.x == 0 && threadIdx.x == 0) { ws->prefix[p] = out; ws->rank[p] = rank - before; }
   return out;
