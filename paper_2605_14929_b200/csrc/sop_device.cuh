@@ -63,6 +63,9 @@ inline cudaError_t launch(void (*kernel)(P...), dim3 grid, int block, size_t sme
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+// Zeros: a kernel of the chain instead of a memset, which would neither start early nor let its successor.
+cudaError_t clear(void* words, size_t bytes, cudaStream_t st);      // whole 32-bit words
+
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -316,11 +316,15 @@ __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __
         in |= (pool_key(v[q].w, a.flags) <= tau_key ? 1u : 0u) << (4 * q + 3);
       }
     } else {
-#pragma unroll 4
+      float v[16];                       // (in flight together as well)
+#pragma unroll
       for (int x = 0; x < 16; ++x) {
         const long long i = i0 + 128 * (x >> 2) + (x & 3);
-        if (i < a.NB && pool_key(__ldg(row + i), a.flags) <= tau_key) in |= 1u << x;
+        v[x] = i < a.NB ? __ldg(row + i) : 0.0f;
       }
+#pragma unroll
+      for (int x = 0; x < 16; ++x)
+        if (i0 + 128 * (x >> 2) + (x & 3) < a.NB && pool_key(v[x], a.flags) <= tau_key) in |= 1u << x;
     }
     unsigned mine = 0;                   // a lane's four counts, a byte each (a warp's sum is at most 128)
 #pragma unroll

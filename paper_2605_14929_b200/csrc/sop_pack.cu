@@ -782,7 +782,7 @@ int sop_pack(const void* W_dev, long long M, long long K, long long ldw, const f
   if (winner) {}
   else if (container_bits == 12) SOP_CUDA_TRY(cudaMemsetAsync(words_dev, 0, padded, st));
   else SOP_CUDA_TRY(cudaMemsetAsync(words_dev + padded - 4, 0, 4, st));
-  if (counts_dev) SOP_CUDA_TRY(cudaMemsetAsync(counts_dev, 0, 2 * sizeof(long long), st));
+  if (counts_dev) SOP_CUDA_TRY(clear(counts_dev, 2 * sizeof(long long), st));
   long long grid = (a.NB + PTB - 1) / PTB;
   const int sms = num_sms();
   const long long resident = (long long)sms * 4;

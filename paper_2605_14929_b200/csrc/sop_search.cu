@@ -1732,8 +1732,8 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   while (((n_tiles + rgrid - 1) / rgrid) * units * (RUNIT / 32) > 4095) ++rgrid;
 
   // the prepass adds to its histograms; the reduction's counters are cleared by the sweep where there is one
-  if (!k_from_result && !reuse_prepass) SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, ws_part_off(), st));
-  else if (!eval_mask) SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, ws_hist_off(), st));
+  if (!k_from_result && !reuse_prepass) SOP_CUDA_TRY(clear(ws, ws_part_off(), st));
+  else if (!eval_mask) SOP_CUDA_TRY(clear(ws, ws_hist_off(), st));
   if ((rc = profile_mark(SOP_PROFILE_PREPASS, 0, st))) return rc;
   if (reuse_prepass) {
     SOP_CUDA_TRY(launch(kselect_kernel, 1, 256, 0, st, P, F, hist, hdr));
