@@ -53,11 +53,11 @@ SM_COUNT, SCHEDULERS, LANES = 148, 4, 32
 # file (dram__bytes_read.sum + dram__bytes_write.sum of one launch on the 8192x8192 layer at E5M6 divided by its
 # elements; traffic grows in proportion to the elements, so a launch of the block is scaled by its elements).
 # None: no capture of the kernel as it is now.
-NCU_SWEEP_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=5.1796,
-                         bytes_per_element_dd_columns=2.5803)
+NCU_SWEEP_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=5.2154,
+                         bytes_per_element_dd_columns=2.5740)
 # the same for the reduction kernel (first call: the fixed candidates' entries; second call: the DD columns' entries)
-NCU_REDUCE_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=4.0759,
-                          bytes_per_element_dd_columns=5.0753)
+NCU_REDUCE_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=4.0624,
+                          bytes_per_element_dd_columns=5.0582)
 
 
 # ---------------------------------------------------------------------------------------------------------
@@ -334,20 +334,20 @@ def sparse_streams_table(dev, hbm_peak, of, flush):
     E = M * K
     opq_ms, wr_ms, all_ms = sorted(t_opq)[2], sorted(t_wr)[2], sorted(t_all)[2]
     opq_bytes = (2.0 + 2.0 + 2 * 2.0 / 16.0) * E + 4.0 * sp["opq"]["count"]
-    wr_bytes = 2 * (2.0 + 0.5 + sw.container / 8.0 / 16.0) * E + 4.0 * sp["wr"]["count"]
+    wr_bytes = (2.0 + 0.5 + sw.container / 8.0 / 16.0 + 2 * 2.0 / 16.0) * E + 4.0 * sp["wr"]["count"]      # one decode pass, the bins out and in
 
     def hbm(b, ms):
         return dict(achieved=b / (ms * 1e-3) / 1e9, peak=hbm_peak, unit="GB/s", frac=b / (ms * 1e-3) / 1e9 / hbm_peak, of=of)
     return dict(workload="8192x8192 at E5M6, ROM4 + DD4, outlier quantile 0.92, correction sparsity 0.001", elements=E,
                 opq=dict(ms=opq_ms, records=sp["opq"]["count"], rate=sp["opq"]["count"] / E, threshold_m=sp["opq"]["m"],
                          bpw=32.0 * sp["opq"]["count"] / E, algorithmic_bytes=opq_bytes, hbm=hbm(opq_bytes, opq_ms),
-                         note="three launches: mask + zeroed copy (W read once, written once), scan of the tile counts, records"),
+                         note="three launches: mask, zeroed copy and the tiles' records (W read once, written once), scan of the tile counts, "
+                              "the records move to their place"),
                 wr=dict(ms=wr_ms, records=sp["wr"]["count"], n_keep=sp["wr"]["n_keep"], scale_exp=sp["wr"]["scale_exp"],
                         bpw=32.0 * sp["wr"]["count"] / E, algorithmic_bytes=wr_bytes, hbm=hbm(wr_bytes, wr_ms),
-                        note="two passes decode W, codes and scale words (2.6 bytes per element) into the residual: block maxima, then the "
-                             "candidates above the bound they give; threshold, kept set and counts come from the candidate list, the "
-                             "write pass decodes only blocks with a kept entry (eighteen launches, seven of them the unused "
-                             "full-decode path that returns at once)"),
+                        note="one pass decodes W, codes and scale words (2.6 bytes per element) into the residual and keeps the bin of every "
+                             "block's largest metric; the blocks above the bound they give are decoded again into the candidate list that "
+                             "the threshold, the kept set, the counts and the records come from (seven launches)"),
                 whole_path_ms=all_ms, whole_path_value=E / all_ms / 1e6)
 
 
