@@ -766,6 +766,8 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
 #pragma unroll
     for (int q = 0; q < 8; ++q) wb[q] = wn[q];
     if (it + 1 < X.n_rows) wp += X.w_step;
+    // (the rows after that on their way into L2, there are no registers to hold them: 14336 x 4096, two formats, a pass 183.8 us, 186 us without)
+    if (it + 3 < X.n_rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(wp + 2 * X.w_step));
     load_block_bits(wp, wn);
     float s_hat, rcp;
     X.scale(absmax_bits(wb), F, s_hat, rcp);
