@@ -563,7 +563,9 @@ def run_gpu(args) -> None:
             ops_per_element=dict(fixed_candidates=sweep_kernel_ops_n_step(n_lut - n_dd, nb, 0), dd_columns=sweep_kernel_ops_n_step(n_dd, nb, 0)),
             algorithmic_bytes_per_launch=sweep_bytes / 2.0 * units / n_pass,
             note="the dominant kernel of the step: the evaluation of every candidate on every block (two launches per layer and "
-                 "format: the fixed candidates, then the DD columns), against its own share of the n-step operation count; "
+                 "format: the fixed candidates, then the DD columns), against its own share of the n-step operation count; the "
+                 "joint rows of the candidates need fewer instructions than that model counts (59 and 30 per element by ncu, at 61 "
+                 "and 68 % of the issue slots), so the fraction may pass 1; "
                  "`search` below is the whole search (evaluation + reduction of the table entries) against the whole count",
             search=dict(
                 kernels=["sweep_kernel", "reduce_kernel"], launches_per_step=4 * n_pass, ms_per_step=search_t * 1e3,

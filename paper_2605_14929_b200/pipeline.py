@@ -197,7 +197,7 @@ class LayerSweep:
             B.sop_pair_search(W, self.c, self.fmt_c, self.atoms_c, self.pair_table, self.signed_table, self.rom_result,
                               self.ws_search, block_cos=self.full_cos, block_sse=self.full_sse, eval_mask=self.fixed_mask,
                               stream=stream, reuse_prepass=reuse_prepass)
-            n += 3
+            n += 3 if reuse_prepass else 4          # the clear of the histograms, prepass (or the shifts alone), sweep, reduction
             B.sop_dd4_lloyd(W, self.c, self.fmt_c, self.atoms_c, self.full_cos, self.pool_rank, self.dd_iters, self.dd_lut,
                             self.distortion, self.pool_count, self.ws_lloyd, search_result=self.rom_result, stream=stream,
                             grid_dp=self.grid_dp)
@@ -210,14 +210,14 @@ class LayerSweep:
             B.sop_pair_search(W, self.c, self.fmt_c, self.atoms_c, self.pair_table, self.signed_table, self.result,
                               self.ws_search, block_cos=self.full_cos, block_sse=self.full_sse, stream=stream,
                               reuse_prepass=reuse_prepass)
-            n += 1
+            n += 1 if reuse_prepass else 2
         n += 2
         B.sop_pack(W, self.c, self.fmt_c, self.atoms_c, codes, words, search_result=self.result,
                    index_a=0 if self.single else B.PAIR_FROM_RESULT, index_b=B.NO_ATOM if self.single else B.PAIR_FROM_RESULT,
                    use_sign=self.use_sign, container_bits=self.container, word_sign_bits=self.use_sign,
                    counts=self.counts, dd_lut=self.dd_lut if self.dd_mask else None, dd_mask=self.dd_mask,
                    block_cos=self.full_cos, stream=stream)
-        n += 1
+        n += 2                                      # the clear of the counts, the packer
         if self.wr_keep:
             B.sop_wr_extract(W, self.c, self.fmt_c, self.atoms_c, codes, words, self.wr_keep, self.wr_row_start,
                              self.wr_records, self.wr_count, self.wr_exp, self.ws_wr, tau=self.wr_tau,
