@@ -636,16 +636,18 @@ template <int NP>
 __device__ __forceinline__ void sweep_emit(float nw, float2 (&nq)[NP], float2 (&dot)[NP], float2 (&sse)[NP], const ColumnPtr* cols,
                                            unsigned at, bool on) {
   float2 nx[NP];
-  float lo = 3.0e38f, hi = 0.0f, dl = 3.0e38f;
+  unsigned lo = 0xFFFFFFFFu, hi = 0u;
+  float dl = 3.0e38f;
   const float2 nnw = make_float2(-nw, -nw);
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
     nx[p] = __fmul2_rn(nnw, nq[p]);
-    lo = fminf(lo, fminf(-nx[p].x, -nx[p].y));
-    hi = fmaxf(hi, fmaxf(-nx[p].x, -nx[p].y));
+    // compared as patterns: a product that is no number (a sum that overflowed times one that underflowed) lies outside too
+    lo = min(lo, min(__float_as_uint(nx[p].x), __float_as_uint(nx[p].y)));
+    hi = max(hi, max(__float_as_uint(nx[p].x), __float_as_uint(nx[p].y)));
     dl = fminf(dl, fminf(fabsf(dot[p].x), fabsf(dot[p].y)));
   }
-  if (lo >= COS_LO && hi <= COS_HI && dl >= COS_DOT) {
+  if (lo >= __float_as_uint(-COS_LO) && hi <= __float_as_uint(-COS_HI) && dl >= COS_DOT) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) dot[p] = cosine_pair(nx[p], dot[p]);
   } else {

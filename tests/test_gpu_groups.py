@@ -50,3 +50,16 @@ def test_block_sums_of_any_magnitude(B, fmt_name):
     W[5] = 0
     W[6] = torch.where(torch.arange(256) % 16 == 3, W[6], torch.zeros(256))
     check_search(B, I.Layer(W.to(torch.bfloat16), L.X), fmt_name, I.alphabet(["NF4", "SH4"], fp=["E2M3", "E4M3"]))
+
+
+@pytest.mark.parametrize("fmt_name", ["E8M7", "UE8M0"])
+def test_a_norm_that_overflows_against_one_that_underflows(B, fmt_name):
+    # per block one huge weight on a channel without activations and fifteen smaller ones that reconstruct as 1e-25: <w, w>
+    # overflows, <q, q> underflows to zero, their product is no number and the cosine is zero
+    L = I.tiny_layer(23, 24, 256)
+    first = (torch.arange(256) % 16 == 0)
+    W = torch.where(first, torch.full((), 2.0 ** 100), (L.W.float().abs() + 1.0) * 2.0 ** 66)
+    X = torch.where(first, torch.zeros(()), L.X)
+    a = _table("small", np.concatenate([np.linspace(-1.0, -0.1, 7), [1e-25], np.linspace(0.1, 1.0, 8)]))
+    got, _ = check_search(B, I.Layer(W.to(torch.bfloat16), X), fmt_name, [a, a.negation()])
+    assert not got["block_cos"].any()
