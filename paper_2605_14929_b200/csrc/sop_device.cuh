@@ -202,7 +202,8 @@ __device__ __forceinline__ float fp_quantize(float u) {
 
 // The same for two values at once through the conversion instructions of the two formats (round to nearest even, saturating,
 // sign of zero kept; every E2M3 and E4M3 value is an fp16 number): fp_quantize<KIND> and fp_code<KIND> of x and y, compared for
-// every finite fp32 pattern.  The codes come back as bytes, x in the lower one.
+// every finite fp32 pattern.  The codes come back as bytes, x in the lower one.  A NaN would stay one in E4M3, where
+// fp_quantize saturates it: saturate_zeros keeps the one there is away from it.
 template <int KIND>
 __device__ __forceinline__ float2 fp_quantize2(float x, float y, uint32_t& codes) {
   unsigned short c;
@@ -216,6 +217,17 @@ __device__ __forceinline__ float2 fp_quantize2(float x, float y, uint32_t& codes
   }
   codes = c;
   return __half22float2(*reinterpret_cast<const __half2*>(&h));
+}
+
+// The weights of a block whose reciprocal scale is infinite (a scale of 2^-128 or below): a zero times it is no number, every other
+// weight saturates.  The zeros become the smallest positive weight, which saturates as well, as fp_quantize has it; in the norms of
+// such a block it is as good as zero (its square and that of its error underflow).
+__device__ __forceinline__ void saturate_zeros(uint32_t (&wb)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const uint32_t zero = __vcmpeq2(wb[q] & 0x7FFF7FFFu, 0u);
+    wb[q] = (wb[q] & ~zero) | (zero & 0x00010001u);
+  }
 }
 
 // Element grid given by parameters (SOP_KIND_FP_GRID): min_eb = biased fp32 exponent of the smallest normal

@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
   for (unsigned base = base0; base < NB; base += stride) {
     const unsigned blk = base + lane;
     const bool on = blk < NB;
-    const uint32_t wb[8] = {nv0.x, nv0.y, nv0.z, nv0.w, nv1.x, nv1.y, nv1.z, nv1.w};
+    uint32_t wb[8] = {nv0.x, nv0.y, nv0.z, nv0.w, nv1.x, nv1.y, nv1.z, nv1.w};
     // the winner in the priority order a, (-a), b, (-b): ties keep the earlier
     int pick = 0;
     float best = ncs[0];
@@ -559,6 +559,7 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
       else { const QScale qs = scale_quantize(sigma, T.k, F); s_hat = qs.s_hat; scode = qs.code; }
       rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
     }
+    if (KIND == SOP_KIND_FP_E4M3 && isinf(rcp)) saturate_zeros(wb);
     uint32_t code4[4];       // sixteen codes as bytes
     if (LUT) {
       const float r = (sg ? 1 - T.neg : T.neg) ? -rcp : rcp;       // a negated table runs on -u

@@ -773,6 +773,7 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
     load_block_bits(wp, wn);
     float s_hat, rcp;
     X.scale(absmax_bits(wb), F, s_hat, rcp);
+    if (MODE == SOP_KIND_FP_E4M3 && isinf(rcp)) saturate_zeros(wb);
     float cc[16];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {

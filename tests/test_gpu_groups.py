@@ -63,3 +63,12 @@ def test_a_norm_that_overflows_against_one_that_underflows(B, fmt_name):
     a = _table("small", np.concatenate([np.linspace(-1.0, -0.1, 7), [1e-25], np.linspace(0.1, 1.0, 8)]))
     got, _ = check_search(B, I.Layer(W.to(torch.bfloat16), X), fmt_name, [a, a.negation()])
     assert not got["block_cos"].any()
+
+
+@pytest.mark.parametrize("fmt_name", ["E8M7", "UE8M0"])
+def test_element_formats_where_the_reciprocal_scale_overflows(B, fmt_name):
+    # rows from 2^-136 to 2^-100 with zeros among the weights: scales of 2^-128 and below
+    L = I.tiny_layer(24, 24, 256)
+    W = L.W.float() * (2.0 ** torch.linspace(-131, -95, 24).round())[:, None]
+    W = torch.where(torch.rand(24, 256, generator=torch.Generator().manual_seed(2)) < 0.4, torch.zeros(()), W)
+    check_search(B, I.Layer(W.to(torch.bfloat16), L.X), fmt_name, I.alphabet([], fp=["E2M3", "E4M3", "E4M3^0"]), k_mode=0)

@@ -63,3 +63,23 @@ def test_packed_bytes_match_oracle(B, M, K, kind, fmt_name, b):
         assert np.array_equal(codes.cpu().numpy()[:NB * 2 * n].reshape(want["codes"].shape), want["codes"])
         assert np.array_equal(words.cpu().numpy()[:want["words"].size], want["words"])
         assert bool((codes[NB * 2 * n:] == 0x5A).all()) and bool((words[B.words_nbytes(NB, b):] == 0x5A).all())
+
+
+@pytest.mark.parametrize("kind", ["E2M3", "E4M3"])
+def test_both_packers_agree_where_the_reciprocal_scale_overflows(B, kind):
+    # zeros among weights of 2^-136 and above at a format that has scales below 2^-128
+    M, K = 24, 256
+    W = I.tiny_layer(62, M, K).W.float() * (2.0 ** torch.linspace(-131, -95, M).round())[:, None]
+    W = torch.where(torch.rand(M, K, generator=torch.Generator().manual_seed(3)) < 0.4, torch.zeros(()), W).to(torch.bfloat16).to(dev())
+    atoms, fmt, NB = [I.fp_atom(kind)], I.scale_format("UE8M7"), M * K // 16
+    cd = torch.ones(K, device=dev())
+    bc = torch.zeros((1, NB), device=dev())
+    out = []
+    for metric in (bc, None):
+        codes = torch.zeros(NB * 2 * atoms[0].n_bits, dtype=torch.uint8, device=dev())
+        words = torch.zeros(B.words_nbytes(NB, 16), dtype=torch.uint8, device=dev())
+        B.sop_pack(W, cd, fmt, atoms, codes, words, index_a=0, index_b=B.NO_ATOM, k_mode=0, container_bits=16, block_cos=metric)
+        out.append((codes, words))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    if kind == "E4M3":
+        assert int(((out[0][0] & 0x7F) == 0x7F).sum()) == 0           # no code that is not a number
