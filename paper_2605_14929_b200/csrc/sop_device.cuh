@@ -306,4 +306,52 @@ __device__ __forceinline__ float block_cosine(float nw, float nq, float dot) {
   return __fdiv_rn(dot, __fsqrt_rn(__fmul_rn(nw, nq)));
 }
 
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Cosines of two candidates at once: RN(dot / RN(sqrt(RN(nw nq)))), the value of block_cosine.  Square root and quotient by
+// Newton steps with exact fused residuals and a final correction (P. Markstein, "Computation of elementary functions on the
+// IBM RISC System/6000 processor", 1990): from the reciprocal root y the pair g ~ sqrt(x), h ~ 1 / (2 sqrt(x)) is refined once
+// and g corrected by its residual x - g^2; 2 h, refined once against the rounded root, is its rounded reciprocal, with which the
+// quotient is corrected by its residual.  The signs are chosen so that no operand needs a negation: G = -g, S = -sqrt(x).
+// Valid for x in [2^-80, 2^80] and |dot| >= 2^-60 (no intermediate result leaves the normal range) where the rounded root has a
+// zero in its significand: the reciprocal of an all-ones significand is halfway between two numbers up to a term that the last
+// refinement rounds away, and the quotient of a power of two by it then comes out one step low.  The caller checks both.
+constexpr float COS_LO = 8.271806125530277e-25f, COS_HI = 1.2089258196146292e24f, COS_DOT = 8.673617379884035e-19f;
+__device__ __forceinline__ float2 cosine_pair(const float2 nx, const float2 dot) {       // nx = -(nw nq)
+  const float2 y = make_float2(rsqrt_approx(-nx.x), rsqrt_approx(-nx.y));
+  const float2 half = make_float2(0.5f, 0.5f), one = make_float2(1.0f, 1.0f);
+  float2 G = __fmul2_rn(nx, y), h = __fmul2_rn(y, half);
+  const float2 r = __ffma2_rn(G, h, half);
+  G = __ffma2_rn(G, r, G);
+  h = __ffma2_rn(h, r, h);
+  const float2 D = __ffma2_rn(G, G, nx);
+  const float2 S = __ffma2_rn(D, h, G);
+  float2 z = __fadd2_rn(h, h);
+  const float2 e = __ffma2_rn(S, z, one);
+  z = __ffma2_rn(z, e, z);
+  const float2 q = __fmul2_rn(dot, z);
+  const float2 m = __ffma2_rn(S, q, dot);
+  return __ffma2_rn(m, z, q);
+}
+
+__device__ __forceinline__ float cosine_one(float nx, float dot) {      // the same steps for one candidate
+  const float y = rsqrt_approx(-nx);
+  float G = __fmul_rn(nx, y), h = __fmul_rn(y, 0.5f);
+  const float r = __fmaf_rn(G, h, 0.5f);
+  G = __fmaf_rn(G, r, G);
+  h = __fmaf_rn(h, r, h);
+  const float S = __fmaf_rn(__fmaf_rn(G, G, nx), h, G);
+  float z = __fadd_rn(h, h);
+  z = __fmaf_rn(z, __fmaf_rn(S, z, 1.0f), z);
+  const float q = __fmul_rn(dot, z);
+  return __fmaf_rn(__fmaf_rn(S, q, dot), z, q);
+}
+
+// Zero exactly where sqrt(x) rounds to an all-ones significand (the two largest numbers below a power of four, the sign aside).
+__device__ __forceinline__ unsigned all_ones_root(float x) { return (__float_as_uint(x) ^ 0x007FFFFEu) & 0x00FFFFFEu; }
+
 }  // namespace sop

@@ -486,49 +486,6 @@ __device__ __forceinline__ float4 lds_f4(unsigned addr) {
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
   return v;
 }
-__device__ __forceinline__ float rsqrt_approx(float x) {
-  float y;
-  asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Cosines of two candidates at once: RN(dot / RN(sqrt(RN(nw nq)))), the value of block_cosine.  Square root and quotient by
-// Newton steps with exact fused residuals and a final correction (P. Markstein, "Computation of elementary functions on the
-// IBM RISC System/6000 processor", 1990): from the reciprocal root y the pair g ~ sqrt(x), h ~ 1 / (2 sqrt(x)) is refined once
-// and g corrected by its residual x - g^2; 2 h, refined once against the rounded root, is its rounded reciprocal, with which the
-// quotient is corrected by its residual.  The signs are chosen so that no operand needs a negation: G = -g, S = -sqrt(x).
-// Valid for x in [2^-80, 2^80] and |dot| >= 2^-60 (no intermediate result leaves the normal range); the caller checks.
-constexpr float COS_LO = 8.271806125530277e-25f, COS_HI = 1.2089258196146292e24f, COS_DOT = 8.673617379884035e-19f;
-__device__ __forceinline__ float2 cosine_pair(const float2 nx, const float2 dot) {       // nx = -(nw nq)
-  const float2 y = make_float2(rsqrt_approx(-nx.x), rsqrt_approx(-nx.y));
-  const float2 half = make_float2(0.5f, 0.5f), one = make_float2(1.0f, 1.0f);
-  float2 G = __fmul2_rn(nx, y), h = __fmul2_rn(y, half);
-  const float2 r = __ffma2_rn(G, h, half);
-  G = __ffma2_rn(G, r, G);
-  h = __ffma2_rn(h, r, h);
-  const float2 D = __ffma2_rn(G, G, nx);
-  const float2 S = __ffma2_rn(D, h, G);
-  float2 z = __fadd2_rn(h, h);
-  const float2 e = __ffma2_rn(S, z, one);
-  z = __ffma2_rn(z, e, z);
-  const float2 q = __fmul2_rn(dot, z);
-  const float2 m = __ffma2_rn(S, q, dot);
-  return __ffma2_rn(m, z, q);
-}
-
-__device__ __forceinline__ float cosine_one(float nx, float dot) {      // the same steps for one candidate
-  const float y = rsqrt_approx(-nx);
-  float G = __fmul_rn(nx, y), h = __fmul_rn(y, 0.5f);
-  const float r = __fmaf_rn(G, h, 0.5f);
-  G = __fmaf_rn(G, r, G);
-  h = __fmaf_rn(h, r, h);
-  const float S = __fmaf_rn(__fmaf_rn(G, G, nx), h, G);
-  float z = __fadd_rn(h, h);
-  z = __fmaf_rn(z, __fmaf_rn(S, z, 1.0f), z);
-  const float q = __fmul_rn(dot, z);
-  return __fmaf_rn(__fmaf_rn(S, q, dot), z, q);
-}
-
 __device__ __noinline__ float block_cosine_any(float nw, float nq, float dot) { return block_cosine(nw, nq, dot); }
 
 // Rounding of a scale in its usual range, with what does not change from block to block worked out beforehand: the pattern of
@@ -636,7 +593,7 @@ template <int NP>
 __device__ __forceinline__ void sweep_emit(float nw, float2 (&nq)[NP], float2 (&dot)[NP], float2 (&sse)[NP], const ColumnPtr* cols,
                                            unsigned at, bool on) {
   float2 nx[NP];
-  unsigned lo = 0xFFFFFFFFu, hi = 0u;
+  unsigned lo = 0xFFFFFFFFu, hi = 0u, ones = 0xFFFFFFFFu;
   float dl = 3.0e38f;
   const float2 nnw = make_float2(-nw, -nw);
 #pragma unroll
@@ -645,9 +602,10 @@ __device__ __forceinline__ void sweep_emit(float nw, float2 (&nq)[NP], float2 (&
     // compared as patterns: a product that is no number (a sum that overflowed times one that underflowed) lies outside too
     lo = min(lo, min(__float_as_uint(nx[p].x), __float_as_uint(nx[p].y)));
     hi = max(hi, max(__float_as_uint(nx[p].x), __float_as_uint(nx[p].y)));
+    ones = min(ones, min(all_ones_root(nx[p].x), all_ones_root(nx[p].y)));
     dl = fminf(dl, fminf(fabsf(dot[p].x), fabsf(dot[p].y)));
   }
-  if (lo >= __float_as_uint(-COS_LO) && hi <= __float_as_uint(-COS_HI) && dl >= COS_DOT) {
+  if (lo >= __float_as_uint(-COS_LO) && hi <= __float_as_uint(-COS_HI) && ones && dl >= COS_DOT) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) dot[p] = cosine_pair(nx[p], dot[p]);
   } else {
@@ -805,7 +763,7 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
     }
     const float nw = fold(nw2[0], nw2[1]), nqs = fold(nq[0], nq[1]), dots = fold(dot[0], dot[1]), err = fold(sse[0], sse[1]);
     const float x = __fmul_rn(nw, nqs);
-    const float cosv = x >= COS_LO && x <= COS_HI && fabsf(dots) >= COS_DOT ? cosine_one(-x, dots) : block_cosine_any(nw, nqs, dots);
+    const float cosv = x >= COS_LO && x <= COS_HI && all_ones_root(x) && fabsf(dots) >= COS_DOT ? cosine_one(-x, dots) : block_cosine_any(nw, nqs, dots);
     if (it < X.n_rows)
       for (int ci = 0; ci < n_cand; ++ci) {      // (candidates of one format and scale have the same values)
         const size_t col = (size_t)K.cand[ci] * NB + (at >> 2);

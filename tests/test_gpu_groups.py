@@ -5,9 +5,10 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2605_14929_b200 import inputs as I
 
-from .test_gpu_parity import B, check_search  # noqa: F401  (B is a fixture)
+from .test_gpu_parity import B, check_search, gpu_search  # noqa: F401  (B is a fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -72,3 +73,25 @@ def test_element_formats_where_the_reciprocal_scale_overflows(B, fmt_name):
     W = L.W.float() * (2.0 ** torch.linspace(-131, -95, 24).round())[:, None]
     W = torch.where(torch.rand(24, 256, generator=torch.Generator().manual_seed(2)) < 0.4, torch.zeros(()), W)
     check_search(B, I.Layer(W.to(torch.bfloat16), L.X), fmt_name, I.alphabet([], fp=["E2M3", "E4M3", "E4M3^0"]), k_mode=0)
+
+
+def test_a_norm_product_whose_root_is_all_ones(B):
+    # <w, w> <q, q> = 4 - 2^-22 and <w, q> = 1 (table) or 1/4 (element format): the root rounds to 2 - 2^-23, the quotient of a power
+    # of two by it is just above the middle of two numbers
+    W, c = torch.zeros(2, 16), np.ones(16, np.float32)
+    W[0, 0], W[0, 4], c[4] = 1.0, 0.125, 64.0 * (3.0 - 2.0 ** -22)           # the table reconstructs (1, 0.125) as (1, 0)
+    W[1] = W[0]
+    three = _table("three", np.array([-1.0, 0.0, 1.0]), n_bits=2)
+    for atoms, fmt_name in (([three, three.negation()], "E5M6"), ([three], "UE4M4")):
+        want = oracle.pair_search(W.to(torch.bfloat16), c, I.scale_format(fmt_name), atoms, want_blocks=True)
+        got = gpu_search(B, W.to(torch.bfloat16), c, I.scale_format(fmt_name), atoms)
+        assert want["block_cos"][0, 0] == np.float32(0.5 + 2.0 ** -24)
+        assert np.array_equal(got["block_cos"].view(np.uint32), want["block_cos"].view(np.uint32))
+    # E2M3 under the layer scale 1/4: (1, 2^-7) is (4, 2^-5) and reconstructs as (4, 0)
+    W, c = torch.zeros(2, 16), np.ones(16, np.float32)
+    W[:, 0], W[:, 4], c[0], c[4] = 1.0, 2.0 ** -7, 1.0 / 16.0, 2.0 ** 14 * (4.0 - 1.0 / 16.0 - 2.0 ** -22)
+    pot = I.Atom("E2M3^0", 6, I.KIND_FP_E2M3, 0, I.SCOPE_LAYER_POT, 7.5)
+    want = oracle.pair_search(W.to(torch.bfloat16), c, I.scale_format("UE4M4"), [pot], want_blocks=True)
+    got = gpu_search(B, W.to(torch.bfloat16), c, I.scale_format("UE4M4"), [pot])
+    assert want["block_cos"][0, 0] == np.float32((0.5 + 2.0 ** -24) / 4.0)
+    assert np.array_equal(got["block_cos"].view(np.uint32), want["block_cos"].view(np.uint32))
