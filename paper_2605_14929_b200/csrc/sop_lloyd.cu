@@ -622,9 +622,10 @@ __global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev 
 //   elements of one split cell in one tile; eight lanes take a run (neighbouring 8-byte elements), four tiles per warp and step,
 //   the next step's elements are loaded ahead.  The warps take the runs cell by cell: the sums of a cell (all of it, and the part
 //   above its threshold) stay in registers until the warp moves to the next cell, one to three times per iteration.
-//   The cells without a threshold are a matter of CTA 0: prefix sums over all cells, built once, make an entry's share the
-//   difference of two of them.  (About the origin, in FP64: the distortion is a few thousandths of the second moment, so 1e-16 of
-//   that leaves it 1e-13.)
+//   The cells without a threshold are a matter of CTA 0: prefix sums over all cells, built once, make an entry's share of the sums
+//   the difference of two of them.  Their distortion comes from the moments about the cells' centres, a cell per thread: what
+//   cancels is of the size of a cell, so elements that lie on their entries leave zero and rounding leaves nothing below it (with
+//   differences of moments about the origin a layer of seven weight values ended at -2e-13).
 //   Every CTA adds its sums to the iteration's global ones, waits (bounded) until all have and then works out the next table for
 //   itself: the sums are integers, so all get the same one and nobody has to hand it on.  A sum carries the number of CTAs that have
 //   added to it in its top byte, so that neither a fence nor an arrival stands between the additions and their readers.
@@ -653,8 +654,21 @@ struct IterSmem {
   // CTA 0: sums over the cells before r
   unsigned long long preN[SORT_ROWS + 1];
   long long preS[SORT_ROWS + 1];
-  double preA[3][SORT_ROWS + 1];
 };
+
+// CTA 0: the moments of the thread's cell.
+struct CellMoments { double a0, a1, a2; };
+
+// sum omega (u - q)^2 of the cell, q the entry that its elements belong to; zero for a cell that is walked element by element.
+__device__ __forceinline__ double cell_distortion(const IterDesc& d, const CellMoments& m, int cell) {
+  int j = 0;                                   // thresholds in lower cells (padded with SORT_ROWS from n_entries - 1 on)
+#pragma unroll
+  for (int step = 16; step >= 1; step >>= 1)
+    if (d.thr_cell[j + step - 1] < cell) j += step;
+  const double e = 256.0 * (double)d.lut[j] - (double)(cell - SORT_CHALF);
+  const double t = m.a2 - e * (2.0 * m.a1 - e * m.a0);
+  return d.thr_cell[j] == cell || t < 0.0 ? 0.0 : t * (1.0 / 65536.0);
+}
 
 __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v, unsigned lanes = 0xFFFFFFFFu) {      // modulo 2^64, by 32-bit sums of 27-bit limbs
   const unsigned a = __reduce_add_sync(lanes, (unsigned)v & 0x7FFFFFFu), b = __reduce_add_sync(lanes, (unsigned)(v >> 27) & 0x7FFFFFFu),
@@ -735,7 +749,7 @@ __device__ void new_table(IterSmem& S, unsigned long long n, long long sv) {
 // The whole CTA: adds its share of one iteration to the sums of that iteration and arrives.
 template <bool ALL>
 __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __restrict__ ws, IterSmem& S, const unsigned short* __restrict__ ts,
-                                                unsigned tile0, int T, int it, bool last) {
+                                                const CellMoments& mom, unsigned tile0, int T, int it, bool last) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, sub = lane >> 3, ln = lane & 7;
   constexpr int NW = ITB / 32;
   const int n_split = S.n_split, Tc = (T + 3) / 4, total = n_split * Tc;
@@ -757,6 +771,7 @@ __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __r
     for (int i = 0; i < PRE; ++i) v[i] = p0 + 8u * i < p1 ? __ldg(src + tile_slot(p0 + 8u * i)) : make_uint2(0u, 0u);
   };
   open_run(warp, l, ch);
+  if (blockIdx.x == 0 && tid < SORT_ROWS) D = cell_distortion(S.d, mom, tid);        // (the first elements are on their way)
   unsigned long long nA = 0, nH = 0;
   long long sA = 0, sH = 0;
 #pragma unroll 1
@@ -851,11 +866,6 @@ __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __r
     double dsum = 0.0;
 #pragma unroll 8
     for (int i = lane; i < ITB; i += 32) dsum += S.lane_D[i];
-    if (lo < hi) {
-      const double q = 256.0 * (double)S.d.lut[lane];
-      const double b0 = S.preA[0][hi] - S.preA[0][lo], b1 = S.preA[1][hi] - S.preA[1][lo], b2 = S.preA[2][hi] - S.preA[2][lo];
-      dsum += (b2 - q * (2.0 * b1 - q * b0)) * (1.0 / 65536.0);
-    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) dsum += __shfl_xor_sync(0xFFFFFFFFu, dsum, o);
     if (lane == 0 && dsum != 0.0) atomicAdd(&ws->accD[it], dsum);
@@ -908,39 +918,34 @@ __global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs
   }
   if (tid < 2 * LIMBS * SOP_MAX_ENTRIES) (&S.limb[0][0][0])[tid] = 0u;
   if (tid < 2 * SOP_MAX_ENTRIES) (&S.sum[0][0])[tid] = 0ull;
+  CellMoments mom = {0.0, 0.0, 0.0};
   if (blockIdx.x == 0) {
     // prefix sums over the cells, one cell per thread: inside the warps, then the warps' totals
     __shared__ unsigned long long t_n[32];
     __shared__ long long t_s[32];
-    __shared__ double t_a[3][32];
     static_assert(SORT_ROWS <= ITB, "one cell per thread");
     const bool in = tid < SORT_ROWS;
     unsigned long long n = in ? ws->cellN[tid] : 0ull;
     long long s = in ? ws->cellS[tid] : 0ll;
-    const double a0 = in ? ws->cellA[0][tid] : 0.0, a1 = in ? ws->cellA[1][tid] : 0.0, a2 = in ? ws->cellA[2][tid] : 0.0;
-    const double r = (double)(tid - SORT_CHALF);
-    double b[3] = {a0, a1 + r * a0, a2 + r * (2.0 * a1 + r * a0)};              // about the origin, in units of a cell
+    if (in) mom = {ws->cellA[0][tid], ws->cellA[1][tid], ws->cellA[2][tid]};
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned long long un = __shfl_up_sync(0xFFFFFFFFu, n, o);
       const long long us = __shfl_up_sync(0xFFFFFFFFu, s, o);
-      double ub[3];
-#pragma unroll
-      for (int x = 0; x < 3; ++x) ub[x] = __shfl_up_sync(0xFFFFFFFFu, b[x], o);
-      if (lane >= o) { n += un; s += us; b[0] += ub[0]; b[1] += ub[1]; b[2] += ub[2]; }
+      if (lane >= o) { n += un; s += us; }
     }
-    if (lane == 31) { t_n[warp] = n; t_s[warp] = s; t_a[0][warp] = b[0]; t_a[1][warp] = b[1]; t_a[2][warp] = b[2]; }
+    if (lane == 31) { t_n[warp] = n; t_s[warp] = s; }
     __syncthreads();
-    for (int w = 0; w < warp && w < 32; ++w) { n += t_n[w]; s += t_s[w]; b[0] += t_a[0][w]; b[1] += t_a[1][w]; b[2] += t_a[2][w]; }
-    if (in) { S.preN[tid + 1] = n; S.preS[tid + 1] = s; S.preA[0][tid + 1] = b[0]; S.preA[1][tid + 1] = b[1]; S.preA[2][tid + 1] = b[2]; }
-    if (tid == 0) { S.preN[0] = 0; S.preS[0] = 0; S.preA[0][0] = S.preA[1][0] = S.preA[2][0] = 0.0; }
+    for (int w = 0; w < warp && w < 32; ++w) { n += t_n[w]; s += t_s[w]; }
+    if (in) { S.preN[tid + 1] = n; S.preS[tid + 1] = s; }
+    if (tid == 0) { S.preN[0] = 0; S.preS[0] = 0; }
   }
   __syncthreads();
   if (warp == 0) split_cells(S);
   __syncthreads();
   for (int it = it0;; ++it) {
     const bool last = it == iters;
-    iteration_share<ALL>(a, ws, S, ts, tile0, T, it, last);
+    iteration_share<ALL>(a, ws, S, ts, mom, tile0, T, it, last);
     if (warp == 0) {
       bool go = true;
       unsigned long long n = 0;

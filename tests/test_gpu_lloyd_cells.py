@@ -53,7 +53,7 @@ def test_scales_that_saturate(B, k):
 
 
 def test_more_tiles_than_a_cta_keeps_the_cell_starts_of(B):
-    # 200 tiles on one iteration CTA (153 fit), in both launch forms
+    # 200 tiles on one iteration CTA (165 fit), in both launch forms
     L = I.outlier_channel_layer(44, 300, 4096, 16)
     fmt = I.scale_format("E5M6")
     atoms = I.alphabet(["NF4"])
@@ -71,3 +71,26 @@ def test_more_tiles_than_a_cta_keeps_the_cell_starts_of(B):
             assert np.allclose(got[1], want[1], rtol=REL, atol=0)
     finally:
         B.dd4_lloyd_tuning()
+
+
+def _levels(seed, M, K):
+    """Weights of seven values per block (bf16 times a power of two), channel norms over many orders of magnitude."""
+    g = torch.Generator().manual_seed(seed)
+    v = torch.tensor([-256.0, -179.0, -77.0, 0.0, 77.0, 179.0, 256.0])[torch.randint(0, 7, (M, K // 16, 16), generator=g)] / 256.0
+    v[..., 0] = 1.0
+    W = (v * 2.0 ** torch.randint(-6, -2, (M, K // 16, 1), generator=g)).reshape(M, K).to(torch.bfloat16)
+    return W, torch.exp(2.5 * torch.randn(K, generator=g)).numpy()
+
+
+@pytest.mark.parametrize("per_iteration", [False, True])
+def test_elements_on_their_entries_leave_no_distortion(B, per_iteration):
+    # the table finds the seven values: the distortion is zero then, and rounding must not take it below (a negative last entry is the
+    # mark of a call that did not finish)
+    fmt, atoms = I.scale_format("E5M6"), I.alphabet(["NF4"])
+    for seed in range(6):
+        W, c = _levels(seed, 256, 1024)
+        NB = W.numel() // 16
+        bc = torch.rand(2, NB, generator=torch.Generator().manual_seed(seed)).to(dev())
+        lut, dist, _ = gpu_lloyd(B, W, c, fmt, atoms, bc, NB // 2, 8, 0, 0, launch_per_iteration=per_iteration)
+        assert set(np.array([-256, -179, -77, 0, 77, 179, 256], np.float32) / 256) <= set(lut[:16])
+        assert (dist >= 0).all() and dist[8] == 0.0, dist
