@@ -261,7 +261,9 @@ int sop_profile_last_sweep_ms(float* ms);   /* = sop_profile_last_ms(SOP_PROFILE
  *       nearest to S / H (clamped to +-1.25) and its cost Q - 2 q S + q^2 H in FP64; a dynamic programme finds the
  *       cut of least total cost (ties to the earliest cut).  iters must be 0; out_lut_dev receives the code points in
  *       ascending order (padded with the last one when there are fewer cells than entries) and distortion_dev[0]
- *       the least total cost.  With fmta_index = SOP_FMTA_FROM_RESULT every table atom must have the same n_entries.
+ *       the least total cost (of integer sums rounded element by element: where a cut costs nothing they may leave it
+ *       a little below zero; nothing waits in this construction, and -1 itself marks a call that did not run).
+ *       With fmta_index = SOP_FMTA_FROM_RESULT every table atom must have the same n_entries.
  *   k_mode: a shift in [-64, 64], or SOP_K_FROM_RESULT to use search_dev->k[fmta].
  *   out_lut_dev: SOP_MAX_ENTRIES floats (first n_entries valid, ascending).
  *   distortion_dev: iters + 1 doubles, sum omega (u - q)^2 before each update and after the last.
@@ -269,7 +271,8 @@ int sop_profile_last_sweep_ms(float* ms);   /* = sop_profile_last_ms(SOP_PROFILE
  *     distortion (never negative) by the closing iteration.  When the iterations run in one launch, its CTAs
  *     wait for one another between iterations; every wait is bounded (about half a second).  A CTA that gives
  *     up makes all of them leave and the last entry stays (or is set back to) -1: the table is then not valid.
- *     A caller reads distortion_dev[iters] after synchronising and treats a negative value as a failed call.
+ *     A caller reads distortion_dev[iters] after synchronising and treats a negative value as a failed call
+ *     (with SOP_LLOYD_GRID_DP: the value -1).
  *   pool_count_dev: one long long, number of blocks in the pool.
  * Workspace: 8 bytes per weight element (u and omega of every pool element are kept across the
  *   iterations), 4 bytes per block (the pool list) and 4 bytes per channel, plus a fixed header (2 MB). */

@@ -178,11 +178,13 @@ class LloydNotFinished(RuntimeError):
     never ran to its end), so the codebook it wrote must not be used."""
 
 
-def check_lloyd_status(distortion: torch.Tensor, iters: int) -> None:
+def check_lloyd_status(distortion: torch.Tensor, iters: int, grid_dp: bool = False) -> None:
     """Reads the status entry ``distortion[iters]`` of a finished (synchronised) ``sop_dd4_lloyd`` call and
-    raises ``LloydNotFinished`` when it is negative."""
-    if float(distortion[iters].item()) < 0.0:
-        raise LloydNotFinished(f"sop_dd4_lloyd did not finish: distortion[{iters}] = {float(distortion[iters].item())}")
+    raises ``LloydNotFinished`` when it is negative.  With ``grid_dp`` the entry is a least cost of rounded integer
+    sums, which a cut that costs nothing may leave a little below zero: only -1 itself is the mark then."""
+    status = float(distortion[iters].item())
+    if status == -1.0 if grid_dp else status < 0.0:
+        raise LloydNotFinished(f"sop_dd4_lloyd did not finish: distortion[{iters}] = {status}")
 
 
 def alloc_workspace(nbytes: int, device) -> torch.Tensor:

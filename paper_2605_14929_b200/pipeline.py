@@ -266,7 +266,7 @@ class LayerSweep:
     def outputs(self) -> SweepOutputs:
         torch.cuda.synchronize(self.dev)
         if self.iters > 0:
-            B.check_lloyd_status(self.distortion, self.dd_iters)  # a codebook from an unfinished call is not handed out
+            B.check_lloyd_status(self.distortion, self.dd_iters, self.grid_dp)  # a codebook from an unfinished call is not handed out
         nF, nR = len(self.full_atoms), len(self.rom_atoms)
         return SweepOutputs(
             c=self.c.cpu(), pair_table=B.read_pair_table(self.pair_table, nF),
@@ -386,7 +386,7 @@ class LayerStream:
         self.out_done[slot].synchronize()
         for f, q in enumerate(self.sweeps):
             if q.iters > 0:
-                B.check_lloyd_status(self.host_out[slot][f]["distortion"], q.dd_iters)
+                B.check_lloyd_status(self.host_out[slot][f]["distortion"], q.dd_iters, q.grid_dp)
         return self.host_out[slot][0] if self.single else self.host_out[slot]
 
 
@@ -443,4 +443,4 @@ class LayerSetSweep:
         for row in self.sweeps:
             for sw in row:
                 if sw.iters > 0:
-                    B.check_lloyd_status(sw.distortion, sw.dd_iters)
+                    B.check_lloyd_status(sw.distortion, sw.dd_iters, sw.grid_dp)

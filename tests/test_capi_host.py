@@ -162,6 +162,17 @@ def test_lloyd_status_entry_is_read_on_the_host(lib):
     B.check_lloyd_status(d, 1)
 
 
+def test_a_cost_that_rounds_below_zero_is_no_failure(lib):
+    # the dynamic programme's least cost is one of rounded integer sums: only -1 marks a call that did not run
+    import torch
+    d = torch.tensor([-1.124e-05], dtype=torch.float64)
+    B.check_lloyd_status(d, 0, grid_dp=True)
+    with pytest.raises(B.LloydNotFinished):
+        B.check_lloyd_status(d, 0)
+    with pytest.raises(B.LloydNotFinished):
+        B.check_lloyd_status(torch.tensor([-1.0], dtype=torch.float64), 0, grid_dp=True)
+
+
 def test_lloyd_tuning_ranges(lib):
     assert lib.sop_dd4_lloyd_tuning(0, 0, 4, 0) == -7 and lib.sop_dd4_lloyd_tuning(129, 0, 4, 0) == -7
     assert lib.sop_dd4_lloyd_tuning(128, -1, 4, 0) == -7 and lib.sop_dd4_lloyd_tuning(128, 0, 4, -1) == -7

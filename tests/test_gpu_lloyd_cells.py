@@ -94,3 +94,14 @@ def test_elements_on_their_entries_leave_no_distortion(B, per_iteration):
         lut, dist, _ = gpu_lloyd(B, W, c, fmt, atoms, bc, NB // 2, 8, 0, 0, launch_per_iteration=per_iteration)
         assert set(np.array([-256, -179, -77, 0, 77, 179, 256], np.float32) / 256) <= set(lut[:16])
         assert (dist >= 0).all() and dist[8] == 0.0, dist
+
+
+def test_a_layer_whose_least_cost_rounds_below_zero_is_handed_out(B):
+    from paper_2605_14929_b200.pipeline import LayerSweep
+    below = 0
+    for seed in range(6):
+        W, c = _levels(seed, 256, 1024)
+        sw = LayerSweep(256, 1024, 2, I.scale_format("E5M6"), ["NF4"], device=dev(), grid_dp=True)
+        sw.run(W.to(dev()), torch.from_numpy(np.stack([c, c])).to(dev()))
+        below += sw.outputs().distortion[0] < 0
+    assert below          # the sums of some of these layers round below zero
