@@ -891,6 +891,10 @@ __global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArg
 // tail of the last CTA (see finalize_body): 256 x 1024 takes 11 us, 16 us with the serial tail.
 // ---------------------------------------------------------------------------------------------
 constexpr int RUNIT = 128;            // blocks of a run: four per lane
+constexpr int RED_UNITS = 6;          // runs of a tile, at most
+// A lane counts its blocks in 12 bits until they are folded away: after every 128 tiles, of which it sees at most 24 blocks each.
+constexpr unsigned COUNT_TILES = 128;
+static_assert(COUNT_TILES * RED_UNITS * (RUNIT / 32) < 4096, "a lane's counts fit 12 bits");
 constexpr int MAX_STAGE = 4;          // tile buffers of the ring
 
 __device__ void finalize_body(const LayerArgs& L, const RedPlan& P, int grid, PartialSums partials, unsigned char* smem, sop_pair_stat* pair_table,
@@ -1032,91 +1036,98 @@ __device__ __forceinline__ void reduce_run(const ReduceCtx& X, const BundleDev& 
 #pragma unroll
     for (int q = 0; q < NE; ++q) { dg[q] += (double)g[q]; de[q] += (double)e[q]; g[q] = e[q] = 0.0f; }
   };
+  if (lane < BUNDLE_ENT) part->counts[lane] = make_uint2(0u, 0u);
   int stage = 0, run = k, half = 0;                 // run: of this tile, counted from its first
   unsigned parity = 0;
   const unsigned last_full = (unsigned)(X.NB / (X.units * RUNIT));      // tiles below this one are whole
-  for (unsigned t = 0; t < X.n_tiles; ++t) {
-    mbar_wait(X.full + 8u * stage, parity, X.hdr);
-    const float* buf = X.ring + (size_t)stage * (2 * X.n_cols) * row_len;
-    const long long tile = (long long)blockIdx.x + (long long)t * gridDim.x;
-    const int live = tile < last_full ? 1 << 30 : (int)(X.NB - tile * (X.units * RUNIT));       // blocks of this tile
 #pragma unroll 1
-    for (; run < X.units; run += nk) {
+  for (unsigned t = 0; t < X.n_tiles;) {
+    const unsigned t_end = min(t + COUNT_TILES, X.n_tiles);
 #pragma unroll 1
-      for (int h = 0; h < 4 / BL; ++h) {
-        const int at = run * RUNIT + h * (32 * BL);
-        const float* bu = buf + at;
-        float c[NC][BL], er[NC][BL], va[NC][BL];
+    for (; t < t_end; ++t) {
+      mbar_wait(X.full + 8u * stage, parity, X.hdr);
+      const float* buf = X.ring + (size_t)stage * (2 * X.n_cols) * row_len;
+      const long long tile = (long long)blockIdx.x + (long long)t * gridDim.x;
+      const int live = tile < last_full ? 1 << 30 : (int)(X.NB - tile * (X.units * RUNIT));       // blocks of this tile
+#pragma unroll 1
+      for (; run < X.units; run += nk) {
+#pragma unroll 1
+        for (int h = 0; h < 4 / BL; ++h) {
+          const int at = run * RUNIT + h * (32 * BL);
+          const float* bu = buf + at;
+          float c[NC][BL], er[NC][BL], va[NC][BL];
 #pragma unroll
-        for (int i = 0; i < NC; ++i) {
-          load(bu, col[SGN ? 2 * i : i], 0, c[i]);
-          load(bu, col[SGN ? 2 * i : i], 1, er[i]);
-          if constexpr (SGN) {
-            float mc[BL], me[BL];
-            load(bu, col[2 * i + 1], 0, mc);
-            load(bu, col[2 * i + 1], 1, me);
+          for (int i = 0; i < NC; ++i) {
+            load(bu, col[SGN ? 2 * i : i], 0, c[i]);
+            load(bu, col[SGN ? 2 * i : i], 1, er[i]);
+            if constexpr (SGN) {
+              float mc[BL], me[BL];
+              load(bu, col[2 * i + 1], 0, mc);
+              load(bu, col[2 * i + 1], 1, me);
 #pragma unroll
-            for (int r = 0; r < BL; ++r) {
-              const bool neg = SEL_ERR ? me[r] < er[i][r] : mc[r] > c[i][r];                    // ties to the atom
-              c[i][r] = neg ? mc[r] : c[i][r]; er[i][r] = neg ? me[r] : er[i][r]; va[i][r] = neg ? NEG : 0.0f;
+              for (int r = 0; r < BL; ++r) {
+                const bool neg = SEL_ERR ? me[r] < er[i][r] : mc[r] > c[i][r];                    // ties to the atom
+                c[i][r] = neg ? mc[r] : c[i][r]; er[i][r] = neg ? me[r] : er[i][r]; va[i][r] = neg ? NEG : 0.0f;
+              }
+            } else {
+#pragma unroll
+              for (int r = 0; r < BL; ++r) va[i][r] = 0.0f;
             }
-          } else {
-#pragma unroll
-            for (int r = 0; r < BL; ++r) va[i][r] = 0.0f;
           }
-        }
-        if (at + 32 * BL > live) {                   // blocks beyond the layer: cosine 1, error 0
+          if (at + 32 * BL > live) {                   // blocks beyond the layer: cosine 1, error 0
 #pragma unroll
-          for (int i = 0; i < NC; ++i)
+            for (int i = 0; i < NC; ++i)
 #pragma unroll
-            for (int r = 0; r < BL; ++r)
-              if (at + lane0 + (VEC ? r : 32 * r) >= live) { c[i][r] = 1.0f; er[i][r] = va[i][r] = 0.0f; }
-        }
+              for (int r = 0; r < BL; ++r)
+                if (at + lane0 + (VEC ? r : 32 * r) >= live) { c[i][r] = 1.0f; er[i][r] = va[i][r] = 0.0f; }
+          }
 #pragma unroll
-        for (int r = 0; r < BL; ++r) {
-          float gp[NC];
+          for (int r = 0; r < BL; ++r) {
+            float gp[NC];
 #pragma unroll
-          for (int i = 0; i < NC; ++i) gp[i] = __fsub_rn(1.0f, c[i][r]);
-          int q = 0;
-          if (SHAPE < 2) {
-#pragma unroll
-            for (int i = 0; i < NA; ++i, ++q) {
-              g[q] = __fadd_rn(g[q], gp[i]); e[q] = __fadd_rn(e[q], er[i][r]);
-              if (SGN) n[q] = __fadd_rn(n[q], va[i][r]);
-            }
-#pragma unroll
-            for (int i = 0; i < NA; ++i)
-#pragma unroll
-              for (int j = i + 1; j < NA; ++j, ++q)
-                entry_add<SEL_ERR, SGN>(g[q], e[q], n[q], c[i][r], c[j][r], gp[i], gp[j], er[i][r], er[j][r], va[i][r], SGN ? __fadd_rn(va[j][r], 1.0f) : 1.0f);
-          } else {
-#pragma unroll
-            for (int j = NA; j < NC; ++j)
+            for (int i = 0; i < NC; ++i) gp[i] = __fsub_rn(1.0f, c[i][r]);
+            int q = 0;
+            if (SHAPE < 2) {
 #pragma unroll
               for (int i = 0; i < NA; ++i, ++q) {
-                const int x = SHAPE == 4 ? j : i, y = SHAPE == 4 ? i : j;        // first and second candidate
-                entry_add<SEL_ERR, SGN>(g[q], e[q], n[q], c[x][r], c[y][r], gp[x], gp[y], er[x][r], er[y][r], va[x][r], SGN ? __fadd_rn(va[y][r], 1.0f) : 1.0f);
+                g[q] = __fadd_rn(g[q], gp[i]); e[q] = __fadd_rn(e[q], er[i][r]);
+                if (SGN) n[q] = __fadd_rn(n[q], va[i][r]);
               }
+#pragma unroll
+              for (int i = 0; i < NA; ++i)
+#pragma unroll
+                for (int j = i + 1; j < NA; ++j, ++q)
+                  entry_add<SEL_ERR, SGN>(g[q], e[q], n[q], c[i][r], c[j][r], gp[i], gp[j], er[i][r], er[j][r], va[i][r], SGN ? __fadd_rn(va[j][r], 1.0f) : 1.0f);
+            } else {
+#pragma unroll
+              for (int j = NA; j < NC; ++j)
+#pragma unroll
+                for (int i = 0; i < NA; ++i, ++q) {
+                  const int x = SHAPE == 4 ? j : i, y = SHAPE == 4 ? i : j;        // first and second candidate
+                  entry_add<SEL_ERR, SGN>(g[q], e[q], n[q], c[x][r], c[y][r], gp[x], gp[y], er[x][r], er[y][r], va[x][r], SGN ? __fadd_rn(va[y][r], 1.0f) : 1.0f);
+                }
+            }
           }
         }
+        half ^= 1;
+        if (!half) fold_sums();                        // eight blocks per lane
       }
-      half ^= 1;
-      if (!half) fold_sums();                        // eight blocks per lane
+      run -= X.units;
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(X.empty + 8u * stage) : "memory");
+      if (++stage == X.n_stage) { stage = 0; parity ^= 1u; }
     }
-    run -= X.units;
-    __syncwarp();
-    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(X.empty + 8u * stage) : "memory");
-    if (++stage == X.n_stage) { stage = 0; parity ^= 1u; }
+    // the lanes' counts go to the CTA's (lane q keeps those of entry q)
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      const unsigned c = __float2uint_rn(n[q]);                // exact: below 2^24
+      const unsigned a = __reduce_add_sync(0xFFFFFFFFu, SGN ? c & 4095u : c), b = SGN ? __reduce_add_sync(0xFFFFFFFFu, c >> 12) : 0u;
+      if (lane == q) { part->counts[q].x += a; part->counts[q].y += b; }
+      n[q] = 0.0f;
+    }
   }
   fold_sums();
-  unsigned n1 = 0, nn = 0, slot = 255;
-#pragma unroll
-  for (int q = 0; q < NE; ++q) {
-    const unsigned c = __float2uint_rn(n[q]);                  // exact: below 2^24
-    const unsigned a = __reduce_add_sync(0xFFFFFFFFu, SGN ? c & 4095u : c), b = SGN ? __reduce_add_sync(0xFFFFFFFFu, c >> 12) : 0u;
-    if (lane == q) { n1 = a; nn = b; slot = k == 0 ? B.slot[q] : 255u; }
-  }
-  if (lane < BUNDLE_ENT) { part->counts[lane] = make_uint2(n1, nn); part->slot[lane] = (unsigned char)slot; }
+  if (lane < BUNDLE_ENT) part->slot[lane] = lane < NE && k == 0 ? B.slot[lane] : (unsigned char)255;
   if (lane == 0) part->n_warps = nk;
   const int q = lane_sums<NE>(dg, lane);
   lane_sums<NE>(de, lane);
@@ -1556,6 +1567,14 @@ static void deal_bundles(const BundleDev* b, int n, BundlesDev* Q) {
   Q->n_warps = at;
 }
 
+// Tiles of 768 blocks, of 256 where those would leave SMs without one; at most one CTA per SM, and never more than the workspace has
+// partials for.
+static long long reduce_grid(long long NB, int sms, int* units) {
+  *units = NB >= (long long)sms * RED_UNITS * RUNIT ? RED_UNITS : 2;
+  const long long n_tiles = (NB + *units * RUNIT - 1) / (*units * RUNIT), most = sms < MAX_GRID ? sms : MAX_GRID;
+  return n_tiles < most ? n_tiles : most;
+}
+
 // the ring of tile buffers; at least the room the closing reduction of the last CTA needs
 static size_t reduce_smem_bytes(int n_cols, int units, int n_stage) {
   const size_t ring = (size_t)n_stage * n_cols * 2 * (units * RUNIT + 4) * sizeof(float);
@@ -1682,17 +1701,13 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   const long long min_grid = (L.nbk + tba - 1) / tba;
   if (grid < min_grid) grid = min_grid;
   if (grid > MAX_GRID) return SOP_ERR_SHAPE;
-  // the reduction: up to fifteen bundles per launch; persistent grid over tiles of 768 blocks, 256 where those would leave SMs
-  // without one.  16-byte copies need 16-byte aligned column starts and runs: a block count that is a multiple of four.
+  // the reduction: up to fifteen bundles per launch; persistent grid over its tiles.  16-byte copies need 16-byte aligned column starts and runs: a block count that is a multiple of four.
   std::vector<BundleDev> bundles;
   build_bundles(Rp, &bundles);
   const int n_launch = bundles.empty() ? 1 : (int)((bundles.size() + MAX_BUNDLES - 1) / MAX_BUNDLES);
   const bool vec = (L.NB % 4) == 0 && (((uintptr_t)cos_cols | (uintptr_t)sse_cols) & 15u) == 0;
-  const int units = L.NB >= (long long)sms * 6 * RUNIT ? 6 : 2;
-  const long long n_tiles = (L.NB + units * RUNIT - 1) / (units * RUNIT);
-  long long rgrid = n_tiles < (long long)sms ? n_tiles : (long long)sms;
-  // a lane counts its blocks in 12 bits: at most 4095 of them even where a bundle has one warp only
-  while (((n_tiles + rgrid - 1) / rgrid) * units * (RUNIT / 32) > 4095) ++rgrid;
+  int units = 0;
+  const long long rgrid = reduce_grid(L.NB, sms, &units);
 
   // the prepass adds to its histograms; the reduction's counters are cleared by the sweep where there is one
   if (!k_from_result && !reuse_prepass) SOP_CUDA_TRY(clear(ws, ws_part_off(), st));

@@ -67,3 +67,45 @@ def test_table_entries_match_the_per_block_values(B, M, K, rom, fp, by_error):
                     gap = 1.0 - wc.astype(np.float64)
                     assert abs((1.0 - got["acos"]) - gap.mean()) <= TOL * np.abs(gap).mean() + 4e-16, (a, b)
                     assert got["mse"] == pytest.approx(we.astype(np.float64).sum() / (M * K), rel=TOL), (a, b)
+
+
+# more blocks than a lane of the reduction counts in 12 bits at one CTA per SM: with two candidates where as many CTAs as 12 bits
+# ask for would not find room in the workspace (137,871,360 blocks), with sixteen where a warp has a bundle for itself
+@pytest.mark.parametrize("M,K,tables", [(135300, 16384, 1), (20500, 16384, 8)])
+def test_more_blocks_than_a_lane_counts_at_once(B, M, K, tables):
+    rng = np.random.default_rng(4)
+    bases = [I.rom_atom("NF4")] + [I.Atom(f"r{i}", 4, I.KIND_LUT, 0, 16, 1.0, np.sort(np.concatenate([[-1.0, 1.0], I.snap_bf16(rng.uniform(-0.95, 0.95, 14))]).astype(np.float32)))
+                                   for i in range(tables - 1)]
+    atoms = [x for a in bases for x in (a, a.negation())]
+    A, NB = len(atoms), M * K // 16
+    W = torch.randn((M, K), dtype=torch.bfloat16, device=dev(), generator=torch.Generator(device=dev()).manual_seed(1))
+    c = torch.rand(K, device=dev(), generator=torch.Generator(device=dev()).manual_seed(2)) + 0.1
+    pt, st, res = B.new_pair_table(A, dev()), B.new_pair_table(A, dev()), B.new_result(dev())
+    bc, bs = torch.empty((A, NB), device=dev()), torch.empty((A, NB), device=dev())
+    need = B.pair_search_workspace(M, K, A)
+    ws = B.alloc_workspace(need + (1 << 22), dev())
+    ws[need:] = 0x5A
+    B.sop_pair_search(W, c, I.scale_format("E5M6"), atoms, pt, st, res, ws, block_cos=bc, block_sse=bs)
+    P, S = B.read_pair_table(pt, A), B.read_pair_table(st, A)
+    assert bool((ws[need:] == 0x5A).all())
+
+    def entry(got, mu, x, y, n1, nn):
+        cos = torch.where(mu, bc[y], bc[x])
+        assert (got["n_sel1"], got["n_neg"]) == (n1, nn)
+        assert abs(got["acos"] - float(cos.double().mean())) <= TOL * (1.0 - got["acos"]) + 1e-15
+        assert got["mse"] == pytest.approx(float(torch.where(mu, bs[y], bs[x]).double().sum()) / (M * K), rel=TOL)
+    for x in range(A):
+        entry(P[x, x], torch.zeros(1, dtype=torch.bool, device=dev()), x, x, 0, 0)
+        for y in range(x + 1, A):
+            mu = bc[y] > bc[x]
+            if y == x + 1 or tables == 1:
+                entry(P[x, y], mu, x, y, int(mu.sum()), 0)
+            else:
+                assert P[x, y]["n_sel1"] == int(mu.sum())
+    for x in range(0, A, 2):
+        neg = bc[x + 1] > bc[x]
+        entry(S[x, x], neg, x, x + 1, 0, int(neg.sum()))
+        for y in range(x + 2, A, 2):
+            negy = bc[y + 1] > bc[y]
+            mu = torch.maximum(bc[y], bc[y + 1]) > torch.maximum(bc[x], bc[x + 1])
+            assert (S[x, y]["n_sel1"], S[x, y]["n_neg"]) == (int(mu.sum()), int(torch.where(mu, negy, neg).sum()))
