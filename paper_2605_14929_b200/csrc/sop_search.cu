@@ -345,7 +345,7 @@ constexpr int SLOW_STEPS = 8;                        // a binary search over at 
 
 // Shared-memory scratch: while the tables are built, the candidates' values and decision points; for the sweep the merged
 // decision points (for a group that is searched).
-struct __align__(16) ColumnPtr { char *cos, *sse; };      // a candidate's columns
+struct __align__(16) ColumnPtr { float *cos, *sse; };      // a candidate's columns
 struct GroupScratch {
   ColumnPtr col[SOP_MAX_CLASSES][GROUP_CAND];
   float vals[GROUP_CAND][32];          // the values of a candidate, in ascending order of u
@@ -517,7 +517,7 @@ struct SweepCtx {
   // blocks
   const uint16_t* w0;
   long long w_step;
-  unsigned n_rows, off0, off_step; // this thread's blocks, the byte offset of the first in a column, the step
+  unsigned n_rows, blk0, blk_step; // this thread's blocks, the number of the first, the step (31 bits: widened where a column is indexed)
   unsigned n_iter;                 // blocks of the thread that has the most
 
   __device__ __forceinline__ void scale(float amax, const FmtDev& F, float& s_hat, float& rcp) const {
@@ -616,10 +616,10 @@ __device__ __forceinline__ void sweep_emit(float nw, float2 (&nq)[NP], float2 (&
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const ColumnPtr a = cols[2 * p], b = cols[2 * p + 1];          // (the last candidate again where their number is odd)
-      *reinterpret_cast<float*>(a.cos + at) = dot[p].x;
-      *reinterpret_cast<float*>(a.sse + at) = sse[p].x;
-      *reinterpret_cast<float*>(b.cos + at) = dot[p].y;
-      *reinterpret_cast<float*>(b.sse + at) = sse[p].y;
+      a.cos[at] = dot[p].x;
+      a.sse[at] = sse[p].x;
+      b.cos[at] = dot[p].y;
+      b.sse[at] = sse[p].y;
     }
   }
 }
@@ -638,7 +638,7 @@ __device__ __forceinline__ void sweep_group(const SweepCtx& X, const FmtDev& F, 
   const unsigned plane_bytes = G.plane_bytes;
   const float inv_range = G.inv_range, n_cells = (float)G.n_cells;
   const uint16_t* wp = X.w0;
-  unsigned at = X.off0;
+  unsigned at = X.blk0;
   uint32_t wn[8];
   load_block_bits(wp, wn);
 #pragma unroll 1
@@ -701,7 +701,7 @@ __device__ __forceinline__ void sweep_group(const SweepCtx& X, const FmtDev& F, 
         sweep_emit<LAST>(nw, nq, dot, sse, cols + 2 * b, at, it < X.n_rows);
       }
     }
-    at += X.off_step;
+    at += X.blk_step;
   }
 }
 
@@ -716,7 +716,7 @@ template <int MODE, bool PAIRED>
 __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F, const ClassDev& K, size_t NB, float* __restrict__ block_cos,
                                              float* __restrict__ block_sse) {
   const uint16_t* wp = X.w0;
-  unsigned at = X.off0;
+  unsigned at = X.blk0;
   const int n_cand = K.n_cand;
   uint32_t wn[8];
   load_block_bits(wp, wn);
@@ -766,11 +766,11 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
     const float cosv = x >= COS_LO && x <= COS_HI && all_ones_root(x) && fabsf(dots) >= COS_DOT ? cosine_one(-x, dots) : block_cosine_any(nw, nqs, dots);
     if (it < X.n_rows)
       for (int ci = 0; ci < n_cand; ++ci) {      // (candidates of one format and scale have the same values)
-        const size_t col = (size_t)K.cand[ci] * NB + (at >> 2);
+        const size_t col = (size_t)K.cand[ci] * NB + at;
         block_cos[col] = cosv;
         block_sse[col] = err;
       }
-    at += X.off_step;
+    at += X.blk_step;
   }
 }
 
@@ -806,11 +806,11 @@ __global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArg
   X.n_rows = r0 < R && r0 < M ? (M - r0 + R - 1) / R : 0u;
   X.w0 = L.W + (size_t)j * SOP_G + (long long)min(r0, M - 1) * L.ldw;
   X.w_step = (long long)R * L.ldw;
-  X.off0 = (r0 * nbk + j) * 4u;                                  // at most 2^27 blocks
-  X.off_step = R * nbk * 4u;
+  X.blk0 = r0 * nbk + j;
+  X.blk_step = R * nbk;
   for (int i = tid; i < P.n_groups * GROUP_CAND; i += TB) {
     const size_t at = (size_t)P.groups[i / GROUP_CAND].cand[i % GROUP_CAND] * (size_t)L.NB;
-    S.col[i / GROUP_CAND][i % GROUP_CAND] = {reinterpret_cast<char*>(block_cos + at), reinterpret_cast<char*>(block_sse + at)};
+    S.col[i / GROUP_CAND][i % GROUP_CAND] = {block_cos + at, block_sse + at};
   }
   {
     const float4* cp = reinterpret_cast<const float4*>(L.c + (size_t)j * SOP_G);

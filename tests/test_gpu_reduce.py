@@ -109,3 +109,31 @@ def test_more_blocks_than_a_lane_counts_at_once(B, M, K, tables):
             negy = bc[y + 1] > bc[y]
             mu = torch.maximum(bc[y], bc[y + 1]) > torch.maximum(bc[x], bc[x + 1])
             assert (S[x, y]["n_sel1"], S[x, y]["n_neg"]) == (int(mu.sum()), int(torch.where(mu, negy, neg).sum()))
+
+
+@pytest.mark.parametrize("kind", ["NF4", "E4M3"])
+def test_blocks_beyond_two_to_the_thirty(B, kind):
+    # the byte offset of a block in a column passes 32 bits: only a few rows hold weights, among them some beyond 2^30, and each must
+    # get its own value (43 GB)
+    M, K = (1 << 30) + 64, 16
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 60 GB of device memory")
+    rows = torch.tensor([0, 1, 5, 63, 64, (1 << 29) + 3, (1 << 30) - 1, 1 << 30, (1 << 30) + 1, (1 << 30) + 5, (1 << 30) + 63], device=dev())
+    few = torch.randn((len(rows), K), device=dev(), generator=torch.Generator(device=dev()).manual_seed(7)).to(torch.bfloat16)
+    W = torch.zeros((M, K), dtype=torch.bfloat16, device=dev())
+    W[rows] = few
+    c = torch.rand(K, device=dev(), generator=torch.Generator(device=dev()).manual_seed(8)) + 0.1
+    atoms, out = [I.rom_atom("NF4") if kind == "NF4" else I.fp_atom("E4M3")], []
+    for Wx in (few, W):
+        NB = Wx.shape[0]
+        pt, st, res = B.new_pair_table(1, dev()), B.new_pair_table(1, dev()), B.new_result(dev())
+        bc, bs = torch.full((1, NB), -7.0, device=dev()), torch.full((1, NB), -7.0, device=dev())
+        B.sop_pair_search(Wx, c, I.scale_format("E8M7"), atoms, pt, st, res, B.alloc_workspace(B.pair_search_workspace(NB, K, 1), dev()),
+                          k_mode=0, block_cos=bc, block_sse=bs)
+        out.append((bc, bs))
+    for small, large in zip(*out):
+        assert torch.equal(large[0, rows], small[0])
+    rest = torch.ones(M, dtype=torch.bool, device=dev())
+    rest[rows] = False
+    assert bool((out[1][0][0][rest] == 1.0).all()) and not bool(out[1][1][0][rest].any())           # zero blocks: cosine 1, error 0
+    assert B.read_pair_table(pt, 1)[0, 0]["mse"] == pytest.approx(float(out[0][1].double().sum()) / (M * K), rel=TOL)
