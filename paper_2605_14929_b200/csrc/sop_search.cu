@@ -1151,7 +1151,8 @@ __global__ void __launch_bounds__(RTB, 1) reduce_kernel(LayerArgs L, RedPlan P, 
   X.NB = L.NB; X.n_cols = Q.n_cols; X.units = units; X.n_stage = n_stage;
   X.row_len = units * RUNIT + (VEC ? 0 : 4);
   const unsigned tiles = (unsigned)((L.NB + units * RUNIT - 1) / (units * RUNIT));
-  X.n_tiles = blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
+  // (no entry to form: no columns, no warp that would hand a buffer back, nothing to copy)
+  X.n_tiles = Q.n_warps && blockIdx.x < tiles ? (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
   X.ring = reinterpret_cast<const float*>(smem);
   X.full = smem_u32(s_bar); X.empty = X.full + 8u * MAX_STAGE;
   X.row_off = s_off; X.hdr = hdr;
@@ -1161,7 +1162,7 @@ __global__ void __launch_bounds__(RTB, 1) reduce_kernel(LayerArgs L, RedPlan P, 
     s_off[tid] = tid * X.row_len + (int)((a & 15u) >> 2);      // (tiles are multiples of four blocks)
   }
   if (tid == 0) {
-    for (int i = 0; i < n_stage; ++i) {
+    for (int i = 0; i < n_stage && Q.n_warps; ++i) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(X.full + 8u * i) : "memory");
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(X.empty + 8u * i), "r"(Q.n_warps) : "memory");
     }

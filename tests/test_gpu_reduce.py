@@ -111,6 +111,26 @@ def test_more_blocks_than_a_lane_counts_at_once(B, M, K, tables):
             assert (S[x, y]["n_sel1"], S[x, y]["n_neg"]) == (int(mu.sum()), int(torch.where(mu, negy, neg).sum()))
 
 
+@pytest.mark.parametrize("M,K", [(3, 64), (2048, 4096)])
+def test_a_call_that_forms_no_entry_keeps_the_tables(B, M, K):
+    # every candidate loaded and every entry kept: the call closes over what an earlier one left (more than four tiles per CTA)
+    L = I.student_layer(6, 0, M, K, 4, 4.0, device="cuda")
+    atoms = I.alphabet(["NF4", "SH4"], fp=["E2M3"])
+    A, NB = len(atoms), M * K // 16
+    c = torch.rand(K, device=dev()) + 0.1
+    pt, st, res, again = B.new_pair_table(A, dev()), B.new_pair_table(A, dev()), B.new_result(dev()), B.new_result(dev())
+    bc, bs = torch.empty((A, NB), device=dev()), torch.empty((A, NB), device=dev())
+    ws = B.alloc_workspace(B.pair_search_workspace(M, K, A), dev())
+    B.sop_pair_search(L.W, c, I.scale_format("E5M6"), atoms, pt, st, res, ws, block_cos=bc, block_sse=bs)
+    before = [t.clone() for t in (pt, st, bc, bs)]
+    for kw in (dict(k_mode=B.K_FROM_RESULT, prev_result=res), dict()):
+        again.zero_()
+        B.sop_pair_search(L.W, c, I.scale_format("E5M6"), atoms, pt, st, again, ws, block_cos=bc, block_sse=bs, eval_mask=0,
+                          load_mask=(1 << A) - 1, keep_loaded=True, **kw)
+        assert all(torch.equal(x, y) for x, y in zip(before, (pt, st, bc, bs)))
+        assert torch.equal(again, res)
+
+
 @pytest.mark.parametrize("kind", ["NF4", "E4M3"])
 def test_blocks_beyond_two_to_the_thirty(B, kind):
     # the byte offset of a block in a column passes 32 bits: only a few rows hold weights, among them some beyond 2^30, and each must
