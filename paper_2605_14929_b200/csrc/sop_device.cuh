@@ -48,7 +48,9 @@ int profile_mark(int which, int edge, cudaStream_t st);
 // dependent launch): a pass is a chain of twenty short kernels, and the time from the end of one to the start of the next was a
 // sixth of a small layer's pass.  Rules that each kernel keeps: pdl_trigger() first (its successor may then be scheduled as its CTAs
 // leave), and pdl_wait() -- which returns when the kernels before it have completed and their writes are visible -- before the
-// first access to global memory; only what depends on the parameters alone comes before the wait.
+// first access to global memory; only what depends on the parameters alone comes before the wait.  Global memory is read by plain
+// loads: __ldg and const __restrict__ promise data that does not change while the kernel lives, and a kernel that starts before its
+// predecessor ends lives while that one still writes what it will read.
 template <typename... P, typename... A>
 inline cudaError_t launch(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};

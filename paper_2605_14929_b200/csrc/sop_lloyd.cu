@@ -134,7 +134,7 @@ __device__ __forceinline__ int resolve_fmta(const LloydArgs& a, const sop_search
 // CTA of LTB threads: the bin of `hist` (LTB PER bins) holding the element of 1-based rank `rank`; *before = elements in lower bins.
 // Every CTA of the pass that follows does this before it can start, so a thread's bins are loaded together.
 template <int PER>
-__device__ void find_bin(const unsigned* __restrict__ hist, long long rank, int* bin, long long* before) {
+__device__ void find_bin(const unsigned* hist, long long rank, int* bin, long long* before) {
   __shared__ unsigned s_warp[LTB / 32];
   __shared__ int s_bin;
   __shared__ unsigned s_before;
@@ -187,7 +187,7 @@ __device__ unsigned derive_prefix(LloydWs* ws, long long pool_rank, int passes) 
 }
 
 template <int PASS>
-__global__ void __launch_bounds__(LTB) select_kernel(LloydArgs a, const sop_search_result* __restrict__ res, LloydWs* __restrict__ ws) {
+__global__ void __launch_bounds__(LTB) select_kernel(LloydArgs a, const sop_search_result* res, LloydWs* ws) {
   pdl_trigger();
   pdl_wait();
   __shared__ unsigned sh[2048];
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(LTB) select_kernel(LloydArgs a, const sop_sear
   for (long long i = (long long)blockIdx.x * LTB + threadIdx.x; i < nv; i += 4 * stride) {
     float4 v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = i + q * stride < nv ? __ldg(reinterpret_cast<const float4*>(row) + i + q * stride) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int q = 0; q < 4; ++q) v[q] = i + q * stride < nv ? *(reinterpret_cast<const float4*>(row) + i + q * stride) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (i + q * stride >= nv) break;
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(LTB) select_kernel(LloydArgs a, const sop_sear
   for (long long i = 4 * nv + (long long)blockIdx.x * LTB + threadIdx.x; i < a.NB; i += 4 * stride) {
     float v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = i + q * stride < a.NB ? __ldg(row + i + q * stride) : 0.0f;
+    for (int q = 0; q < 4; ++q) v[q] = i + q * stride < a.NB ? row[i + q * stride] : 0.0f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (i + q * stride >= a.NB) break;
@@ -239,8 +239,8 @@ __device__ __forceinline__ int sort_cell(float u) {
 __device__ void make_desc(IterDesc* d, const float* table, int ne);
 
 // CTA 0: max(c) and what the first table needs; the others clear the header.
-__global__ void __launch_bounds__(INIT_TB) lloyd_init_kernel(LloydArgs a, AtomsDev A, const sop_search_result* __restrict__ res,
-                                                             LloydWs* __restrict__ ws, double* __restrict__ distortion, int iters) {
+__global__ void __launch_bounds__(INIT_TB) lloyd_init_kernel(LloydArgs a, AtomsDev A, const sop_search_result* res,
+                                                             LloydWs* ws, double* distortion, int iters) {
   __shared__ float red[INIT_TB / 32];
   __shared__ float s_lut[SOP_MAX_ENTRIES];
   pdl_trigger();
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(INIT_TB) lloyd_init_kernel(LloydArgs a, AtomsD
     return;
   }
   float mx = 0.0f;
-  for (long long i = tid; i < a.K; i += INIT_TB) mx = fmaxf(mx, __ldg(a.c + i));
+  for (long long i = tid; i < a.K; i += INIT_TB) mx = fmaxf(mx, a.c[i]);
   for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
   if ((tid & 31) == 0) red[tid >> 5] = mx;
   const int f = resolve_fmta(a, res), ne = A.atoms[f].n_entries;
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(INIT_TB) lloyd_init_kernel(LloydArgs a, AtomsD
 // memory and leave in whole lines.  The order of the list depends on the scheduling of the CTAs; nothing downstream depends on it
 // (integer sums, and FP64 sums compared with a tolerance).
 constexpr int LIST_ROUND = (LTB / 32) * 512;
-__global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __restrict__ ws) {
+__global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* ws) {
   __shared__ unsigned s_cnt[LTB / 32 + 1];
   __shared__ unsigned s_base;
   __shared__ unsigned s_idx[LIST_ROUND];
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __
   {
     const float cmax = ws->cmax;
     for (long long i = (long long)blockIdx.x * LTB + tid; i < a.K; i += (long long)gridDim.x * LTB)
-      a.omega[i] = (a.flags & SOP_LLOYD_UNIFORM_WEIGHTS) ? 1.0f : (cmax > 0.0f ? __fdiv_rn(__ldg(a.c + i), cmax) : 0.0f);
+      a.omega[i] = (a.flags & SOP_LLOYD_UNIFORM_WEIGHTS) ? 1.0f : (cmax > 0.0f ? __fdiv_rn(a.c[i], cmax) : 0.0f);
   }
   const float* row = a.cosrow_base + (size_t)ws->fmta * a.NB;
   const bool vec = (reinterpret_cast<uintptr_t>(row) & 15u) == 0;
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __
     if (vec && base + warp * 512 + 512 <= a.NB) {
       float4 v[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] = __ldg(reinterpret_cast<const float4*>(row + i0 + 128 * q));
+      for (int q = 0; q < 4; ++q) v[q] = *reinterpret_cast<const float4*>(row + i0 + 128 * q);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         in |= (pool_key(v[q].x, a.flags) <= tau_key ? 1u : 0u) << (4 * q);
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(LTB) pool_list_kernel(LloydArgs a, LloydWs* __
 #pragma unroll
       for (int x = 0; x < 16; ++x) {
         const long long i = i0 + 128 * (x >> 2) + (x & 3);
-        v[x] = i < a.NB ? __ldg(row + i) : 0.0f;
+        v[x] = i < a.NB ? row[i] : 0.0f;
       }
 #pragma unroll
       for (int x = 0; x < 16; ++x)
@@ -422,7 +422,7 @@ __device__ void spill_cells(CacheSmem& S, LloydWs* ws) {
 // asynchronous bulk copy.  8192 x 8192, half the blocks in the pool: 167 us (228 us with limb atomics per run, executed for one lane
 // at a time); 28672 x 8192: 563 us (772 us).
 template <bool DP>
-__global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev F, LloydWs* __restrict__ ws, long long* __restrict__ pool_count_out,
+__global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev F, LloydWs* ws, long long* pool_count_out,
                                                          unsigned spill_tiles) {
   pdl_trigger();
   pdl_wait();
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev 
       const unsigned m = blk / nbk;
       jn = blk - m * nbk;
       const uint4* p = reinterpret_cast<const uint4*>(a.W + (long long)m * a.ldw + (long long)jn * SOP_G);
-      wn0 = __ldg(p); wn1 = __ldg(p + 1);
+      wn0 = *p; wn1 = p[1];
     }
   };
   load_w(load_idx(blockIdx.x));
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(CTB, 2) pool_cache_kernel(LloydArgs a, FmtDev 
       const float4* op = reinterpret_cast<const float4*>(a.omega + (size_t)jn * SOP_G);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float4 o = __ldg(op + q);
+        const float4 o = op[q];
         om[4 * q] = o.x; om[4 * q + 1] = o.y; om[4 * q + 2] = o.z; om[4 * q + 3] = o.w;
       }
     } else {
@@ -748,7 +748,7 @@ __device__ void new_table(IterSmem& S, unsigned long long n, long long sv) {
 
 // The whole CTA: adds its share of one iteration to the sums of that iteration and arrives.
 template <bool ALL>
-__device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __restrict__ ws, IterSmem& S, const unsigned short* __restrict__ ts,
+__device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* ws, IterSmem& S, const unsigned short* ts,
                                                 const CellMoments& mom, unsigned tile0, int T, int it, bool last) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, sub = lane >> 3, ln = lane & 7;
   constexpr int NW = ITB / 32;
@@ -768,7 +768,7 @@ __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __r
       src = a.cache + (size_t)(tile0 + (unsigned)t) * TILE_ELEMS;
     }
 #pragma unroll
-    for (int i = 0; i < PRE; ++i) v[i] = p0 + 8u * i < p1 ? __ldg(src + tile_slot(p0 + 8u * i)) : make_uint2(0u, 0u);
+    for (int i = 0; i < PRE; ++i) v[i] = p0 + 8u * i < p1 ? src[tile_slot(p0 + 8u * i)] : make_uint2(0u, 0u);
   };
   open_run(warp, l, ch);
   if (blockIdx.x == 0 && tid < SORT_ROWS) D = cell_distortion(S.d, mom, tid);        // (the first elements are on their way)
@@ -811,7 +811,7 @@ __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __r
         q += 8u * PRE;
         if (!__any_sync(0xFFFFFFFFu, q < q1)) break;
 #pragma unroll
-        for (int i = 0; i < PRE; ++i) w[i] = q + 8u * i < q1 ? __ldg(from + tile_slot(q + 8u * i)) : make_uint2(0u, 0u);
+        for (int i = 0; i < PRE; ++i) w[i] = q + 8u * i < q1 ? from[tile_slot(q + 8u * i)] : make_uint2(0u, 0u);
       }
       if ((l != l_now || x + NW >= total) && !last) {
         const unsigned long long ta = warp_sum64(nA), th = warp_sum64(nH), ua = warp_sum64((unsigned long long)sA), uh = warp_sum64((unsigned long long)sH);
@@ -825,7 +825,7 @@ __device__ __forceinline__ void iteration_share(const LloydArgs& a, LloydWs* __r
     } else {
 #pragma unroll 1
       for (; q < q1; q += 8u) {
-        const uint2 y = __ldg(from + tile_slot(q));
+        const uint2 y = from[tile_slot(q)];
         const float u = __uint_as_float(y.x), om = __uint_as_float(y.y);
         const int code = count_below(S.d.tau, u);
         const float dd = __fsub_rn(u, S.d.lut[code]);
@@ -895,8 +895,8 @@ __device__ __forceinline__ bool read_sums(const unsigned long long (*acc)[SOP_MA
 // The wait is bounded: a CTA that gives up raises ws->error, every CTA then leaves, and the last distortion entry stays -1 (a
 // distortion is never negative) so that the caller can tell.
 template <bool ALL>
-__global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs* __restrict__ ws, double* __restrict__ distortion, int it0, int iters,
-                                                           float* __restrict__ out_lut, int smem_tiles) {
+__global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs* ws, double* distortion, int it0, int iters,
+                                                           float* out_lut, int smem_tiles) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(16) unsigned char iter_smem[];
@@ -909,7 +909,7 @@ __global__ void __launch_bounds__(ITB, 1) lloyd_iter_kernel(LloydArgs a, LloydWs
   const unsigned short* ts = a.tile_start + (size_t)tile0 * TS_PITCH;
   if (T <= smem_tiles) {                  // the cell starts of this CTA's tiles, kept over the iterations
     const uint4* from = reinterpret_cast<const uint4*>(ts);
-    for (int i = tid; i < T * (TS_PITCH / 8); i += ITB) reinterpret_cast<uint4*>(s_ts)[i] = __ldg(from + i);
+    for (int i = tid; i < T * (TS_PITCH / 8); i += ITB) reinterpret_cast<uint4*>(s_ts)[i] = from[i];
     ts = s_ts;
   }
   {
@@ -1046,7 +1046,7 @@ __device__ __forceinline__ double dp_run_cost(const long long* pH, const long lo
   return __dadd_rn(__dsub_rn(qq, a), c);
 }
 
-__global__ void __launch_bounds__(DP_TB) grid_dp_cost_kernel(const LloydWs* __restrict__ ws, DpScratch* __restrict__ dp) {
+__global__ void __launch_bounds__(DP_TB) grid_dp_cost_kernel(const LloydWs* ws, DpScratch* dp) {
   __shared__ long long pre[3][SORT_ROWS + 1];
   __shared__ long long tot[4][32];
   pdl_trigger();
@@ -1100,9 +1100,9 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__global__ void __cluster_dims__(DP_CL, 1, 1) __launch_bounds__(DP_TB) grid_dp_rows_kernel(const DpScratch* __restrict__ dp, int n_entries,
-                                                                                         short* __restrict__ cut, float* __restrict__ out_lut,
-                                                                                         double* __restrict__ cost_out) {
+__global__ void __cluster_dims__(DP_CL, 1, 1) __launch_bounds__(DP_TB) grid_dp_rows_kernel(const DpScratch* dp, int n_entries,
+                                                                                         short* cut, float* out_lut,
+                                                                                         double* cost_out) {
   extern __shared__ __align__(16) unsigned char dp_smem[];
   DpSmem& S = *reinterpret_cast<DpSmem*>(dp_smem);
   pdl_trigger();

@@ -39,10 +39,10 @@ struct PackCand { int table; int kind; int neg; int scope; int k; float tmax; Gr
 // The 16 codes come back as bytes, four per word (element i in byte i % 4 of word i / 4).
 // METRIC: 0 = codes only, 1 = also the block cosine, 2 = also the block squared error (in cos_out).
 template <int METRIC, int KIND>
-__device__ __forceinline__ void eval_block_kind(const float (&w)[16], const float (&c)[16], const float* __restrict__ tau,
-                                                const float* __restrict__ lutv, int neg, float rcp, float s_hat,
+__device__ __forceinline__ void eval_block_kind(const float (&w)[16], const float (&c)[16], const float* tau,
+                                                const float* lutv, int neg, float rcp, float s_hat,
                                                 float& cos_out, uint32_t (&code4)[4], const GridDev grid = GridDev(), int sign_pos = 0,
-                                                const uint2* __restrict__ cells = nullptr, float invh = 0.0f, int c_half = 0) {
+                                                const uint2* cells = nullptr, float invh = 0.0f, int c_half = 0) {
   float qn[4], qd[4], qw[4];
 #pragma unroll
   for (int h = 0; h < 4; ++h) {
@@ -96,10 +96,10 @@ __device__ __forceinline__ void eval_block_kind(const float (&w)[16], const floa
 // the quantiser kind is decided once per block, outside the element loops: a kind test inside them lets
 // the compiler hoist the FP-grid arithmetic into the table path
 template <int METRIC>
-__device__ __forceinline__ void eval_block_regs(const float (&w)[16], const float (&c)[16], const float* __restrict__ tau,
-                                                const float* __restrict__ lutv, int kind, int neg, float rcp, float s_hat,
+__device__ __forceinline__ void eval_block_regs(const float (&w)[16], const float (&c)[16], const float* tau,
+                                                const float* lutv, int kind, int neg, float rcp, float s_hat,
                                                 float& cos_out, uint32_t (&code4)[4], const GridDev grid, int sign_pos,
-                                                const uint2* __restrict__ cells, float invh, int c_half) {
+                                                const uint2* cells, float invh, int c_half) {
   if (kind == KIND_LUT_CELL) eval_block_kind<METRIC, KIND_LUT_CELL>(w, c, tau, lutv, neg, rcp, s_hat, cos_out, code4, grid, sign_pos, cells, invh, c_half);
   else if (kind == KIND_LUT16) eval_block_kind<METRIC, KIND_LUT16>(w, c, tau, lutv, neg, rcp, s_hat, cos_out, code4);
   else if (kind == SOP_KIND_LUT) eval_block_kind<METRIC, SOP_KIND_LUT>(w, c, tau, lutv, neg, rcp, s_hat, cos_out, code4);
@@ -111,7 +111,7 @@ __device__ __forceinline__ void eval_block_regs(const float (&w)[16], const floa
 // USE_COS: the winner of each block is read off the per-block cosines of a sweep and only it is encoded
 // (no channel norms needed); otherwise every candidate of the choice is evaluated here.
 template <bool USE_COS>
-__global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res) {
+__global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* res) {
   pdl_trigger();
   pdl_wait();
   __shared__ float lutv[2][32], tau[2][32];
@@ -242,12 +242,12 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
   auto fetch = [&](unsigned blk, uint4& v0, uint4& v1, float (&cs4)[4]) {
     const unsigned m = blk / nbk32, j = blk - m * nbk32;
     const uint4* p = reinterpret_cast<const uint4*>(a.W + (long long)m * a.ldw + (long long)j * SOP_G);
-    v0 = __ldg(p); v1 = __ldg(p + 1);
+    v0 = *p; v1 = p[1];
     if (USE_COS) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int slot = n_sign == 2 ? q : 2 * q;          // candidate q of the order a, (-a), b, (-b)
-        cs4[q] = q < n_cand ? __ldg(a.block_cos + (size_t)s_row[slot] * a.NB + blk) : 0.0f;
+        cs4[q] = q < n_cand ? a.block_cos[(size_t)s_row[slot] * a.NB + blk] : 0.0f;
       }
     }
   };
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
       const float4* cp = reinterpret_cast<const float4*>(a.c + j * SOP_G);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float4 v = __ldg(cp + q);
+        const float4 v = cp[q];
         c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
       }
     }
@@ -421,7 +421,7 @@ __device__ __forceinline__ unsigned pack_cell(float u, float inv_range) {
 // KIND: SOP_KIND_LUT (any pair or single table), SOP_KIND_FP_E2M3 or SOP_KIND_FP_E4M3 (a single format).  N: bits of a code (0: as the
 // atom says).  NC: candidates of the choice, 1, 2 (a pair, or a table and its negation) or 4.
 template <int KIND, int N, int NC>
-__global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res) {
+__global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* res) {
   constexpr bool LUT = KIND == SOP_KIND_LUT;
   __shared__ __align__(16) uint2 cells[LUT ? 2 * (PCELLS + 1) * PCOPIES : 1];      // {threshold, code below | code above << 8}
   __shared__ float tau[2][32], lutv[2][32];
@@ -516,10 +516,10 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
     if (blk < NB) {
       const uint16_t* p = a.W + (size_t)blk * SOP_G;
       if (!packed_rows) { const unsigned m = blk / nbk; p = a.W + (long long)m * a.ldw + (long long)(blk - m * nbk) * SOP_G; }
-      nv0 = __ldg(reinterpret_cast<const uint4*>(p)); nv1 = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+      nv0 = *reinterpret_cast<const uint4*>(p); nv1 = *(reinterpret_cast<const uint4*>(p) + 1);
       if (NC > 1) {
 #pragma unroll
-        for (int q = 0; q < NC; ++q) ncs[q] = __uint_as_float(__float_as_uint(__ldg(row[q] + blk)) ^ flip);
+        for (int q = 0; q < NC; ++q) ncs[q] = __uint_as_float(__float_as_uint(row[q][blk]) ^ flip);
       }
     }
   };

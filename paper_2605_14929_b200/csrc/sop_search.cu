@@ -121,8 +121,8 @@ struct LayerArgs {
 
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void load_block_bits(const uint16_t* p, uint32_t (&v)[8]) {
-  const uint4 a = __ldg(reinterpret_cast<const uint4*>(p));
-  const uint4 b = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+  const uint4 a = *reinterpret_cast<const uint4*>(p);
+  const uint4 b = *(reinterpret_cast<const uint4*>(p) + 1);
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
   v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
@@ -156,7 +156,7 @@ __device__ __forceinline__ int sigma_exponent(float a, float tmax) {
 // shared-memory addition per class and block, and max|W| added up by every warp), latency on a small one.
 constexpr int PPB = 256;                 // threads per CTA
 constexpr int PP_FLY = 4;                // blocks in flight per thread
-__global__ void __launch_bounds__(PPB) prepass_kernel(LayerArgs L, Plan P, FmtDev F, unsigned* __restrict__ hist, WsHeader* __restrict__ hdr, unsigned rows) {
+__global__ void __launch_bounds__(PPB) prepass_kernel(LayerArgs L, Plan P, FmtDev F, unsigned* hist, WsHeader* hdr, unsigned rows) {
   pdl_trigger();
   __shared__ unsigned s_cnt[(SOP_MAX_CLASSES + 1) * 256];      // [region][exponent]
   __shared__ unsigned s_mark[4];                               // mantissas that are a cut point
@@ -207,19 +207,17 @@ __global__ void __launch_bounds__(PPB) prepass_kernel(LayerArgs L, Plan P, FmtDe
     while (left) {
       uint4 v[PP_FLY][2];
 #pragma unroll
-      for (int q = 0; q < PP_FLY; ++q)
-        if (q < (int)left) {
-          v[q][0] = __ldg(reinterpret_cast<const uint4*>(p + q * step));
-          v[q][1] = __ldg(reinterpret_cast<const uint4*>(p + q * step) + 1);
-        } else {
-          v[q][0] = v[q][1] = make_uint4(0u, 0u, 0u, 0u);
-        }
+      for (int q = 0; q < PP_FLY; ++q) {           // (past the last one the first again: the loads go out together)
+        const uint4* w = reinterpret_cast<const uint4*>(q < (int)left ? p + q * step : p);
+        v[q][0] = w[0]; v[q][1] = w[1];
+      }
+      const int n = (int)min(left, (unsigned)PP_FLY);
       p += PP_FLY * step;
-      left -= min(left, (unsigned)PP_FLY);
+      left -= (unsigned)n;
 #pragma unroll
       for (int q = 0; q < PP_FLY; ++q) {
         const uint32_t wb[8] = {v[q][0].x, v[q][0].y, v[q][0].z, v[q][0].w, v[q][1].x, v[q][1].y, v[q][1].z, v[q][1].w};
-        const unsigned pat = __float_as_uint(absmax_bits(wb)) >> 16;
+        const unsigned pat = q < n ? __float_as_uint(absmax_bits(wb)) >> 16 : 0u;
         wmax = max(wmax, pat);
         if (pat) {
           const int e = (int)(pat >> 7);
@@ -264,7 +262,7 @@ __global__ void __launch_bounds__(PPB) prepass_kernel(LayerArgs L, Plan P, FmtDe
 }
 
 // The shifts of another scale format from the histograms that an earlier prepass of the same layer left in the workspace.
-__global__ void __launch_bounds__(256) kselect_kernel(Plan P, FmtDev F, const unsigned* __restrict__ hist, WsHeader* __restrict__ hdr) {
+__global__ void __launch_bounds__(256) kselect_kernel(Plan P, FmtDev F, const unsigned* hist, WsHeader* hdr) {
   pdl_trigger();
   pdl_wait();
   if (threadIdx.x == 0) hdr->wmax_bits = hist[SOP_MAX_CLASSES * SOP_HIST_BINS];
@@ -539,7 +537,7 @@ constexpr unsigned C_STEP = TB * 16u;
 // in the halves of word 4 p + i), their rows at `plane`.  The sums run in the order of the quad tree: four quads of consecutive
 // elements, sequential inside a quad, (Q0 + Q1) + (Q2 + Q3).
 template <int NP>
-__device__ __forceinline__ void sweep_pass(const unsigned char* __restrict__ plane, const uint32_t (&wb)[8], const uint32_t (&off)[8],
+__device__ __forceinline__ void sweep_pass(const unsigned char* plane, const uint32_t (&wb)[8], const uint32_t (&off)[8],
                                            unsigned c_addr, float s_hat, float2 (&nq)[NP], float2 (&dot)[NP], float2 (&sse)[NP]) {
   const float2 ns = make_float2(-s_hat, -s_hat);
   float2 n2[NP], d2[NP], s2[NP];
@@ -713,11 +711,13 @@ __device__ __forceinline__ float fold(const float2 a, const float2 b) {
 }
 
 template <int MODE, bool PAIRED>
-__device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F, const ClassDev& K, size_t NB, float* __restrict__ block_cos,
-                                             float* __restrict__ block_sse) {
+__device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F, const ClassDev& K, size_t NB, float* block_cos,
+                                             float* block_sse) {
   const uint16_t* wp = X.w0;
   unsigned at = X.blk0;
   const int n_cand = K.n_cand;
+  const GridDev grid = K.grid;
+  float *cos0 = block_cos + (size_t)K.cand[0] * NB, *sse0 = block_sse + (size_t)K.cand[0] * NB;
   uint32_t wn[8];
   load_block_bits(wp, wn);
 #pragma unroll 1
@@ -726,7 +726,7 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
 #pragma unroll
     for (int q = 0; q < 8; ++q) wb[q] = wn[q];
     if (it + 1 < X.n_rows) wp += X.w_step;
-    // (the rows after that on their way into L2, there are no registers to hold them: 14336 x 4096, two formats, a pass 183.8 us, 186 us without)
+    // (the rows after that on their way into L2, there are no registers to hold them: 14336 x 4096, two formats, a pass 178.7 us; 2 us more without)
     if (it + 3 < X.n_rows) asm volatile("prefetch.global.L2 [%0];" ::"l"(wp + 2 * X.w_step));
     load_block_bits(wp, wn);
     float s_hat, rcp;
@@ -751,7 +751,7 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
         const float2 c = make_float2(cc[ix], cc[iy]);
         const float2 u = __fmul2_rn(w, r2);
         float2 q;
-        if constexpr (MODE == SOP_KIND_FP_GRID) { q.x = grid_quantize(u.x, K.grid); q.y = grid_quantize(u.y, K.grid); }
+        if constexpr (MODE == SOP_KIND_FP_GRID) { q.x = grid_quantize(u.x, grid); q.y = grid_quantize(u.y, grid); }
         else { uint32_t codes; q = fp_quantize2<MODE>(u.x, u.y, codes); }
         nw2[p] = __ffma2_rn(__fmul2_rn(c, w), w, nw2[p]);
         const float2 cq = __fmul2_rn(c, q);
@@ -764,12 +764,15 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
     const float nw = fold(nw2[0], nw2[1]), nqs = fold(nq[0], nq[1]), dots = fold(dot[0], dot[1]), err = fold(sse[0], sse[1]);
     const float x = __fmul_rn(nw, nqs);
     const float cosv = x >= COS_LO && x <= COS_HI && all_ones_root(x) && fabsf(dots) >= COS_DOT ? cosine_one(-x, dots) : block_cosine_any(nw, nqs, dots);
-    if (it < X.n_rows)
-      for (int ci = 0; ci < n_cand; ++ci) {      // (candidates of one format and scale have the same values)
+    if (it < X.n_rows) {
+      cos0[at] = cosv;
+      sse0[at] = err;
+      for (int ci = 1; ci < n_cand; ++ci) {      // (candidates of one format and scale have the same values)
         const size_t col = (size_t)K.cand[ci] * NB + at;
         block_cos[col] = cosv;
         block_sse[col] = err;
       }
+    }
     at += X.blk_step;
   }
 }
@@ -777,9 +780,9 @@ __device__ __forceinline__ void sweep_format(const SweepCtx& X, const FmtDev& F,
 // Evaluates the candidates of eval_mask on every block and writes their columns of block_cos / block_sse: group by group, then
 // format by format (W is read again for each: it is a tenth of the time of one).
 template <int MAX_NP>
-__global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArgs L, Plan P, AtomsDev A, FmtDev F, WsHeader* __restrict__ hdr,
-                                                      float* __restrict__ block_cos, float* __restrict__ block_sse,
-                                                      const sop_search_result* __restrict__ prev, unsigned c_off, unsigned tba) {
+__global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArgs L, Plan P, AtomsDev A, FmtDev F, WsHeader* hdr,
+                                                      float* block_cos, float* block_sse,
+                                                      const sop_search_result* prev, unsigned c_off, unsigned tba) {
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smem[];
   GroupScratch& S = *reinterpret_cast<GroupScratch*>(smem);
@@ -815,7 +818,7 @@ __global__ void __launch_bounds__(TB, MAX_NP == 0 ? 2 : 1) sweep_kernel(LayerArg
   {
     const float4* cp = reinterpret_cast<const float4*>(L.c + (size_t)j * SOP_G);
     float4* dst = reinterpret_cast<float4*>(smem + c_off);
-    const float4 v0 = __ldg(cp), v1 = __ldg(cp + 1), v2 = __ldg(cp + 2), v3 = __ldg(cp + 3);
+    const float4 v0 = *cp, v1 = cp[1], v2 = cp[2], v3 = cp[3];
     asm volatile("prefetch.global.L2 [%0];" ::"l"(X.w0));          // the first block arrives while the tables are built
     if (MAX_NP == 0) {
       dst[tid] = make_float4(v0.x, v1.x, v0.y, v1.y);
@@ -1136,9 +1139,9 @@ __device__ __forceinline__ void reduce_run(const ReduceCtx& X, const BundleDev& 
 
 template <bool SEL_ERR, bool VEC>
 __global__ void __launch_bounds__(RTB, 1) reduce_kernel(LayerArgs L, RedPlan P, BundlesDev Q, int units, int n_stage, int do_final,
-                                                        WsHeader* __restrict__ hdr, PartialSums partials, const float* __restrict__ block_cos,
-                                                        const float* __restrict__ block_sse, sop_pair_stat* pair_table, sop_pair_stat* signed_table,
-                                                        sop_search_result* __restrict__ res, const sop_search_result* __restrict__ prev) {
+                                                        WsHeader* hdr, PartialSums partials, const float* block_cos,
+                                                        const float* block_sse, sop_pair_stat* pair_table, sop_pair_stat* signed_table,
+                                                        sop_search_result* res, const sop_search_result* prev) {
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ BundleSums s_part[RED_WARPS];

@@ -88,9 +88,9 @@ __device__ __forceinline__ unsigned cta_excl_scan(unsigned v, unsigned* s_warp, 
 // In place: tile_sums[t] becomes the number of records before tile t.  One CTA; a thread holds 16 consecutive tiles of a
 // chunk of 16384 in registers (four loads in flight, one scan of the CTA per chunk).  The total goes to row_start[M] and
 // *count.  With `wr` the kernel also turns the largest kept |E| into the layer exponent of the Wr values.
-__global__ void __launch_bounds__(1024) tile_scan_kernel(unsigned* __restrict__ tile_sums, long long n_tiles, unsigned* __restrict__ row_start,
-                                                         long long M, long long* __restrict__ count, SparseWs* __restrict__ ws, int wr,
-                                                         int* __restrict__ scale_exp_out, float* __restrict__ tau_out) {
+__global__ void __launch_bounds__(1024) tile_scan_kernel(unsigned* tile_sums, long long n_tiles, unsigned* row_start,
+                                                         long long M, long long* count, SparseWs* ws, int wr,
+                                                         int* scale_exp_out, float* tau_out) {
   pdl_trigger();
   pdl_wait();
   __shared__ unsigned s_warp[2][32];
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(STB) opq_mask_kernel(OpqArgs a) {
     if (tile < n_tiles && blk < NB) {
       m = blk / nbk; j = blk - m * nbk;
       const uint4* p = reinterpret_cast<const uint4*>(a.W + (long long)m * a.ldw + (long long)j * SOP_G);
-      v0 = __ldg(p); v1 = __ldg(p + 1);
+      v0 = *p; v1 = p[1];
     }
   };
   fetch(blockIdx.x);
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(STB) opq_mask_kernel(OpqArgs a) {
       const uint16_t* p = a.W + (long long)cm * a.ldw + (long long)cj * SOP_G;
       for (unsigned rest = mask; rest; rest &= rest - 1u, ++pos) {
         const int i = __ffs((int)rest) - 1;
-        if (pos < OPQ_LOCAL) a.local[(size_t)tile * OPQ_LOCAL + pos] = (cj * SOP_G + (unsigned)i) | ((unsigned)__ldg(p + i) << 16);
+        if (pos < OPQ_LOCAL) a.local[(size_t)tile * OPQ_LOCAL + pos] = (cj * SOP_G + (unsigned)i) | ((unsigned)p[i] << 16);
       }
     }
   }
@@ -249,20 +249,20 @@ __global__ void __launch_bounds__(STB) opq_write_kernel(OpqArgs a) {
   const int tid = threadIdx.x, lane = tid & 31;
   const unsigned NB = (unsigned)a.NB, nbk = (unsigned)a.nbk, n_tiles = (NB + STB - 1) / STB;   // the block count fits 31 bits
   for (unsigned tile = blockIdx.x * (STB / 32) + (tid >> 5); tile < n_tiles; tile += gridDim.x * (STB / 32)) {
-    const unsigned base = __ldg(a.tile_sums + tile);
-    const unsigned cnt = (tile + 1 < n_tiles ? __ldg(a.tile_sums + tile + 1) : __ldg(a.row_start + a.M)) - base;
+    const unsigned base = a.tile_sums[tile];
+    const unsigned cnt = (tile + 1 < n_tiles ? a.tile_sums[tile + 1] : a.row_start[a.M]) - base;
     const bool local = cnt <= OPQ_LOCAL;
     if (local) {
       const unsigned* from = a.local + (size_t)tile * OPQ_LOCAL;
       for (unsigned i = lane; i < cnt; i += 32)
-        if ((long long)base + i < a.capacity) a.records[base + i] = __ldg(from + i);
+        if ((long long)base + i < a.capacity) a.records[base + i] = from[i];
     }
     const unsigned t0 = tile * STB, jt = t0 % nbk;
     if (jt == 0 && lane == 0) a.row_start[t0 / nbk] = base;
     if (local && jt + min((unsigned)STB, NB - t0) <= nbk) continue;          // no other row starts here
     const unsigned b0 = t0 + 8 * lane;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (b0 < NB) v = __ldg(reinterpret_cast<const uint4*>(a.masks + b0));      // the array is padded to 256 bytes
+    if (b0 < NB) v = *reinterpret_cast<const uint4*>(a.masks + b0);      // the array is padded to 256 bytes
     const unsigned n_here = b0 < NB ? (NB - b0 < 8u ? NB - b0 : 8u) : 0u;
     unsigned u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -349,7 +349,7 @@ __device__ __forceinline__ float scale_decode(uint32_t code, int k, const FmtDev
 }
 
 // the first warp of every CTA; the caller synchronises afterwards
-__device__ void wr_setup(const WrArgs& a, const AtomsDev& A, const sop_search_result* __restrict__ res, WrShared& sh) {
+__device__ void wr_setup(const WrArgs& a, const AtomsDev& A, const sop_search_result* res, WrShared& sh) {
   const int lane = threadIdx.x;
   if (lane >= 32) return;
   int ia = a.index_a, ib = a.index_b;
@@ -398,37 +398,37 @@ struct WrRaw {
 };
 
 template <bool LUT4>
-__device__ __forceinline__ WrRaw<LUT4> wr_fetch(const WrArgs& a, int n_bits, unsigned blk, const uint16_t* __restrict__ wrow) {
+__device__ __forceinline__ WrRaw<LUT4> wr_fetch(const WrArgs& a, int n_bits, unsigned blk, const uint16_t* wrow) {
   WrRaw<LUT4> r;
   const uint4* p = reinterpret_cast<const uint4*>(wrow);
-  r.v0 = __ldg(p); r.v1 = __ldg(p + 1);
+  r.v0 = *p; r.v1 = p[1];
   r.w1 = 0;
   const int b = a.container_bits;
-  if (b == 16) r.w0 = (unsigned)__ldg(reinterpret_cast<const unsigned short*>(a.words) + blk);
-  else if (b == 8) r.w0 = (unsigned)__ldg(reinterpret_cast<const unsigned char*>(a.words) + blk);
+  if (b == 16) r.w0 = (unsigned)*(reinterpret_cast<const unsigned short*>(a.words) + blk);
+  else if (b == 8) r.w0 = (unsigned)*(reinterpret_cast<const unsigned char*>(a.words) + blk);
   else {
     const unsigned long long bit = (unsigned long long)blk * 12u;
     const unsigned* q = a.words + (bit >> 5);
-    r.w0 = __ldg(q);
-    if (((unsigned)bit & 31u) > 20u) r.w1 = __ldg(q + 1);
+    r.w0 = *q;
+    if (((unsigned)bit & 31u) > 20u) r.w1 = q[1];
   }
   if constexpr (LUT4) {
-    r.c4 = __ldg(reinterpret_cast<const uint2*>(a.codes) + blk);
+    r.c4 = *(reinterpret_cast<const uint2*>(a.codes) + blk);
   } else {
     const int n = n_bits;
     const unsigned char* cp = a.codes + (size_t)blk * 2 * n;
     r.lo = r.hi = 0;
     if (n == 4) {
-      const uint2 t = __ldg(reinterpret_cast<const uint2*>(cp));
+      const uint2 t = *reinterpret_cast<const uint2*>(cp);
       r.lo = (unsigned long long)t.x | ((unsigned long long)t.y << 32);
     } else if (n == 8) {
-      const uint4 t = __ldg(reinterpret_cast<const uint4*>(cp));
+      const uint4 t = *reinterpret_cast<const uint4*>(cp);
       r.lo = (unsigned long long)t.x | ((unsigned long long)t.y << 32);
       r.hi = (unsigned long long)t.z | ((unsigned long long)t.w << 32);
     } else {
       const unsigned short* sp = reinterpret_cast<const unsigned short*>(cp);
       for (int i = 0; i < n; ++i) {
-        const unsigned long long v = (unsigned long long)__ldg(sp + i);
+        const unsigned long long v = (unsigned long long)sp[i];
         if (i < 4) r.lo |= v << (16 * i); else r.hi |= v << (16 * (i - 4));
       }
     }
@@ -440,7 +440,7 @@ __device__ __forceinline__ void wr_weights(const WrArgs& a, unsigned j, float (&
   const float4* cq = reinterpret_cast<const float4*>(a.c + (size_t)j * SOP_G);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const float4 v = __ldg(cq + q);
+    const float4 v = cq[q];
     c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
   }
 }
@@ -526,7 +526,7 @@ struct WrPick {
 };
 
 // Adds a CTA's histogram to the layer's; true in the CTA that comes last (all threads of the CTA call it).
-__device__ __forceinline__ bool wr_flush(const unsigned* hist, unsigned* __restrict__ out, unsigned* __restrict__ done, WrPick& s) {
+__device__ __forceinline__ bool wr_flush(const unsigned* hist, unsigned* out, unsigned* done, WrPick& s) {
   __syncthreads();
   for (int i = threadIdx.x; i < 2048; i += STB)
     if (hist[i]) atomicAdd(&out[i], hist[i]);
@@ -542,7 +542,7 @@ __device__ __forceinline__ bool wr_flush(const unsigned* hist, unsigned* __restr
 // pass; after the last pass the threshold itself.  Pass -1: the bin of the n_keep-th largest block maximum.  A rank
 // beyond the histogram's total (no pair to correct, so the histogram is empty) leaves a NaN threshold: nothing
 // compares >= to it.
-__device__ void wr_pick(SparseWs* __restrict__ ws, int pass, long long n_keep, WrPick& s) {
+__device__ void wr_pick(SparseWs* ws, int pass, long long n_keep, WrPick& s) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned long long rank = pass <= 0 ? (unsigned long long)n_keep : ws->rank;
   const unsigned prev = pass > 0 ? ws->prefix : 0u;
@@ -590,8 +590,8 @@ __device__ void wr_pick(SparseWs* __restrict__ ws, int pass, long long n_keep, W
 // What bounds it: instruction issue (67 % of the slots) beside 184 MB of DRAM traffic; 50 us at 8192 x 8192, 28 us of which the bytes need
 // (82 us with a block per thread in storage order, weights re-read per block, and both tables in the same sixteen banks).
 template <bool LUT4>
-__global__ void __launch_bounds__(STB, LUT4 ? 4 : 2) wr_max_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
-                                                                   SparseWs* __restrict__ ws, unsigned rows) {
+__global__ void __launch_bounds__(STB, LUT4 ? 4 : 2) wr_max_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* res,
+                                                                   SparseWs* ws, unsigned rows) {
   pdl_trigger();
   __shared__ WrShared sh;
   __shared__ WrPick pk;
@@ -660,8 +660,8 @@ struct WrValue {
 // the chain bins -> block -> list bounds it.
 constexpr int WR_BPL = 32;               // blocks per lane and step
 template <bool LUT4>
-__global__ void __launch_bounds__(STB) wr_collect_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
-                                                         SparseWs* __restrict__ ws) {
+__global__ void __launch_bounds__(STB) wr_collect_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* res,
+                                                         SparseWs* ws) {
   pdl_trigger();
   __shared__ WrShared sh;
   __shared__ WrPick pk;
@@ -757,8 +757,8 @@ __global__ void __launch_bounds__(STB) wr_collect_kernel(WrArgs a, AtomsDev A, F
 
 // The second and third digit of the threshold: over the candidate list, or over the layer when it overflowed.
 template <int PASS, bool LUT4>
-__global__ void __launch_bounds__(STB) wr_select_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
-                                                        SparseWs* __restrict__ ws) {
+__global__ void __launch_bounds__(STB) wr_select_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* res,
+                                                        SparseWs* ws) {
   pdl_trigger();
   __shared__ WrShared sh;
   __shared__ WrPick pk;
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(STB) wr_select_kernel(WrArgs a, AtomsDev A, Fm
   if (!ws->overflow) {
     __syncthreads();
     const unsigned n = ws->n_cand;
-    for (unsigned i = blockIdx.x * STB + tid; i < n; i += gridDim.x * STB) add(__uint_as_float(__ldg(a.cand_m + i)));
+    for (unsigned i = blockIdx.x * STB + tid; i < n; i += gridDim.x * STB) add(__uint_as_float(a.cand_m[i]));
   } else {
     wr_setup(a, A, res, sh);
     __syncthreads();
@@ -793,8 +793,8 @@ __global__ void __launch_bounds__(STB) wr_select_kernel(WrArgs a, AtomsDev A, Fm
 // The kept candidates: their bit in the per-block masks (two blocks per 32-bit word), their tile's record count, the
 // largest |E| among them.  After an overflow: the counts and the largest |E| from the layer.
 template <bool LUT4>
-__global__ void __launch_bounds__(STB) wr_mark_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
-                                                      SparseWs* __restrict__ ws) {
+__global__ void __launch_bounds__(STB) wr_mark_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* res,
+                                                      SparseWs* ws) {
   pdl_trigger();
   __shared__ WrShared sh;
   __shared__ unsigned s_cnt;
@@ -806,8 +806,8 @@ __global__ void __launch_bounds__(STB) wr_mark_kernel(WrArgs a, AtomsDev A, FmtD
     const unsigned n = ws->n_cand;
     unsigned* map = reinterpret_cast<unsigned*>(a.kept);
     for (unsigned i = blockIdx.x * STB + tid; i < n; i += gridDim.x * STB) {
-      const unsigned pos = __ldg(a.cand_pos + i), e = __ldg(a.cand_e + i);
-      if (!wr_kept(__uint_as_float(__ldg(a.cand_m + i)), tau)) continue;
+      const unsigned pos = a.cand_pos[i], e = a.cand_e[i];
+      if (!wr_kept(__uint_as_float(a.cand_m[i]), tau)) continue;
       atomicOr(&map[pos >> 5], 1u << (pos & 31u));
       atomicAdd(&a.tile_sums[pos >> 12], 1u);          // a tile is 256 blocks of 16 elements
       emax = max(emax, e & 0x7FFFFFFFu);
@@ -858,8 +858,8 @@ __device__ __forceinline__ unsigned wr_bits_before(const uint4& v, unsigned pos,
 // latency.
 // After an overflow: every block is decoded and its entries are compared with the threshold.
 template <bool LUT4>
-__global__ void __launch_bounds__(STB) wr_write_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* __restrict__ res,
-                                                       const SparseWs* __restrict__ ws) {
+__global__ void __launch_bounds__(STB) wr_write_kernel(WrArgs a, AtomsDev A, FmtDev F, const sop_search_result* res,
+                                                       const SparseWs* ws) {
   pdl_trigger();
   __shared__ WrShared sh;
   __shared__ unsigned s_warp[STB / 32];
@@ -872,8 +872,8 @@ __global__ void __launch_bounds__(STB) wr_write_kernel(WrArgs a, AtomsDev A, Fmt
     for (unsigned m = wid; m < (unsigned)a.M; m += n_warps) {
       const unsigned b = m * nbk;
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (lane * 8 < (b & 255u)) v = __ldg(reinterpret_cast<const uint4*>(a.kept + (b & ~255u)) + lane);
-      const unsigned base = __ldg(a.tile_sums + (b >> 8));
+      if (lane * 8 < (b & 255u)) v = *(reinterpret_cast<const uint4*>(a.kept + (b & ~255u)) + lane);
+      const unsigned base = a.tile_sums[b >> 8];
       const unsigned cnt = wr_bits_before(v, b * 16u, lane);
       if (lane == 0) a.row_start[m] = base + cnt;
     }
@@ -881,13 +881,13 @@ __global__ void __launch_bounds__(STB) wr_write_kernel(WrArgs a, AtomsDev A, Fmt
       bool keep = false;
       unsigned pos = 0, rec = 0;
       if (i0 + lane < n) {
-        pos = __ldg(a.cand_pos + i0 + lane);
-        const float e = __uint_as_float(__ldg(a.cand_e + i0 + lane));
-        keep = wr_kept(__uint_as_float(__ldg(a.cand_m + i0 + lane)), tau);
+        pos = a.cand_pos[i0 + lane];
+        const float e = __uint_as_float(a.cand_e[i0 + lane]);
+        keep = wr_kept(__uint_as_float(a.cand_m[i0 + lane]), tau);
         const unsigned blk = pos >> 4;
         rec = ((blk % nbk) * SOP_G + (pos & 15u)) | (V.code(e) << 16);
       }
-      const unsigned first = keep ? __ldg(a.tile_sums + (pos >> 12)) : 0u;
+      const unsigned first = keep ? a.tile_sums[pos >> 12] : 0u;
       unsigned before = 0;
       for (unsigned rest = __ballot_sync(0xFFFFFFFFu, keep); rest; ) {
         int src[4];
@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(STB) wr_write_kernel(WrArgs a, AtomsDev A, Fmt
           rest &= rest - 1u;                                      // 0 stays 0
           p[q] = __shfl_sync(0xFFFFFFFFu, pos, src[q] & 31);
           v[q] = make_uint4(0u, 0u, 0u, 0u);
-          if (src[q] >= 0 && 128u * lane < (p[q] & 4095u)) v[q] = __ldg(reinterpret_cast<const uint4*>(a.kept + ((p[q] >> 4) & ~255u)) + lane);
+          if (src[q] >= 0 && 128u * lane < (p[q] & 4095u)) v[q] = *(reinterpret_cast<const uint4*>(a.kept + ((p[q] >> 4) & ~255u)) + lane);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
