@@ -21,8 +21,6 @@
 #include <math.h>
 #include <string.h>
 
-#include <vector>
-
 #include "sop_device.cuh"
 
 namespace sop {
@@ -1460,7 +1458,9 @@ int build_plan(const AtomsDev& A, const FmtDev& F, int k_mode, unsigned eval_mas
 // fours (twos for a rest of two) with the pairs among them, then the remaining pairs as rectangles -- the second candidate with
 // the most pairs left and the one that shares the most first candidates with it, against up to four of those; where one first
 // candidate meets many second ones the rectangle is taken the other way round.
-static void build_bundles(const RedPlan& P, std::vector<BundleDev>* out) {
+struct BundleList { int n; BundleDev b[MAX_SLOTS]; };      // (every bundle forms at least one entry)
+static void build_bundles(const RedPlan& P, BundleList* out) {
+  out->n = 0;
   for (int ty = 0; ty < 2; ++ty) {
     int slot_of[SOP_MAX_ATOMS][SOP_MAX_ATOMS];
     for (int i = 0; i < SOP_MAX_ATOMS; ++i)
@@ -1488,7 +1488,7 @@ static void build_bundles(const RedPlan& P, std::vector<BundleDev>* out) {
       for (int i = 0; i < na; ++i)
         for (int j = i + 1; j < na; ++j, ++q)
           if (j < take) { B.slot[q] = (unsigned char)slot_of[B.a[i]][B.a[j]]; slot_of[B.a[i]][B.a[j]] = 255; }
-      out->push_back(B);
+      out->b[out->n++] = B;
       at += take;
     }
     for (;;) {
@@ -1525,7 +1525,7 @@ static void build_bundles(const RedPlan& P, std::vector<BundleDev>* out) {
           B.slot[4 * j + i] = (unsigned char)s;
           s = 255;
         }
-      out->push_back(B);
+      out->b[out->n++] = B;
     }
   }
 }
@@ -1706,9 +1706,9 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   if (grid < min_grid) grid = min_grid;
   if (grid > MAX_GRID) return SOP_ERR_SHAPE;
   // the reduction: up to fifteen bundles per launch; persistent grid over its tiles.  16-byte copies need 16-byte aligned column starts and runs: a block count that is a multiple of four.
-  std::vector<BundleDev> bundles;
+  BundleList bundles;
   build_bundles(Rp, &bundles);
-  const int n_launch = bundles.empty() ? 1 : (int)((bundles.size() + MAX_BUNDLES - 1) / MAX_BUNDLES);
+  const int n_launch = bundles.n ? (bundles.n + MAX_BUNDLES - 1) / MAX_BUNDLES : 1;
   const bool vec = (L.NB % 4) == 0 && (((uintptr_t)cos_cols | (uintptr_t)sse_cols) & 15u) == 0;
   int units = 0;
   const long long rgrid = reduce_grid(L.NB, sms, &units);
@@ -1759,9 +1759,9 @@ int sop_pair_search(const void* W_dev, long long M, long long K, long long ldw, 
   if ((rc = profile_mark(SOP_PROFILE_REDUCE, 0, st))) return rc;
   const bool sel_err = (flags & SOP_SEARCH_SELECT_MSE) != 0;
   for (int l = 0; l < n_launch; ++l) {
-    const int b0 = l * MAX_BUNDLES, nb = (int)bundles.size() - b0 < MAX_BUNDLES ? (int)bundles.size() - b0 : MAX_BUNDLES;
+    const int b0 = l * MAX_BUNDLES, nb = bundles.n - b0 < MAX_BUNDLES ? bundles.n - b0 : MAX_BUNDLES;
     BundlesDev Q;
-    deal_bundles(bundles.data() + b0, nb, &Q);
+    deal_bundles(bundles.b + b0, nb, &Q);
     int n_stage = g_reduce_ring ? MAX_STAGE : 2;             // (sixteen columns: two buffers of 98 KB)
     while (n_stage > 2 && reduce_smem_bytes(Q.n_cols, units, n_stage) > RED_SMEM_MAX) --n_stage;
     const size_t rs = reduce_smem_bytes(Q.n_cols, units, n_stage);
