@@ -325,7 +325,8 @@ int sop_dd4_lloyd(const void* W_dev, long long M, long long K, long long ldw, co
  *     the remaining m-1 metabits.  Unused metabits are zero.
  *   counts_dev (may be NULL): two long long {n_sel1, n_neg}, overwritten.  With index_a = SOP_PAIR_FROM_RESULT
  *     the search result may hold no pair (a singles-only search, a search without a signed table while
- *     use_sign = 1, an alphabet with one base atom): nothing is packed then, codes_dev is left as it was and
+ *     use_sign = 1, an alphabet with one base atom): nothing is packed then, codes_dev is left as it was, of
+ *     words_dev a 12-bit stream is cleared (else only its last 32 bits are) and
  *     counts_dev receives {-1, -1}; pass counts_dev whenever the pair comes from a result block.
  *   flags: SOP_PACK_SELECT_MSE (paragraph "Pair-search design axes", axis ii): the smallest block squared
  *     error wins instead of the largest block cosine, ties keep the earlier candidate.

@@ -440,6 +440,11 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
     ib = a.use_sign ? res->best_sb : res->best_b;
     if (ia < 0 || ib < 0 || ia >= A.n_atoms || ib >= A.n_atoms || (a.use_sign && (ia + 1 >= A.n_atoms || ib + 1 >= A.n_atoms))) {
       if (a.counts && blockIdx.x == 0 && tid < 2) a.counts[tid] = ~0ull;     // {-1, -1}: the result holds no pair
+      // the words as the other packer leaves them: a stream of 12-bit words cleared, else the last 32 bits
+      const unsigned long long n_words = ((unsigned long long)a.NB * (unsigned)a.container_bits + 31ull) / 32ull;
+      unsigned long long i = (unsigned long long)blockIdx.x * PTB + (unsigned)tid;
+      if (a.container_bits != 12) i += n_words - 1ull;
+      for (; i < n_words; i += (unsigned long long)gridDim.x * PTB) a.words[i] = 0u;
       return;
     }
   }

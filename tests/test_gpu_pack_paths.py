@@ -83,3 +83,22 @@ def test_both_packers_agree_where_the_reciprocal_scale_overflows(B, kind):
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     if kind == "E4M3":
         assert int(((out[0][0] & 0x7F) == 0x7F).sum()) == 0           # no code that is not a number
+
+
+@pytest.mark.parametrize("b", [8, 12, 16])
+def test_both_packers_leave_the_same_words_where_there_is_no_pair(B, b):
+    # a result without a pair: nothing is packed, a 12-bit stream is cleared, else its last 32 bits
+    M, K = 37, 272
+    fmt, atoms, NB = I.scale_format("UE4M3"), I.alphabet(["NF4", "SH4"]), M * K // 16
+    W, cd, res = I.tiny_layer(63, M, K).W.to(dev()), torch.ones(K, device=dev()), B.new_result(dev())
+    B.sop_pair_search(W, cd, fmt, atoms, B.new_pair_table(4, dev()), None, res, B.alloc_workspace(B.pair_search_workspace(M, K, 4), dev()),
+                      singles_only=True, block_cos=torch.empty((4, NB), device=dev()), block_sse=torch.empty((4, NB), device=dev()))
+    n, out = B.words_nbytes(NB, b), []
+    for metric in (torch.zeros((4, NB), device=dev()), None):
+        codes, words = torch.full((NB * 8,), 0x5A, dtype=torch.uint8, device=dev()), torch.full((n + 64,), 0x5A, dtype=torch.uint8, device=dev())
+        counts = torch.zeros(2, dtype=torch.int64, device=dev())
+        B.sop_pack(W, cd, fmt, atoms, codes, words, search_result=res, container_bits=b, counts=counts, block_cos=metric)
+        assert counts.tolist() == [-1, -1] and bool((codes == 0x5A).all())
+        out.append(words)
+    assert torch.equal(out[0], out[1])
+    assert int((out[0] == 0).sum()) == (n if b == 12 else 4) and bool((out[0][n:] == 0x5A).all())
