@@ -219,11 +219,9 @@ __global__ void __launch_bounds__(STB) opq_mask_kernel(OpqArgs a) {
     if (lane == 0) s_cnt[par][warp] = cnt;
     __syncthreads();
     const unsigned other = lane < STB / 32 ? s_cnt[par][lane] : 0u;
-    if (warp == 0) {
-      const unsigned sum = __reduce_add_sync(0xFFFFFFFFu, other);
-      if (lane == 0) a.tile_sums[tile] = sum;
-    }
-    if (cnt) {
+    const unsigned sum = __reduce_add_sync(0xFFFFFFFFu, other);
+    if (tid == 0) a.tile_sums[tile] = sum;
+    if (cnt && sum <= OPQ_LOCAL) {
       unsigned incl = mine;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -234,7 +232,7 @@ __global__ void __launch_bounds__(STB) opq_mask_kernel(OpqArgs a) {
       const uint16_t* p = a.W + (long long)cm * a.ldw + (long long)cj * SOP_G;
       for (unsigned rest = mask; rest; rest &= rest - 1u, ++pos) {
         const int i = __ffs((int)rest) - 1;
-        if (pos < OPQ_LOCAL) a.local[(size_t)tile * OPQ_LOCAL + pos] = (cj * SOP_G + (unsigned)i) | ((unsigned)p[i] << 16);
+        a.local[(size_t)tile * OPQ_LOCAL + pos] = (cj * SOP_G + (unsigned)i) | ((unsigned)p[i] << 16);
       }
     }
   }
@@ -251,15 +249,36 @@ __global__ void __launch_bounds__(STB) opq_write_kernel(OpqArgs a) {
   for (unsigned tile = blockIdx.x * (STB / 32) + (tid >> 5); tile < n_tiles; tile += gridDim.x * (STB / 32)) {
     const unsigned base = a.tile_sums[tile];
     const unsigned cnt = (tile + 1 < n_tiles ? a.tile_sums[tile + 1] : a.row_start[a.M]) - base;
-    const bool local = cnt <= OPQ_LOCAL;
-    if (local) {
-      const unsigned* from = a.local + (size_t)tile * OPQ_LOCAL;
-      for (unsigned i = lane; i < cnt; i += 32)
-        if ((long long)base + i < a.capacity) a.records[base + i] = from[i];
+    const unsigned t0 = tile * STB;
+    if (cnt > OPQ_LOCAL) {
+      // the tile's records did not fit their share: from the masks and W, 32 neighbouring blocks at a time
+      unsigned run = base;
+      for (unsigned blk = t0 + lane; blk < t0 + STB; blk += 32) {
+        const unsigned mask = blk < NB ? (unsigned)a.masks[blk] : 0u, m = blk / nbk, j = blk - m * nbk;
+        const unsigned mine = (unsigned)__popc(mask);
+        unsigned incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+          if (lane >= o) incl += t;
+        }
+        unsigned pos = run + incl - mine;
+        run += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        if (blk < NB && j == 0) a.row_start[m] = pos;
+        const uint16_t* p = a.W + (long long)m * a.ldw + (long long)j * SOP_G;
+        for (unsigned rest = mask; rest; rest &= rest - 1u, ++pos) {
+          const int i = __ffs((int)rest) - 1;
+          if ((long long)pos < a.capacity) a.records[pos] = (j * SOP_G + (unsigned)i) | ((unsigned)p[i] << 16);
+        }
+      }
+      continue;
     }
-    const unsigned t0 = tile * STB, jt = t0 % nbk;
+    const unsigned* from = a.local + (size_t)tile * OPQ_LOCAL;
+    for (unsigned i = lane; i < cnt; i += 32)
+      if ((long long)base + i < a.capacity) a.records[base + i] = from[i];
+    const unsigned jt = t0 % nbk;
     if (jt == 0 && lane == 0) a.row_start[t0 / nbk] = base;
-    if (local && jt + min((unsigned)STB, NB - t0) <= nbk) continue;          // no other row starts here
+    if (jt + min((unsigned)STB, NB - t0) <= nbk) continue;          // no other row starts here
     const unsigned b0 = t0 + 8 * lane;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
     if (b0 < NB) v = *reinterpret_cast<const uint4*>(a.masks + b0);      // the array is padded to 256 bytes
@@ -281,16 +300,7 @@ __global__ void __launch_bounds__(STB) opq_write_kernel(OpqArgs a) {
     for (int e = 0; e < 8; ++e) {
       if ((unsigned)e < n_here) {
         if (j == 0) a.row_start[m] = pos;
-        const unsigned mask = (u[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
-        if (local) pos += (unsigned)__popc(mask);
-        else {
-          const uint16_t* p = a.W + (long long)m * a.ldw + (long long)j * SOP_G;
-          for (unsigned rest = mask; rest; rest &= rest - 1u) {
-            const int i = __ffs((int)rest) - 1;
-            if ((long long)pos < a.capacity) a.records[pos] = (j * SOP_G + (unsigned)i) | ((unsigned)p[i] << 16);
-            ++pos;
-          }
-        }
+        pos += (unsigned)__popc((u[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
         if (++j == nbk) { j = 0; ++m; }
       }
     }
