@@ -36,3 +36,15 @@ def test_the_fast_cosine_is_the_rounded_quotient_by_the_rounded_root():
     for x in xs:
         bad = _run(lib.check_cosine, C.c_uint(int(x)), C.c_uint(1), C.c_void_p(every.data_ptr()), every.numel())
         assert bad[0] == 0, (hex(int(x)), bad)
+
+
+@pytest.mark.parametrize("exponent", [4, 5, 126, 127, 128, 249, 250])
+def test_the_reciprocal_of_a_scale_is_rounded_to_nearest(exponent):
+    # every significand; 4 .. 250 are the exponent fields that the sweep and the packer take this path for
+    assert _run(device_checks.lib().check_reciprocal, C.c_uint(exponent))[0] == 0
+
+
+@pytest.mark.parametrize("kind", [1, 2])
+def test_the_conversion_instructions_quantise_and_encode_like_the_arithmetic(kind):
+    # every finite fp32 pattern, in both places of the pair
+    assert _run(device_checks.lib().check_quantize, C.c_int(kind))[:2] == [0, 0]
