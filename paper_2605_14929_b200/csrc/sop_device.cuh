@@ -272,17 +272,12 @@ __device__ __forceinline__ uint32_t fp_code(float q) {
   return (sign << (xb + 3)) | mag;
 }
 
-// Decision thresholds of a table: tau[j] = largest fp32 <= (lut[j] + lut[j+1]) / 2, so that for
-// every fp32 u "u > tau[j]" is exactly "u is strictly closer to lut[j+1] than to lut[j]".  A repeated
-// entry takes the threshold above it, so its upper copy is never chosen.  tau[j] = +inf for j >= ne-1.
-__device__ __forceinline__ void build_thresholds(const float* lut, int ne, float* tau /* 32 */) {
-  float next = __int_as_float(0x7F800000);
-  for (int j = 31; j >= 0; --j) {
-    float t = __int_as_float(0x7F800000);
-    if (j < ne - 1) t = (lut[j] == lut[j + 1]) ? next : __double2float_rd(0.5 * ((double)lut[j] + (double)lut[j + 1]));
-    tau[j] = t;
-    next = t;
-  }
+// Decision threshold of a table above entry j: the largest fp32 <= (lut[j] + lut[j + 1]) / 2, so that for every fp32 u
+// "u > threshold" is exactly "u is strictly closer to lut[j + 1] than to lut[j]".  A repeated entry takes the threshold above
+// it, so its upper copy is never chosen.  +inf from the last of ne entries on.
+__device__ __forceinline__ float table_threshold(const float* lut, int j, int ne) {
+  while (j < ne - 1 && lut[j] == lut[j + 1]) ++j;
+  return j < ne - 1 ? __double2float_rd(0.5 * ((double)lut[j] + (double)lut[j + 1])) : __int_as_float(0x7F800000);
 }
 
 // number of thresholds strictly below u: branch-free binary search over 2^STEPS - 1 sorted entries (+inf

@@ -703,15 +703,12 @@ __device__ void split_cells(IterSmem& S) {
 }
 
 // One warp: the descriptor of a table (entry j of the sorted table, padded with its last value, in lane j): the decision
-// thresholds (the same rule as build_thresholds: the largest fp32 <= the midpoint, a repeated entry takes the threshold above
-// it, +inf from n_entries - 1 on) and their lookup cells.  sort_cell is monotone, so an element in a lower cell than a
+// thresholds and their lookup cells.  sort_cell is monotone, so an element in a lower cell than a
 // threshold's is below the threshold and one in a higher cell is above it: only the elements of the cells listed here need the
 // comparison itself.
 __device__ void make_desc(IterDesc* d, const float* table, int ne) {
   const int j = threadIdx.x & 31;
-  int jj = j;
-  while (jj < ne - 1 && table[jj] == table[jj + 1]) ++jj;
-  const float t = jj < ne - 1 ? __double2float_rd(0.5 * ((double)table[jj] + (double)table[jj + 1])) : __int_as_float(0x7F800000);
+  const float t = table_threshold(table, j, ne);
   d->lut[j] = table[j];
   d->tau[j] = t;
   d->thr_cell[j] = j < ne - 1 ? sort_cell(t) : SORT_ROWS;

@@ -3,8 +3,7 @@
 // encoded: 2n bytes of codes plus one b-bit scale word (sign, exponent, mantissa, selector).  Reads W once,
 // writes ~n/8 + b/128 bytes per element; bound by instruction issue (the encode), not by bytes.  Table codes
 // come from a uniform cell grid on u where the table allows it, else from a binary search over the thresholds.
-// pack_winner_kernel serves winners whose cosines or errors a sweep has written (tables, E2M3, E4M3);
-// pack_kernel serves parametric grids and choices that have to be evaluated here.
+// pack_winner_kernel serves choices whose cosines or errors a sweep has written; pack_kernel evaluates the candidates itself.
 #include <string.h>
 
 #include "sop_device.cuh"
@@ -37,7 +36,7 @@ struct PackCand { int table; int kind; int neg; int scope; int k; float tmax; Gr
 
 // One candidate on one block, everything in registers; same operation order as the sweep kernel.
 // The 16 codes come back as bytes, four per word (element i in byte i % 4 of word i / 4).
-// METRIC: 0 = codes only, 1 = also the block cosine, 2 = also the block squared error (in cos_out).
+// METRIC: 1 = with the block cosine, 2 = with the block squared error (in cos_out).
 template <int METRIC, int KIND>
 __device__ __forceinline__ void eval_block_kind(const float (&w)[16], const float (&c)[16], const float* tau,
                                                 const float* lutv, int neg, float rcp, float s_hat,
@@ -82,7 +81,7 @@ __device__ __forceinline__ void eval_block_kind(const float (&w)[16], const floa
         aw = __fmaf_rn(cw, w[i], aw);
         ad = __fmaf_rn(cq, w[i], ad);
         an = __fmaf_rn(cq, q, an);
-      } else if (METRIC == 2) {
+      } else {
         const float e = __fmaf_rn(-s_hat, q, w[i]);     // w - s q with one rounding, as the sweep forms it
         an = __fmaf_rn(e, e, an);
       }
@@ -90,7 +89,7 @@ __device__ __forceinline__ void eval_block_kind(const float (&w)[16], const floa
     qn[h] = an; qd[h] = ad; qw[h] = aw;
     code4[h] = packed;
   }
-  cos_out = METRIC == 1 ? block_cosine(quad_tree(qw), quad_tree(qn), quad_tree(qd)) : (METRIC == 2 ? quad_tree(qn) : 0.0f);
+  cos_out = METRIC == 1 ? block_cosine(quad_tree(qw), quad_tree(qn), quad_tree(qd)) : quad_tree(qn);
 }
 
 // the quantiser kind is decided once per block, outside the element loops: a kind test inside them lets
@@ -108,10 +107,8 @@ __device__ __forceinline__ void eval_block_regs(const float (&w)[16], const floa
   else eval_block_kind<METRIC, SOP_KIND_FP_E4M3>(w, c, tau, lutv, neg, rcp, s_hat, cos_out, code4);
 }
 
-// USE_COS: the winner of each block is read off the per-block cosines of a sweep and only it is encoded
-// (no channel norms needed); otherwise every candidate of the choice is evaluated here.
-template <bool USE_COS>
-__global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* res) {
+// Every candidate of the choice is evaluated here.
+__global__ void __launch_bounds__(PTB, 1) pack_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* res) {
   pdl_trigger();
   pdl_wait();
   __shared__ float lutv[2][32], tau[2][32];
@@ -120,7 +117,6 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
   __shared__ int s_nb, s_nbits;
   __shared__ float s_pot[2];
   __shared__ unsigned s_cnt[2];
-  __shared__ int s_row[4];   // rows of block_cos for the candidates a, -a, b, -b (-1: none)
   __shared__ int s_idx[2];   // the two atoms
   __shared__ int s_no_pair;  // the search result holds no pair to pack
   const int tid = threadIdx.x;
@@ -153,11 +149,6 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
       s_pot[t] = at.scope == 0 ? layer_pot_scale(wmax, at.tmax) : 0.0f;
       s_idx[t] = idx;
     }
-    // from a search result with signs, a and b are base atoms and each is followed by its negation
-    s_row[0] = ia;
-    s_row[1] = from_result ? ia + 1 : a.cos_neg_a;
-    s_row[2] = nb == 2 ? ib : -1;
-    s_row[3] = nb == 2 ? (from_result ? ib + 1 : a.cos_neg_b) : -1;
     s_cnt[0] = s_cnt[1] = 0;
   }
   __syncthreads();
@@ -166,8 +157,7 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
     return;
   }
   const int nb = s_nb, n = s_nbits, b = a.container_bits;
-  // table values and decision thresholds of the (up to two) tables: one thread per entry (the same rule as
-  // build_thresholds: the largest fp32 <= the midpoint, a repeated entry takes the threshold above it)
+  // table values and decision thresholds of the (up to two) tables: one thread per entry
   if (tid < 32 * nb) {
     const int t = tid >> 5, j = tid & 31, idx = s_idx[t];
     const sop_atom& at = A.atoms[idx];
@@ -175,9 +165,7 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
     const int ne = at.kind == SOP_KIND_LUT ? at.n_entries : 2;
     lutv[t][j] = at.kind == SOP_KIND_LUT ? (dd ? A.dd_lut[min(j, ne - 1)] : at.lut[min(j, ne - 1)]) : 0.0f;
     __syncwarp();
-    int jj = j;
-    while (jj < ne - 1 && lutv[t][jj] == lutv[t][jj + 1]) ++jj;
-    tau[t][j] = jj < ne - 1 ? __double2float_rd(0.5 * ((double)lutv[t][jj] + (double)lutv[t][jj + 1])) : __int_as_float(0x7F800000);
+    tau[t][j] = table_threshold(lutv[t], j, ne);
   }
   __syncthreads();
   // Cell grids of the tables.  A grid of width h <= (smallest gap between two thresholds) / 2 puts at most one threshold
@@ -236,44 +224,28 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
   const int n_sign = a.use_sign ? 2 : 1;
   unsigned my_sel = 0, my_neg = 0;
   const unsigned nbk32 = (unsigned)a.nbk, NB32 = (unsigned)a.NB;       // the block count fits 31 bits
-  const int n_cand = nb * n_sign;
-  // the loads of a block (its weights and, when the winner is read off a sweep, the candidates' values) are
-  // issued one iteration ahead
-  auto fetch = [&](unsigned blk, uint4& v0, uint4& v1, float (&cs4)[4]) {
+  // the weights of a block are loaded one iteration ahead
+  auto fetch = [&](unsigned blk, uint4& v0, uint4& v1) {
     const unsigned m = blk / nbk32, j = blk - m * nbk32;
     const uint4* p = reinterpret_cast<const uint4*>(a.W + (long long)m * a.ldw + (long long)j * SOP_G);
     v0 = *p; v1 = p[1];
-    if (USE_COS) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int slot = n_sign == 2 ? q : 2 * q;          // candidate q of the order a, (-a), b, (-b)
-        cs4[q] = q < n_cand ? a.block_cos[(size_t)s_row[slot] * a.NB + blk] : 0.0f;
-      }
-    }
   };
   const unsigned stride = gridDim.x * PTB;
   uint4 nv0 = make_uint4(0u, 0u, 0u, 0u), nv1 = nv0;
-  float ncs4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  if (blockIdx.x * PTB + tid < NB32) fetch(blockIdx.x * PTB + tid, nv0, nv1, ncs4);
+  if (blockIdx.x * PTB + tid < NB32) fetch(blockIdx.x * PTB + tid, nv0, nv1);
   for (unsigned blk = blockIdx.x * PTB + tid; blk < NB32; blk += stride) {
     const unsigned j = blk % nbk32;
     const uint4 v0 = nv0, v1 = nv1;
-    float cs4[4] = {ncs4[0], ncs4[1], ncs4[2], ncs4[3]};
-    if (blk + stride < NB32) fetch(blk + stride, nv0, nv1, ncs4);
+    if (blk + stride < NB32) fetch(blk + stride, nv0, nv1);
     const uint32_t wb[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
     float w[16], c[16];
 #pragma unroll
     for (int i = 0; i < 8; ++i) { w[2 * i] = bf16lo(wb[i]); w[2 * i + 1] = bf16hi(wb[i]); }
-    if (USE_COS) {
+    const float4* cp = reinterpret_cast<const float4*>(a.c + j * SOP_G);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) c[i] = 0.0f;
-    } else {
-      const float4* cp = reinterpret_cast<const float4*>(a.c + j * SOP_G);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 v = cp[q];
-        c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
-      }
+    for (int q = 0; q < 4; ++q) {
+      const float4 v = cp[q];
+      c[4 * q] = v.x; c[4 * q + 1] = v.y; c[4 * q + 2] = v.z; c[4 * q + 3] = v.w;
     }
     // bf16 magnitudes order like their bit patterns: the maximum of the sixteen 15-bit patterns, two per word at a time
     uint32_t mb = 0;
@@ -284,53 +256,28 @@ __global__ void __launch_bounds__(PTB, USE_COS ? 4 : 1) pack_kernel(PackArgs a, 
     float best_cos = 0.0f;
     uint32_t best_scode = 0, best4[4] = {0u, 0u, 0u, 0u};
     int pick = -1;
-    if (USE_COS) {
-      // the winner follows from the cosines of the sweep (same arithmetic, bit for bit): only it is encoded
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q >= n_cand) break;
-        const float cs = cs4[q];
-        const int slot = n_sign == 2 ? q : 2 * q;
-        if (pick < 0 || (a.select_err ? cs < best_cos : cs > best_cos)) { best_cos = cs; pick = slot; }
-      }
-      const int t = pick >> 1, sg = pick & 1;
+    for (int t = 0; t < nb; ++t) {
       const PackCand cd = base[t];
       float s_hat;
+      uint32_t sc = 0;
       if (cd.scope == 0) {
         s_hat = amax > 0.0f ? s_pot[t] : 0.0f;
       } else {
         const float sigma = cd.tmax == 1.0f ? amax : __fdiv_rn(amax, cd.tmax);
         const QScale qs = scale_quantize(sigma, cd.k, F);
         s_hat = qs.s_hat;
-        best_scode = qs.code;
+        sc = qs.code;
       }
       const float rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
-      float unused;
-      eval_block_regs<0>(w, c, tau[t], lutv[t], cd.kind, sg ? 1 - cd.neg : cd.neg, rcp, s_hat, unused, best4, cd.grid, cd.sign_pos, cells[t], cd.invh, cd.c_half);
-    } else {
-      for (int t = 0; t < nb; ++t) {
-        const PackCand cd = base[t];
-        float s_hat;
-        uint32_t sc = 0;
-        if (cd.scope == 0) {
-          s_hat = amax > 0.0f ? s_pot[t] : 0.0f;
-        } else {
-          const float sigma = cd.tmax == 1.0f ? amax : __fdiv_rn(amax, cd.tmax);
-          const QScale qs = scale_quantize(sigma, cd.k, F);
-          s_hat = qs.s_hat;
-          sc = qs.code;
-        }
-        const float rcp = s_hat > 0.0f ? __frcp_rn(s_hat) : 0.0f;
-        for (int sg = 0; sg < n_sign; ++sg) {
-          float cs;
-          uint32_t c4[4];
-          if (a.select_err) eval_block_regs<2>(w, c, tau[t], lutv[t], cd.kind, sg ? 1 - cd.neg : cd.neg, rcp, s_hat, cs, c4, cd.grid, cd.sign_pos, cells[t], cd.invh, cd.c_half);
-          else eval_block_regs<1>(w, c, tau[t], lutv[t], cd.kind, sg ? 1 - cd.neg : cd.neg, rcp, s_hat, cs, c4, cd.grid, cd.sign_pos, cells[t], cd.invh, cd.c_half);
-          if (pick < 0 || (a.select_err ? cs < best_cos : cs > best_cos)) {
-            best_cos = cs; best_scode = sc; pick = 2 * t + sg;
+      for (int sg = 0; sg < n_sign; ++sg) {
+        float cs;
+        uint32_t c4[4];
+        if (a.select_err) eval_block_regs<2>(w, c, tau[t], lutv[t], cd.kind, sg ? 1 - cd.neg : cd.neg, rcp, s_hat, cs, c4, cd.grid, cd.sign_pos, cells[t], cd.invh, cd.c_half);
+        else eval_block_regs<1>(w, c, tau[t], lutv[t], cd.kind, sg ? 1 - cd.neg : cd.neg, rcp, s_hat, cs, c4, cd.grid, cd.sign_pos, cells[t], cd.invh, cd.c_half);
+        if (pick < 0 || (a.select_err ? cs < best_cos : cs > best_cos)) {
+          best_cos = cs; best_scode = sc; pick = 2 * t + sg;
 #pragma unroll
-            for (int h = 0; h < 4; ++h) best4[h] = c4[h];
-          }
+          for (int h = 0; h < 4; ++h) best4[h] = c4[h];
         }
       }
     }
@@ -418,7 +365,7 @@ __device__ __forceinline__ unsigned pack_cell(float u, float inv_range) {
   return __float_as_uint(__fmaf_rn(__saturatef(__fmaf_rn(u, inv_range, 0.5f)), (float)PCELLS, PMAGIC));      // cell number + bits of PMAGIC
 }
 
-// KIND: SOP_KIND_LUT (any pair or single table), SOP_KIND_FP_E2M3 or SOP_KIND_FP_E4M3 (a single format).  N: bits of a code (0: as the
+// KIND: SOP_KIND_LUT (any pair or single table), SOP_KIND_FP_E2M3, SOP_KIND_FP_E4M3 or SOP_KIND_FP_GRID (a single format).  N: bits of a code (0: as the
 // atom says).  NC: candidates of the choice, 1, 2 (a pair, or a table and its negation) or 4.
 template <int KIND, int N, int NC>
 __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDev A, FmtDev F, const sop_search_result* res) {
@@ -476,10 +423,7 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
       const int t = tid >> 5, j = tid & 31, idx = s_idx[t], ne = A.atoms[idx].n_entries;
       lutv[t][j] = ((A.dd_mask >> idx) & 1u) ? A.dd_lut[min(j, ne - 1)] : A.atoms[idx].lut[min(j, ne - 1)];
       __syncwarp();
-      // decision thresholds (the rule of build_thresholds)
-      int jj = j;
-      while (jj < ne - 1 && lutv[t][jj] == lutv[t][jj + 1]) ++jj;
-      const float x = jj < ne - 1 ? __double2float_rd(0.5 * ((double)lutv[t][jj] + (double)lutv[t][jj + 1])) : __int_as_float(0x7F800000);
+      const float x = table_threshold(lutv[t], j, ne);
       tau[t][j] = x;
       const unsigned c = x < __int_as_float(0x7F800000) ? pack_cell(x, tab[t].inv_range) - __float_as_uint(PMAGIC) : 0xFFFFu;
       tcell[t][j] = (unsigned short)c;
@@ -504,6 +448,13 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
   const bool signs = NC == 4 || (NC == 2 && a.use_sign);      // the candidates are a table and its negation, once or twice
   const unsigned nbk = (unsigned)a.nbk, NB = (unsigned)a.NB;       // the block count fits 31 bits
   const bool packed_rows = a.ldw == a.K;
+  GridDev grid = {};
+  int sign_pos = 0;
+  if (KIND == SOP_KIND_FP_GRID) {
+    const sop_atom& at = A.atoms[ia];
+    grid.min_eb = 128 - at.grid_bias; grid.sh = 23 - at.grid_man_bits; grid.vpos = at.tmax; grid.vneg = at.grid_neg_max;
+    sign_pos = at.grid_exp_bits + at.grid_man_bits;
+  }
   const unsigned flip = a.select_err ? 0x80000000u : 0u;      // errors are compared as their negatives
   const float* row[NC];
 #pragma unroll
@@ -596,12 +547,24 @@ __global__ void __launch_bounds__(PTB, 4) pack_winner_kernel(PackArgs a, AtomsDe
           }
         }
       }
+    } else if (KIND == SOP_KIND_FP_GRID) {
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        code4[h] = 0;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int i = 4 * h + x;
+          const float u = __fmul_rn((i & 1) ? bf16hi(wb[i >> 1]) : bf16lo(wb[i >> 1]), rcp);
+          code4[h] |= grid_code(grid_quantize(u, grid), grid, sign_pos) << (8 * x);      // at most 8 bits: the host refuses wider grids here
+        }
+      }
     } else {
+      constexpr int FORMAT = KIND == SOP_KIND_FP_E4M3 ? SOP_KIND_FP_E4M3 : SOP_KIND_FP_E2M3;
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
         uint32_t lo2, hi2;
-        fp_quantize2<KIND == SOP_KIND_LUT ? SOP_KIND_FP_E2M3 : KIND>(__fmul_rn(bf16lo(wb[2 * h]), rcp), __fmul_rn(bf16hi(wb[2 * h]), rcp), lo2);
-        fp_quantize2<KIND == SOP_KIND_LUT ? SOP_KIND_FP_E2M3 : KIND>(__fmul_rn(bf16lo(wb[2 * h + 1]), rcp), __fmul_rn(bf16hi(wb[2 * h + 1]), rcp), hi2);
+        fp_quantize2<FORMAT>(__fmul_rn(bf16lo(wb[2 * h]), rcp), __fmul_rn(bf16hi(wb[2 * h]), rcp), lo2);
+        fp_quantize2<FORMAT>(__fmul_rn(bf16lo(wb[2 * h + 1]), rcp), __fmul_rn(bf16hi(wb[2 * h + 1]), rcp), hi2);
         code4[h] = lo2 | (hi2 << 16);
       }
     }
@@ -784,7 +747,7 @@ int sop_pack(const void* W_dev, long long M, long long K, long long ldw, const f
   const size_t padded = (word_bytes + 3) & ~(size_t)3;
   const bool negs_known = !use_sign || from_result || (a.cos_neg_a >= 0 && (!pair || a.cos_neg_b >= 0));
   const int kind = from_result ? SOP_KIND_LUT : atoms[index_a].kind;
-  const bool winner = block_cos_dev && negs_known && kind != SOP_KIND_FP_GRID;       // (pack_winner_kernel writes whole words)
+  const bool winner = block_cos_dev && negs_known;       // (pack_winner_kernel writes whole words)
   if (winner) {}
   else if (container_bits == 12) SOP_CUDA_TRY(cudaMemsetAsync(words_dev, 0, padded, st));
   else SOP_CUDA_TRY(cudaMemsetAsync(words_dev + padded - 4, 0, 4, st));
@@ -799,13 +762,13 @@ int sop_pack(const void* W_dev, long long M, long long K, long long ldw, const f
   const int n_cand = (pair ? 2 : 1) * (use_sign ? 2 : 1);
   if (winner && kind == SOP_KIND_FP_E2M3) SOP_PACK(SOP_KIND_FP_E2M3, 6, 1);
   else if (winner && kind == SOP_KIND_FP_E4M3) SOP_PACK(SOP_KIND_FP_E4M3, 8, 1);
+  else if (winner && kind == SOP_KIND_FP_GRID) SOP_PACK(SOP_KIND_FP_GRID, 0, 1);
   else if (winner && n_bits == 4) SOP_PACK_LUT(4);
   else if (winner && n_bits == 5) SOP_PACK_LUT(5);
   else if (winner) SOP_PACK_LUT(0);
 #undef SOP_PACK_LUT
 #undef SOP_PACK
-  else if (block_cos_dev && negs_known) SOP_CUDA_TRY(launch(pack_kernel<true>, grid, PTB, 0, st, a, A, F, search_dev));
-  else SOP_CUDA_TRY(launch(pack_kernel<false>, grid, PTB, 0, st, a, A, F, search_dev));
+  else SOP_CUDA_TRY(launch(pack_kernel, grid, PTB, 0, st, a, A, F, search_dev));
   if ((rc = profile_mark(SOP_PROFILE_PACK, 1, st))) return rc;
   SOP_CUDA_TRY(cudaGetLastError());
   return SOP_OK;

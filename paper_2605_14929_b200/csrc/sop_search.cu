@@ -384,13 +384,9 @@ __device__ void build_group(const Plan& P, const AtomsDev& A, int g, unsigned ch
     const int jj = min(j, ne - 1);
     const float v = lut[neg ? ne - 1 - jj : jj];
     S.vals[q][j] = neg ? -v : v;
-    // threshold of the table below entry t (the rule of build_thresholds: the largest fp32 <= the midpoint, a repeated
-    // entry takes the threshold above it, +inf from the last entry on)
     float x = __int_as_float(0x7F800000);
     if (j < ne - 1) {
-      int t = neg ? ne - 2 - j : j;
-      while (t < ne - 1 && lut[t] == lut[t + 1]) ++t;
-      if (t < ne - 1) x = __double2float_rd(0.5 * ((double)lut[t] + (double)lut[t + 1]));
+      x = table_threshold(lut, neg ? ne - 2 - j : j, ne);
       if (neg) {
         const float y = -x;
         const unsigned b = __float_as_uint(y);

@@ -102,3 +102,20 @@ def test_both_packers_leave_the_same_words_where_there_is_no_pair(B, b):
         out.append(words)
     assert torch.equal(out[0], out[1])
     assert int((out[0] == 0).sum()) == (n if b == 12 else 4) and bool((out[0][n:] == 0x5A).all())
+
+
+@pytest.mark.parametrize("M,K", [(1, 16), (5, 112), (37, 272)])
+@pytest.mark.parametrize("grid", [(3, 4, 3, 15.5), (2, 3, 1, 7.5), (2, 2, 1, 7.0), (3, 3, 3, 30.0)])      # 8, 6, 5 and 7 bits
+def test_parametric_grids_in_both_packers(B, M, K, grid):
+    x, y, bias, top = grid
+    atoms, fmt, NB, n = [I.Atom("grid", 1 + x + y, I.KIND_FP_GRID, 0, 16, top, None, (x, y, bias, top))], I.scale_format("UE4M4"), M * K // 16, 1 + x + y
+    W, cd, res = I.tiny_layer(64, M, K).W.to(dev()), torch.ones(K, device=dev()), B.new_result(dev())
+    bc, bs = torch.empty((1, NB), device=dev()), torch.empty((1, NB), device=dev())
+    B.sop_pair_search(W, cd, fmt, atoms, B.new_pair_table(1, dev()), None, res, B.alloc_workspace(B.pair_search_workspace(M, K, 1), dev()),
+                      block_cos=bc, block_sse=bs)
+    out = []
+    for metric in (bc, None):
+        codes, words = torch.full((NB * 2 * n + 64,), 0x5A, dtype=torch.uint8, device=dev()), torch.full((B.words_nbytes(NB, 12) + 64,), 0x5A, dtype=torch.uint8, device=dev())
+        B.sop_pack(W, cd, fmt, atoms, codes, words, index_a=0, index_b=B.NO_ATOM, search_result=res, container_bits=12, block_cos=metric)
+        out.append((codes, words))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
