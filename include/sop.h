@@ -292,7 +292,7 @@ int sop_dd4_lloyd_launches(long long M, long long K, int iters, int flags, int* 
  * not depend on them).  cell_spill_tiles in [1, 128]: cache tiles a CTA sorts between two transfers of its
  * per-cell partial sums to the global sums (default 128);
  * cache_ctas >= 0: largest grid of the cache kernel (0 = default, two CTAs per SM);
- * tiles_per_warp in [1, 4]: accepted, without effect;
+ * tiles_per_warp in [1, 4]: reserved (accepted, nothing depends on it);
  * iter_ctas >= 0: largest grid of the iteration kernels (0 = default: a CTA per four cache tiles of the expected pool,
  *   at most one per SM).
  * SOP_ERR_RANGE outside these ranges. */

@@ -44,8 +44,8 @@ int num_sms();
 int profile_mark(int which, int edge, cudaStream_t st);
 
 // ---- launches ------------------------------------------------------------------------------
-// Every kernel of the library is launched so that it may start while the one before it on the stream still runs (programmatic
-// dependent launch): a pass is a chain of twenty short kernels, and the time from the end of one to the start of the next was a
+// Every kernel of the library but one is launched so that it may start while the one before it on the stream still runs (programmatic
+// dependent launch); the Lloyd iterations, whose CTAs wait for one another, are launched cooperatively instead and start in their turn.  A pass is a chain of twenty short kernels, and the time from the end of one to the start of the next was a
 // sixth of a small layer's pass.  Rules that each kernel keeps: pdl_trigger() first (its successor may then be scheduled as its CTAs
 // leave), and pdl_wait() -- which returns when the kernels before it have completed and their writes are visible -- before the
 // first access to global memory; only what depends on the parameters alone comes before the wait.  Global memory is read by plain

@@ -370,7 +370,7 @@ __device__ __forceinline__ long long fix24(float v) {   // llrint(v * 2^24): exa
 }
 
 constexpr int CELL_SPILL_TILES_MAX = 128;     // cache tiles a CTA sorts between two transfers of its per-cell sums to the global ones (any number is safe)
-constexpr int TILES_PER_WARP_MAX = 4;         // range of a tuning argument that has no effect any more
+constexpr int TILES_PER_WARP_MAX = 4;         // range of a reserved tuning argument
 
 // Launch-shape parameters of the pool cache and of the iteration grid; sop_dd4_lloyd_tuning lowers them (tests reach the
 // mid-loop transfer and CTAs with many tiles on small layers that way).  Results do not depend on them.

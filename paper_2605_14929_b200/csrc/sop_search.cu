@@ -617,8 +617,8 @@ __device__ __forceinline__ void sweep_emit(float nw, float2 (&nq)[NP], float2 (&
 }
 
 // The candidates of one group on every block of the thread: first the rows of its sixteen elements (kept as 16-bit offsets),
-// then the metrics of two pairs of candidates at a time -- the sums of all eight at once would take more registers than leave
-// enough warps resident.
+// then the metrics of two pairs of candidates at a time -- the sums of all eight at once do not fit the 128 registers that a thread
+// of 512 has.
 //   KT: decision points per cell that are compared (0: the group is searched).
 template <int NP, int KT>
 __device__ __forceinline__ void sweep_group(const SweepCtx& X, const FmtDev& F, const GroupDev& G, const float* merged, const ColumnPtr* cols) {
@@ -1583,7 +1583,7 @@ static size_t reduce_smem_bytes(int n_cols, int units, int n_stage) {
 }
 
 // Shared memory of the sweep: per group its rows (one more than its decision points) and its cells, 128 bytes per cell and
-// 128 or 256 per row with the copies; every group gets the same number of cells, the largest of 1280, 640, 320, ... that fits
+// 128 or 256 per row with the copies; every group gets the same number of cells, the largest of 640, 320, 160, ... that fits
 // `limit` bytes in all (a cell then rarely holds more than three decision points; a group where one does is searched instead).
 constexpr size_t SWEEP_C_BYTES = (size_t)TB * SOP_G * sizeof(float);
 static size_t sweep_layout(const AtomsDev& A, Plan* P, size_t limit) {

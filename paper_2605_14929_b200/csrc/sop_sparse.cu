@@ -1099,7 +1099,8 @@ int sop_wr_extract(const void* W_dev, long long M, long long K, long long ldw, c
   const long long fit = cap * STB / a.nbk;
   const unsigned rows = (unsigned)(fit < 1 ? 1 : fit < M ? fit : M);
   const int mgrid = (int)((rows * a.nbk + STB - 1) / STB);
-  // (a memset, not clear(): with the launch chain unbroken between the packer and the first decode pass 8192 x 8192 takes 1069 us instead of 1051)
+  // (a memset, not clear(), which ends the chain of early starts between the packer and the first decode pass: with clear() here a pass over
+  // 8192 x 8192 with both streams takes 1078 us instead of 1056, in three comparisons.  Why has not been established; elsewhere clear() wins.)
   SOP_CUDA_TRY(cudaMemsetAsync(ws, 0, sizeof(SparseWs), st));
   if ((rc = profile_mark(SOP_PROFILE_WR, 0, st))) return rc;
   // both codebooks tables of at most 16 entries: the decode with constant shifts (a pair taken from a search result is
