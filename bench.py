@@ -53,11 +53,13 @@ SM_COUNT, SCHEDULERS, LANES = 148, 4, 32
 # file (dram__bytes_read.sum + dram__bytes_write.sum of one launch on the 8192x8192 layer at E5M6 divided by its
 # elements; traffic grows in proportion to the elements, so a launch of the block is scaled by its elements).
 # None: no capture of the kernel as it is now.
-NCU_SWEEP_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=5.2154,
-                         bytes_per_element_dd_columns=2.5740)
+NCU_SWEEP_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=5.1928,
+                         bytes_per_element_dd_columns=2.5279)
+# thread instructions that the sweep kernel executes per weight element, from the same capture (warp instructions x 32)
+NCU_SWEEP_INSTR = dict(fixed_candidates=59.45, dd_columns=30.53)
 # the same for the reduction kernel (first call: the fixed candidates' entries; second call: the DD columns' entries)
-NCU_REDUCE_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=4.0624,
-                          bytes_per_element_dd_columns=5.0582)
+NCU_REDUCE_TRAFFIC = dict(source="profiles/kernels_config5_layer_8192x8192_E5M6.md", bytes_per_element_fixed_candidates=4.0097,
+                          bytes_per_element_dd_columns=5.0165)
 
 
 # ---------------------------------------------------------------------------------------------------------
@@ -547,7 +549,9 @@ def run_gpu(args) -> None:
         search_t = sweep_t + reduce_t
         # the evaluation kernel by itself: its own share of the operation count
         ops_sweep = sweep_kernel_ops_n_step(n_lut - n_dd, nb, 0) + sweep_kernel_ops_n_step(n_dd, nb, 0)
-        ach_sweep = ops_sweep * units / sweep_t / 1e12
+        ach_model = ops_sweep * units / sweep_t / 1e12
+        # what it executes: the bound that cannot be passed
+        ach_sweep = sum(NCU_SWEEP_INSTR.values()) * units / sweep_t / 1e12
         ach = ops_n_step * units / search_t / 1e12
         ach_cell = ops_cell * units / search_t / 1e12
         alg_bytes = search_bytes(n_lut, n_dd)
@@ -560,12 +564,15 @@ def run_gpu(args) -> None:
             frac=ach_sweep / alu_peak, traffic=traffic, traffic_source=NCU_SWEEP_TRAFFIC["source"],
             peak_source=f"{SM_COUNT} SMs x {SCHEDULERS} schedulers x {LANES} lanes x {sm_max:.0f} MHz (clocks.max.sm, {of})",
             avg_launch_ms=sweep_t * 1e3 / (2 * n_pass),
-            ops_per_element=dict(fixed_candidates=sweep_kernel_ops_n_step(n_lut - n_dd, nb, 0), dd_columns=sweep_kernel_ops_n_step(n_dd, nb, 0)),
+            executed_per_element=NCU_SWEEP_INSTR,
+            n_step_model=dict(ops_per_element=dict(fixed_candidates=sweep_kernel_ops_n_step(n_lut - n_dd, nb, 0), dd_columns=sweep_kernel_ops_n_step(n_dd, nb, 0)),
+                              achieved=ach_model, frac=ach_model / alu_peak,
+                              note="the kernel's share of the n-step operation count over the same time; the joint rows of the candidates need "
+                                   "fewer instructions than that model counts, so this fraction may pass 1"),
             algorithmic_bytes_per_launch=sweep_bytes / 2.0 * units / n_pass,
             note="the dominant kernel of the step: the evaluation of every candidate on every block (two launches per layer and "
-                 "format: the fixed candidates, then the DD columns), against its own share of the n-step operation count; the "
-                 "joint rows of the candidates need fewer instructions than that model counts (59 and 30 per element by ncu, at 61 "
-                 "and 68 % of the issue slots), so the fraction may pass 1; "
+                 "format: the fixed candidates, then the DD columns): the thread instructions that it executes per element (by ncu) "
+                 "over its time, against the issue peak; "
                  "`search` below is the whole search (evaluation + reduction of the table entries) against the whole count",
             search=dict(
                 kernels=["sweep_kernel", "reduce_kernel"], launches_per_step=4 * n_pass, ms_per_step=search_t * 1e3,
